@@ -216,6 +216,7 @@ PW_PLAN(48, 192, 16, 3)
 PW_PLAN(64, 256, 8, 8)
 PW_PLAN(96, 384, 8, 4, 3)
 PW_PLAN(128, 512, 16, 8)
+PW_PLAN(256, 256, 16, 16)  // single lines only (gsm3.cuh)
 #undef PW_PLAN
 
 template <int N, int I> struct StageInfo {

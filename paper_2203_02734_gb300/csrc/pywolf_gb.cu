@@ -20,6 +20,7 @@
 #include "dense_tc.cuh"
 #include "t256.cuh"
 #include "grad.cuh"
+#include "plane.cuh"
 #include "r128.cuh"
 #include "r96.cuh"
 
@@ -57,6 +58,7 @@ namespace pwi {
 // Sets the thread's message returned by pw_last_error() (used by other translation units).
 void set_last_error(const char* msg) { g_err = msg; }
 pw_status encode_vmap(CUtensorMap* map, void* work, int N);
+pw_status encode_wmap(CUtensorMap* map, void* W, int N);
 cudaError_t launch_batch_instance(int N, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
                                   const float2* Ein, const float2* mask, int ap_ithr, cudaStream_t s);
 }  // namespace pwi
@@ -105,6 +107,7 @@ struct pw_csd {
   CUtensorMap ymap;  // N = 256: the second pass's tiles of the work buffer
   CUtensorMap y3map;  // N = 256: the third pass's tiles of the work buffer
   CUtensorMap y1map;  // N = 256: the first pass's stores (four rows per warp) into the work buffer
+  CUtensorMap wmap;   // planes of W, at N = 256 its column tiles (plane.cuh)
   int dft_mode;      // PW_DFT_AUTO, PW_DFT_FP32 or PW_DFT_TC_BF16X3
   int Nz;            // zero padding: transform size (0 = none); the dense path runs when set
   void* qbuf;        // split DFT matrices of the tensor-core dense path (allocated on first use)
@@ -425,6 +428,98 @@ cudaError_t dispatch(int N, int src, bool herm, bool grad, const CUtensorMap& vm
   }
 }
 
+// Propagation of a GSM source plane by plane (plane.cuh).
+struct PlaneArgs {
+  const float2* F;
+  const float* G;
+  const float2* tw;
+  const float2* Eout;
+  float2* work;  // 2 N^3 table values
+  float2* W;
+  float* S;
+  float A, scale;
+  float2* row;  // W(P1, .) or nullptr
+  int iP, jP;
+};
+
+template <int N>
+cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
+  namespace P = pw::plane;
+  constexpr size_t N3 = (size_t)N * N * N;
+  static int grid = 0;  // of the plane kernel
+  cudaError_t e;
+  constexpr auto kernel = [] {
+    if constexpr (N == 96) return P::plane96_kernel;
+    else if constexpr (N == 128) return P::plane128_kernel;
+    else return P::plane_kernel<N>;
+  }();
+  constexpr int nt = N == 96 ? pw::r96::NT : N == 128 ? pw::r128::NT : pw::Plan<N>::NT;
+  constexpr size_t smem = N == 96 ? P::plane96_smem() : N == 128 ? P::plane128_smem() : P::plane_smem<N>();
+  if (grid == 0) {
+    if ((e = cudaFuncSetAttribute(P::table_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)P::tab_smem<N>())) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+        (e = persistent_grid(kernel, nt, smem, N * N, &grid)) != cudaSuccess)
+      return e;
+  }
+  if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
+  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, q.A};
+  P::table_kernel<N><<<dim3(N * (N / P::tab_lines<N>()), 2), P::tab_nt<N>(), P::tab_smem<N>(), s>>>(ta);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
+  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, q.row, q.iP, q.jP};
+  kernel<<<grid, nt, smem, s>>>(wmap, a);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+cudaError_t launch_planes256(const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s, cudaEvent_t* ev) {
+  namespace P = pw::plane;
+  constexpr int N = 256;
+  constexpr size_t N3 = (size_t)N * N * N;
+  static int grid = 0;  // of the column kernel
+  cudaError_t e;
+  if (grid == 0) {
+    if ((e = cudaFuncSetAttribute(P::table_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)P::tab_smem<N>())) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(P::rows256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)P::rows256_smem())) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(P::cols256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)P::cols256_smem())) != cudaSuccess ||
+        (e = persistent_grid(P::cols256_kernel, P::NT256, P::cols256_smem(), 1 << 30, &grid)) != cudaSuccess)
+      return e;
+  }
+  if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
+  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, q.A};
+  P::table_kernel<N><<<dim3(N * (N / P::tab_lines<N>()), 2), P::tab_nt<N>(), P::tab_smem<N>(), s>>>(ta);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, nullptr, 0, 0};
+  P::rows256_kernel<<<N * (N / 16) * (N / P::ROWS_C), P::NT256, P::rows256_smem(), s>>>(a);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
+  P::cols256_kernel<<<grid, P::NT256, P::cols256_smem(), s>>>(wmap, a, err);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s,
+                            cudaEvent_t* ev) {
+  switch (N) {
+#define PW_CASE(NN) \
+  case NN:          \
+    return launch_planes<NN>(wmap, q, s, ev);
+    PW_CASE(2) PW_CASE(4) PW_CASE(6) PW_CASE(8) PW_CASE(12) PW_CASE(16) PW_CASE(24)
+    PW_CASE(32) PW_CASE(48) PW_CASE(64) PW_CASE(96) PW_CASE(128)
+#undef PW_CASE
+    case 256:
+      return launch_planes256(wmap, q, err, s, ev);
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda).
 PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
@@ -474,6 +569,7 @@ pw_status make_t256_maps(pw_csd* h) {
 
 pw_status make_vmap(pw_csd* h) {
   pw_status st = pwi::encode_vmap(&h->vmap, h->work, h->N);
+  if (st == PW_OK) st = pwi::encode_wmap(&h->wmap, h->W, h->N);
   if (st == PW_OK && h->N == 256) st = make_t256_maps(h);
   return st;
 }
@@ -516,6 +612,18 @@ pw_status build_tables(pw_csd* h, double z, bool farfield) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "table kernel launch");
   return PW_OK;
+}
+
+// The output plane becomes the current plane: its CSDA is in W, its masks are unset.
+void to_output_plane(pw_csd* h, double dx, bool herm) {
+  h->d = dx;
+  h->kind = SRC_PROPAGATED;
+  h->hermitian = herm ? 1 : 0;
+  h->W0 = nullptr;
+  h->diag = nullptr;
+  h->aperture = 0.0;
+  h->lens_f = 0.0;
+  h->mask = nullptr;
 }
 
 bool has_masks(const pw_csd* h) { return h->aperture > 0.0 || h->lens_f != 0.0 || h->mask != nullptr; }
@@ -628,30 +736,20 @@ pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dense propagation launch");
   if (ev && (e = cudaEventRecord(ev[2], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
-  h->d = dx;
-  h->kind = SRC_PROPAGATED;
-  h->hermitian = herm ? 1 : 0;
-  h->W0 = nullptr;
-  h->diag = nullptr;
-  h->aperture = 0.0;
-  h->lens_f = 0.0;
-  h->mask = nullptr;
+  to_output_plane(h, dx, herm);
   return PW_OK;
 }
 
 // N = 256, three streaming passes (t256.cuh): the source with the point-2 DFT over (m, d) into the
 // work buffer, the radix-4 over r and the DFT over b in place there, the DFT over a with the output
-// factors and S from the work buffer into W.  Any source (Hermitian or not; an uploaded W0 may be W
+// factors and S from the work buffer into W.  Any source but the GSM model (Hermitian or not; an uploaded W0 may be W
 // itself, since the first pass writes only the work buffer).  Events: the first pass, then the
 // second and third apart.
 pw_status propagate_t256(pw_csd* h, double z, bool herm) {
   namespace T = pw::t256;
-  const int src = h->kind == SRC_GSM ? pw::SRC_GSM
-                  : h->kind == SRC_DIAGONAL ? pw::SRC_DIAG
-                  : h->kind == SRC_ADJOINT ? pw::SRC_ADJ : pw::SRC_ARRAY;
+  const int src = h->kind == SRC_DIAGONAL ? pw::SRC_DIAG : h->kind == SRC_ADJOINT ? pw::SRC_ADJ : pw::SRC_ARRAY;
   pw::PassAArgs a{};
   a.F = h->F;
-  a.G = h->G;
   a.tw = h->tw;
   a.W0 = src == pw::SRC_ARRAY ? reinterpret_cast<const float2*>(h->kind == SRC_PROPAGATED ? h->W : h->W0) : nullptr;
   a.diag = h->diag;
@@ -700,7 +798,6 @@ pw_status propagate_t256(pw_csd* h, double z, bool herm) {
   }
   if (ev && (e = cudaEventRecord(ev[0], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
   switch (src) {
-    case pw::SRC_GSM: e = kernel1(T::pass1_kernel<pw::SRC_GSM>, ready1[pw::SRC_GSM]); break;
     case pw::SRC_DIAG: e = kernel1(T::pass1_kernel<pw::SRC_DIAG>, ready1[pw::SRC_DIAG]); break;
     case pw::SRC_ADJ: e = kernel1(T::pass1_kernel<pw::SRC_ADJ>, ready1[pw::SRC_ADJ]); break;
     default: e = kernel1(T::pass1_kernel<pw::SRC_ARRAY>, ready1[pw::SRC_ARRAY]); break;
@@ -713,14 +810,32 @@ pw_status propagate_t256(pw_csd* h, double z, bool herm) {
   T::pass3_kernel<<<g3, T::NT2, T::pass3_smem(), h->stream>>>(h->y3map, b, h->err);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "third-pass launch (N = 256)");
   if (ev && (e = cudaEventRecord(ev[2], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
-  h->d = lz / (h->N * h->d);
-  h->kind = SRC_PROPAGATED;
-  h->hermitian = herm ? 1 : 0;
-  h->W0 = nullptr;
-  h->diag = nullptr;
-  h->aperture = 0.0;
-  h->lens_f = 0.0;
-  h->mask = nullptr;
+  to_output_plane(h, lz / (h->N * h->d), herm);
+  return PW_OK;
+}
+
+// GSM sources, plane by plane (plane.cuh).  The work buffer holds the two tables.  Events: the tables
+// (at N = 256 with the row pass) as the first pass, the planes (the column pass) as the second.
+pw_status propagate_planes(pw_csd* h, double z) {
+  cudaEvent_t* ev = nullptr;
+  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) {
+    h->three[h->timed] = 0;
+    ev = &h->events[4 * h->timed++];
+  }
+  const double lz = h->lambda * z;
+  PlaneArgs q{};
+  q.F = h->F;
+  q.G = h->G;
+  q.tw = h->tw;
+  q.Eout = h->Eout;
+  q.work = reinterpret_cast<float2*>(h->work);
+  q.W = reinterpret_cast<float2*>(h->W);
+  q.S = h->S;
+  q.A = (float)h->A;
+  q.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
+  cudaError_t e = dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
+  if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch (GSM source)");
+  to_output_plane(h, lz / (h->N * h->d), true);
   return PW_OK;
 }
 
@@ -736,9 +851,14 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
     return fail(PW_EUNSUPPORTED, "the tensor-core first stage is built for Gaussian Schell-model sources only");
   pw_status st = build_tables(h, z, farfield);
   if (st != PW_OK) return st;
-  // N = 256: the three streaming passes (t256.cuh), any source; the cluster engine (d256.cuh) runs
+  // GSM sources: plane by plane, one 2D transform over (a, d) per (b', c') from tables of N^3 values
+  // (N = 128: 0.97 against 1.67 ms on the two general passes; N = 256: 16.5 against 31.3 ms; N = 32: 2 us
+  // less).  The exception is the tensor-core comparison mode at N = 256.
+  const bool tc256 = h->N == 256 && h->dft_mode == PW_DFT_TC_BF16X3;
+  if (h->kind == SRC_GSM && !tc256) return propagate_planes(h, z);
+  // N = 256: the three streaming passes (t256.cuh), any other source; the cluster engine (d256.cuh) runs
   // only the comparison mode with the tensor-core first stage
-  if (h->N == 256 && h->dft_mode != PW_DFT_TC_BF16X3) return propagate_t256(h, z, herm);
+  if (h->N == 256 && !tc256) return propagate_t256(h, z, herm);
   const int src = h->kind == SRC_GSM ? pw::SRC_GSM
                   : h->kind == SRC_DIAGONAL ? pw::SRC_DIAG
                   : h->kind == SRC_ADJOINT ? pw::SRC_ADJ : pw::SRC_ARRAY;
@@ -782,15 +902,7 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
   if (grad) b.gr = *h->adj_grad;
   cudaError_t e = dispatch(h->N, src, herm, grad, h->vmap, a, b, x, h->stream, ev);
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
-  // The output plane becomes the current plane; its CSDA is in W, its masks are unset.
-  h->d = lz / (h->N * h->d);
-  h->kind = SRC_PROPAGATED;
-  h->hermitian = herm ? 1 : 0;
-  h->W0 = nullptr;
-  h->diag = nullptr;
-  h->aperture = 0.0;
-  h->lens_f = 0.0;
-  h->mask = nullptr;
+  to_output_plane(h, lz / (h->N * h->d), herm);
   return PW_OK;
 }
 
@@ -844,6 +956,32 @@ pw_status encode_vmap(CUtensorMap* map, void* work, int N) {
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(PW_ECUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", (int)r);
+  return PW_OK;
+}
+
+// 5D map of W for the plane kernels: a plane (b', c') is the N rows W(a', b', c', .), left whole (N <= 96), or
+// at N = 128 as the eight rows a' = w + 16 i of one warp; at N = 256 the column pass's tiles, 64 floats
+// of every a.
+pw_status encode_wmap(CUtensorMap* map, void* W, int N) {
+  auto enc = encode_tiled();
+  if (!enc) return fail(PW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  if (N == 256) {
+    const cuuint64_t dims[5] = {64, 256 * 256 * 8, 256, 1, 1};
+    const cuuint64_t strides[4] = {256, (cuuint64_t)256 * 256 * 256 * 8, (cuuint64_t)1 << 35, (cuuint64_t)1 << 35};
+    const cuuint32_t box[5] = {64, 1, 256, 1, 1};
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, W, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(PW_ECUDA, "cuTensorMapEncodeTiled (column tiles of W) failed (CUresult %d)", (int)r);
+    return PW_OK;
+  }
+  const cuuint64_t n = N, row = 2 * n * sizeof(float), lo = N == 128 ? 16 : n;
+  const cuuint64_t dims[5] = {2 * n, n, n, lo, n / lo};
+  const cuuint64_t strides[4] = {row, row * n, row * n * n, row * n * n * lo};
+  const cuuint32_t box[5] = {(cuuint32_t)(2 * N), 1, 1, (cuuint32_t)(N == 128 ? 1 : N), (cuuint32_t)(N == 128 ? 8 : 1)};
+  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, W, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(PW_ECUDA, "cuTensorMapEncodeTiled (planes of W) failed (CUresult %d)", (int)r);
   return PW_OK;
 }
 

@@ -31,7 +31,8 @@ template <int SIGN> __device__ __forceinline__ float2 twid(const float2* tw, int
   return w;
 }
 
-template <int RP, int RQ, int SIGN> __device__ __forceinline__ void dft2d(float2 (&v)[RP][RQ]) {
+// SIGN along p, SQ along q (the same unless given).
+template <int RP, int RQ, int SIGN, int SQ = SIGN> __device__ __forceinline__ void dft2d(float2 (&v)[RP][RQ]) {
 #pragma unroll
   for (int rq = 0; rq < RQ; ++rq) {
     float2 c[RP];
@@ -42,11 +43,11 @@ template <int RP, int RQ, int SIGN> __device__ __forceinline__ void dft2d(float2
     for (int rp = 0; rp < RP; ++rp) v[rp][rq] = c[rp];
   }
 #pragma unroll
-  for (int rp = 0; rp < RP; ++rp) Dft<RQ, SIGN>::run(v[rp]);
+  for (int rp = 0; rp < RP; ++rp) Dft<RQ, SQ>::run(v[rp]);
 }
 
 // v[rp][rq] *= tw[mp * rp] (rp >= 1) and tw[mq * rq] (rq >= 1)
-template <int RP, int RQ, int SIGN>
+template <int RP, int RQ, int SIGN, int SQ = SIGN>
 __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], const float2* tw, int mp, int mq) {
 #pragma unroll
   for (int rp = 1; rp < RP; ++rp) {
@@ -56,7 +57,7 @@ __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], const float2* tw,
   }
 #pragma unroll
   for (int rq = 1; rq < RQ; ++rq) {
-    const float2 w = twid<SIGN>(tw, mq * rq);
+    const float2 w = twid<SQ>(tw, mq * rq);
 #pragma unroll
     for (int rp = 0; rp < RP; ++rp) v[rp][rq] = cmul(v[rp][rq], w);
   }
@@ -67,7 +68,10 @@ __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], const float2* tw,
 // ROWS: the second exchange puts row p at buffer row vrow(p), so that the rows stage 3 of a warp
 // reads (c' = warp + 16 i + 32 rp) are the eight buffer rows 8 warp .. 8 warp + 7.
 // Contract: buf is free on entry (all threads passed a barrier after its last use).
-template <int SIGN, bool ROWS = false>
+// PAIR: the thread's stage-3 butterflies are the column pair 2 (lane mod 16) + i of row
+// jp3 = warp + 16 (lane / 16) instead, read 16 bytes at a time: w3[i][rp][rq] then holds the
+// transform at (jp3 + 32 rp, 2 (lane mod 16) + i + 32 rq).  Signs: SIGN along p, SQ along q.
+template <int SIGN, bool ROWS = false, int SQ = SIGN, bool PAIR = false>
 __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][4], float2* buf,
                                          const float2* tw) {
   auto row = [](int p) { return ROWS ? vrow<N>(p) : p; };
@@ -83,8 +87,8 @@ __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][
   for (int rp = 0; rp < 4; ++rp)
 #pragma unroll
     for (int rq = 0; rq < 8; ++rq) u[rp][rq] = buf[(jp2 + 32 * rp) * N + sw1(jq2 + 16 * rq)];
-  twiddle2d<4, 8, SIGN>(u, tw, 4 * (jp2 & 7), 4 * (jq2 & 3));
-  dft2d<4, 8, SIGN>(u);
+  twiddle2d<4, 8, SIGN, SQ>(u, tw, 4 * (jp2 & 7), 4 * (jq2 & 3));
+  dft2d<4, 8, SIGN, SQ>(u);
   __syncthreads();
 #pragma unroll
   for (int rp = 0; rp < 4; ++rp)
@@ -92,15 +96,32 @@ __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][
     for (int rq = 0; rq < 8; ++rq)
       buf[row((jp2 >> 3) * 32 + (jp2 & 7) + 8 * rp) * N + sw2((jq2 >> 2) * 32 + (jq2 & 3) + 4 * rq)] = u[rp][rq];
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int jp3 = warp + 16 * i;
+  if constexpr (PAIR) {
+    const int jp3 = warp + 16 * (lane >> 4), jq = 2 * (lane & 15);
 #pragma unroll
     for (int rp = 0; rp < 4; ++rp)
 #pragma unroll
-      for (int rq = 0; rq < 4; ++rq) w3[i][rp][rq] = buf[row(jp3 + 32 * rp) * N + sw2(lane + 32 * rq)];
-    twiddle2d<4, 4, SIGN>(w3[i], tw, jp3, lane);
-    dft2d<4, 4, SIGN>(w3[i]);
+      for (int rq = 0; rq < 4; ++rq) {
+        const float4 x = *reinterpret_cast<const float4*>(buf + row(jp3 + 32 * rp) * N + sw2(jq + 32 * rq));
+        w3[0][rp][rq] = make_float2(x.x, x.y);
+        w3[1][rp][rq] = make_float2(x.z, x.w);
+      }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      twiddle2d<4, 4, SIGN, SQ>(w3[i], tw, jp3, jq + i);
+      dft2d<4, 4, SIGN, SQ>(w3[i]);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int jp3 = warp + 16 * i;
+#pragma unroll
+      for (int rp = 0; rp < 4; ++rp)
+#pragma unroll
+        for (int rq = 0; rq < 4; ++rq) w3[i][rp][rq] = buf[row(jp3 + 32 * rp) * N + sw2(lane + 32 * rq)];
+      twiddle2d<4, 4, SIGN, SQ>(w3[i], tw, jp3, lane);
+      dft2d<4, 4, SIGN, SQ>(w3[i]);
+    }
   }
 }
 

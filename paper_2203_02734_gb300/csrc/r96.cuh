@@ -29,7 +29,7 @@ constexpr int NT = 192;
 constexpr int P = N + 1;  // exchange pitch
 
 // v[kp][kq] *= (p twiddle of stage (RP, NSP) for jp) x (q twiddle of stage (RQ, NSQ) for jq)
-template <int RP, int NSP, int RQ, int NSQ, int SIGN>
+template <int RP, int NSP, int RQ, int NSQ, int SIGN, int SQ = SIGN>
 __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], int jp, int jq, const float2* tw) {
   if constexpr (NSP > 1) {
     const int k = jp % NSP;
@@ -48,7 +48,7 @@ __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], int jp, int jq, c
 #pragma unroll
     for (int r = 1; r < RQ; ++r) {
       float2 w = tw[r * k * STEP];
-      if (SIGN > 0) w.y = -w.y;
+      if (SQ > 0) w.y = -w.y;
 #pragma unroll
       for (int c = 0; c < RP; ++c) v[c][r] = cmul(v[c][r], w);
     }
@@ -59,12 +59,13 @@ __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], int jp, int jq, c
 // through X.  On return w3[i][kp][kq] holds the transform at (jp3 + 24 kp, jq3 + 24 kq), with
 // u = t + 192 i, jq3 = u mod 24, jp3 = u / 24.  Contract: X is free on entry; on return every
 // thread has finished reading X (a block barrier has been passed).
-template <int SIGN>
+// Signs: SIGN along p, SQ along q.
+template <int SIGN, int SQ = SIGN>
 __device__ __forceinline__ void stages(float2 (&v)[2][8][3], float2 (&w3)[3][4][4], float2* X, const float2* tw) {
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    r128::dft2d<8, 3, SIGN>(v[i]);
+    r128::dft2d<8, 3, SIGN, SQ>(v[i]);
     const int jp = warp + 6 * i, jq = lane;
 #pragma unroll
     for (int kp = 0; kp < 8; ++kp)
@@ -80,8 +81,8 @@ __device__ __forceinline__ void stages(float2 (&v)[2][8][3], float2 (&w3)[3][4][
     for (int kp = 0; kp < 3; ++kp)
 #pragma unroll
       for (int kq = 0; kq < 8; ++kq) u2[i][kp][kq] = X[(jp + 32 * kp) * P + jq + 12 * kq];
-    twiddle2d<3, 8, 8, 3, SIGN>(u2[i], jp, jq, tw);
-    r128::dft2d<3, 8, SIGN>(u2[i]);
+    twiddle2d<3, 8, 8, 3, SIGN, SQ>(u2[i], jp, jq, tw);
+    r128::dft2d<3, 8, SIGN, SQ>(u2[i]);
   }
   __syncthreads();
 #pragma unroll
@@ -101,8 +102,8 @@ __device__ __forceinline__ void stages(float2 (&v)[2][8][3], float2 (&w3)[3][4][
     for (int kp = 0; kp < 4; ++kp)
 #pragma unroll
       for (int kq = 0; kq < 4; ++kq) w3[i][kp][kq] = X[(jp + 24 * kp) * P + jq + 24 * kq];
-    twiddle2d<4, 24, 4, 24, SIGN>(w3[i], jp, jq, tw);
-    r128::dft2d<4, 4, SIGN>(w3[i]);
+    twiddle2d<4, 24, 4, 24, SIGN, SQ>(w3[i], jp, jq, tw);
+    r128::dft2d<4, 4, SIGN, SQ>(w3[i]);
   }
   __syncthreads();
 }

@@ -11,8 +11,9 @@
 // intermediate array lives in the work buffer as
 //   Y[a][b][kperm(k_l)][g][r][j]  (after pass 1)  and  Y[a][b'][kperm(k_l)][g][k_h][j]  (after pass 2),
 // so that the 4 x 8 values one pass-2 line group needs are one 256-byte run (kperm: below).
-//   pass 1, tile (a, b, r): the source rows c = r + 4 m of slice (a, b) are generated in registers
-//     (W1(c, d) = conj F(a, b) F(c, d) x source), transformed over (m, d) as a 64 x 256 2D DFT in
+// It runs every source but the GSM model, which has no need of the point-2 pass (plane.cuh).
+//   pass 1, tile (a, b, r): the source rows c = r + 4 m of slice (a, b) are read or generated in
+//     registers (W1(c, d) = conj F(a, b) F(c, d) x source), transformed over (m, d) as a 64 x 256 2D DFT in
 //     registers through one shared buffer, and stored to Y by TMA (64-byte pieces of the 256-byte
 //     runs; the four r tiles of a slice run side by side and fill each run together).
 //   pass 2, tile (a, k_l, g): the 256 runs Y[a][.][k_l][g] (all b, r, j) arrive by one TMA tensor
@@ -158,32 +159,24 @@ __global__ void __launch_bounds__(NT1, 1) pass1_kernel(const __grid_constant__ C
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   for (int i = t; i < N; i += NT1) tw[i] = p.tw[i];
   const float2* __restrict__ F = p.F;
-  const float* __restrict__ G = p.G;
   for (int tile = blockIdx.x; tile < N * N * 4; tile += gridDim.x) {
     const int ab = tile >> 2, r = tile & 3;
     const int a = ab / N, b = ab - a * N;
     float2 s_ab = cconj(__ldg(F + ab));
-    if (SRC == SRC_GSM || SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
+    if (SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
     if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
     const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
     AdjSlice adj{};
     if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
     // stage 1 inputs: m = w + 16 rp (c = r + 4 m), d = l + 32 rq
-    float gb[8];
-    if (SRC == SRC_GSM) {
-#pragma unroll
-      for (int rq = 0; rq < 8; ++rq) gb[rq] = __ldg(G + b * N + lane + 32 * rq);
-    }
     float2 v[4][8];
 #pragma unroll
     for (int rp = 0; rp < 4; ++rp) {
       const int c = r + 4 * (w + 16 * rp);
-      const float ga = SRC == SRC_GSM ? __ldg(G + a * N + c) : 1.f;
 #pragma unroll
       for (int rq = 0; rq < 8; ++rq) {
         const int d = lane + 32 * rq;
         float2 x = cmul(s_ab, __ldg(F + c * N + d));
-        if (SRC == SRC_GSM) x = cscale(x, ga * gb[rq]);
         if (ARRAY) x = cmul(x, __ldg(W0 + c * N + d));
         if (DIAG) x = (c == a && d == b) ? x : make_float2(0.f, 0.f);
         if (SRC == SRC_ADJ) x = cmul(x, adj.at(p.cross, c * N + d));
