@@ -277,17 +277,16 @@ pw_status pw_csd_pass_times3(pw_csd* h, double* ms_first, double* ms_second, dou
  * spectrum), several distances and uneven grid sizes.  Each instance is one propagation of a
  * GSM source (Sec. 5.4) times an optional aperture, thin lens and mask from its source plane;
  * it yields S (Eq. defS) and mu(P1, .) (Eq. defMu) of its output plane, and the whole propagated
- * CSDA when dev_W is given.  Two execution modes (pw_batch_set_mode, chosen by pw_batch_autotune):
- *   PW_BATCH_PERSISTENT: all instances in one persistent launch that walks a work list of
+ * CSDA when dev_W is given.  Instances without dev_W need no CSDA at all: S is the transform of the
+ * correlation of the source field times its coherence and mu's row two convolutions, O(N^2 log N)
+ * work each, all of them together in a few launches in either mode.  For the instances with dev_W
+ * there are two execution modes (pw_batch_set_mode, chosen by pw_batch_autotune):
+ *   PW_BATCH_PERSISTENT: all of them in one persistent launch that walks a work list of
  *     (instance, pass, slice chunk) items; pass-B work of an instance starts after its pass-A
  *     work (bounded waits, see pw_batch_check);
- *   PW_BATCH_SEQUENCED: the instances one after the other on the single-instance kernels (each
- *     fills the GPU): pass A, then pass B with S, the mu numerator and W when dev_W is given;
- *     without dev_W the second pass computes only the two outputs per column that S and the mu
- *     numerator use (dot products over the point-1 pair, Eq. W_fresnel's point-1 sum at X1 = X2
- *     and at X1 = P1), reading the half-transformed CSDA in its own layout.
+ *   PW_BATCH_SEQUENCED: one after the other on the single-instance kernels (each fills the GPU).
  * The default is SEQUENCED when every instance has N >= 64, else PERSISTENT.  In both modes the
- * half-transformed CSDAs share a pool of `pool` buffers of the largest N (instance i uses slot
+ * intermediate arrays share a pool of `pool` buffers of the largest N (instance i uses slot
  * i mod pool).  pw_batch_run enqueues only device work (no allocation, no synchronisation), so
  * the caller may capture it in a CUDA graph and replay it. */
 typedef struct pw_instance {
@@ -344,7 +343,8 @@ pw_status pw_batch_autotune(pw_batch* b, int* chunk_out);
 /* Failure-detection test hook (no counterpart in the paper): leave the pass-A work of
  * `instance` out of the work list and bound every dependency wait to wait_s seconds, so that
  * the pass-B work of that instance gives up waiting and the next pw_batch_check returns
- * PW_ETIMEOUT while the other instances complete.  No device fault is involved. */
+ * PW_ETIMEOUT while the other instances complete.  In the persistent mode every instance, with or
+ * without dev_W, then runs in the persistent launch.  No device fault is involved. */
 pw_status pw_batch_inject_stall(pw_batch* b, int instance, double wait_s);
 
 /* Polychromatic intensity (Sec. 3.5: I(x) = integral of S(x, omega) over frequency; the paper

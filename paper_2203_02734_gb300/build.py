@@ -1,6 +1,6 @@
 """Compile the CUDA library (csrc/) into libpywolf_gb.so next to this file, for sm_103a.
 
-One translation unit, one -gencode, no cmake: a single nvcc call.  Rebuilds only when a
+A few translation units compiled in parallel, one -gencode, no cmake: a single nvcc call.  Rebuilds only when a
 source or the public header is newer than the library (or when forced).
 """
 import glob
@@ -12,7 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libpywolf_gb.so")
 SRC = os.path.join(HERE, "csrc", "pywolf_gb.cu")
-SRCS = [SRC, os.path.join(HERE, "csrc", "noalloc.cu"), os.path.join(HERE, "csrc", "batch.cu")]
+SRCS = [SRC, os.path.join(HERE, "csrc", "noalloc.cu"), os.path.join(HERE, "csrc", "batch.cu"),
+        os.path.join(HERE, "csrc", "smu.cu")]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 
@@ -39,7 +40,7 @@ def build(force=False, verbose=False):
     if not force and up_to_date():
         return LIB
     tmp = LIB + ".tmp%d" % os.getpid()
-    cmd = [_nvcc(), "-std=c++17", "-O3", ARCH, "-lineinfo", "-Xptxas", "-v" if verbose else "-O3",
+    cmd = [_nvcc(), "-std=c++17", "-O3", "-t", "0", ARCH, "-lineinfo", "-Xptxas", "-v" if verbose else "-O3",
            "-shared", "-Xcompiler", "-fPIC", "-o", tmp] + SRCS
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:

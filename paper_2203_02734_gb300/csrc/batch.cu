@@ -1,9 +1,11 @@
 // batch.cu -- C ABI of the batched run (pw_batch_*): instance descriptors, workspace layout,
-// item list, launch sequence (counter reset, FP64 tables, one persistent launch, mu) and the
-// chunk-size autotuner.
+// item list, launch sequence and the chunk-size autotuner.  Instances that keep no W run on smu.cuh
+// (S and mu without the CSDA); the others on the plane kernels one after the other, or in the
+// persistent launch.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -11,13 +13,8 @@
 
 #include "../../include/pywolf_gb.h"
 #include "batch.cuh"
-
-namespace pwi {  // pywolf_gb.cu
-void set_last_error(const char* msg);
-pw_status encode_vmap(CUtensorMap* map, void* work, int N);
-cudaError_t launch_batch_instance(int N, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
-                                  const float2* Ein, const float2* mask, int ap_ithr, cudaStream_t s);
-}
+#include "internal.h"
+#include "smu.cuh"
 
 namespace {
 
@@ -98,7 +95,20 @@ Layout layout(const pw_instance* in, int n, int pool) {
 struct pw_batch {
   int n, pool, chunk;
   int mode;  // PW_BATCH_PERSISTENT or PW_BATCH_SEQUENCED
-  std::vector<CUtensorMap> vmaps;  // per instance: its V slot in the layout of its N
+  std::vector<CUtensorMap> wmaps;  // per instance with W: its planes (plane.cuh)
+  std::vector<pw::TableArgs> targs;   // FP64 tables, uploaded with N = 0 for the instances on smu.cuh
+  std::vector<pw::smu::Inst> smu;     // the instances on smu.cuh, by pw_instance index where direct
+  std::vector<pw::smu::TabArgs> smu_t;
+  std::vector<float2*> mus;           // dev_mu of every instance
+  struct Round {                      // one launch round of the instances on smu.cuh
+    int chunk;
+    bool mu;
+    std::vector<int> Ns;
+  };
+  std::vector<Round> rounds;
+  int ndirect;                        // instances on smu.cuh
+  const pw::smu::Inst* dev_smu;
+  const pw::smu::TabArgs* dev_smu_t;
   char* base;
   Layout L;
   cudaStream_t stream;
@@ -111,6 +121,14 @@ struct pw_batch {
 
 namespace {
 
+// Instances that keep no W need no half-transformed array and run on smu.cuh, in either mode (192
+// instances of N = 64 to 128: 87 ms on the half-transformed arrays).  With a stall injected the whole list
+// stays in the persistent launch, whose waits are under test.
+bool stalled(const pw_batch* b) { return std::find(b->stalled.begin(), b->stalled.end(), 1) != b->stalled.end(); }
+bool direct(const pw_batch* b, int i) {
+  return b->inst[i].W == nullptr && !(b->mode == PW_BATCH_PERSISTENT && stalled(b));
+}
+
 pw_status build_items(pw_batch* b) {
   std::vector<pw::batch::Item> items;
   // One pass = J = ceil(S / chunk) items.  N = 128 (register-resident engine, whose pass B
@@ -118,7 +136,7 @@ pw_status build_items(pw_batch* b) {
   // j + 2 J, ..., so that neighbouring CTAs gather the columns of one run together.  Other sizes:
   // contiguous ranges of chunk slices (measured slightly faster there).
   auto add = [&](int i, int pass) {
-    if (pass == 0 && b->stalled[i]) return;
+    if (direct(b, i) || (pass == 0 && b->stalled[i])) return;
     const int S = b->inst[i].slices;
     const int J = (S + b->chunk - 1) / b->chunk;
     for (int j = 0; j < J; ++j) {
@@ -144,6 +162,60 @@ pw_status build_items(pw_batch* b) {
   if (e != cudaSuccess) return cuda_fail(e, "uploading the item list");
   return PW_OK;
 }
+
+// Uploads what depends on which instances run on smu.cuh: the FP64 table arguments, the mu outputs of
+// the others, the smu.cuh descriptors, and the item list.  The descriptors sit at the end of the
+// item area, in the room of the items that these instances do not have (2560 bytes each at least);
+// their scratch is the V pool, in as many rounds as it takes.
+pw_status upload(pw_batch* b) {
+  const int n = b->n;
+  const size_t pool_bytes = b->L.slot_bytes * b->pool;
+  std::vector<pw::TableArgs> targs(b->targs);
+  std::vector<float2*> mus(b->mus);
+  std::vector<pw::smu::Inst> list;
+  std::vector<pw::smu::TabArgs> tabs;
+  b->rounds.clear();
+  size_t used = 0;
+  int chunk = 0;
+  for (int i = 0; i < n; ++i) {
+    if (!direct(b, i)) continue;
+    targs[i].N = 0;
+    mus[i] = nullptr;
+    pw::smu::Inst q = b->smu[i];
+    const size_t need = align256((size_t)6 * q.N * q.N * sizeof(float2));
+    if (used + need > pool_bytes) {
+      ++chunk;
+      used = 0;
+    }
+    if (b->rounds.empty() || b->rounds.back().chunk != chunk) b->rounds.push_back({chunk, false, {}});
+    auto& r = b->rounds.back();
+    r.mu = r.mu || q.mu;
+    if (std::find(r.Ns.begin(), r.Ns.end(), q.N) == r.Ns.end()) r.Ns.push_back(q.N);
+    q.chunk = chunk;
+    q.scratch = reinterpret_cast<float2*>(b->base + b->L.pool + used);
+    used += need;
+    list.push_back(q);
+    tabs.push_back(b->smu_t[i]);
+  }
+  b->ndirect = (int)list.size();
+  const size_t lb = align256(list.size() * sizeof(pw::smu::Inst)), tb = align256(tabs.size() * sizeof(pw::smu::TabArgs));
+  char* tail = b->base + (b->L.items + sizeof(pw::batch::Item) * (size_t)b->L.max_items) / 256 * 256 - lb - tb;
+  b->dev_smu = reinterpret_cast<pw::smu::Inst*>(tail);
+  b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs*>(tail + lb);
+  cudaError_t e = cudaMemcpyAsync(b->base + b->L.targs, targs.data(), sizeof(pw::TableArgs) * n, cudaMemcpyHostToDevice,
+                                  b->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->base + b->L.mu, mus.data(), sizeof(float2*) * n, cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess && b->ndirect)
+    e = cudaMemcpyAsync(tail, list.data(), list.size() * sizeof(pw::smu::Inst), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess && b->ndirect)
+    e = cudaMemcpyAsync(tail + lb, tabs.data(), tabs.size() * sizeof(pw::smu::TabArgs), cudaMemcpyHostToDevice, b->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "uploading the batch descriptors");
+  return build_items(b);
+}
+
+__global__ void __launch_bounds__(256) smu_tables_kernel(const pw::smu::TabArgs* t) { pw::smu::tables(t[blockIdx.x]); }
 
 int num_sms() {
   int dev = 0, n = 0;
@@ -196,16 +268,20 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
   bool all_large = true;
   for (int i = 0; i < n; ++i) all_large = all_large && in[i].N >= 64;
   b->mode = all_large ? PW_BATCH_SEQUENCED : PW_BATCH_PERSISTENT;
-  b->vmaps.resize(n);
+  b->wmaps.resize(n);
   for (int i = 0; i < n; ++i) {
-    pw_status st = pwi::encode_vmap(&b->vmaps[i], b->base + L.pool + L.slot_bytes * (i % pool), in[i].N);
+    pw_status st = in[i].dev_W ? pwi::encode_wmap(&b->wmaps[i], in[i].dev_W, in[i].N) : PW_OK;
     if (st != PW_OK) {
       delete b;
       return st;
     }
   }
-  std::vector<pw::TableArgs> targs(n);
-  std::vector<float2*> mus(n);
+  std::vector<pw::TableArgs>& targs = b->targs;
+  std::vector<float2*>& mus = b->mus;
+  targs.resize(n);
+  mus.resize(n);
+  b->smu.resize(n);
+  b->smu_t.resize(n);
   b->inst.resize(n);
   size_t off = L.tables;
   for (int i = 0; i < n; ++i) {
@@ -269,6 +345,32 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     t.tw = tw;
     t.Eout = Eo;
     t.Ein = Ei;
+    // smu.cuh: its tables take the place of F (11 N of the N^2 values)
+    pw::smu::TabArgs& ta = b->smu_t[i];
+    ta.N = N;
+    ta.Kin = t.Kin;
+    ta.Kout = t.Kout;
+    ta.gs = t.gs;
+    ta.gm = t.gm;
+    ta.tw = F;
+    ta.P1 = ta.tw + 2 * N;
+    ta.Eout = ta.P1 + N;
+    ta.k = reinterpret_cast<float*>(ta.Eout + N);
+    ta.K = ta.k + N;
+    pw::smu::Inst& si = b->smu[i];
+    si.N = N;
+    si.iP = q.iP;
+    si.jP = q.jP;
+    si.factor = (float)((double)d.scale * q.amplitude / (4.0 * (double)NN));
+    si.tw = ta.tw;
+    si.P1 = ta.P1;
+    si.Eout = ta.Eout;
+    si.k = ta.k;
+    si.K = ta.K;
+    si.mask = d.mask;
+    si.ap_ithr = d.ap_ithr;
+    si.S = q.dev_S;
+    si.mu = mus[i];
   }
   bool any128 = false;
   for (int i = 0; i < n; ++i) any128 = any128 || in[i].N == 128;
@@ -287,10 +389,6 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
   if (e == cudaSuccess && any128)
     e = cudaMemcpyAsync(b->base + L.tmaps, maps.data(), sizeof(CUtensorMap) * pool, cudaMemcpyHostToDevice,
                         b->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->base + L.targs, targs.data(), sizeof(pw::TableArgs) * n, cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(b->base + L.mu, mus.data(), sizeof(float2*) * n, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)  // counters and the error flag start at zero (the workspace may hold old data)
     e = cudaMemsetAsync(b->base + L.counters, 0, sizeof(int) * (2 * (size_t)n + 2), b->stream);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(pw::batch::batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -299,7 +397,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     delete b;
     return cuda_fail(e, "batch set-up");
   }
-  pw_status st = build_items(b);
+  pw_status st = upload(b);
   if (st != PW_OK) {
     delete b;
     return st;
@@ -311,8 +409,16 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
 pw_status pw_batch_run(pw_batch* b) {
   pwi::set_last_error("");
   if (!b) return fail(PW_EINVAL, "null batch");
-  int* cnt = reinterpret_cast<int*>(b->base + b->L.counters);
   cudaError_t e;
+  if (b->ndirect) {
+    smu_tables_kernel<<<b->ndirect, 256, 0, b->stream>>>(b->dev_smu_t);
+    for (const auto& r : b->rounds)
+      for (int N : r.Ns)
+        if ((e = pwi::launch_smu(N, b->dev_smu, pw::smu::Inst{}, b->ndirect, r.chunk, r.mu, b->stream)) != cudaSuccess)
+          return cuda_fail(e, "batch S/mu launch");
+    if (b->ndirect == b->n) return PW_OK;
+  }
+  int* cnt = reinterpret_cast<int*>(b->base + b->L.counters);
   if (b->mode == PW_BATCH_PERSISTENT) {
     e = cudaMemsetAsync(cnt, 0, sizeof(int) * (2 * (size_t)b->n + 1), b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "resetting the batch counters");
@@ -320,35 +426,39 @@ pw_status pw_batch_run(pw_batch* b) {
   int maxNN = 0;
   for (const auto& d : b->inst) maxNN = d.slices > maxNN ? d.slices : maxNN;
   dim3 tg((maxNN + 255) / 256, b->n);
-  pw::batch::batch_tables_kernel<<<tg, 256, 0, b->stream>>>(reinterpret_cast<const pw::TableArgs*>(b->base + b->L.targs));
+  pw::batch::batch_tables_kernel<<<tg, 256, 0, b->stream>>>(reinterpret_cast<const pw::TableArgs*>(b->base + b->L.targs),
+                                                          b->mode == PW_BATCH_PERSISTENT ? cnt + b->n : nullptr);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "batch tables launch");
-  if (b->mode == PW_BATCH_SEQUENCED) {
-    // one instance after the other on the single-instance kernels (stream order reuses the slots)
-    for (int i = 0; i < b->n; ++i) {
-      const pw::batch::Inst& d = b->inst[i];
-      pw::PassAArgs a{};
-      a.F = d.F;
-      a.G = d.G;
-      a.tw = d.tw;
-      a.A = d.A;
-      pw::PassBArgs pb{};
-      pb.V = d.V;
-      pb.tw = d.tw;
-      pb.Eout = d.Eout;
-      pb.W = d.W;
-      pb.S = d.S;
-      pb.scale = d.scale;
-      pb.row = d.row;
-      pb.iP = d.iP;
-      pb.jP = d.jP;
-      e = pwi::launch_batch_instance(d.N, b->vmaps[i], a, pb, d.Ein, d.mask, d.ap_ithr, b->stream);
-      if (e != cudaSuccess) return cuda_fail(e, "batch instance launch");
-    }
+  // mu of the instances that are not on smu.cuh (the others' entries are null)
+  auto mu = [&]() -> pw_status {
     dim3 mg((maxNN + 255) / 256, b->n);
     pw::batch::batch_mu_kernel<<<mg, 256, 0, b->stream>>>(reinterpret_cast<const pw::batch::Inst*>(b->base + b->L.inst),
                                                           reinterpret_cast<float2* const*>(b->base + b->L.mu));
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "batch mu launch");
-    return PW_OK;
+    const cudaError_t r = cudaGetLastError();
+    return r == cudaSuccess ? PW_OK : cuda_fail(r, "batch mu launch");
+  };
+  if (b->mode == PW_BATCH_SEQUENCED) {
+    // one instance after the other on the plane kernels (stream order reuses the slots)
+    for (int i = 0; i < b->n; ++i) {
+      const pw::batch::Inst& d = b->inst[i];
+      if (direct(b, i)) continue;
+      pwi::PlaneArgs q{};
+      q.F = d.F;
+      q.G = d.G;
+      q.tw = d.tw;
+      q.Eout = d.Eout;
+      q.work = d.V;
+      q.W = d.W;
+      q.S = d.S;
+      q.A = d.A;
+      q.scale = d.scale;
+      q.row = d.row;
+      q.iP = d.iP;
+      q.jP = d.jP;
+      e = pwi::dispatch_planes(d.N, b->wmaps[i], q, nullptr, b->stream, nullptr);
+      if (e != cudaSuccess) return cuda_fail(e, "batch instance launch");
+    }
+    return mu();
   }
   pw::batch::Args g{};
   g.inst = reinterpret_cast<const pw::batch::Inst*>(b->base + b->L.inst);
@@ -362,10 +472,7 @@ pw_status pw_batch_run(pw_batch* b) {
   g.wait_cycles = b->wait_cycles;
   pw::batch::batch_kernel<<<num_sms(), pw::batch::NT, pw::batch::smem_bytes(), b->stream>>>(g);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "batch kernel launch");
-  dim3 mg((maxNN + 255) / 256, b->n);
-  pw::batch::batch_mu_kernel<<<mg, 256, 0, b->stream>>>(g.inst, reinterpret_cast<float2* const*>(b->base + b->L.mu));
-  if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "batch mu launch");
-  return PW_OK;
+  return mu();
 }
 
 pw_status pw_batch_check(pw_batch* b) {
@@ -414,12 +521,18 @@ pw_status pw_batch_spectral_sum(pw_batch* b, const double* weights, float* dev_I
   return PW_OK;
 }
 
+// The mode decides where a stalled batch runs its instances without W.
+static pw_status change_mode(pw_batch* b, int mode) {
+  const bool again = mode != b->mode && stalled(b);
+  b->mode = mode;
+  return again ? upload(b) : PW_OK;
+}
+
 pw_status pw_batch_set_mode(pw_batch* b, int mode) {
   pwi::set_last_error("");
   if (!b) return fail(PW_EINVAL, "null batch");
   if (mode != PW_BATCH_PERSISTENT && mode != PW_BATCH_SEQUENCED) return fail(PW_EINVAL, "unknown batch mode %d", mode);
-  b->mode = mode;
-  return PW_OK;
+  return change_mode(b, mode);
 }
 
 pw_status pw_batch_get_mode(const pw_batch* b, int* mode) {
@@ -449,7 +562,7 @@ pw_status pw_batch_autotune(pw_batch* b, int* chunk_out) {
   int best_m = b->mode, best_c = b->chunk;
   pw_status st = PW_OK;
   for (const auto& mc : cand) {
-    b->mode = mc[0];
+    if ((st = change_mode(b, mc[0])) != PW_OK) break;
     if (mc[0] == PW_BATCH_PERSISTENT && (st = pw_batch_set_chunk(b, mc[1])) != PW_OK) break;
     if ((st = pw_batch_run(b)) != PW_OK) break;  // warm-up
     cudaEventRecord(e0, b->stream);
@@ -468,7 +581,7 @@ pw_status pw_batch_autotune(pw_batch* b, int* chunk_out) {
   cudaEventDestroy(e1);
   if (st != PW_OK) return st;
   if ((st = pw_batch_check(b)) != PW_OK) return st;
-  b->mode = best_m;
+  if ((st = change_mode(b, best_m)) != PW_OK) return st;
   if (chunk_out) *chunk_out = best_c;
   return pw_batch_set_chunk(b, best_c);
 }
@@ -480,7 +593,7 @@ pw_status pw_batch_inject_stall(pw_batch* b, int instance, double wait_s) {
   if (!(wait_s > 0.0) || !std::isfinite(wait_s)) return fail(PW_EINVAL, "wait must be finite and > 0");
   b->stalled[instance] = 1;
   b->wait_cycles = (long long)(wait_s * 2.0e9);
-  return build_items(b);
+  return upload(b);
 }
 
 pw_status pw_batch_destroy(pw_batch* b) {

@@ -408,8 +408,14 @@ __global__ void __launch_bounds__(NT, 1) batch_kernel(Args g) {
 }
 
 // The FP64 tables of every instance (blockIdx.y = instance), as tables_kernel does for one.
-__global__ void batch_tables_kernel(const TableArgs* targs) {
+// An instance with N = 0 is not in the launch (smu.cuh): its passes count as done for the instances
+// that take its slot (doneB: nullptr outside the persistent mode).
+__global__ void batch_tables_kernel(const TableArgs* targs, int* doneB) {
   const TableArgs t = targs[blockIdx.y];
+  if (t.N == 0) {
+    if (doneB && blockIdx.x == 0 && threadIdx.x == 0) doneB[blockIdx.y] = 1 << 30;
+    return;
+  }
   const int N = t.N, M = N / 2, NN = N * N;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < NN; idx += gridDim.x * blockDim.x) {
     const int i = idx / N, j = idx - i * N;

@@ -189,6 +189,34 @@ __device__ __forceinline__ void fft_stage_stream(const float2* tw, Load load, St
   }
 }
 
+// The same stage over LINES independent lines, lanes walking across lines (x[pos * pitch + line] in
+// shared memory is then read and written contiguously by a warp).
+template <int N, int R, int NS, int SIGN, int LINES, int NT, class Load, class Mid, class Store>
+__device__ __forceinline__ void line_stage(const float2* tw, Load load, Mid mid, Store store) {
+  constexpr int NJ = N / R, NB = NJ * LINES, PER = (NB + NT - 1) / NT;
+  float2 v[PER][R];
+#pragma unroll
+  for (int it = 0; it < PER; ++it) {
+    const int u = threadIdx.x + it * NT, line = u % LINES, j = u / LINES;
+    if (NB % NT == 0 || u < NB) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[it][r] = load(line, j + r * NJ);
+      twiddle<N, R, NS, SIGN>(v[it], j, tw);
+      Dft<R, SIGN>::run(v[it]);
+    }
+  }
+  mid();
+#pragma unroll
+  for (int it = 0; it < PER; ++it) {
+    const int u = threadIdx.x + it * NT, line = u % LINES, j = u / LINES;
+    if (NB % NT == 0 || u < NB) {
+      const int base = (j / NS) * NS * R + (j % NS);
+#pragma unroll
+      for (int r = 0; r < R; ++r) store(line, base + r * NS, v[it][r]);
+    }
+  }
+}
+
 struct SyncMid {
   __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
@@ -216,7 +244,9 @@ PW_PLAN(48, 192, 16, 3)
 PW_PLAN(64, 256, 8, 8)
 PW_PLAN(96, 384, 8, 4, 3)
 PW_PLAN(128, 512, 16, 8)
-PW_PLAN(256, 256, 16, 16)  // single lines only (gsm3.cuh)
+PW_PLAN(192, 256, 8, 8, 3)   // 192, 256, 512: single lines only (plane.cuh, smu.cuh)
+PW_PLAN(256, 256, 16, 16)
+PW_PLAN(512, 256, 8, 8, 8)
 #undef PW_PLAN
 
 template <int N, int I> struct StageInfo {

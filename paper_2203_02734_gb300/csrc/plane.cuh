@@ -37,34 +37,6 @@ struct TabArgs {
   float A;
 };
 
-// One Stockham stage (the convention of fft.cuh) over LINES lines stored as x[pos * LINES + line]:
-// lanes walk across lines, so every shared-memory access of a warp is contiguous.
-template <int N, int R, int NS, int SIGN, int LINES, int NT, class Load, class Mid, class Store>
-__device__ __forceinline__ void line_stage(const float2* tw, Load load, Mid mid, Store store) {
-  constexpr int NJ = N / R, NB = NJ * LINES, PER = (NB + NT - 1) / NT;
-  float2 v[PER][R];
-#pragma unroll
-  for (int it = 0; it < PER; ++it) {
-    const int u = threadIdx.x + it * NT, line = u % LINES, j = u / LINES;
-    if (NB % NT == 0 || u < NB) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[it][r] = load(line, j + r * NJ);
-      twiddle<N, R, NS, SIGN>(v[it], j, tw);
-      Dft<R, SIGN>::run(v[it]);
-    }
-  }
-  mid();
-#pragma unroll
-  for (int it = 0; it < PER; ++it) {
-    const int u = threadIdx.x + it * NT, line = u % LINES, j = u / LINES;
-    if (NB % NT == 0 || u < NB) {
-      const int base = (j / NS) * NS * R + (j % NS);
-#pragma unroll
-      for (int r = 0; r < R; ++r) store(line, base + r * NS, v[it][r]);
-    }
-  }
-}
-
 // In-place stages I .. IEND - 1 of the plan on the shared buffer x (a barrier after each).
 template <int N, int SIGN, int LINES, int NT, int I, int IEND>
 __device__ __forceinline__ void line_stages(float2* x, const float2* tw) {

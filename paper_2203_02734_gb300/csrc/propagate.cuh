@@ -295,15 +295,13 @@ struct PassBArgs {
   float2* W;
   float* S;
   float scale;
-  float2* row;   // optional: row[x] = W(P1, x) (the mu numerator), P1 = (iP, jP); nullptr = none
-  int iP, jP;
   GradEpi gr;    // W_GRAD only
 };
 
-// What pass B stores of the propagated CSDA: nothing (S and the optional row only), the
-// conjugated column as the contiguous row (Hermitian CSDA), every element at its own place, or
-// (W_GRAD) nothing but the GSM parameter-gradient sums of the adjoint.
-enum WStore { W_NONE = 0, W_HERM = 1, W_GENERAL = 2, W_GRAD = 3 };
+// What pass B stores of the propagated CSDA: the conjugated column as the contiguous row (Hermitian
+// CSDA), every element at its own place, or (W_GRAD) nothing but the GSM parameter-gradient sums of
+// the adjoint.
+enum WStore { W_HERM = 1, W_GENERAL = 2, W_GRAD = 3 };
 
 // W_GRAD epilogue for one column x2 = (c, d).  With R = Re(W_B conj-factors) the per-point terms
 //   t = R G(a, c) G(b, d) m(a, b),  sum t r^2,  sum t |x1 - x2|^2,  sum t
@@ -371,10 +369,10 @@ __device__ __forceinline__ void grad_reduce(const GradEpi& g, int N, int cd, con
 
 // Pass B, persistent: CTA blockIdx.x handles point-2 output pairs cd = blockIdx.x + k gridDim.x.
 // Per slice: gather V(., ., c', d') + DFT along a (lanes along b), DFT along b with the
-// epilogue (scale, output propagators, S on the diagonal, and with ROW the P1 row).  WST = W_HERM:
+// epilogue (scale, output propagators, S on the diagonal).  WST = W_HERM:
 // the conjugated column is the contiguous row W(c', d', ., .), written to shared memory and left
-// by one bulk store; W_GENERAL: strided stores; W_NONE: no store of W.
-template <int N, int WST, bool ROW = false>
+// by one bulk store; W_GENERAL: strided stores.
+template <int N, int WST>
 __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_b_kernel(PassBArgs p) {
   constexpr int NT = Plan<N>::NT, P = pitch<N>(), S = Plan<N>::stages;
   constexpr size_t NN = (size_t)N * N;
@@ -413,13 +411,10 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_b_kernel(PassBArgs p) {
     const float2 ecd = cscale(cmul(eo[c], eo[d]), p.scale);
     float* Sd = p.S;
     auto ld0 = [buf](int a, int b) { return buf[a * P + b]; };
-    float2* rw = p.row;
-    const int iP = p.iP, jP = p.jP;
     if constexpr (WST == W_HERM) {
       auto epi = [=](int a, int b, float2 y) {
         const float2 w = cmul(cmul(cconj(cmul(eo[a], eo[b])), ecd), y);
         if (a == c && b == d) Sd[cd] = w.x;
-        if (ROW && a == iP && b == jP) rw[cd] = w;
         buf[a * N + b] = cconj(w);
       };
       fft_stage<N, StageInfo<N, S - 1>::R, StageInfo<N, S - 1>::NS, +1, true, NT>(tw, ld0, SyncMid{}, epi);
@@ -444,7 +439,6 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_b_kernel(PassBArgs p) {
       auto epi = [=](int a, int b, float2 y) {
         const float2 w = cmul(cmul(cconj(cmul(eo[a], eo[b])), ecd), y);
         if (a == c && b == d) Sd[cd] = w.x;
-        if (ROW && a == iP && b == jP) rw[cd] = w;
         if (WST == W_GENERAL) W[(size_t)(a * N + b) * NN + cd] = w;
       };
       fft_stage<N, StageInfo<N, S - 1>::R, StageInfo<N, S - 1>::NS, +1, true, NT>(tw, ld0, NoMid{}, epi);
@@ -504,84 +498,6 @@ static __global__ void s_mu_kernel(SMuArgs a) {
       if (a.M0) w = cmul(cmul(cconj(a.M0[xp]), a.M0[x]), w);
       const float den = sp * sx;
       a.mu_out[x] = den > 0.f ? cscale(w, rsqrtf(den)) : make_float2(0.f, 0.f);
-    }
-  }
-}
-
-// S and the P1 row of one propagation from V alone, for callers that keep no W (the batch).  Of
-// the sign-+1 2D DFT over x1 = (a, b) that pass B runs on column x2 = (c, d), only two outputs are
-// used: (a', b') = (c, d) for S and (a', b') = P1 for the mu numerator.  Each is one dot product
-//   X(a', b') = sum_{a,b} e^{+2 pi i (a a' + b b') / N} V(a, b; c, d)
-// with a separable phase, so V is streamed in its own layout V[c][d/4][a][b][d mod 4]: one block of
-// 4 N^2 contiguous values per (c, d/4) (row vrow(c)), four columns, no gather.  The block has one thread per value
-// of an a-row (4 N, at most 512; SMU_SLOTS rows' worth otherwise): thread t owns the (b, j) pairs
-// k = t + SMU_NT s (j = d mod 4 = t mod 4), sums over a with e^{+2 pi i a c / N} and
-// e^{+2 pi i a iP / N}, then applies the b phase, and the block reduces over b.  The epilogue is
-// pass B's: W(a', b'; c, d) = s conj(E(a') E(b')) E(c) E(d) X(a', b').
-template <int N> __host__ __device__ constexpr int smu_nt() { return 4 * N < 512 ? 4 * N : 512; }
-
-template <int N>
-__global__ void __launch_bounds__(smu_nt<N>(), 2048 / smu_nt<N>()) smu_from_v_kernel(PassBArgs p) {
-  constexpr int G = 4, ROW = N * G, NT = smu_nt<N>(), SLOTS = ROW / NT, NW = NT / 32, NG = N * N / G;
-  static_assert(ROW % NT == 0 && NT % 32 == 0, "a-rows split evenly over the block");
-  __shared__ float2 phc[N], php[N];
-  __shared__ float2 red[NW][4][2];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, j = t & 3;
-  const bool row = p.row != nullptr;
-  for (int q = blockIdx.x; q < NG; q += gridDim.x) {
-    const int cr = q / (N / G), dg = q - cr * (N / G), c = vrow_inv<N>(cr);  // block q holds V row cr
-    __syncthreads();  // the previous group's tables and partial sums are consumed
-    for (int a = t; a < N; a += NT) {
-      phc[a] = cconj(__ldg(p.tw + (a * c) % N));
-      php[a] = cconj(__ldg(p.tw + (a * p.iP) % N));
-    }
-    __syncthreads();
-    const float2* __restrict__ Vq = p.V + (size_t)q * N * ROW;
-    float2 ad[SLOTS], ap[SLOTS];
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) ad[s] = ap[s] = make_float2(0.f, 0.f);
-#pragma unroll 8
-    for (int a = 0; a < N; ++a) {
-      const float2 pc = phc[a], pp = php[a];
-#pragma unroll
-      for (int s = 0; s < SLOTS; ++s) {
-        const float2 v = __ldg(Vq + a * ROW + t + NT * s);
-        ad[s] = cadd(ad[s], cmul(pc, v));
-        ap[s] = cadd(ap[s], cmul(pp, v));
-      }
-    }
-    float2 sd = make_float2(0.f, 0.f), sp = make_float2(0.f, 0.f);
-    const int d = G * dg + j;
-#pragma unroll
-    for (int s = 0; s < SLOTS; ++s) {
-      const int b = (t + NT * s) >> 2;
-      sd = cadd(sd, cmul(cconj(__ldg(p.tw + (b * d) % N)), ad[s]));
-      sp = cadd(sp, cmul(cconj(__ldg(p.tw + (b * p.jP) % N)), ap[s]));
-    }
-#pragma unroll
-    for (int o = 4; o < 32; o <<= 1) {
-      sd.x += __shfl_xor_sync(0xffffffffu, sd.x, o);
-      sd.y += __shfl_xor_sync(0xffffffffu, sd.y, o);
-      sp.x += __shfl_xor_sync(0xffffffffu, sp.x, o);
-      sp.y += __shfl_xor_sync(0xffffffffu, sp.y, o);
-    }
-    if (lane < 4) {
-      red[warp][lane][0] = sd;
-      red[warp][lane][1] = sp;
-    }
-    __syncthreads();
-    if (t < 4) {
-      float2 xd = make_float2(0.f, 0.f), xp = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int w = 0; w < NW; ++w) {
-        xd = cadd(xd, red[w][t][0]);
-        xp = cadd(xp, red[w][t][1]);
-      }
-      const int dd = G * dg + t, cd = c * N + dd;
-      const float2 ecd = cscale(cmul(__ldg(p.Eout + c), __ldg(p.Eout + dd)), p.scale);
-      const float2 wd = cmul(cmul(cmul(cconj(__ldg(p.Eout + c)), ecd), cconj(__ldg(p.Eout + dd))), xd);
-      p.S[cd] = wd.x;
-      if (row) p.row[cd] = cmul(cmul(cmul(cconj(__ldg(p.Eout + p.iP)), ecd), cconj(__ldg(p.Eout + p.jP))), xp);
     }
   }
 }

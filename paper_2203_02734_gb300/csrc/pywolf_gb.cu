@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/pywolf_gb.h"
+#include "internal.h"
 #include "propagate.cuh"
 #include "d256.cuh"
 #include "dense.cuh"
@@ -55,12 +56,7 @@ enum SourceKind { SRC_NONE = 0, SRC_GSM = 1, SRC_ARRAY = 2, SRC_PROPAGATED = 3, 
 }  // namespace
 
 namespace pwi {
-// Sets the thread's message returned by pw_last_error() (used by other translation units).
 void set_last_error(const char* msg) { g_err = msg; }
-pw_status encode_vmap(CUtensorMap* map, void* work, int N);
-pw_status encode_wmap(CUtensorMap* map, void* W, int N);
-cudaError_t launch_batch_instance(int N, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
-                                  const float2* Ein, const float2* mask, int ap_ithr, cudaStream_t s);
 }  // namespace pwi
 
 struct pw_csd {
@@ -202,18 +198,18 @@ cudaError_t launch_a_r128(const CUtensorMap& vmap, const pw::PassAArgs& a, const
 }
 
 // N = 128, Hermitian store or none: register-resident pass B with prefetched gather (r128.cuh).
-template <int WST, bool ROW = false>
+template <int WST>
 cudaError_t launch_b_r128(const pw::PassBArgs& b, cudaStream_t s) {
   constexpr size_t smem = pw::r128::pass_b_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_b_r128<WST, ROW>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_b_r128<WST>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r128::pass_b_r128<WST, ROW>, pw::r128::NT, smem, 128 * 128, &grid);
+    e = persistent_grid(pw::r128::pass_b_r128<WST>, pw::r128::NT, smem, 128 * 128, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r128::pass_b_r128<WST, ROW><<<grid, pw::r128::NT, smem, s>>>(b);
+  pw::r128::pass_b_r128<WST><<<grid, pw::r128::NT, smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -233,18 +229,18 @@ cudaError_t launch_a_r96(const CUtensorMap& vmap, const pw::PassAArgs& a, const 
   return cudaGetLastError();
 }
 
-template <int WST, bool ROW = false>
+template <int WST>
 cudaError_t launch_b_r96(const pw::PassBArgs& b, cudaStream_t s) {
   constexpr size_t smem = pw::r96::pass_b_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_b_r96<WST, ROW>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_b_r96<WST>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r96::pass_b_r96<WST, ROW>, pw::r96::NT, smem, 96 * 96, &grid);
+    e = persistent_grid(pw::r96::pass_b_r96<WST>, pw::r96::NT, smem, 96 * 96, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r96::pass_b_r96<WST, ROW><<<grid, pw::r96::NT, smem, s>>>(b);
+  pw::r96::pass_b_r96<WST><<<grid, pw::r96::NT, smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -322,18 +318,18 @@ cudaError_t launch_b_d256(const pw::PassBArgs& b, cudaStream_t s) {
                          s, b);
 }
 
-template <int N, int WST, bool ROW = false>
+template <int N, int WST>
 cudaError_t launch_b(const pw::PassBArgs& b, cudaStream_t s) {
   constexpr size_t smem = pw::pass_b_smem<N>();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::pass_b_kernel<N, WST, ROW>,
+    cudaError_t e = cudaFuncSetAttribute(pw::pass_b_kernel<N, WST>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::pass_b_kernel<N, WST, ROW>, pw::Plan<N>::NT, smem, N * N, &grid);
+    e = persistent_grid(pw::pass_b_kernel<N, WST>, pw::Plan<N>::NT, smem, N * N, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::pass_b_kernel<N, WST, ROW><<<grid, pw::Plan<N>::NT, smem, s>>>(b);
+  pw::pass_b_kernel<N, WST><<<grid, pw::Plan<N>::NT, smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -389,8 +385,10 @@ cudaError_t launch_passes(int src, bool herm, bool grad, const CUtensorMap& vmap
                           const pw::PassBArgs& b, const R128Extra& x, cudaStream_t s, cudaEvent_t* ev) {
   cudaError_t e;
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  if (src == pw::SRC_GSM) e = launch_a_mode<N, pw::SRC_GSM>(vmap, a, x, s);
-  else if (src == pw::SRC_DIAG) e = launch_a_sparse<N, pw::SRC_DIAG>(vmap, a, b, x, s);
+  if (src == pw::SRC_GSM) {  // the tensor-core comparison mode only (plane.cuh runs the others)
+    if constexpr (N == 256) e = launch_a_mode<N, pw::SRC_GSM>(vmap, a, x, s);
+    else e = cudaErrorNotSupported;
+  } else if (src == pw::SRC_DIAG) e = launch_a_sparse<N, pw::SRC_DIAG>(vmap, a, b, x, s);
   else if (src == pw::SRC_ADJ) e = launch_a_sparse<N, pw::SRC_ADJ>(vmap, a, b, x, s);
   else e = launch_a_mode<N, pw::SRC_ARRAY>(vmap, a, x, s);
   if (e != cudaSuccess) return e;
@@ -428,19 +426,7 @@ cudaError_t dispatch(int N, int src, bool herm, bool grad, const CUtensorMap& vm
   }
 }
 
-// Propagation of a GSM source plane by plane (plane.cuh).
-struct PlaneArgs {
-  const float2* F;
-  const float* G;
-  const float2* tw;
-  const float2* Eout;
-  float2* work;  // 2 N^3 table values
-  float2* W;
-  float* S;
-  float A, scale;
-  float2* row;  // W(P1, .) or nullptr
-  int iP, jP;
-};
+using pwi::PlaneArgs;
 
 template <int N>
 cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
@@ -504,6 +490,9 @@ cudaError_t launch_planes256(const CUtensorMap& wmap, const PlaneArgs& q, int* e
   return cudaSuccess;
 }
 
+}  // namespace
+
+namespace pwi {
 cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s,
                             cudaEvent_t* ev) {
   switch (N) {
@@ -519,6 +508,10 @@ cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, 
       return cudaErrorInvalidValue;
   }
 }
+
+}  // namespace pwi
+
+namespace {
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda).
 PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
@@ -833,7 +826,7 @@ pw_status propagate_planes(pw_csd* h, double z) {
   q.S = h->S;
   q.A = (float)h->A;
   q.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
-  cudaError_t e = dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
+  cudaError_t e = pwi::dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch (GSM source)");
   to_output_plane(h, lz / (h->N * h->d), true);
   return PW_OK;
@@ -985,49 +978,6 @@ pw_status encode_wmap(CUtensorMap* map, void* W, int N) {
   return PW_OK;
 }
 
-// The S / P1-row pass of an instance without W: one wave of resident blocks, each taking the same
-// number of column groups (blocks left for a second wave, or a last round of a few blocks, stream V
-// at a fraction of the bandwidth).  The grid is cached per N.
-template <int NN>
-cudaError_t launch_smu(const pw::PassBArgs& b, cudaStream_t s) {
-  static int grid = 0;
-  if (grid == 0) {
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pw::smu_from_v_kernel<NN>, pw::smu_nt<NN>(), 0);
-    if (e != cudaSuccess) return e;
-    const int groups = NN * NN / 4, resident = std::max(1, per_sm) * num_sms();
-    const int rounds = (groups + resident - 1) / resident;
-    grid = (groups + rounds - 1) / rounds;
-  }
-  pw::smu_from_v_kernel<NN><<<grid, pw::smu_nt<NN>(), 0, s>>>(b);
-  return cudaGetLastError();
-}
-
-// One propagation of a batched GSM instance on the single-instance kernels, from the instance's
-// tables: pass A, then pass B with S, the P1 row and, if b.W is set, the Hermitian W store.
-cudaError_t launch_batch_instance(int N, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
-                                  const float2* Ein, const float2* mask, int ap_ithr, cudaStream_t s) {
-  R128Extra x{};
-  x.Ein = Ein;
-  x.mask = mask;
-  x.ap_ithr = ap_ithr;
-  cudaError_t e;
-  // Without W (S and the P1 row only) the second pass is smu_from_v_kernel: two dot products per
-  // column instead of the full DFT over point 1, reading V in its own layout.
-  switch (N) {
-#define PW_BCASE(NN)                                                                                        \
-  case NN:                                                                                                  \
-    if ((e = launch_a_mode<NN, pw::SRC_GSM>(vmap, a, x, s)) != cudaSuccess) return e;                       \
-    if (!b.W) return launch_smu<NN>(b, s);                                                                  \
-    if constexpr (NN == 128) return launch_b_r128<pw::W_HERM, true>(b, s);                                 \
-    else if constexpr (NN == 96) return launch_b_r96<pw::W_HERM, true>(b, s);                              \
-    else return launch_b<NN, pw::W_HERM, true>(b, s);
-    PW_BCASE(16) PW_BCASE(32) PW_BCASE(64) PW_BCASE(96) PW_BCASE(128)
-#undef PW_BCASE
-    default:
-      return cudaErrorInvalidValue;
-  }
-}
 }  // namespace pwi
 
 extern "C" {

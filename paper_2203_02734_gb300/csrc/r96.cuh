@@ -209,10 +209,10 @@ constexpr size_t pass_b_smem() {
 // cd = blockIdx.x + k gridDim.x: every thread loads its 48 stage-1 inputs of the strided column
 // V(., ., c', d') (8 bytes from each 32-byte run) straight into registers -- the other CTA of the
 // SM computes meanwhile -- with the column group's block brought into L2 two columns ahead; the
-// inverse-sign 2D DFT; the epilogue (scale, output propagators, S on the diagonal, with ROW the P1
-// row) and, for WST = W_HERM, the conjugated column as the contiguous row W(c', d', ., .) from
-// registers (W_NONE: no W store).
-template <int WST, bool ROW = false>
+// inverse-sign 2D DFT; the epilogue (scale, output propagators, S on the diagonal)
+// and, for WST = W_HERM, the conjugated column as the contiguous row W(c', d', ., .) from
+// registers.
+template <int WST>
 __global__ void __launch_bounds__(NT, 2) pass_b_r96(PassBArgs p) {
   extern __shared__ __align__(1024) float2 smem[];
   float2* X = smem;
@@ -235,8 +235,6 @@ __global__ void __launch_bounds__(NT, 2) pass_b_r96(PassBArgs p) {
   prefetch(blockIdx.x);
   prefetch(blockIdx.x + gridDim.x);
   __syncthreads();
-  float2* rw = p.row;
-  const int iP = p.iP, jP = p.jP;
   for (int cd = blockIdx.x; cd < N * N; cd += gridDim.x) {
     const int c = cd / N, d = cd - c * N;
     prefetch(cd + 2 * gridDim.x);
@@ -286,7 +284,6 @@ __global__ void __launch_bounds__(NT, 2) pass_b_r96(PassBArgs p) {
             const int b = jq + 24 * kq;
             const float2 w = cmul(cmul(ea, cconj(eo[b])), w3[i][kp][kq]);
             if (a == c && b == d) p.S[cd] = w.x;
-            if (ROW && a == iP && b == jP) rw[cd] = w;
             if (WST == W_HERM) Wrow[a * N + b] = cconj(w);
           }
         }

@@ -1,0 +1,304 @@
+// smu.cuh -- S and mu(P1, .) of a propagated Gaussian Schell-model source without its CSDA.
+//
+// The GSM axis factor is a product, G(a, c) = h(a) h(c) k(a - c) with h(n) = exp(-n^2 d^2/(4 sigma_S^2)) and
+// k(u) = exp(-u^2 d^2/(2 sigma_mu^2)), so with the source field P(a, b) = F(a, b) h(a) h(b)
+//   S(a', b') = s A sum_{u,v} e^{-2 pi i (u a' + v b')/N} k(u) k(v) C(u, v),
+//   C(u, v) = sum_{a,b} conj P(a, b) P(a + u, b + v)
+// (the output propagators cancel), and the numerator of mu is
+//   W(P1; c', d') = s A conj(E(iP) E(jP)) E(c') E(d') sum_{c,d} e^{-2 pi i (c c' + d d')/N} P(c, d) R(c, d),
+//   R = (k x k) * [conj P(a, b) e^{+2 pi i (a iP + b jP)/N}].
+// Both the correlation C and the convolution R come from the zero-padded transform P^ of P (L = 2 N per
+// axis): C is the inverse transform of |P^|^2, and R that of
+//   K(m) K(n) conj P^(2 iP - m, 2 jP - n), K = the transform of k,
+// so an instance costs a few FFTs of (2N)^2 points in place of an N^4 array.  (The 4D route took 0.99 ms
+// for one instance at N = 128, 87 ms for a batch of 192.)  Everything but the small tables is FP32, as
+// on the 4D route.
+//   k1: columns b, transform over a              -> X1[m][b]   (L x N)
+//   k2: rows m, transform over b; |P^|^2 back to v, times k(v), to b' -> Z1[m][b'];
+//       the R product back to d                  -> Z2[m][d]   (L x N each)
+//   k3: columns, Z1 back to u, times k(u), to a' -> S;  Z2 back to c, times P(c, d), to c' -> X3[c'][d]
+//   k4: rows c', transform over d                -> mu
+// One launch of each covers every instance of one N (blockIdx.y).  A block holds LINES lines in shared
+// memory as x[pos * (LINES + 1) + line], so lanes may walk along lines or across them without bank
+// conflicts and every global access is contiguous along one of the two.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "propagate.cuh"
+
+namespace pw {
+namespace smu {
+
+struct Inst {
+  int N, iP, jP;
+  int chunk;            // launch round: instances of one round have scratch of their own
+  float factor;         // s A / L^2
+  const float2* tw;     // L twiddles exp(-2 pi i m / L)
+  const float2* P1;     // N: Ein(i) h(i)
+  const float2* Eout;   // N
+  const float* k;       // N: k(u)
+  const float* K;       // L: transform of k over |u| < N
+  const float2* mask;   // N x N or nullptr
+  int ap_ithr;          // aperture, as in batch.cuh
+  float2* scratch;      // 3 L N values
+  float* S;             // N x N
+  float2* mu;           // N x N or nullptr
+};
+
+template <int N> __host__ __device__ constexpr int lines() { return N % 16 == 0 ? (N >= 256 ? 8 : 16) : N % 8 == 0 ? 8 : N; }
+template <int N> __host__ __device__ constexpr int threads() { return N >= 64 ? 256 : 128; }
+template <int N> constexpr size_t smem_bytes() {
+  return (size_t)(2 * 2 * N * (lines<N>() + 1) + 3 * N) * sizeof(float2);
+}
+
+// In-place transform of the block's lines (length LEN, natural order), after a barrier and ending with one.
+template <int LEN, int SIGN, int LINES, int NT, int I = 0>
+__device__ __forceinline__ void fft_lines(float2* x, const float2* tw) {
+  if constexpr (I < Plan<LEN>::stages) {
+    constexpr int LP = LINES + 1;
+    auto ld = [x](int line, int pos) { return x[pos * LP + line]; };
+    auto st = [x](int line, int pos, float2 v) { x[pos * LP + line] = v; };
+    line_stage<LEN, StageInfo<LEN, I>::R, StageInfo<LEN, I>::NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
+    __syncthreads();
+    fft_lines<LEN, SIGN, LINES, NT, I + 1>(x, tw);
+  }
+}
+
+// The tables of a block: tw (L) and twN (N = every other entry).
+template <int N>
+__device__ __forceinline__ void load_tw(const Inst& in, float2* tw, float2* twN) {
+  for (int i = threadIdx.x; i < 2 * N; i += threads<N>()) {
+    const float2 v = in.tw[i];
+    tw[i] = v;
+    if (!(i & 1)) twN[i >> 1] = v;
+  }
+}
+
+// P(a, b): source field at a point.
+template <int N>
+__device__ __forceinline__ float2 field(const Inst& in, int a, int b) {
+  const int na = a - N / 2, nb = b - N / 2;
+  if (in.ap_ithr >= 0 && na * na + nb * nb > in.ap_ithr) return make_float2(0.f, 0.f);
+  float2 v = cmul(__ldg(in.P1 + a), __ldg(in.P1 + b));
+  if (in.mask) v = cmul(v, __ldg(in.mask + a * N + b));
+  return v;
+}
+
+// x[v] <- k(v) x[v] + k(N - v) x[v + N] for v < N: the weighted lags v and v - N, folded mod N.
+template <int N, int LINES, int NT>
+__device__ __forceinline__ void fold(float2* x, const float* k) {
+  constexpr int LP = LINES + 1;
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int line = e % LINES, v = e / LINES;
+    float2 y = cscale(x[v * LP + line], __ldg(k + v));
+    if (v > 0) y = cadd(y, cscale(x[(v + N) * LP + line], __ldg(k + N - v)));
+    x[v * LP + line] = y;
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ Inst pick(const Inst* list, const Inst& one) { return list ? list[blockIdx.y] : one; }
+
+template <int N>
+__global__ void __launch_bounds__(threads<N>()) k1(const Inst* list, Inst one, int chunk) {
+  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  const Inst in = pick(list, one);
+  if (in.N != N || in.chunk != chunk) return;
+  extern __shared__ __align__(16) float2 smem[];
+  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  load_tw<N>(in, tw, twN);
+  const int b0 = blockIdx.x * LINES;
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int line = e % LINES, a = e / LINES;
+    x[a * LP + line] = a < N ? field<N>(in, a, b0 + line) : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  fft_lines<L, -1, LINES, NT>(x, tw);
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int line = e % LINES, m = e / LINES;
+    in.scratch[m * N + b0 + line] = x[m * LP + line];
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(threads<N>()) k2(const Inst* list, Inst one, int chunk) {
+  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  const Inst in = pick(list, one);
+  if (in.N != N || in.chunk != chunk) return;
+  extern __shared__ __align__(16) float2 smem[];
+  float2 *x = smem, *y = x + L * LP, *tw = y + L * LP, *twN = tw + L;
+  load_tw<N>(in, tw, twN);
+  const int m0 = blockIdx.x * LINES;
+  const float2* X1 = in.scratch;
+  float2* Z1 = in.scratch + (size_t)L * N;
+  float2* Z2 = Z1 + (size_t)L * N;
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int b = e % L, line = e / L;
+    x[b * LP + line] = b < N ? X1[(m0 + line) * N + b] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  fft_lines<L, -1, LINES, NT>(x, tw);  // P^(m, n)
+  if (in.mu) {
+    for (int e = threadIdx.x; e < L * LINES; e += NT) {  // row m' = 2 iP - m of the R product
+      const int line = e % LINES, n = e / LINES;
+      int mm = 2 * in.iP - (m0 + line), nn = 2 * in.jP - n;
+      mm += mm < 0 ? L : 0;
+      nn += nn < 0 ? L : 0;
+      y[n * LP + line] = cscale(cconj(x[nn * LP + line]), __ldg(in.K + mm) * __ldg(in.K + n));
+    }
+    __syncthreads();
+  }
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int line = e % LINES, n = e / LINES;
+    const float2 v = x[n * LP + line];
+    x[n * LP + line] = make_float2(fmaf(v.x, v.x, v.y * v.y), 0.f);
+  }
+  __syncthreads();
+  fft_lines<L, +1, LINES, NT>(x, tw);
+  fold<N, LINES, NT>(x, in.k);
+  fft_lines<N, -1, LINES, NT>(x, twN);
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int b = e % N, line = e / N;
+    Z1[(m0 + line) * N + b] = x[b * LP + line];
+  }
+  if (in.mu) {
+    fft_lines<L, +1, LINES, NT>(y, tw);
+    for (int e = threadIdx.x; e < N * LINES; e += NT) {
+      const int d = e % N, line = e / N;
+      int mm = 2 * in.iP - (m0 + line);
+      mm += mm < 0 ? L : 0;
+      Z2[mm * N + d] = y[d * LP + line];
+    }
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(threads<N>()) k3(const Inst* list, Inst one, int chunk) {
+  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  const Inst in = pick(list, one);
+  if (in.N != N || in.chunk != chunk) return;
+  extern __shared__ __align__(16) float2 smem[];
+  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  load_tw<N>(in, tw, twN);
+  const int b0 = blockIdx.x * LINES;
+  float2* X3 = in.scratch;
+  const float2* Z1 = in.scratch + (size_t)L * N;
+  const float2* Z2 = Z1 + (size_t)L * N;
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int line = e % LINES, m = e / LINES;
+    x[m * LP + line] = Z1[m * N + b0 + line];
+  }
+  __syncthreads();
+  fft_lines<L, +1, LINES, NT>(x, tw);
+  fold<N, LINES, NT>(x, in.k);
+  fft_lines<N, -1, LINES, NT>(x, twN);
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int line = e % LINES, a = e / LINES;
+    in.S[a * N + b0 + line] = x[a * LP + line].x * in.factor;
+  }
+  if (!in.mu) return;
+  __syncthreads();
+  for (int e = threadIdx.x; e < L * LINES; e += NT) {
+    const int line = e % LINES, m = e / LINES;
+    x[m * LP + line] = Z2[m * N + b0 + line];
+  }
+  __syncthreads();
+  fft_lines<L, +1, LINES, NT>(x, tw);
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int line = e % LINES, c = e / LINES;
+    x[c * LP + line] = cmul(field<N>(in, c, b0 + line), x[c * LP + line]);
+  }
+  __syncthreads();
+  fft_lines<N, -1, LINES, NT>(x, twN);
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int line = e % LINES, c = e / LINES;
+    X3[c * N + b0 + line] = x[c * LP + line];
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(threads<N>()) k4(const Inst* list, Inst one, int chunk) {
+  constexpr int LINES = lines<N>(), LP = LINES + 1, NT = threads<N>(), L = 2 * N;
+  const Inst in = pick(list, one);
+  if (in.N != N || in.chunk != chunk || !in.mu) return;
+  extern __shared__ __align__(16) float2 smem[];
+  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  load_tw<N>(in, tw, twN);
+  const int c0 = blockIdx.x * LINES;
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int d = e % N, line = e / N;
+    x[d * LP + line] = in.scratch[(c0 + line) * N + d];
+  }
+  __syncthreads();
+  fft_lines<N, -1, LINES, NT>(x, twN);
+  const float sp = in.S[in.iP * N + in.jP];
+  const float2 ep = cscale(cconj(cmul(__ldg(in.Eout + in.iP), __ldg(in.Eout + in.jP))), in.factor);
+  for (int e = threadIdx.x; e < N * LINES; e += NT) {
+    const int d = e % N, line = e / N, c = c0 + line;
+    const float den = sp * in.S[c * N + d];
+    const float2 row = cmul(cmul(ep, cmul(__ldg(in.Eout + c), __ldg(in.Eout + d))), x[d * LP + line]);
+    in.mu[c * N + d] = den > 0.f ? cscale(row, rsqrtf(den)) : make_float2(0.f, 0.f);
+  }
+}
+
+// FP64-derived tables of one instance (one block): twiddles, per-axis factors, coherence and its
+// transform.
+struct TabArgs {
+  int N;
+  double Kin, Kout;  // turns per n^2 of the input factor (propagator, lens) and of the output propagator
+  double gs, gm;     // d^2/(4 sigma_S^2), d^2/(2 sigma_mu^2)
+  float2 *tw, *P1, *Eout;
+  float *k, *K;
+};
+
+// The N = blockDim.x-strided work of each table; a block barrier separates k, tw from K.
+__device__ __forceinline__ void tables(const TabArgs& t) {
+  const int N = t.N, L = 2 * N, M = N / 2;
+  // one FP64 evaluation per thread and step: tasks 0..L-1 tw, then P1, Eout and k of each index
+  for (int q = threadIdx.x; q < L + 3 * N; q += blockDim.x) {
+    if (q < L) {
+      t.tw[q] = cis_turns(-(double)q / (double)L);
+      continue;
+    }
+    const int kind = (q - L) / N, i = (q - L) - kind * N;
+    const double n2 = (double)(i - M) * (double)(i - M);
+    if (kind == 0) t.P1[i] = cscale(cis_turns(frac_turns(n2 * t.Kin) + 0.5 * (i & 1)), (float)exp(-n2 * t.gs));
+    else if (kind == 1) t.Eout[i] = cis_turns(frac_turns(n2 * t.Kout) + 0.5 * (i & 1));
+    else t.k[i] = (float)exp(-(double)i * (double)i * t.gm);
+  }
+  __syncthreads();
+  for (int m = threadIdx.x; m < L; m += blockDim.x) {
+    float acc = 0.f;
+    int j = 0;  // m u mod L
+    for (int u = 1; u < N; ++u) {
+      j += m;
+      j -= j >= L ? L : 0;
+      acc = fmaf(t.k[u], t.tw[j].x, acc);
+    }
+    t.K[m] = fmaf(2.f, acc, t.k[0]);
+  }
+}
+
+template <int N>
+cudaError_t launch(const Inst* list, const Inst& one, int n, int chunk, bool any_mu, cudaStream_t s) {
+  constexpr int LINES = lines<N>(), NT = threads<N>();
+  constexpr size_t sm = smem_bytes<N>();
+  static bool ready = false;
+  cudaError_t e = cudaSuccess;
+  if (!ready) {
+    if ((e = cudaFuncSetAttribute(k1<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k3<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k4<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+      return e;
+    ready = true;
+  }
+  k1<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k2<N><<<dim3(2 * N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k3<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  if (any_mu) k4<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  return cudaGetLastError();
+}
+
+}  // namespace smu
+}  // namespace pw
