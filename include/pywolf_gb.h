@@ -238,9 +238,11 @@ pw_status pw_csd_get_padding(const pw_csd* h, int* Nz);
  *     the FFT paths, the tensor cores for the dense contractions (N <= 256; FP32 above).
  *   PW_DFT_FP32: FP32 on the CUDA cores everywhere (codelets with FP64-derived twiddles, dense FP32
  *     complex products).
- *   PW_DFT_TC_BF16X3: the products as GEMMs on the tensor cores (tcgen05, BF16 operands,
- *     FP32 accumulation in tensor memory), each FP32 operand split into three BF16 parts and six
- *     partial products kept (relative error ~5e-7 per stage).
+ *   PW_DFT_TC_BF16X3: the products as GEMMs on the tensor cores (tcgen05, FP32 accumulation in tensor
+ *     memory) with each FP32 operand split into 16-bit parts: at N = 256 on the FFT path three BF16
+ *     parts and six partial products (relative error ~5e-7 per stage), in the dense contractions two
+ *     FP16 parts of operands scaled by powers of two and three partial products (2e-6 to 3e-6 of W over
+ *     a whole propagation, the error of the accumulation).
  * Returns PW_EINVAL for an unknown mode, PW_EUNSUPPORTED for PW_DFT_TC_BF16X3 at N > 256.  On the
  * FFT path at N = 256 a later propagation of a source other than the Gaussian Schell model
  * returns PW_EUNSUPPORTED while the tensor-core mode is set; at other FFT grid sizes the mode has

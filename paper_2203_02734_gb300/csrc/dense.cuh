@@ -31,12 +31,14 @@ struct TabArgs {
   double Kin;   // turns per n^2 of the input propagator (0 for the far field)
   double Kout;  // turns per k^2 of the output propagator
   float2* E;    // N x N, row k (output), column n (input)
+  unsigned* max;  // 8 magnitude slots of the tensor-core contractions, zeroed here
 };
 
 // E(k, n) in FP64 turns: Kout (k-M)^2 - ((k-M)(n-M) mod Nz) / Nz + Kin (n-M)^2, M = N/2.
 __global__ void tables_kernel(TabArgs t) {
   const int N = t.N, M = N / 2;
   const int NN = N * N;
+  if (blockIdx.x == 0 && threadIdx.x < 8) t.max[threadIdx.x] = 0u;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < NN; idx += gridDim.x * blockDim.x) {
     const int k = idx / N, n = idx - k * N;
     const long long pk = k - M, pn = n - M;
@@ -58,6 +60,7 @@ struct SrcArgs {
   const float* diag;    // N x N diagonal (SRC_DIAG)
   float A;              // GSM amplitude or diagonal weight
   float2* W;            // output, N^4
+  unsigned* max;        // SRC_DIAG, tensor cores: bits of the largest component, or nullptr
 };
 
 __global__ void source_kernel(SrcArgs s) {
@@ -74,6 +77,7 @@ __global__ void source_kernel(SrcArgs s) {
       v = cmul(cmul(m1, s.W0[idx]), m2);
     } else {
       v = (a == c && b == d) ? cscale(cmul(m1, m2), s.A * s.diag[ab]) : make_float2(0.f, 0.f);
+      if (s.max && a == c && b == d) atomicMax(s.max, __float_as_uint(fmaxf(fabsf(v.x), fabsf(v.y))));
     }
     s.W[idx] = v;
   }
@@ -95,15 +99,6 @@ struct AxisArgs {
   const float2* in;
   float2* out;
   float* S;
-  int stall;  // failure-detection test (0 = off): CTA 0 of the tensor-core kernel never copies operand chunk
-              // `stall` (> 0), or never announces A tile -stall (< 0)
-  // Tensor-core kernel, first contraction (L = 1) of a GSM source: gen != 0 builds the input
-  // W0(a, b, c, d) = A conj(M0(a, b)) G(a, c) G(b, d) M0(c, d) in the converters instead of reading
-  // `in` (source_kernel is then not run).
-  int gen;
-  const float* G;
-  const float2* M0;
-  float A;
 };
 
 constexpr int BM = 64, BN = 64, BK = 16, PITCH = 66, NT = 256;

@@ -86,6 +86,7 @@ struct pw_csd {
   float2* Ein;    // per-axis input factors
   float* S;       // S of the last propagated plane (pass-B epilogue)
   int* err;       // device flag: a bounded wait in a kernel gave up
+  unsigned* maxes;  // dense path: bits of the largest input component of each contraction (8 slots)
   // adjoint scratch (O(N^2)): the adjoint source (diagonal, P1 row), per-column gradient sums, the
   // GSM factor and far-field factors of the source grid, and a spare gradient triple
   float* adj_d;
@@ -621,27 +622,66 @@ void to_output_plane(pw_csd* h, double dx, bool herm) {
 
 bool has_masks(const pw_csd* h) { return h->aperture > 0.0 || h->lens_f != 0.0 || h->mask != nullptr; }
 
-// Zero padding (Nz > N) or a grid size without an FFT plan: four dense axis contractions
-// (dense.cuh).  W0 is built in W (for a GSM source on the tensor cores, inside the first
-// contraction instead), then d (W -> work), c (work -> W), b (W -> work) and a (work -> W, with the
-// scale and S).  Events as for the FFT passes: the first two contractions count as the first pass.
+// Launches one tensor-core contraction of the dense path.
+cudaError_t launch_axis_tc(const pw::dense_tc::Args& ax, int mode, const unsigned char* q, int* err, cudaStream_t s) {
+  namespace T = pw::dense_tc;
+  static size_t smem_set = 0;  // the limit is raised once per size
+  const size_t smem = T::smem_bytes(ax.N);
+  auto set = [&](auto k) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); };
+  auto all = [&](auto f) -> cudaError_t {
+    cudaError_t e;
+    if ((e = f(T::axis_tc_kernel<2, T::IN_COLS>)) != cudaSuccess || (e = f(T::axis_tc_kernel<2, T::IN_ROWS>)) != cudaSuccess ||
+        (e = f(T::axis_tc_kernel<2, T::IN_MASK>)) != cudaSuccess || (e = f(T::axis_tc_kernel<2, T::IN_PRODUCT>)) != cudaSuccess ||
+        (e = f(T::axis_tc_kernel<3, T::IN_COLS>)) != cudaSuccess || (e = f(T::axis_tc_kernel<3, T::IN_ROWS>)) != cudaSuccess ||
+        (e = f(T::axis_tc_kernel<3, T::IN_MASK>)) != cudaSuccess)
+      return e;
+    return f(T::axis_tc_kernel<3, T::IN_PRODUCT>);
+  };
+  if (smem > smem_set) {
+    const cudaError_t e = all(set);
+    if (e != cudaSuccess) return e;
+    smem_set = smem;
+  }
+  const dim3 grid((unsigned)((ax.ncols + 127) / 128 * T::parts(ax.N)));
+  auto go = [&](auto k) { k<<<grid, T::NT, smem, s>>>(ax, q, err); };
+  const bool two = T::b_buffers(ax.N) == 2;
+  switch (mode) {
+    case T::IN_COLS: two ? go(T::axis_tc_kernel<2, T::IN_COLS>) : go(T::axis_tc_kernel<3, T::IN_COLS>); break;
+    case T::IN_ROWS: two ? go(T::axis_tc_kernel<2, T::IN_ROWS>) : go(T::axis_tc_kernel<3, T::IN_ROWS>); break;
+    case T::IN_MASK: two ? go(T::axis_tc_kernel<2, T::IN_MASK>) : go(T::axis_tc_kernel<3, T::IN_MASK>); break;
+    default: two ? go(T::axis_tc_kernel<2, T::IN_PRODUCT>) : go(T::axis_tc_kernel<3, T::IN_PRODUCT>); break;
+  }
+  return cudaGetLastError();
+}
+
+// Zero padding (Nz > N) or a grid size without an FFT plan: dense axis contractions (dense.cuh).
+//   Tensor cores (dense_tc.cuh), GSM source: the tables H and T (in W), then d (-> work) and a (-> W, with
+//     the scale and S).  Other sources: d (masks applied on the way in), c, b, a, alternating between
+//     work and W.
+//   CUDA cores: W0 is built in W, then d (W -> work), c (work -> W), b (W -> work) and a (work -> W).
+// Events as for the FFT passes: the first half of the contractions counts as the first pass.
 pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   const int N = h->N, Nz = h->Nz > 0 ? h->Nz : N;
   pw_status st = build_tables(h, z, farfield);  // G and M0 (the FFT factors are not used here)
   if (st != PW_OK) return st;
   const double d = h->d, lz = h->lambda * z, dx = lz / (Nz * d);
+  cudaStream_t s = h->stream;
   cudaEvent_t* ev = nullptr;
-  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) ev = &h->events[4 * h->timed++];
+  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) {
+    h->three[h->timed] = 0;
+    ev = &h->events[4 * h->timed++];
+  }
   cudaError_t e = cudaSuccess;
-  if (ev && (e = cudaEventRecord(ev[0], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+  if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return cuda_fail(e, "event record");
   pw::dense::TabArgs t{};
   t.N = N;
   t.Nz = Nz;
   t.Kin = farfield ? 0.0 : d * d / (2.0 * lz);
   t.Kout = dx * dx / (2.0 * lz);
   t.E = h->F;  // the FFT input factor's storage (N x N complex) holds E on this path
+  t.max = h->maxes;
   const int NN = N * N;
-  pw::dense::tables_kernel<<<(NN + 255) / 256, 256, 0, h->stream>>>(t);
+  pw::dense::tables_kernel<<<(NN + 255) / 256, 256, 0, s>>>(t);
   pw::dense::SrcArgs sa{};
   sa.N = N;
   sa.mode = h->kind == SRC_GSM ? pw::SRC_GSM : (h->kind == SRC_DIAGONAL ? pw::SRC_DIAG : pw::SRC_ARRAY);
@@ -652,83 +692,115 @@ pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   sa.A = (float)h->A;
   sa.W = reinterpret_cast<float2*>(h->W);
   const bool tc = h->dft_mode != PW_DFT_FP32 && N <= pw::dense_tc::MAX_N;
-  const bool gen = tc && sa.mode == pw::SRC_GSM;  // the first tensor-core contraction builds W0 itself
-  if (!gen) pw::dense::source_kernel<<<num_sms() * 8, 256, 0, h->stream>>>(sa);
-  pw::dense::AxisArgs ax{};
-  ax.G = h->G;
-  ax.M0 = h->M0;
-  ax.A = (float)h->A;
-  ax.N = N;
-  ax.ncols = (long long)N * N * N;
-  ax.E = h->F;
-  ax.S = h->S;
-  const dim3 grid((unsigned)(((ax.ncols + pw::dense::BN - 1) / pw::dense::BN) * ((N + pw::dense::BM - 1) / pw::dense::BM)));
   float2* Wf = reinterpret_cast<float2*>(h->W);
   float2* Xf = reinterpret_cast<float2*>(h->work);
   const long long L[4] = {1, N, (long long)N * N, (long long)N * N * N};
-  if (tc) {  // the split matrices of E (point 2) and conj(E) (point 1), then four tensor-core passes
-    const size_t qb = (size_t)pw::dense_tc::nchunks(N) * pw::dense_tc::chunk_bytes(N);
+  const float scale = (float)((d * d / lz) * (d * d / lz));
+  if (tc) {
+    namespace T = pw::dense_tc;
+    // the split matrices of E (point 2) and conj(E) (point 1)
+    const size_t qb = T::q_bytes(N);
     if (!h->qbuf && (e = cudaMalloc(&h->qbuf, 2 * qb)) != cudaSuccess) return cuda_fail(e, "cudaMalloc of the split DFT matrices");
-    const int abuf = pw::dense_tc::a_buffers(N);
-    const size_t smem = pw::dense_tc::smem_bytes(N, abuf);
-    static size_t smem_set = 0;
-    if (smem > smem_set) {
-      if ((e = cudaFuncSetAttribute(pw::dense_tc::axis_tc_kernel<false, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem)) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(pw::dense_tc::axis_tc_kernel<true, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem)) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(pw::dense_tc::axis_tc_kernel<false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem)) != cudaSuccess ||
-          (e = cudaFuncSetAttribute(pw::dense_tc::axis_tc_kernel<true, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem)) != cudaSuccess)
-        return cuda_fail(e, "shared memory of the tensor-core contraction");
-      smem_set = smem;
-    }
     unsigned char* q = reinterpret_cast<unsigned char*>(h->qbuf);
     for (int cj = 0; cj < 2; ++cj) {
-      pw::dense_tc::QArgs qa{N, h->F, cj, reinterpret_cast<__nv_bfloat16*>(q + cj * qb)};
-      pw::dense_tc::qsplit_kernel<<<num_sms() * 4, 256, 0, h->stream>>>(qa);
+      T::QArgs qa{N, h->F, cj, q + cj * qb};
+      T::qsplit_kernel<<<num_sms() * 4, 256, 0, s>>>(qa);
     }
-    const dim3 tgrid((unsigned)((ax.ncols + 127) / 128));
-    ax.stall = h->stall;  // first contraction only, then cleared
+    unsigned* mx = h->maxes;  // zeroed by tables_kernel
+    T::Args ax{};
+    ax.N = N;
+    ax.scale = 1.0f;
+    ax.vec = 1;
+    const int stall = h->stall;  // first contraction of the N^4 array only, then cleared
     h->stall = 0;
+    if (sa.mode == pw::SRC_GSM) {
+      const size_t N3 = (size_t)N * N * N;
+      T::TableArgs ta{N, h->G, h->M0, (float)h->A, Xf, Xf + N3, mx};
+      T::table_source_kernel<<<num_sms() * 8, 256, 0, s>>>(ta);
+      float2 *H = Wf, *Tt = Wf + N3;
+      ax.L = N;
+      ax.ncols = (long long)NN;
+      ax.in = ta.H0;
+      ax.out = H;
+      ax.max_in = mx;
+      if ((e = launch_axis_tc(ax, T::IN_COLS, q + qb, h->err, s)) != cudaSuccess) return cuda_fail(e, "table contraction");
+      ax.in = ta.T0;
+      ax.out = Tt;
+      ax.max_in = mx + 1;
+      if ((e = launch_axis_tc(ax, T::IN_COLS, q, h->err, s)) != cudaSuccess) return cuda_fail(e, "table contraction");
+      T::table_max_kernel<<<(NN + 255) / 256, 256, 0, s>>>(N, H, Tt, mx + 2);
+      ax.L = 1;
+      ax.ncols = (long long)N3;
+      ax.in = nullptr;
+      ax.H = H;
+      ax.T = Tt;
+      ax.out = Xf;
+      ax.max_in = mx + 2;
+      ax.max_out = mx + 3;
+      ax.stall = stall;
+      if ((e = launch_axis_tc(ax, T::IN_PRODUCT, q, h->err, s)) != cudaSuccess) return cuda_fail(e, "dense contraction");
+      if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return cuda_fail(e, "event record");
+      ax.stall = 0;
+      ax.L = L[3];
+      ax.in = Xf;
+      ax.out = Wf;
+      ax.scale = scale;
+      ax.S = h->S;
+      ax.max_in = mx + 3;
+      ax.max_out = nullptr;
+      if ((e = launch_axis_tc(ax, T::IN_COLS, q + qb, h->err, s)) != cudaSuccess) return cuda_fail(e, "dense contraction");
+    } else {
+      const float2* src = sa.W0;
+      int mode = T::IN_MASK;
+      if (sa.mode == pw::SRC_DIAG) {  // N^2 non-zeros: built in W
+        sa.max = mx;
+        pw::dense::source_kernel<<<num_sms() * 8, 256, 0, s>>>(sa);
+        src = Wf;
+        mode = T::IN_ROWS;
+      } else {
+        T::masked_max_kernel<<<std::min(NN, num_sms() * 8), 256, 0, s>>>(N, src, h->M0, mx);
+      }
+      ax.ncols = (long long)N * NN;
+      ax.M0 = h->M0;
+      for (int pass = 0; pass < 4; ++pass) {
+        ax.L = L[pass];
+        ax.in = pass == 0 ? src : pass % 2 == 0 ? Wf : Xf;
+        ax.vec = aligned(ax.in, 16) ? 1 : 0;
+        ax.out = pass % 2 == 0 ? Xf : Wf;
+        ax.scale = pass == 3 ? scale : 1.0f;
+        ax.S = pass == 3 ? h->S : nullptr;
+        ax.max_in = mx + pass;
+        ax.max_out = pass < 3 ? mx + pass + 1 : nullptr;
+        ax.stall = pass == 0 ? stall : 0;
+        if ((e = launch_axis_tc(ax, pass == 0 ? mode : T::IN_COLS, q + (pass < 2 ? 0 : qb), h->err, s)) != cudaSuccess)
+          return cuda_fail(e, "dense contraction");
+        if (pass == 1 && ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return cuda_fail(e, "event record");
+      }
+    }
+  } else {
+    pw::dense::source_kernel<<<num_sms() * 8, 256, 0, s>>>(sa);
+    pw::dense::AxisArgs ax{};
+    ax.N = N;
+    ax.ncols = (long long)N * NN;
+    ax.E = h->F;
+    ax.S = h->S;
+    const dim3 grid((unsigned)(((ax.ncols + pw::dense::BN - 1) / pw::dense::BN) * ((N + pw::dense::BM - 1) / pw::dense::BM)));
     for (int pass = 0; pass < 4; ++pass) {
       ax.L = L[pass];
       ax.in = pass % 2 == 0 ? Wf : Xf;
       ax.out = pass % 2 == 0 ? Xf : Wf;
-      ax.scale = pass == 3 ? (float)((d * d / lz) * (d * d / lz)) : 1.0f;
-      const unsigned char* qm = q + (pass < 2 ? 0 : qb);
-      if (pass > 0) ax.stall = 0;
-      ax.gen = gen && pass == 0 ? 1 : 0;
-      if (abuf == 2) {
-        if (pass < 3)
-          pw::dense_tc::axis_tc_kernel<false, 2><<<tgrid, pw::dense_tc::NT, smem, h->stream>>>(ax, qm, h->err);
-        else
-          pw::dense_tc::axis_tc_kernel<true, 2><<<tgrid, pw::dense_tc::NT, smem, h->stream>>>(ax, qm, h->err);
-      } else {
-        if (pass < 3)
-          pw::dense_tc::axis_tc_kernel<false, 1><<<tgrid, pw::dense_tc::NT, smem, h->stream>>>(ax, qm, h->err);
-        else
-          pw::dense_tc::axis_tc_kernel<true, 1><<<tgrid, pw::dense_tc::NT, smem, h->stream>>>(ax, qm, h->err);
-      }
-      if (pass == 1 && ev && (e = cudaEventRecord(ev[1], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+      ax.scale = pass == 3 ? scale : 1.0f;
+      if (pass < 2)
+        pw::dense::axis_kernel<false, false><<<grid, pw::dense::NT, 0, s>>>(ax);
+      else if (pass == 2)
+        pw::dense::axis_kernel<true, false><<<grid, pw::dense::NT, 0, s>>>(ax);
+      else
+        pw::dense::axis_kernel<true, true><<<grid, pw::dense::NT, 0, s>>>(ax);
+      if (pass == 1 && ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return cuda_fail(e, "event record");
     }
   }
-  for (int pass = 0; pass < 4 && !tc; ++pass) {
-    ax.L = L[pass];
-    ax.in = pass % 2 == 0 ? Wf : Xf;
-    ax.out = pass % 2 == 0 ? Xf : Wf;
-    ax.scale = pass == 3 ? (float)((d * d / lz) * (d * d / lz)) : 1.0f;
-    if (pass < 2)
-      pw::dense::axis_kernel<false, false><<<grid, pw::dense::NT, 0, h->stream>>>(ax);
-    else if (pass == 2)
-      pw::dense::axis_kernel<true, false><<<grid, pw::dense::NT, 0, h->stream>>>(ax);
-    else
-      pw::dense::axis_kernel<true, true><<<grid, pw::dense::NT, 0, h->stream>>>(ax);
-    if (pass == 1 && ev && (e = cudaEventRecord(ev[1], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
-  }
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "dense propagation launch");
-  if (ev && (e = cudaEventRecord(ev[2], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+  if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return cuda_fail(e, "event record");
   to_output_plane(h, dx, herm);
   return PW_OK;
 }
@@ -1055,6 +1127,7 @@ pw_status pw_csd_create(pw_csd** out, int N, double dxi_m, double lambda_m, pw_c
   h->Ein = reinterpret_cast<float2*>(p);
   p += N * sizeof(float2);
   h->err = reinterpret_cast<int*>(p);
+  h->maxes = reinterpret_cast<unsigned*>(p + 64);
   p += 256;
   auto carve = [&](size_t bytes) {
     char* q = p;
