@@ -130,7 +130,7 @@ template <int CS, int SRC, bool MASK, bool TC = false>
 __global__ void __launch_bounds__(Geo<CS>::NT, Geo<CS>::MINB)
     pass_a_d256(const __grid_constant__ CUtensorMap vmap, PassAArgs p, const float2* __restrict__ Ein,
                 const float2* __restrict__ mask, int ap_ithr, int* err) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY, DIAG = SRC == SRC_DIAG;
+  constexpr bool ARRAY = SRC == SRC_ARRAY;
   constexpr int RPC = Geo<CS>::RPC, NT = Geo<CS>::NT, HALF = Geo<CS>::HALF;
   static_assert(!TC || NT == 256, "the tensor-core stage maps thread t to vector t of two 128-row tiles");
   extern __shared__ __align__(1024) float2 smem[];
@@ -176,11 +176,8 @@ __global__ void __launch_bounds__(Geo<CS>::NT, Geo<CS>::MINB)
     float2 fab = inside(a, b) ? cmul(ein[a], ein[b]) : make_float2(0.f, 0.f);
     if (MASK) fab = cmul(fab, __ldg(mask + a * N + b));
     float2 s_ab = cconj(fab);
-    if (SRC == SRC_GSM || SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
-    if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
+    if (SRC == SRC_GSM) s_ab = cscale(s_ab, p.A);
     const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
-    AdjSlice adj{};
-    if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
     float2 v[2][16];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -192,9 +189,7 @@ __global__ void __launch_bounds__(Geo<CS>::NT, Geo<CS>::MINB)
         float2 x = cmul(sc, SRC == SRC_GSM ? cscale(ein[d], gB[d]) : ein[d]);
         if (MASK) x = cmul(x, __ldg(mask + c * N + d));
         if (ARRAY) x = cmul(x, __ldg(W0 + (size_t)c * N + d));
-        if (SRC == SRC_ADJ) x = cmul(x, adj.at(p.cross, c * N + d));
         bool keep = inside(c, d);
-        if (DIAG) keep = keep && c == a && d == b;
         v[h][r] = keep ? x : make_float2(0.f, 0.f);
       }
       if (!TC) Dft<16, -1>::run(v[h]);

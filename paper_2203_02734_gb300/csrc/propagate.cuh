@@ -85,51 +85,16 @@ static __global__ void tables_kernel(TableArgs t) {
   }
 }
 
-// Source of pass A: the GSM model, an uploaded CSDA, a diagonal (delta-correlated, incoherent)
-// source W0 = w d(xi1) delta(xi1 - xi2) with d real, or the adjoint source of a loss on S and mu
-// (SRC_ADJ): the diagonal d plus the row of the coherence point P1,
-//   Y(x1, x2) = d(x1) delta(x1 - x2) + delta(x1 - P1) r(x2),
-// completed to its Hermitian part (r halved on the row, conj(r)/2 on the column of P1) when the
-// propagated array must be Hermitian.
-enum SrcMode { SRC_GSM = 0, SRC_ARRAY = 1, SRC_DIAG = 2, SRC_ADJ = 3 };
+// Sources: the GSM model, an uploaded CSDA, and (dense path) a diagonal source.
+enum SrcMode { SRC_GSM = 0, SRC_ARRAY = 1, SRC_DIAG = 2 };
 
 struct PassAArgs {
   const float2* F;
   const float* G;
   const float2* tw;
   const float2* W0;   // uploaded source (SRC_ARRAY) or nullptr
-  const float* diag;  // N x N diagonal (SRC_DIAG, SRC_ADJ) or nullptr
-  float A;            // GSM amplitude, or the weight w of the diagonal / adjoint source
-  const float2* cross;  // SRC_ADJ: N x N row r of P1, or nullptr
-  int iP, jP;           // SRC_ADJ: P1
-  int herm;             // SRC_ADJ: nonzero = Hermitian part (row and column of P1, halved)
+  float A;            // GSM amplitude
 };
-
-// The adjoint source of one slice x1 = ab, evaluated at x2 = cd (SRC_ADJ).
-struct AdjSlice {
-  int ab, p1;
-  float dg;      // d(x1), or 0
-  float2 col;    // conj(r(x1)) / 2 (Hermitian part), or 0
-  bool row;      // x1 == P1: the slice holds the row r
-  float wr;      // weight of the row: 1/2 (Hermitian part) or 1
-  __device__ __forceinline__ float2 at(const float2* __restrict__ cross, int cd) const {
-    float2 v = make_float2(cd == ab ? dg : 0.f, 0.f);
-    if (cd == p1) v = cadd(v, col);
-    if (row) v = cadd(v, cscale(__ldg(cross + cd), wr));
-    return v;
-  }
-};
-
-__device__ __forceinline__ AdjSlice adj_slice(const PassAArgs& p, int ab, int N) {
-  AdjSlice s;
-  s.ab = ab;
-  s.p1 = p.iP * N + p.jP;
-  s.dg = p.diag ? __ldg(p.diag + ab) : 0.f;
-  s.row = p.cross != nullptr && ab == s.p1;
-  s.wr = p.herm ? 0.5f : 1.f;
-  s.col = (p.cross != nullptr && p.herm) ? cscale(cconj(__ldg(p.cross + ab)), 0.5f) : make_float2(0.f, 0.f);
-  return s;
-}
 
 template <int N> __host__ __device__ constexpr int pitch() { return N + 1; }
 // Width g of the d' runs of the V layout: 4 (one 32-byte sector per run; 2 when 4 does not
@@ -155,7 +120,7 @@ template <int N> __host__ __device__ constexpr size_t pass_a_smem() {
   return (size_t)N * pitch<N>() * sizeof(float2) + N * sizeof(float2) + 2 * N * sizeof(float);
 }
 template <int N> __host__ __device__ constexpr size_t pass_b_smem() {
-  return (size_t)N * pitch<N>() * sizeof(float2) + 2 * N * sizeof(float2) + 4 * 32 * sizeof(double);
+  return (size_t)N * pitch<N>() * sizeof(float2) + 2 * N * sizeof(float2);
 }
 
 // ---- bulk asynchronous copies (TMA) issued by one thread, tracked as bulk groups ----
@@ -222,7 +187,7 @@ __device__ __forceinline__ void smem_stages(float2* buf, const float2* tw) {
 // {2g floats, 1, 1, N/g, N} over (d' mod g, b, a, d'/g, c')).
 template <int N, int SRC>
 __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_a_kernel(const __grid_constant__ CUtensorMap vmap, PassAArgs p) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY, DIAG = SRC == SRC_DIAG;
+  constexpr bool ARRAY = SRC == SRC_ARRAY;
   constexpr int NT = Plan<N>::NT, P = pitch<N>(), S = Plan<N>::stages;
   extern __shared__ __align__(1024) float2 smem[];
   float2* buf = smem;
@@ -241,16 +206,11 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_a_kernel(const __grid_con
     }
     __syncthreads();
     float2 s_ab = cconj(__ldg(F + ab));
-    if (SRC == SRC_GSM || SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
-    if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
+    if (SRC == SRC_GSM) s_ab = cscale(s_ab, p.A);
     const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
-    AdjSlice adj{};
-    if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
     auto gen = [&](int d, int c) -> float2 {
       const float2 f = __ldg(F + c * N + d);
       if (ARRAY) return cmul(cmul(s_ab, __ldg(W0 + c * N + d)), f);
-      if (DIAG) return (c * N + d == ab) ? cmul(s_ab, f) : make_float2(0.f, 0.f);
-      if (SRC == SRC_ADJ) return cmul(cmul(s_ab, f), adj.at(p.cross, c * N + d));
       return cscale(cmul(s_ab, f), gA[c] * gB[d]);
     };
     auto st1 = [buf](int d, int c, float2 v) { buf[c * P + d] = v; };
@@ -271,23 +231,6 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_a_kernel(const __grid_con
   if (threadIdx.x == 0) bulk_wait_all();
 }
 
-// Parameter gradients of the amplitude-masked GSM source W0 = A a(x1) a(x2) G(x1, x2) reduced in
-// the epilogue of the adjoint propagation's second pass (W_GRAD): the array R it computes gives
-// conj(W0bar) = c R ff (ff = q(x1) q*(x2) after a far-field forward propagation, else 1), and per
-// output column x2 the kernel adds, over x1, t = Re(R ff) G(x1, x2) a(x1):
-//   part[x2][0] = a(x2) d^2 sum t (r^2(x1) + r^2(x2)),  part[x2][1] = a(x2) d^2 sum t |x1 - x2|^2,
-//   part[x2][2] = a(x2) sum t  (r^2 and |x1 - x2|^2 in pixels^2),  gmask[x2] = gscale sum t,
-// the same per-point sums the standalone gradient kernel forms row by row (R and G symmetric).
-struct GradEpi {
-  const float* gtab;   // N x N GSM axis factor G(i, k), the same table for both axes
-  const float* amask;  // N x N amplitude mask, or nullptr (a = 1)
-  const float2* qff;   // far field: q(x_i) per axis (N entries), or nullptr
-  double* part;        // N^2 x 3 per-column sums
-  float* gmask;        // N^2 mask gradient (4 c A sum t), or nullptr
-  float gscale;        // 4 c A
-  float d2;            // d^2 of the source grid
-};
-
 struct PassBArgs {
   const float2* V;
   const float2* tw;
@@ -295,77 +238,11 @@ struct PassBArgs {
   float2* W;
   float* S;
   float scale;
-  GradEpi gr;    // W_GRAD only
 };
 
 // What pass B stores of the propagated CSDA: the conjugated column as the contiguous row (Hermitian
-// CSDA), every element at its own place, or (W_GRAD) nothing but the GSM parameter-gradient sums of
-// the adjoint.
-enum WStore { W_HERM = 1, W_GENERAL = 2, W_GRAD = 3 };
-
-// W_GRAD epilogue for one column x2 = (c, d).  With R = Re(W_B conj-factors) the per-point terms
-//   t = R G(a, c) G(b, d) m(a, b),  sum t r^2,  sum t |x1 - x2|^2,  sum t
-// are separable in a and b: r^2 = (a-M)^2 + (b-M)^2 + (c-M)^2 + (d-M)^2 and |x1 - x2|^2 =
-// (a-c)^2 + (b-d)^2, so each point-1 index carries its own G factor, squares and output factor
-// (GradAxis), set up once per row / column of the thread; the column's (c-M)^2 + (d-M)^2 enters
-// in grad_reduce.  In the far field W_B is also multiplied by q(a) q(b) conj(q(c) q(d)), folded
-// into the same factors (grad_col for the column part).
-struct GradAxis {
-  float g, r, dd;  // G(a, c), (a - M)^2, (a - c)^2
-  float2 e;        // output factor of this index (times q(a) in the far field)
-};
-__device__ __forceinline__ GradAxis grad_axis(const GradEpi& g, int N, int a, int c, float2 e) {
-  GradAxis x;
-  x.g = __ldg(g.gtab + a * N + c);
-  const float m = (float)(a - N / 2), dd = (float)(a - c);
-  x.r = m * m;
-  x.dd = dd * dd;
-  x.e = g.qff ? cmul(e, __ldg(g.qff + a)) : e;
-  return x;
-}
-// the column factor s E(c) E(d) (times conj(q(c) q(d)) in the far field)
-__device__ __forceinline__ float2 grad_col(const GradEpi& g, int c, int d, float2 ecd) {
-  return g.qff ? cmul(ecd, cconj(cmul(__ldg(g.qff + c), __ldg(g.qff + d)))) : ecd;
-}
-struct GradSums {
-  float sS = 0.f, sM = 0.f, sA = 0.f;  // sS without the column's (c-M)^2 + (d-M)^2 (grad_reduce)
-  // transform value y at x1 = (a, b) (axis factors A of a, B of b; m = mask value m(a, b))
-  __device__ __forceinline__ void add(const GradAxis& A, const GradAxis& B, float m, float2 y) {
-    const float2 e = cmul(A.e, B.e);
-    const float t = (e.x * y.x - e.y * y.y) * (A.g * B.g) * m;
-    sS = fmaf(t, A.r + B.r, sS);
-    sM = fmaf(t, A.dd + B.dd, sM);
-    sA += t;
-  }
-};
-__device__ __forceinline__ float grad_mask(const GradEpi& g, int N, int a, int b) {
-  return g.amask ? __ldg(g.amask + a * N + b) : 1.f;
-}
-
-// Block reduction of the W_GRAD sums of column cd (red: 4 x 32 doubles of shared memory); writes
-// part[cd] and gmask[cd].  Every thread of the block must call it.
-__device__ __forceinline__ void grad_reduce(const GradEpi& g, int N, int cd, const GradSums& s, double* red) {
-  const float a2 = g.amask ? __ldg(g.amask + cd) : 1.f;
-  const int c = cd / N, d = cd - c * N;
-  const float rc = (float)((c - N / 2) * (c - N / 2) + (d - N / 2) * (d - N / 2));
-  const float sS = fmaf(rc, s.sA, s.sS);
-  double v[4] = {(double)sS * a2 * g.d2, (double)s.sM * a2 * g.d2, (double)s.sA * a2, (double)s.sA};
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    double x = v[k];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if (lane == 0) red[k * 32 + warp] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    double x = 0.0;
-    for (int w = 0; w < nw; ++w) x += red[threadIdx.x * 32 + w];
-    if (threadIdx.x < 3) g.part[(size_t)cd * 3 + threadIdx.x] = x;
-    else if (g.gmask) g.gmask[cd] = (float)(g.gscale * x);
-  }
-  __syncthreads();
-}
+// CSDA) or every element at its own place.
+enum WStore { W_HERM = 1, W_GENERAL = 2 };
 
 // Pass B, persistent: CTA blockIdx.x handles point-2 output pairs cd = blockIdx.x + k gridDim.x.
 // Per slice: gather V(., ., c', d') + DFT along a (lanes along b), DFT along b with the
@@ -380,7 +257,6 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_b_kernel(PassBArgs p) {
   float2* buf = smem;
   float2* tw = buf + N * P;
   float2* eo = tw + N;
-  double* red = reinterpret_cast<double*>(eo + N);  // W_GRAD: block reduction
   for (int i = threadIdx.x; i < N; i += NT) {
     tw[i] = p.tw[i];
     eo[i] = p.Eout[i];
@@ -424,22 +300,12 @@ __global__ void __launch_bounds__(Plan<N>::NT, 1) pass_b_kernel(PassBArgs p) {
         bulk_store(p.W + (size_t)cd * NN, buf, (unsigned)(NN * sizeof(float2)));
         bulk_commit();
       }
-    } else if constexpr (WST == W_GRAD) {
-      GradSums gs;
-      const GradEpi& ge = p.gr;
-      const float2 ecg = grad_col(ge, c, d, ecd);
-      auto epi = [&](int a, int b, float2 y) {
-        gs.add(grad_axis(ge, N, a, c, cmul(cconj(eo[a]), ecg)), grad_axis(ge, N, b, d, cconj(eo[b])),
-               grad_mask(ge, N, a, b), y);
-      };
-      fft_stage<N, StageInfo<N, S - 1>::R, StageInfo<N, S - 1>::NS, +1, true, NT>(tw, ld0, NoMid{}, epi);
-      grad_reduce(ge, N, cd, gs, red);
     } else {
       float2* W = p.W;
       auto epi = [=](int a, int b, float2 y) {
         const float2 w = cmul(cmul(cconj(cmul(eo[a], eo[b])), ecd), y);
         if (a == c && b == d) Sd[cd] = w.x;
-        if (WST == W_GENERAL) W[(size_t)(a * N + b) * NN + cd] = w;
+        W[(size_t)(a * N + b) * NN + cd] = w;
       };
       fft_stage<N, StageInfo<N, S - 1>::R, StageInfo<N, S - 1>::NS, +1, true, NT>(tw, ld0, NoMid{}, epi);
     }

@@ -20,6 +20,7 @@
 #include "dense.cuh"
 #include "dense_tc.cuh"
 #include "t256.cuh"
+#include "delta.cuh"
 #include "grad.cuh"
 #include "plane.cuh"
 #include "r128.cuh"
@@ -50,8 +51,7 @@ bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
 // complex values (masks, uploaded arrays, mu) or floats (S, diagonals).
 bool aligned(const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
-// SRC_ADJOINT: the adjoint source of a loss on S and mu, set only inside the adjoint calls.
-enum SourceKind { SRC_NONE = 0, SRC_GSM = 1, SRC_ARRAY = 2, SRC_PROPAGATED = 3, SRC_DIAGONAL = 4, SRC_ADJOINT = 5 };
+enum SourceKind { SRC_NONE = 0, SRC_GSM = 1, SRC_ARRAY = 2, SRC_PROPAGATED = 3, SRC_DIAGONAL = 4 };
 
 }  // namespace
 
@@ -87,7 +87,7 @@ struct pw_csd {
   float* S;       // S of the last propagated plane (pass-B epilogue)
   int* err;       // device flag: a bounded wait in a kernel gave up
   unsigned* maxes;  // dense path: bits of the largest input component of each contraction (8 slots)
-  // adjoint scratch (O(N^2)): the adjoint source (diagonal, P1 row), per-column gradient sums, the
+  // adjoint scratch (O(N^2)): the adjoint source (diagonal, P1 row), partial sums, the
   // GSM factor and far-field factors of the source grid, and a spare gradient triple
   float* adj_d;
   float2* adj_c;
@@ -95,11 +95,6 @@ struct pw_csd {
   float* gtab;
   float2* qtab;
   double* g3tmp;
-  // the adjoint source of the next propagation (kind == SRC_ADJOINT)
-  int adj_herm;     // Hermitian part (row and column of P1) or the general array (row only)
-  int adj_mu;       // the source has a P1 row (a mu term)
-  int adj_iP, adj_jP;
-  const pw::GradEpi* adj_grad;  // non-null: reduce the GSM parameter gradients in pass B (W_GRAD)
   CUtensorMap vmap;  // TMA map of the work buffer in the V layout
   CUtensorMap ymap;  // N = 256: the second pass's tiles of the work buffer
   CUtensorMap y3map;  // N = 256: the third pass's tiles of the work buffer
@@ -159,18 +154,18 @@ cudaError_t persistent_grid(K kernel, int threads, size_t smem, int slices, int*
   return cudaSuccess;
 }
 
-template <int N, int SRC>
+template <int N>
 cudaError_t launch_a(const CUtensorMap& vmap, const pw::PassAArgs& a, cudaStream_t s) {
   constexpr size_t smem = pw::pass_a_smem<N>();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::pass_a_kernel<N, SRC>,
+    cudaError_t e = cudaFuncSetAttribute(pw::pass_a_kernel<N, pw::SRC_ARRAY>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::pass_a_kernel<N, SRC>, pw::Plan<N>::NT, smem, N * N, &grid);
+    e = persistent_grid(pw::pass_a_kernel<N, pw::SRC_ARRAY>, pw::Plan<N>::NT, smem, N * N, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::pass_a_kernel<N, SRC><<<grid, pw::Plan<N>::NT, smem, s>>>(vmap, a);
+  pw::pass_a_kernel<N, pw::SRC_ARRAY><<<grid, pw::Plan<N>::NT, smem, s>>>(vmap, a);
   return cudaGetLastError();
 }
 
@@ -180,68 +175,65 @@ struct R128Extra {
   const float2* mask;
   int ap_ithr;
   int* err;
-  int dft_tc;  // N = 256: first stage of the first pass on the tensor cores
 };
 
-template <int SRC, bool MASK>
+template <bool MASK>
 cudaError_t launch_a_r128(const CUtensorMap& vmap, const pw::PassAArgs& a, const R128Extra& x, cudaStream_t s) {
   constexpr size_t smem = pw::r128::pass_a_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_a_r128<SRC, MASK>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_a_r128<MASK>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r128::pass_a_r128<SRC, MASK>, pw::r128::NT, smem, 128 * 128, &grid);
+    e = persistent_grid(pw::r128::pass_a_r128<MASK>, pw::r128::NT, smem, 128 * 128, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r128::pass_a_r128<SRC, MASK><<<grid, pw::r128::NT, smem, s>>>(vmap, a, x.Ein, x.mask, x.ap_ithr);
+  pw::r128::pass_a_r128<MASK><<<grid, pw::r128::NT, smem, s>>>(vmap, a, x.Ein, x.mask, x.ap_ithr);
   return cudaGetLastError();
 }
 
-// N = 128, Hermitian store or none: register-resident pass B with prefetched gather (r128.cuh).
-template <int WST>
+// N = 128, Hermitian store: register-resident pass B with prefetched gather (r128.cuh).
 cudaError_t launch_b_r128(const pw::PassBArgs& b, cudaStream_t s) {
   constexpr size_t smem = pw::r128::pass_b_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_b_r128<WST>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r128::pass_b_r128,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r128::pass_b_r128<WST>, pw::r128::NT, smem, 128 * 128, &grid);
+    e = persistent_grid(pw::r128::pass_b_r128, pw::r128::NT, smem, 128 * 128, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r128::pass_b_r128<WST><<<grid, pw::r128::NT, smem, s>>>(b);
+  pw::r128::pass_b_r128<<<grid, pw::r128::NT, smem, s>>>(b);
   return cudaGetLastError();
 }
 
 // N = 96: register-resident passes (r96.cuh), two CTAs per SM.
-template <int SRC, bool MASK>
+template <bool MASK>
 cudaError_t launch_a_r96(const CUtensorMap& vmap, const pw::PassAArgs& a, const R128Extra& x, cudaStream_t s) {
   constexpr size_t smem = pw::r96::pass_a_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_a_r96<SRC, MASK>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_a_r96<MASK>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r96::pass_a_r96<SRC, MASK>, pw::r96::NT, smem, 96 * 96, &grid);
+    e = persistent_grid(pw::r96::pass_a_r96<MASK>, pw::r96::NT, smem, 96 * 96, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r96::pass_a_r96<SRC, MASK><<<grid, pw::r96::NT, smem, s>>>(vmap, a, x.Ein, x.mask, x.ap_ithr);
+  pw::r96::pass_a_r96<MASK><<<grid, pw::r96::NT, smem, s>>>(vmap, a, x.Ein, x.mask, x.ap_ithr);
   return cudaGetLastError();
 }
 
-template <int WST>
 cudaError_t launch_b_r96(const pw::PassBArgs& b, cudaStream_t s) {
   constexpr size_t smem = pw::r96::pass_b_smem();
   static int grid = 0;
   if (grid == 0) {
-    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_b_r96<WST>,
+    cudaError_t e = cudaFuncSetAttribute(pw::r96::pass_b_r96,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    e = persistent_grid(pw::r96::pass_b_r96<WST>, pw::r96::NT, smem, 96 * 96, &grid);
+    e = persistent_grid(pw::r96::pass_b_r96, pw::r96::NT, smem, 96 * 96, &grid);
     if (e != cudaSuccess) return e;
   }
-  pw::r96::pass_b_r96<WST><<<grid, pw::r96::NT, smem, s>>>(b);
+  pw::r96::pass_b_r96<<<grid, pw::r96::NT, smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -292,23 +284,24 @@ cudaError_t launch_clusters(K kernel, int cs, int threads, size_t smem, int* gri
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-template <int SRC, bool MASK, bool TC = false>
+// N = 256, GSM source, first stage on the tensor cores: the comparison mode.
+template <bool MASK>
 cudaError_t launch_a_d256(const CUtensorMap& vmap, const pw::PassAArgs& a, const R128Extra& x, cudaStream_t s) {
   static int grid = 0;
   constexpr int CS = pw::d256::CLUSTER_A;
-  if (TC && grid == 0) {
+  if (grid == 0) {
     // The occupancy calculator fits one CTA per SM for a kernel that uses tensor memory (15
     // clusters of 8 instead of 36, measured). This one allocates 128 of an SM's 512 columns and
     // has the registers, threads and shared memory of its FP32 twin, which caps residency at two
     // CTAs per SM, so it takes the twin's grid (two per SM co-resident, measured: 53.8 -> 32.3 ms).
-    cudaError_t e = cudaFuncSetAttribute(pw::d256::pass_a_d256<CS, SRC, MASK, TC>,
+    cudaError_t e = cudaFuncSetAttribute(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw::d256::pass_a_smem<CS>());
     if (e != cudaSuccess) return e;
-    e = cluster_capacity(pw::d256::pass_a_d256<CS, SRC, MASK, false>, CS, pw::d256::Geo<CS>::NT,
+    e = cluster_capacity(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, false>, CS, pw::d256::Geo<CS>::NT,
                          pw::d256::pass_a_smem<CS>(), &grid);
     if (e != cudaSuccess) return e;
   }
-  return launch_clusters(pw::d256::pass_a_d256<CS, SRC, MASK, TC>, CS, pw::d256::Geo<CS>::NT,
+  return launch_clusters(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, true>, CS, pw::d256::Geo<CS>::NT,
                          pw::d256::pass_a_smem<CS>(), &grid, s, vmap, a, x.Ein, x.mask, x.ap_ithr, x.err);
 }
 
@@ -334,91 +327,36 @@ cudaError_t launch_b(const pw::PassBArgs& b, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// ev: nullptr or three events recorded before pass A, between the passes and after pass B.
-// Pass A of the source mode `src` (pw::SrcMode) on the engine for N.
-template <int N, int SRC>
-cudaError_t launch_a_mode(const CUtensorMap& vmap, const pw::PassAArgs& a, const R128Extra& x, cudaStream_t s) {
-  if constexpr (N == 128) {
-    return x.mask ? launch_a_r128<SRC, true>(vmap, a, x, s) : launch_a_r128<SRC, false>(vmap, a, x, s);
-  } else if constexpr (N == 96) {
-    return x.mask ? launch_a_r96<SRC, true>(vmap, a, x, s) : launch_a_r96<SRC, false>(vmap, a, x, s);
-  } else if constexpr (N == 256) {
-    if (x.dft_tc) {
-      if constexpr (SRC == pw::SRC_GSM)
-        return x.mask ? launch_a_d256<SRC, true, true>(vmap, a, x, s) : launch_a_d256<SRC, false, true>(vmap, a, x, s);
-      else
-        return cudaErrorNotSupported;
-    }
-    return x.mask ? launch_a_d256<SRC, true>(vmap, a, x, s) : launch_a_d256<SRC, false>(vmap, a, x, s);
-  } else {
-    return launch_a<N, SRC>(vmap, a, s);
-  }
-}
-
-// Pass A of a source with at most one or two points per slice: the adjoint source (SRC_ADJ) and
-// the delta-correlated source (SRC_DIAG, the adjoint form's diagonal term with the source's d and
-// weight).  At N <= 128 (V layout with runs of 4) V is written directly (grad.cuh: adj_row_kernel
-// for the P1 row of a mu term, then adj_direct_kernel); elsewhere the engine's pass A.
-template <int N, int SRC>
-cudaError_t launch_a_sparse(const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
-                            const R128Extra& x, cudaStream_t s) {
-  if constexpr (N >= 16 && N <= 128 && pw::vgroup<N>() == 4) {
-    if (SRC == pw::SRC_DIAG && a.cross) return cudaErrorInvalidValue;  // a diagonal source has no row
-    float2* V = const_cast<float2*>(b.V);
-    if (a.cross) {
-      pw::adj_row_kernel<N><<<N, N, 0, s>>>(a, V);
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
-    }
-    constexpr int nt = pw::adj_nt<N>(), rows = N * (N / 4) * N;
-    pw::adj_direct_kernel<N><<<std::min(rows, num_sms() * (2048 / nt)), nt, 0, s>>>(a, V);
-    return cudaGetLastError();
-  } else {
-    return launch_a_mode<N, SRC>(vmap, a, x, s);
-  }
-}
-
-// ev: nullptr or three events recorded before pass A, between the passes and after pass B.
-// grad: pass B reduces the GSM parameter gradients of an adjoint propagation (W_GRAD) instead of
-// storing W.
+// The two general passes of an uploaded or propagated array (N <= 128), or at N = 256 of a GSM source in the
+// tensor-core comparison mode.  ev: nullptr or three events recorded before pass A, between the
+// passes and after pass B.
 template <int N>
-cudaError_t launch_passes(int src, bool herm, bool grad, const CUtensorMap& vmap, const pw::PassAArgs& a,
-                          const pw::PassBArgs& b, const R128Extra& x, cudaStream_t s, cudaEvent_t* ev) {
+cudaError_t launch_passes(bool herm, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
+                          const R128Extra& x, cudaStream_t s, cudaEvent_t* ev) {
   cudaError_t e;
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  if (src == pw::SRC_GSM) {  // the tensor-core comparison mode only (plane.cuh runs the others)
-    if constexpr (N == 256) e = launch_a_mode<N, pw::SRC_GSM>(vmap, a, x, s);
-    else e = cudaErrorNotSupported;
-  } else if (src == pw::SRC_DIAG) e = launch_a_sparse<N, pw::SRC_DIAG>(vmap, a, b, x, s);
-  else if (src == pw::SRC_ADJ) e = launch_a_sparse<N, pw::SRC_ADJ>(vmap, a, b, x, s);
-  else e = launch_a_mode<N, pw::SRC_ARRAY>(vmap, a, x, s);
+  if constexpr (N == 256) e = x.mask ? launch_a_d256<true>(vmap, a, x, s) : launch_a_d256<false>(vmap, a, x, s);
+  else if constexpr (N == 128) e = x.mask ? launch_a_r128<true>(vmap, a, x, s) : launch_a_r128<false>(vmap, a, x, s);
+  else if constexpr (N == 96) e = x.mask ? launch_a_r96<true>(vmap, a, x, s) : launch_a_r96<false>(vmap, a, x, s);
+  else e = launch_a<N>(vmap, a, s);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
-  if (grad) {
-    if constexpr (N == 128) e = launch_b_r128<pw::W_GRAD>(b, s);
-    else if constexpr (N == 96) e = launch_b_r96<pw::W_GRAD>(b, s);
-    else if constexpr (N == 256) e = cudaErrorNotSupported;
-    else e = launch_b<N, pw::W_GRAD>(b, s);
-  } else if constexpr (N == 128) {
-    e = herm ? launch_b_r128<pw::W_HERM>(b, s) : launch_b<N, pw::W_GENERAL>(b, s);
-  } else if constexpr (N == 96) {
-    e = herm ? launch_b_r96<pw::W_HERM>(b, s) : launch_b<N, pw::W_GENERAL>(b, s);
-  } else if constexpr (N == 256) {
-    e = herm ? launch_b_d256(b, s) : cudaErrorNotSupported;
-  } else {
-    e = herm ? launch_b<N, pw::W_HERM>(b, s) : launch_b<N, pw::W_GENERAL>(b, s);
-  }
+  if constexpr (N == 256) e = launch_b_d256(b, s);
+  else if (!herm) e = launch_b<N, pw::W_GENERAL>(b, s);
+  else if constexpr (N == 128) e = launch_b_r128(b, s);
+  else if constexpr (N == 96) e = launch_b_r96(b, s);
+  else e = launch_b<N, pw::W_HERM>(b, s);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
-cudaError_t dispatch(int N, int src, bool herm, bool grad, const CUtensorMap& vmap, const pw::PassAArgs& a,
-                     const pw::PassBArgs& b, const R128Extra& x, cudaStream_t s, cudaEvent_t* ev) {
+cudaError_t dispatch(int N, bool herm, const CUtensorMap& vmap, const pw::PassAArgs& a, const pw::PassBArgs& b,
+                     const R128Extra& x, cudaStream_t s, cudaEvent_t* ev) {
   switch (N) {
 #define PW_CASE(NN) \
   case NN:          \
-    return launch_passes<NN>(src, herm, grad, vmap, a, b, x, s, ev);
+    return launch_passes<NN>(herm, vmap, a, b, x, s, ev);
     PW_CASE(2) PW_CASE(4) PW_CASE(6) PW_CASE(8) PW_CASE(12) PW_CASE(16) PW_CASE(24)
     PW_CASE(32) PW_CASE(48) PW_CASE(64) PW_CASE(96) PW_CASE(128) PW_CASE(256)
 #undef PW_CASE
@@ -620,6 +558,13 @@ void to_output_plane(pw_csd* h, double dx, bool herm) {
   h->mask = nullptr;
 }
 
+// The next recorded propagation's events, or nullptr.
+cudaEvent_t* next_events(pw_csd* h) {
+  if (h->events.empty() || (size_t)(4 * (h->timed + 1)) > h->events.size()) return nullptr;
+  h->three[h->timed] = 0;
+  return &h->events[4 * h->timed++];
+}
+
 bool has_masks(const pw_csd* h) { return h->aperture > 0.0 || h->lens_f != 0.0 || h->mask != nullptr; }
 
 // Launches one tensor-core contraction of the dense path.
@@ -666,11 +611,7 @@ pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   if (st != PW_OK) return st;
   const double d = h->d, lz = h->lambda * z, dx = lz / (Nz * d);
   cudaStream_t s = h->stream;
-  cudaEvent_t* ev = nullptr;
-  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) {
-    h->three[h->timed] = 0;
-    ev = &h->events[4 * h->timed++];
-  }
+  cudaEvent_t* ev = next_events(h);
   cudaError_t e = cudaSuccess;
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return cuda_fail(e, "event record");
   pw::dense::TabArgs t{};
@@ -805,28 +746,17 @@ pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   return PW_OK;
 }
 
-// N = 256, three streaming passes (t256.cuh): the source with the point-2 DFT over (m, d) into the
+// N = 256, three streaming passes (t256.cuh): the array with the point-2 DFT over (m, d) into the
 // work buffer, the radix-4 over r and the DFT over b in place there, the DFT over a with the output
-// factors and S from the work buffer into W.  Any source but the GSM model (Hermitian or not; an uploaded W0 may be W
+// factors and S from the work buffer into W.  Uploaded and propagated arrays (Hermitian or not; W0 may be W
 // itself, since the first pass writes only the work buffer).  Events: the first pass, then the
 // second and third apart.
 pw_status propagate_t256(pw_csd* h, double z, bool herm) {
   namespace T = pw::t256;
-  const int src = h->kind == SRC_DIAGONAL ? pw::SRC_DIAG : h->kind == SRC_ADJOINT ? pw::SRC_ADJ : pw::SRC_ARRAY;
   pw::PassAArgs a{};
   a.F = h->F;
   a.tw = h->tw;
-  a.W0 = src == pw::SRC_ARRAY ? reinterpret_cast<const float2*>(h->kind == SRC_PROPAGATED ? h->W : h->W0) : nullptr;
-  a.diag = h->diag;
-  a.A = (float)h->A;
-  if (src == pw::SRC_ADJ) {
-    a.diag = h->adj_d;
-    a.cross = h->adj_mu ? h->adj_c : nullptr;
-    a.iP = h->adj_iP;
-    a.jP = h->adj_jP;
-    a.herm = h->adj_herm;
-    a.A = 1.0f;
-  }
+  a.W0 = reinterpret_cast<const float2*>(h->kind == SRC_PROPAGATED ? h->W : h->W0);
   pw::PassBArgs b{};
   b.tw = h->tw;
   b.Eout = h->Eout;
@@ -836,19 +766,10 @@ pw_status propagate_t256(pw_csd* h, double z, bool herm) {
   b.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
   static int g2 = 0, g3 = 0;
   cudaError_t e = cudaSuccess;
-  // one 512-thread CTA per SM; the shared-memory limit is raised once per source mode
-  auto kernel1 = [&](auto k, bool& ready) -> cudaError_t {
-    if (!ready) {
-      cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::pass1_smem());
-      if (r != cudaSuccess) return r;
-      ready = true;
-    }
-    k<<<num_sms(), T::NT1, T::pass1_smem(), h->stream>>>(h->y1map, a);
-    return cudaGetLastError();
-  };
-  static bool ready1[4] = {false, false, false, false};
   if (g2 == 0) {
-    if ((e = cudaFuncSetAttribute(T::pass2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(T::pass1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)T::pass1_smem())) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(T::pass2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)T::pass2_smem())) != cudaSuccess ||
         (e = cudaFuncSetAttribute(T::pass3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)T::pass3_smem())) != cudaSuccess ||
@@ -862,11 +783,8 @@ pw_status propagate_t256(pw_csd* h, double z, bool herm) {
     ev = &h->events[4 * h->timed++];
   }
   if (ev && (e = cudaEventRecord(ev[0], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
-  switch (src) {
-    case pw::SRC_DIAG: e = kernel1(T::pass1_kernel<pw::SRC_DIAG>, ready1[pw::SRC_DIAG]); break;
-    case pw::SRC_ADJ: e = kernel1(T::pass1_kernel<pw::SRC_ADJ>, ready1[pw::SRC_ADJ]); break;
-    default: e = kernel1(T::pass1_kernel<pw::SRC_ARRAY>, ready1[pw::SRC_ARRAY]); break;
-  }
+  T::pass1_kernel<<<num_sms(), T::NT1, T::pass1_smem(), h->stream>>>(h->y1map, a);  // one CTA per SM
+  e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "first-pass launch (N = 256)");
   if (ev && (e = cudaEventRecord(ev[1], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
   T::pass2_kernel<<<g2, T::NT2, T::pass2_smem(), h->stream>>>(h->ymap, h->tw, reinterpret_cast<float2*>(h->work), h->err);
@@ -882,11 +800,7 @@ pw_status propagate_t256(pw_csd* h, double z, bool herm) {
 // GSM sources, plane by plane (plane.cuh).  The work buffer holds the two tables.  Events: the tables
 // (at N = 256 with the row pass) as the first pass, the planes (the column pass) as the second.
 pw_status propagate_planes(pw_csd* h, double z) {
-  cudaEvent_t* ev = nullptr;
-  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) {
-    h->three[h->timed] = 0;
-    ev = &h->events[4 * h->timed++];
-  }
+  cudaEvent_t* ev = next_events(h);
   const double lz = h->lambda * z;
   PlaneArgs q{};
   q.F = h->F;
@@ -904,13 +818,54 @@ pw_status propagate_planes(pw_csd* h, double z) {
   return PW_OK;
 }
 
+// Tables of a sparse source (delta.cuh) into the work buffer: D, and with a row al and be.
+cudaError_t delta_tables(pw_csd* h, pw::delta::TabArgs& t) {
+  const int N = h->N, G = pw::delta::table_groups(N);
+  const size_t NN = (size_t)N * N;
+  t.N = N;
+  t.F = h->F;
+  t.tw = h->tw;
+  t.Eout = h->Eout;
+  t.D = reinterpret_cast<float2*>(h->work);
+  t.al = t.D + NN;
+  t.be = t.al + NN;
+  pw::delta::tables_kernel<<<dim3(N, t.cross ? 2 : 1), N * G, (size_t)(G + 1) * N * sizeof(float2), h->stream>>>(t, G);
+  return cudaGetLastError();
+}
+
+cudaError_t delta_write(pw_csd* h, const pw::delta::TabArgs& t, bool cross, bool conj, double kappa, float* S) {
+  const int N = h->N, H = N / 2;
+  const pw::delta::WriteArgs w{N, t.Eout, t.q, t.D, t.al, t.be, (float)kappa, reinterpret_cast<float2*>(h->W), S};
+  const int grid = std::min(N * N, num_sms() * 8), nt = 256 / H * H;
+  if (cross && conj) pw::delta::write_kernel<true, true><<<grid, nt, 0, h->stream>>>(w);
+  else if (conj) pw::delta::write_kernel<false, true><<<grid, nt, 0, h->stream>>>(w);
+  else pw::delta::write_kernel<false, false><<<grid, nt, 0, h->stream>>>(w);
+  return cudaGetLastError();
+}
+
+// A delta-correlated source: W depends on x1 - x2 but for the output factors (delta.cuh).  Events: the table
+// as the first pass, the write as the second.
+pw_status propagate_diagonal(pw_csd* h, double z) {
+  const double lz = h->lambda * z, s = (h->d * h->d / lz) * (h->d * h->d / lz);
+  cudaEvent_t* ev = next_events(h);
+  cudaError_t e;
+  pw::delta::TabArgs t{};
+  t.d = h->diag;
+  t.A = (float)h->A;
+  if (ev && (e = cudaEventRecord(ev[0], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+  if ((e = delta_tables(h, t)) != cudaSuccess) return cuda_fail(e, "table launch (delta-correlated source)");
+  if (ev && (e = cudaEventRecord(ev[1], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+  if ((e = delta_write(h, t, false, false, s, h->S)) != cudaSuccess) return cuda_fail(e, "write launch (delta-correlated source)");
+  if (ev && (e = cudaEventRecord(ev[2], h->stream)) != cudaSuccess) return cuda_fail(e, "event record");
+  to_output_plane(h, lz / (h->N * h->d), true);
+  return PW_OK;
+}
+
 pw_status propagate(pw_csd* h, double z, bool farfield) {
   if (!h) return fail(PW_EINVAL, "null handle");
   if (!finite_pos(z)) return fail(PW_EINVAL, "propagation distance must be finite and > 0 (got %g)", z);
   if (h->kind == SRC_NONE) return fail(PW_ESTATE, "no source set for the current plane");
-  const bool herm = h->kind == SRC_GSM || h->kind == SRC_DIAGONAL || (h->kind == SRC_ADJOINT ? h->adj_herm != 0 : h->hermitian != 0);
-  if (h->kind == SRC_ADJOINT && (h->Nz > 0 || !supported(h->N)))
-    return fail(PW_EUNSUPPORTED, "the adjoint propagation needs an unpadded grid with an FFT plan");
+  const bool herm = h->kind == SRC_GSM || h->kind == SRC_DIAGONAL || h->hermitian != 0;
   if (h->Nz > 0 || !supported(h->N)) return propagate_dense(h, z, farfield, herm);
   if (h->dft_mode == PW_DFT_TC_BF16X3 && h->kind != SRC_GSM)
     return fail(PW_EUNSUPPORTED, "the tensor-core first stage is built for Gaussian Schell-model sources only");
@@ -921,27 +876,16 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
   // less).  The exception is the tensor-core comparison mode at N = 256.
   const bool tc256 = h->N == 256 && h->dft_mode == PW_DFT_TC_BF16X3;
   if (h->kind == SRC_GSM && !tc256) return propagate_planes(h, z);
-  // N = 256: the three streaming passes (t256.cuh), any other source; the cluster engine (d256.cuh) runs
+  if (h->kind == SRC_DIAGONAL) return propagate_diagonal(h, z);
+  // N = 256: the three streaming passes (t256.cuh); the cluster engine (d256.cuh) runs
   // only the comparison mode with the tensor-core first stage
   if (h->N == 256 && !tc256) return propagate_t256(h, z, herm);
-  const int src = h->kind == SRC_GSM ? pw::SRC_GSM
-                  : h->kind == SRC_DIAGONAL ? pw::SRC_DIAG
-                  : h->kind == SRC_ADJOINT ? pw::SRC_ADJ : pw::SRC_ARRAY;
   pw::PassAArgs a{};
   a.F = h->F;
   a.G = h->G;
   a.tw = h->tw;
-  a.W0 = src == pw::SRC_ARRAY ? reinterpret_cast<const float2*>(h->kind == SRC_PROPAGATED ? h->W : h->W0) : nullptr;
-  a.diag = h->diag;
+  a.W0 = tc256 ? nullptr : reinterpret_cast<const float2*>(h->kind == SRC_PROPAGATED ? h->W : h->W0);
   a.A = (float)h->A;
-  if (src == pw::SRC_ADJ) {
-    a.diag = h->adj_d;
-    a.cross = h->adj_mu ? h->adj_c : nullptr;
-    a.iP = h->adj_iP;
-    a.jP = h->adj_jP;
-    a.herm = h->adj_herm;
-    a.A = 1.0f;
-  }
   pw::PassBArgs b{};
   b.V = reinterpret_cast<const float2*>(h->work);
   b.tw = h->tw;
@@ -950,22 +894,17 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
   b.S = h->S;
   const double lz = h->lambda * z;
   b.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
-  cudaEvent_t* ev = nullptr;
-  if (!h->events.empty() && (size_t)(4 * (h->timed + 1)) <= h->events.size()) ev = &h->events[4 * h->timed++];
   R128Extra x{};
   x.Ein = h->Ein;
   x.mask = reinterpret_cast<const float2*>(h->mask);
   x.ap_ithr = -1;
   x.err = h->err;
-  x.dft_tc = h->dft_mode == PW_DFT_TC_BF16X3;
   if (h->aperture > 0.0) {
     const double rp = h->aperture / h->d;
     const double thr = rp * rp;  // the FP64 threshold of the table kernel; r^2 is an integer
     x.ap_ithr = thr >= 2147483647.0 ? 2147483647 : (int)std::floor(thr);
   }
-  const bool grad = src == pw::SRC_ADJ && h->adj_grad != nullptr;
-  if (grad) b.gr = *h->adj_grad;
-  cudaError_t e = dispatch(h->N, src, herm, grad, h->vmap, a, b, x, h->stream, ev);
+  cudaError_t e = dispatch(h->N, herm, h->vmap, a, b, x, h->stream, next_events(h));
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
   to_output_plane(h, lz / (h->N * h->d), herm);
   return PW_OK;
@@ -1406,6 +1345,7 @@ pw_status pw_gsm_gradient(pw_csd* h, double sigma_S_m, double sigma_mu_m, double
   g.gmask = dev_grad_mask;
   // the work buffer is scratch between propagations: partial sums, then the FP64-built tables
   g.part = reinterpret_cast<double*>(h->work);
+  g.rows = N * N;
   g.gtab = reinterpret_cast<float*>(g.part + (size_t)N * N * 3);
   g.qtab = reinterpret_cast<float2*>(g.gtab + (size_t)N * N + (N & 1));
   pw::gsm_gradient_tables<<<(N * N + 255) / 256, 256, 0, h->stream>>>(g);
@@ -1454,7 +1394,22 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
   const double c = std::pow(d / dx, 4);
   cudaStream_t st = h->stream;
 
+  // the handle ends at the source plane, with no source recorded
+  auto done = [&](pw_status r) {
+    h->d = d;
+    h->kind = SRC_NONE;
+    h->W0 = nullptr;
+    h->diag = nullptr;
+    h->aperture = 0.0;
+    h->lens_f = 0.0;
+    h->mask = nullptr;
+    return r;
+  };
+  if (h->dft_mode == PW_DFT_TC_BF16X3)
+    return done(fail(PW_EUNSUPPORTED, "the tensor-core first stage is built for Gaussian Schell-model sources only"));
+
   // the (conjugated) adjoint source on the output plane
+  const int NN = N * N, nprep = (NN + 1023) / 1024;
   pw::AdjPrepArgs pa{};
   pa.N = N;
   pa.iP = a->iP;
@@ -1465,7 +1420,8 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
   pa.mu = reinterpret_cast<const float2*>(a->dev_mu);
   pa.d = h->adj_d;
   pa.cross = h->adj_c;
-  pw::adjoint_prep_kernel<<<1, 1024, 0, st>>>(pa);
+  pa.part = h->gpart;
+  pw::adjoint_prep_kernel<<<nprep, 1024, 0, st>>>(pa);
   // the GSM factor (parameter gradients) and the far-field factors of the source grid
   pw::GradArgs g{};
   g.N = N;
@@ -1473,75 +1429,55 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
   g.sigma_S = params ? a->sigma_S_m : 0.0;
   g.sigma_mu = params ? a->sigma_mu_m : 0.0;
   g.A = a->amplitude;
-  g.amask = a->dev_amask;
-  g.R = reinterpret_cast<const float2*>(h->W);
   g.c = c;
-  g.farfield = farfield ? 1 : 0;
   g.Kq = d * d / (2.0 * lam * z);
   g.part = h->gpart;
   g.gtab = h->gtab;
   g.qtab = h->qtab;
   g.g3 = a->dev_grad3 ? a->dev_grad3 : h->g3tmp;
-  g.gmask = a->dev_grad_amask;
-  pw::gsm_gradient_tables<<<(N * N + 255) / 256, 256, 0, st>>>(g);
+  pw::gsm_gradient_tables<<<(NN + 255) / 256, 256, 0, st>>>(g);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "adjoint set-up launch");
+  if (e != cudaSuccess) return done(cuda_fail(e, "adjoint set-up launch"));
 
-  // one adjoint propagation: a Fresnel propagation over z from the output sampling dx of the
-  // conjugated source (back onto the source grid d)
-  auto run = [&](bool herm, const pw::GradEpi* epi) -> pw_status {
-    h->d = dx;
-    h->kind = SRC_ADJOINT;
-    h->adj_herm = herm ? 1 : 0;
-    h->adj_mu = has_mu ? 1 : 0;
-    h->adj_iP = a->iP;
-    h->adj_jP = a->jP;
-    h->adj_grad = epi;
-    pw_status r = propagate(h, z, false);
-    h->adj_grad = nullptr;
-    return r;
-  };
-  bool R_herm_in_W = false;
-  pw_status r = PW_OK;
+  // the adjoint propagation is a Fresnel propagation over z from the output sampling dx of the
+  // conjugated source, back onto the source grid d, in closed form (delta.cuh)
+  h->d = dx;
+  h->kind = SRC_DIAGONAL;  // no GSM table
+  pw_status r = build_tables(h, z, false);
+  if (r != PW_OK) return done(r);
+  const double lz = lam * z, s = (dx * dx / lz) * (dx * dx / lz);
+  cudaEvent_t* ev = next_events(h);
+  if (ev && (e = cudaEventRecord(ev[0], st)) != cudaSuccess) return done(cuda_fail(e, "event record"));
+  pw::delta::TabArgs t{};
+  t.d = h->adj_d;
+  t.A = 1.0f;
+  t.q = farfield ? h->qtab : nullptr;
+  t.cross = has_mu ? h->adj_c : nullptr;
+  t.iP = a->iP;
+  t.jP = a->jP;
+  t.part = has_mu ? h->gpart : nullptr;
+  t.npart = nprep;
+  t.S = a->dev_S;
+  if ((e = delta_tables(h, t)) != cudaSuccess) return done(cuda_fail(e, "adjoint table launch"));
+  if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return done(cuda_fail(e, "event record"));
   if (params) {
     // the Hermitian part of the source suffices: dW0/dtheta is Hermitian
-    if (N != 256) {
-      pw::GradEpi ge{};
-      ge.gtab = h->gtab;
-      ge.amask = a->dev_amask;
-      ge.qff = farfield ? h->qtab : nullptr;
-      ge.part = h->gpart;
-      ge.gmask = a->dev_grad_amask;
-      ge.gscale = (float)(4.0 * c * a->amplitude);
-      ge.d2 = (float)(d * d);
-      r = run(true, &ge);
-    } else {
-      r = run(true, nullptr);  // R stored in W, then the standalone gradient kernel
-      if (r == PW_OK) {
-        const size_t sh = 2 * N * sizeof(float) + 2 * N * sizeof(float2) + 32 * sizeof(double) + 64;
-        if (farfield) pw::gsm_gradient_kernel<true><<<N * N, 256, sh, st>>>(g);
-        else pw::gsm_gradient_kernel<false><<<N * N, 256, sh, st>>>(g);
-        R_herm_in_W = true;
-      }
-    }
-    if (r == PW_OK) pw::gsm_gradient_reduce<<<1, 256, 0, st>>>(g);
+    const int rows = std::max(1, 256 / N), nt = (rows * N + 31) / 32 * 32;
+    const pw::delta::GradArgs ga{N, h->Eout, t.q, t.D, t.al, t.be, h->gtab, a->dev_amask, (float)s, (float)(d * d),
+                                 h->gpart, a->dev_grad_amask, (float)(4.0 * c * a->amplitude)};
+    g.rows = std::min(NN, num_sms() * (2048 / nt));
+    const size_t sh = N * sizeof(float2);
+    if (has_mu) pw::delta::grad_kernel<true><<<g.rows, nt, sh, st>>>(ga);
+    else pw::delta::grad_kernel<false><<<g.rows, nt, sh, st>>>(ga);
+    pw::gsm_gradient_reduce<<<1, 256, 0, st>>>(g);
+    if ((e = cudaGetLastError()) != cudaSuccess) return done(cuda_fail(e, "gradient launch"));
   }
-  if (r == PW_OK && a->grad_W0) {
-    // a general complex W0: the whole adjoint (the P1 row without its mirrored column)
-    if (!(R_herm_in_W && !has_mu)) r = run(!has_mu, nullptr);
-    if (r == PW_OK) {
-      const int blocks = num_sms() * 8;
-      pw::w0_gradient_kernel<<<blocks, 256, 0, st>>>(reinterpret_cast<float2*>(h->W), N, (float)(2.0 * c),
-                                                     farfield ? h->qtab : nullptr);
-    }
-  }
-  if (r == PW_OK && (e = cudaGetLastError()) != cudaSuccess) r = cuda_fail(e, "adjoint kernel launch");
-  // the handle is at the source plane, with no source recorded
-  h->d = d;
-  h->kind = SRC_NONE;
-  h->W0 = nullptr;
-  h->diag = nullptr;
-  return r;
+  // a general complex W0: the whole adjoint (the P1 row without its mirrored column), as
+  // dL/dRe W0 + i dL/dIm W0 = 2 c conj(R)
+  if (a->grad_W0 && (e = delta_write(h, t, has_mu, true, 2.0 * c * s, nullptr)) != cudaSuccess)
+    return done(cuda_fail(e, "gradient write launch"));
+  if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return done(cuda_fail(e, "event record"));
+  return done(PW_OK);
 }
 
 }  // namespace

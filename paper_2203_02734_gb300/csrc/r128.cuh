@@ -125,19 +125,17 @@ __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][
   }
 }
 
-// Pass A at N = 128, persistent.  Per point-1 pair (a, b): build W1(c, d) = s_ab F(c, d) G(a,c)
-// G(b,d) (or W0 x factors) in registers, 2D DFT (sign -1) over (c, d), natural-order slice into
+// Pass A at N = 128, persistent.  Per point-1 pair (a, b): read W1(c, d) = s_ab F(c, d) W0(a, b, c, d)
+// into registers, 2D DFT (sign -1) over (c, d), natural-order slice into
 // shared memory, one TMA tensor store into the V layout.  F(c, d) = Ein(c) Ein(d) Y(c, d) m(c, d)
-// from the per-axis factors, the aperture test and the optional mask; the GSM factors G(a, c),
-// G(b, d) are read through L1.  Stage 3 reads and writes only its warp's eight buffer rows (the
+// from the per-axis factors, the aperture test and the optional mask.  Stage 3 reads and writes only its warp's eight buffer rows (the
 // second exchange permutes rows by vrow), so the natural-order write after it needs only a warp
 // barrier, and each warp leaves its rows by its own TMA store (8 rows of V, 256 runs of 32 bytes),
 // which drains while the next slice is built.
-template <int SRC, bool MASK>
+template <bool MASK>
 __global__ void __launch_bounds__(NT, 1)
     pass_a_r128(const __grid_constant__ CUtensorMap vmap, PassAArgs p, const float2* __restrict__ Ein,
                 const float2* __restrict__ mask, int ap_ithr) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY, DIAG = SRC == SRC_DIAG;
   extern __shared__ __align__(1024) float2 smem[];
   float2* buf = smem;
   float2* tw = buf + N * N;
@@ -163,35 +161,26 @@ __global__ void __launch_bounds__(NT, 1)
   __syncthreads();  // tw, ein
   for (int ab = blockIdx.x; ab < N * N; ab += gridDim.x) {
     const int a = ab / N, b = ab - a * N;
-    // s_ab = A conj(F(a, b)), F(i, j) = Ein(i) Ein(j) Y(i, j) m(i, j)
+    // s_ab = conj(F(a, b)), F(i, j) = Ein(i) Ein(j) Y(i, j) m(i, j)
     float2 fab = inside(a, b) ? cmul(ein[a], ein[b]) : make_float2(0.f, 0.f);
     if (MASK) fab = cmul(fab, __ldg(mask + a * N + b));
-    float2 s_ab = cconj(fab);
-    if (SRC == SRC_GSM || SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
-    if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
-    const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
-    AdjSlice adj{};
-    if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
-    float2 ed[4];  // Ein(d) G(b, d)
+    const float2 s_ab = cconj(fab);
+    const float2* W0 = p.W0 + (size_t)ab * N * N;
+    float2 ed[4];  // Ein(d)
 #pragma unroll
-    for (int rq = 0; rq < 4; ++rq) {
-      const int d = lane + 32 * rq;
-      ed[rq] = SRC == SRC_GSM ? cscale(ein[d], __ldg(p.G + b * N + d)) : ein[d];
-    }
+    for (int rq = 0; rq < 4; ++rq) ed[rq] = ein[lane + 32 * rq];
     float2 v[8][4];
 #pragma unroll
     for (int rp = 0; rp < 8; ++rp) {
       const int c = warp + 16 * rp;
-      const float2 sc = SRC == SRC_GSM ? cmul(s_ab, cscale(ein[c], __ldg(p.G + a * N + c))) : cmul(s_ab, ein[c]);
+      const float2 sc = cmul(s_ab, ein[c]);
 #pragma unroll
       for (int rq = 0; rq < 4; ++rq) {
         const int d = lane + 32 * rq;
         float2 x = cmul(sc, ed[rq]);
         if (MASK) x = cmul(x, __ldg(mask + c * N + d));
-        if (ARRAY) x = cmul(x, __ldg(W0 + c * N + d));
-        if (SRC == SRC_ADJ) x = cmul(x, adj.at(p.cross, c * N + d));
-        bool keep = (inmask >> (rp * 4 + rq)) & 1u;
-        if (DIAG) keep = keep && c == a && d == b;
+        x = cmul(x, __ldg(W0 + c * N + d));
+        const bool keep = (inmask >> (rp * 4 + rq)) & 1u;
         v[rp][rq] = keep ? x : make_float2(0.f, 0.f);
       }
     }
@@ -334,7 +323,7 @@ __device__ __forceinline__ void stages_23_half(float2 (&v)[8][4], float2 (&w3)[2
 
 constexpr size_t kStageBytes = (size_t)N * N * sizeof(float2);  // prefetched stage-1 inputs
 constexpr size_t kXBytes = (size_t)N * N * sizeof(float2) / 2;     // half-size exchange buffer
-constexpr size_t pass_b_smem() { return kStageBytes + kXBytes + 2 * N * sizeof(float2) + 4 * 32 * sizeof(double); }
+constexpr size_t pass_b_smem() { return kStageBytes + kXBytes + 2 * N * sizeof(float2); }
 
 // Pass B at N = 128, persistent.  CTA blockIdx.x handles point-2 output pairs cd = blockIdx.x +
 // k gridDim.x.  Every thread gathers exactly the 32 points (a, b) = (warp + 16 rp, lane + 32 rq)
@@ -345,14 +334,12 @@ constexpr size_t pass_b_smem() { return kStageBytes + kXBytes + 2 * N * sizeof(f
 // output propagators, S on the diagonal) writes, for WST = W_HERM, the
 // conjugated column as the contiguous row W(c', d', ., .) straight from registers (Hermitian
 // store).
-template <int WST>
-__global__ void __launch_bounds__(NT, 1) pass_b_r128(PassBArgs p) {
+static __global__ void __launch_bounds__(NT, 1) pass_b_r128(PassBArgs p) {
   extern __shared__ __align__(1024) float2 smem[];
   float2* stg = smem;
   float2* xb = stg + N * N;
   float2* tw = xb + N * N / 2;
   float2* eo = tw + N;
-  double* red = reinterpret_cast<double*>(eo + N);  // W_GRAD: block reduction
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int g = vgroup<N>();
   for (int i = t; i < N; i += NT) {
@@ -398,37 +385,18 @@ __global__ void __launch_bounds__(NT, 1) pass_b_r128(PassBArgs p) {
     stages_23_half<+1>(v, w3, xb, tw);
     const float2 ecd = cscale(cmul(eo[c], eo[d]), p.scale);
     float2* Wrow = p.W + (size_t)cd * N * N;
-    if constexpr (WST == W_GRAD) {
-      GradSums gs;
-      const float2 ecg = grad_col(p.gr, c, d, ecd);
-      GradAxis B[4];
 #pragma unroll
-      for (int rq = 0; rq < 4; ++rq) B[rq] = grad_axis(p.gr, N, lane + 32 * rq, d, cconj(eo[lane + 32 * rq]));
+    for (int i = 0; i < 2; ++i) {
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
+      for (int rp = 0; rp < 4; ++rp) {
+        const int a = warp + 16 * i + 32 * rp;
+        const float2 ea = cmul(cconj(eo[a]), ecd);
 #pragma unroll
-        for (int rp = 0; rp < 4; ++rp) {
-          const int a = warp + 16 * i + 32 * rp;
-          const GradAxis A = grad_axis(p.gr, N, a, c, cmul(cconj(eo[a]), ecg));
-#pragma unroll
-          for (int rq = 0; rq < 4; ++rq) gs.add(A, B[rq], grad_mask(p.gr, N, a, lane + 32 * rq), w3[i][rp][rq]);
-        }
-      }
-      grad_reduce(p.gr, N, cd, gs, red);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-#pragma unroll
-        for (int rp = 0; rp < 4; ++rp) {
-          const int a = warp + 16 * i + 32 * rp;
-          const float2 ea = cmul(cconj(eo[a]), ecd);
-#pragma unroll
-          for (int rq = 0; rq < 4; ++rq) {
-            const int b = lane + 32 * rq;
-            const float2 w = cmul(cmul(ea, cconj(eo[b])), w3[i][rp][rq]);
-            if (a == c && b == d) p.S[cd] = w.x;
-            if (WST == W_HERM) Wrow[a * N + b] = cconj(w);
-          }
+        for (int rq = 0; rq < 4; ++rq) {
+          const int b = lane + 32 * rq;
+          const float2 w = cmul(cmul(ea, cconj(eo[b])), w3[i][rp][rq]);
+          if (a == c && b == d) p.S[cd] = w.x;
+          Wrow[a * N + b] = cconj(w);
         }
       }
     }

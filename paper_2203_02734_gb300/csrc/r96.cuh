@@ -108,16 +108,15 @@ __device__ __forceinline__ void stages(float2 (&v)[2][8][3], float2 (&w3)[3][4][
   __syncthreads();
 }
 
-// Pass A at N = 96, persistent (two CTAs per SM).  Per point-1 pair (a, b): build W1(c, d) =
-// s_ab F(c, d) G(a,c) G(b,d) (or W0 x factors, or the diagonal source) in registers at the
-// thread's stage-1 input points, 2D DFT (sign -1), natural-order slice into shared memory, one TMA
-// tensor store into the V layout.  F(c, d) = Ein(c) Ein(d) Y(c, d) m(c, d) from the per-axis
-// factors, the aperture test and the optional mask.
-template <int SRC, bool MASK>
+// Pass A at N = 96, persistent (two CTAs per SM).  Per point-1 pair (a, b): read W1(c, d) =
+// s_ab F(c, d) W0(a, b, c, d) into registers at the thread's stage-1 input points, 2D DFT (sign -1),
+// natural-order slice into shared memory, one TMA tensor store into the V layout.
+// F(c, d) = Ein(c) Ein(d) Y(c, d) m(c, d) from the per-axis factors, the aperture test and the optional
+// mask.
+template <bool MASK>
 __global__ void __launch_bounds__(NT, 2)
     pass_a_r96(const __grid_constant__ CUtensorMap vmap, PassAArgs p, const float2* __restrict__ Ein,
                const float2* __restrict__ mask, int ap_ithr) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY, DIAG = SRC == SRC_DIAG;
   extern __shared__ __align__(1024) float2 smem[];
   float2* X = smem;  // exchange buffer; the first N x N entries also stage the slice for TMA
   float2* tw = X + N * P;
@@ -141,40 +140,29 @@ __global__ void __launch_bounds__(NT, 2)
       for (int kq = 0; kq < 3; ++kq)
         if (inside(warp + 6 * i + 12 * kp, lane + 32 * kq)) inmask |= 1ull << (i * 24 + kp * 3 + kq);
   __syncthreads();  // tw, ein
-  // the GSM factors G(a, c), G(b, d) are read through L1 (no per-slice table, no barrier)
-  const float* __restrict__ G = p.G;
   for (int ab = blockIdx.x; ab < N * N; ab += gridDim.x) {
     const int a = ab / N, b = ab - a * N;
     float2 fab = inside(a, b) ? cmul(ein[a], ein[b]) : make_float2(0.f, 0.f);
     if (MASK) fab = cmul(fab, __ldg(mask + a * N + b));
-    float2 s_ab = cconj(fab);
-    if (SRC == SRC_GSM || SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
-    if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
-    const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
-    AdjSlice adj{};
-    if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
-    float2 ed[3];  // Ein(d) G(b, d)
+    const float2 s_ab = cconj(fab);
+    const float2* W0 = p.W0 + (size_t)ab * N * N;
+    float2 ed[3];  // Ein(d)
 #pragma unroll
-    for (int kq = 0; kq < 3; ++kq) {
-      const int d = lane + 32 * kq;
-      ed[kq] = SRC == SRC_GSM ? cscale(ein[d], __ldg(G + b * N + d)) : ein[d];
-    }
+    for (int kq = 0; kq < 3; ++kq) ed[kq] = ein[lane + 32 * kq];
     float2 v[2][8][3];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
       for (int kp = 0; kp < 8; ++kp) {
         const int c = warp + 6 * i + 12 * kp;
-        const float2 sc = SRC == SRC_GSM ? cmul(s_ab, cscale(ein[c], __ldg(G + a * N + c))) : cmul(s_ab, ein[c]);
+        const float2 sc = cmul(s_ab, ein[c]);
 #pragma unroll
         for (int kq = 0; kq < 3; ++kq) {
           const int d = lane + 32 * kq;
           float2 x = cmul(sc, ed[kq]);
           if (MASK) x = cmul(x, __ldg(mask + c * N + d));
-          if (ARRAY) x = cmul(x, __ldg(W0 + c * N + d));
-          if (SRC == SRC_ADJ) x = cmul(x, adj.at(p.cross, c * N + d));
-          bool keep = (inmask >> (i * 24 + kp * 3 + kq)) & 1ull;
-          if (DIAG) keep = keep && c == a && d == b;
+          x = cmul(x, __ldg(W0 + c * N + d));
+          const bool keep = (inmask >> (i * 24 + kp * 3 + kq)) & 1ull;
           v[i][kp][kq] = keep ? x : make_float2(0.f, 0.f);
         }
       }
@@ -202,7 +190,7 @@ __global__ void __launch_bounds__(NT, 2)
 
 constexpr size_t pass_a_smem() { return (size_t)N * P * sizeof(float2) + 2 * N * sizeof(float2); }
 constexpr size_t pass_b_smem() {
-  return (size_t)N * P * sizeof(float2) + 2 * N * sizeof(float2) + 4 * 32 * sizeof(double);
+  return (size_t)N * P * sizeof(float2) + 2 * N * sizeof(float2);
 }
 
 // Pass B at N = 96, persistent (two CTAs per SM).  CTA blockIdx.x handles point-2 output pairs
@@ -212,13 +200,11 @@ constexpr size_t pass_b_smem() {
 // inverse-sign 2D DFT; the epilogue (scale, output propagators, S on the diagonal)
 // and, for WST = W_HERM, the conjugated column as the contiguous row W(c', d', ., .) from
 // registers.
-template <int WST>
 __global__ void __launch_bounds__(NT, 2) pass_b_r96(PassBArgs p) {
   extern __shared__ __align__(1024) float2 smem[];
   float2* X = smem;
   float2* tw = X + N * P;
   float2* eo = tw + N;
-  double* red = reinterpret_cast<double*>(eo + N);  // W_GRAD: block reduction
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   constexpr int g = vgroup<N>();
   constexpr size_t NN = (size_t)N * N;
@@ -253,39 +239,19 @@ __global__ void __launch_bounds__(NT, 2) pass_b_r96(PassBArgs p) {
     stages<+1>(v, w3, X, tw);
     const float2 ecd = cscale(cmul(eo[c], eo[d]), p.scale);
     float2* Wrow = p.W + (size_t)cd * NN;
-    if constexpr (WST == W_GRAD) {
-      GradSums gs;
-      const float2 ecg = grad_col(p.gr, c, d, ecd);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int u = t + NT * i, jq = u % 24, jp = u / 24;
-        GradAxis B[4];
+    for (int i = 0; i < 3; ++i) {
+      const int u = t + NT * i, jq = u % 24, jp = u / 24;
 #pragma unroll
-        for (int kq = 0; kq < 4; ++kq) B[kq] = grad_axis(p.gr, N, jq + 24 * kq, d, cconj(eo[jq + 24 * kq]));
+      for (int kp = 0; kp < 4; ++kp) {
+        const int a = jp + 24 * kp;
+        const float2 ea = cmul(cconj(eo[a]), ecd);
 #pragma unroll
-        for (int kp = 0; kp < 4; ++kp) {
-          const int a = jp + 24 * kp;
-          const GradAxis A = grad_axis(p.gr, N, a, c, cmul(cconj(eo[a]), ecg));
-#pragma unroll
-          for (int kq = 0; kq < 4; ++kq) gs.add(A, B[kq], grad_mask(p.gr, N, a, jq + 24 * kq), w3[i][kp][kq]);
-        }
-      }
-      grad_reduce(p.gr, N, cd, gs, red);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const int u = t + NT * i, jq = u % 24, jp = u / 24;
-#pragma unroll
-        for (int kp = 0; kp < 4; ++kp) {
-          const int a = jp + 24 * kp;
-          const float2 ea = cmul(cconj(eo[a]), ecd);
-#pragma unroll
-          for (int kq = 0; kq < 4; ++kq) {
-            const int b = jq + 24 * kq;
-            const float2 w = cmul(cmul(ea, cconj(eo[b])), w3[i][kp][kq]);
-            if (a == c && b == d) p.S[cd] = w.x;
-            if (WST == W_HERM) Wrow[a * N + b] = cconj(w);
-          }
+        for (int kq = 0; kq < 4; ++kq) {
+          const int b = jq + 24 * kq;
+          const float2 w = cmul(cmul(ea, cconj(eo[b])), w3[i][kp][kq]);
+          if (a == c && b == d) p.S[cd] = w.x;
+          Wrow[a * N + b] = cconj(w);
         }
       }
     }

@@ -11,9 +11,10 @@
 // intermediate array lives in the work buffer as
 //   Y[a][b][kperm(k_l)][g][r][j]  (after pass 1)  and  Y[a][b'][kperm(k_l)][g][k_h][j]  (after pass 2),
 // so that the 4 x 8 values one pass-2 line group needs are one 256-byte run (kperm: below).
-// It runs every source but the GSM model, which has no need of the point-2 pass (plane.cuh).
-//   pass 1, tile (a, b, r): the source rows c = r + 4 m of slice (a, b) are read or generated in
-//     registers (W1(c, d) = conj F(a, b) F(c, d) x source), transformed over (m, d) as a 64 x 256 2D DFT in
+// It runs the uploaded and propagated arrays; the sources given by a formula have shorter ways
+// (plane.cuh, delta.cuh).
+//   pass 1, tile (a, b, r): the source rows c = r + 4 m of slice (a, b) are read into registers
+//     (W1(c, d) = conj F(a, b) F(c, d) W0), transformed over (m, d) as a 64 x 256 2D DFT in
 //     registers through one shared buffer, and stored to Y by TMA (64-byte pieces of the 256-byte
 //     runs; the four r tiles of a slice run side by side and fill each run together).
 //   pass 2, tile (a, k_l, g): the 256 runs Y[a][.][k_l][g] (all b, r, j) arrive by one TMA tensor
@@ -150,9 +151,7 @@ __device__ __forceinline__ int xs2(int q) { return q ^ (((q >> 6) & 3) << 3); }
 
 constexpr size_t pass1_smem() { return (size_t)64 * N * sizeof(float2) + N * sizeof(float2); }
 
-template <int SRC>
 __global__ void __launch_bounds__(NT1, 1) pass1_kernel(const __grid_constant__ CUtensorMap smap, PassAArgs p) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY, DIAG = SRC == SRC_DIAG;
   extern __shared__ __align__(1024) float2 smem[];
   float2* buf = smem;  // 64 x 256
   float2* tw = buf + 64 * N;
@@ -161,13 +160,8 @@ __global__ void __launch_bounds__(NT1, 1) pass1_kernel(const __grid_constant__ C
   const float2* __restrict__ F = p.F;
   for (int tile = blockIdx.x; tile < N * N * 4; tile += gridDim.x) {
     const int ab = tile >> 2, r = tile & 3;
-    const int a = ab / N, b = ab - a * N;
-    float2 s_ab = cconj(__ldg(F + ab));
-    if (SRC == SRC_ADJ) s_ab = cscale(s_ab, p.A);
-    if (DIAG) s_ab = cscale(s_ab, p.A * __ldg(p.diag + ab));
-    const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
-    AdjSlice adj{};
-    if (SRC == SRC_ADJ) adj = adj_slice(p, ab, N);
+    const float2 s_ab = cconj(__ldg(F + ab));
+    const float2* W0 = p.W0 + (size_t)ab * N * N;
     // stage 1 inputs: m = w + 16 rp (c = r + 4 m), d = l + 32 rq
     float2 v[4][8];
 #pragma unroll
@@ -176,11 +170,7 @@ __global__ void __launch_bounds__(NT1, 1) pass1_kernel(const __grid_constant__ C
 #pragma unroll
       for (int rq = 0; rq < 8; ++rq) {
         const int d = lane + 32 * rq;
-        float2 x = cmul(s_ab, __ldg(F + c * N + d));
-        if (ARRAY) x = cmul(x, __ldg(W0 + c * N + d));
-        if (DIAG) x = (c == a && d == b) ? x : make_float2(0.f, 0.f);
-        if (SRC == SRC_ADJ) x = cmul(x, adj.at(p.cross, c * N + d));
-        v[rp][rq] = x;
+        v[rp][rq] = cmul(cmul(s_ab, __ldg(F + c * N + d)), __ldg(W0 + c * N + d));
       }
     }
 #pragma unroll
