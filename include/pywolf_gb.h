@@ -201,6 +201,15 @@ pw_status pw_propagate_fresnel(pw_csd* h, double z_m);
  * propagators and sampling as for Fresnel). */
 pw_status pw_propagate_farfield(pw_csd* h, double z_m);
 
+/* S and mu(P1, .) of the plane that a propagation of the recorded GSM source over z_m would reach (with the
+ * masks recorded for the current plane; farfield selects Eq. W_farfield), without its CSDA: S is the
+ * transform of the correlation of the source field times its coherence (Eq. defS), mu's numerator a
+ * convolution (Eq. defMu), O(N^2 log N) work.  For callers that need only these two, such as the forward
+ * pass of an inverse problem.  Leaves the current plane, its source and dev_W as they are and uses
+ * dev_work as scratch; dev_mu may be NULL (S only).  Asynchronous on the handle's stream.  PW_ESTATE without
+ * a GSM source, PW_EUNSUPPORTED on a zero-padded grid, one without an FFT plan, or N < 4. */
+pw_status pw_gsm_s_mu(pw_csd* h, double z_m, int farfield, int iP, int jP, float* dev_S, pw_c32* dev_mu);
+
 /* Sampling d of the current plane in metres. */
 pw_status pw_get_sampling(const pw_csd* h, double* d_m);
 

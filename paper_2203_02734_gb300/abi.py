@@ -41,6 +41,7 @@ SIGNATURES = {
     "pw_csd_pass_times": (_i, [_vp, ctypes.POINTER(_d), ctypes.POINTER(_d), ctypes.POINTER(_i)]),
     "pw_csd_pass_times3": (_i, [_vp, ctypes.POINTER(_d), ctypes.POINTER(_d), ctypes.POINTER(_d), ctypes.POINTER(_i)]),
     "pw_source_gsm": (_i, [_vp, _d, _d, _d]),
+    "pw_gsm_s_mu": (_i, [_vp, _d, _i, _i, _i, _vp, _vp]),
     "pw_source_aperture": (_i, [_vp, _d]),
     "pw_source_lens": (_i, [_vp, _d]),
     "pw_source_mask": (_i, [_vp, _vp]),
@@ -228,6 +229,10 @@ def pw_gsm_gradient(h, sigma_S_m, sigma_mu_m, amplitude, dev_amask, lambda_m, z_
                     dev_grad_mask):
     _check(LIB.pw_gsm_gradient(h, sigma_S_m, sigma_mu_m, amplitude, dev_amask, lambda_m, z_m, 1 if farfield else 0,
                                dev_grad3, dev_grad_mask))
+
+
+def pw_gsm_s_mu(h, z_m, farfield, iP, jP, dev_S, dev_mu):
+    _check(LIB.pw_gsm_s_mu(h, z_m, 1 if farfield else 0, iP, jP, dev_S, dev_mu))
 
 
 def pw_propagate_fresnel(h, z_m):

@@ -19,24 +19,33 @@ def _ptr(t):
 
 
 class _Model:
-    """The handle, its two N^4 device buffers and the output buffers, reused by every call."""
+    """The handle and its two N^4 device buffers, reused by every call."""
 
     def __init__(self, N, dxi, lam, z, P1, farfield, device):
         self.N, self.dxi, self.lam, self.z, self.farfield = N, float(dxi), float(lam), float(z), bool(farfield)
         self.P1 = (N // 2, N // 2) if P1 is None else (int(P1[0]), int(P1[1]))
         self.dx = self.lam * self.z / (N * self.dxi)
         self.csd = CSD(N, self.dxi, self.lam, device=device)
-        dev = self.csd.W.device
-        self.S = torch.empty((N, N), dtype=torch.float32, device=dev)
-        self.mu = torch.empty((N, N), dtype=torch.complex64, device=dev)
-        self.g3 = torch.zeros(3, dtype=torch.float64, device=dev)
-        self.gmask = torch.empty((N, N), dtype=torch.float32, device=dev)
+        self.dev = self.csd.W.device
+
+    def outputs(self):
+        """New S and mu tensors (they belong to the caller's graph)."""
+        return self.new(torch.float32), self.new(torch.complex64)
+
+    def new(self, dtype, *shape):
+        """A device tensor that the handle's stream may still be writing when it is freed."""
+        t = torch.empty(shape or (self.N, self.N), dtype=dtype, device=self.dev)
+        if torch.cuda.current_stream(self.dev) != self.csd.stream:
+            t.record_stream(self.csd.stream)
+        return t
 
     def propagate_and_read(self):
         h = self.csd.h
+        S, mu = self.outputs()
         (abi.pw_propagate_farfield if self.farfield else abi.pw_propagate_fresnel)(h, self.z)
-        abi.pw_spectral_density(h, self.S.data_ptr())
-        abi.pw_degree_of_coherence(h, self.P1[0], self.P1[1], self.mu.data_ptr())
+        abi.pw_spectral_density(h, S.data_ptr())
+        abi.pw_degree_of_coherence(h, self.P1[0], self.P1[1], mu.data_ptr())
+        return S, mu
 
     def adjoint(self, gS, gmu, S, mu, **kw):
         """One adjoint call from the output plane; gS / gmu are torch's upstream gradients or None."""
@@ -70,7 +79,9 @@ class GSMPropagation:
 
     def __init__(self, N, dxi, lam, z, P1=None, farfield=False, device=None):
         self.m = _Model(N, dxi, lam, z, P1, farfield, device)
-        self.mask_c = torch.zeros((N, N), dtype=torch.complex64, device=self.m.csd.W.device)
+        self.mask_c = torch.zeros((N, N), dtype=torch.complex64, device=self.m.dev)
+        # S and mu need no CSDA where the library has the direct form (an FFT plan, N >= 4)
+        self.direct = N >= 4 and abi.pw_supported_n(N)
 
     def __call__(self, sigma_S, sigma_mu, A, amask):
         return _GSMFn.apply(sigma_S, sigma_mu, A, amask, self)
@@ -97,12 +108,16 @@ class _GSMFn(torch.autograd.Function):
         am = amask.detach().to(torch.float32).contiguous()
         model.mask_c.real.copy_(am)  # the amplitude mask as a complex mask (argument marshalling)
         abi.pw_csd_reset(h, m.dxi)
-        abi.pw_source_gsm(h, float(sigma_S), float(sigma_mu), float(A))
+        params = (float(sigma_S), float(sigma_mu), float(A))
+        abi.pw_source_gsm(h, *params)
         abi.pw_source_mask(h, model.mask_c.data_ptr())
-        m.propagate_and_read()
-        S, mu = m.S.clone(), m.mu.clone()
+        if model.direct:
+            S, mu = m.outputs()
+            abi.pw_gsm_s_mu(h, m.z, m.farfield, m.P1[0], m.P1[1], S.data_ptr(), mu.data_ptr())
+        else:
+            S, mu = m.propagate_and_read()
         ctx.model = model
-        ctx.params = (float(sigma_S), float(sigma_mu), float(A))
+        ctx.params = params
         ctx.like = [(x.device, x.dtype) if torch.is_tensor(x) else None for x in (sigma_S, sigma_mu, A)]
         ctx.save_for_backward(am, S, mu)
         ctx.set_materialize_grads(False)  # an unused output (mu of an S-only loss) gets no adjoint term
@@ -115,12 +130,15 @@ class _GSMFn(torch.autograd.Function):
         if gS is None and gmu is None:
             return None, None, None, None, None
         sS, sM, A = ctx.params
+        g, gmask = m.new(torch.float64, 3), m.new(torch.float32)
         keep = m.adjoint(gS, gmu, S, mu, sigma_S_m=sS, sigma_mu_m=sM, amplitude=A, dev_amask=am.data_ptr(),
-                         dev_grad3=m.g3.data_ptr(), dev_grad_amask=m.gmask.data_ptr())
-        g = m.g3.clone()
+                         dev_grad3=g.data_ptr(), dev_grad_amask=gmask.data_ptr())
         del keep
-        out = [None if lk is None else g[k].to(device=lk[0], dtype=lk[1]) for k, lk in enumerate(ctx.like)]
-        return out[0], out[1], out[2], m.gmask.clone().to(dtype=am.dtype), None
+        if any(lk is not None and lk[0].type == "cpu" for lk in ctx.like):
+            g_host = g.cpu()  # one copy for the parameters that live on the host
+        out = [None if lk is None else (g_host if lk[0].type == "cpu" else g)[k].to(device=lk[0], dtype=lk[1])
+               for k, lk in enumerate(ctx.like)]
+        return out[0], out[1], out[2], gmask, None
 
 
 class CSDPropagation:
@@ -148,8 +166,7 @@ class _CSDFn(torch.autograd.Function):
         W0c = W0.detach().to(torch.complex64).contiguous()
         abi.pw_csd_reset(h, m.dxi)
         abi.pw_source_array(h, W0c.data_ptr(), 1 if model.hermitian else 0)
-        m.propagate_and_read()
-        S, mu = m.S.clone(), m.mu.clone()
+        S, mu = m.propagate_and_read()
         ctx.model = model
         ctx.save_for_backward(S, mu)
         ctx.set_materialize_grads(False)

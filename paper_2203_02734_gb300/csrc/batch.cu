@@ -97,8 +97,8 @@ struct pw_batch {
   int mode;  // PW_BATCH_PERSISTENT or PW_BATCH_SEQUENCED
   std::vector<CUtensorMap> wmaps;  // per instance with W: its planes (plane.cuh)
   std::vector<pw::TableArgs> targs;   // FP64 tables, uploaded with N = 0 for the instances on smu.cuh
-  std::vector<pw::smu::Inst> smu;     // the instances on smu.cuh, by pw_instance index where direct
-  std::vector<pw::smu::TabArgs> smu_t;
+  std::vector<pw::smu::Inst<float2>> smu;     // the instances on smu.cuh, by pw_instance index where direct
+  std::vector<pw::smu::TabArgs<float2>> smu_t;
   std::vector<float2*> mus;           // dev_mu of every instance
   struct Round {                      // one launch round of the instances on smu.cuh
     int chunk;
@@ -107,8 +107,8 @@ struct pw_batch {
   };
   std::vector<Round> rounds;
   int ndirect;                        // instances on smu.cuh
-  const pw::smu::Inst* dev_smu;
-  const pw::smu::TabArgs* dev_smu_t;
+  const pw::smu::Inst<float2>* dev_smu;
+  const pw::smu::TabArgs<float2>* dev_smu_t;
   char* base;
   Layout L;
   cudaStream_t stream;
@@ -172,8 +172,8 @@ pw_status upload(pw_batch* b) {
   const size_t pool_bytes = b->L.slot_bytes * b->pool;
   std::vector<pw::TableArgs> targs(b->targs);
   std::vector<float2*> mus(b->mus);
-  std::vector<pw::smu::Inst> list;
-  std::vector<pw::smu::TabArgs> tabs;
+  std::vector<pw::smu::Inst<float2>> list;
+  std::vector<pw::smu::TabArgs<float2>> tabs;
   b->rounds.clear();
   size_t used = 0;
   int chunk = 0;
@@ -181,7 +181,7 @@ pw_status upload(pw_batch* b) {
     if (!direct(b, i)) continue;
     targs[i].N = 0;
     mus[i] = nullptr;
-    pw::smu::Inst q = b->smu[i];
+    pw::smu::Inst<float2> q = b->smu[i];
     const size_t need = align256((size_t)6 * q.N * q.N * sizeof(float2));
     if (used + need > pool_bytes) {
       ++chunk;
@@ -198,24 +198,22 @@ pw_status upload(pw_batch* b) {
     tabs.push_back(b->smu_t[i]);
   }
   b->ndirect = (int)list.size();
-  const size_t lb = align256(list.size() * sizeof(pw::smu::Inst)), tb = align256(tabs.size() * sizeof(pw::smu::TabArgs));
+  const size_t lb = align256(list.size() * sizeof(pw::smu::Inst<float2>)), tb = align256(tabs.size() * sizeof(pw::smu::TabArgs<float2>));
   char* tail = b->base + (b->L.items + sizeof(pw::batch::Item) * (size_t)b->L.max_items) / 256 * 256 - lb - tb;
-  b->dev_smu = reinterpret_cast<pw::smu::Inst*>(tail);
-  b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs*>(tail + lb);
+  b->dev_smu = reinterpret_cast<pw::smu::Inst<float2>*>(tail);
+  b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs<float2>*>(tail + lb);
   cudaError_t e = cudaMemcpyAsync(b->base + b->L.targs, targs.data(), sizeof(pw::TableArgs) * n, cudaMemcpyHostToDevice,
                                   b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->base + b->L.mu, mus.data(), sizeof(float2*) * n, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess && b->ndirect)
-    e = cudaMemcpyAsync(tail, list.data(), list.size() * sizeof(pw::smu::Inst), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(tail, list.data(), list.size() * sizeof(pw::smu::Inst<float2>), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess && b->ndirect)
-    e = cudaMemcpyAsync(tail + lb, tabs.data(), tabs.size() * sizeof(pw::smu::TabArgs), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(tail + lb, tabs.data(), tabs.size() * sizeof(pw::smu::TabArgs<float2>), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "uploading the batch descriptors");
   return build_items(b);
 }
-
-__global__ void __launch_bounds__(256) smu_tables_kernel(const pw::smu::TabArgs* t) { pw::smu::tables(t[blockIdx.x]); }
 
 int num_sms() {
   int dev = 0, n = 0;
@@ -345,8 +343,8 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     t.tw = tw;
     t.Eout = Eo;
     t.Ein = Ei;
-    // smu.cuh: its tables take the place of F (11 N of the N^2 values)
-    pw::smu::TabArgs& ta = b->smu_t[i];
+    // smu.cuh: its tables take the place of F (6.5 N of the N^2 values)
+    pw::smu::TabArgs<float2>& ta = b->smu_t[i];
     ta.N = N;
     ta.Kin = t.Kin;
     ta.Kout = t.Kout;
@@ -354,16 +352,18 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     ta.gm = t.gm;
     ta.tw = F;
     ta.P1 = ta.tw + 2 * N;
-    ta.Eout = ta.P1 + N;
+    ta.P1l = ta.P1 + N;
+    ta.Eout = ta.P1l + N;
     ta.k = reinterpret_cast<float*>(ta.Eout + N);
     ta.K = ta.k + N;
-    pw::smu::Inst& si = b->smu[i];
+    pw::smu::Inst<float2>& si = b->smu[i];
     si.N = N;
     si.iP = q.iP;
     si.jP = q.jP;
-    si.factor = (float)((double)d.scale * q.amplitude / (4.0 * (double)NN));
+    si.factor = (double)d.scale * q.amplitude / (4.0 * (double)NN);
     si.tw = ta.tw;
     si.P1 = ta.P1;
+    si.P1l = ta.P1l;
     si.Eout = ta.Eout;
     si.k = ta.k;
     si.K = ta.K;
@@ -411,10 +411,11 @@ pw_status pw_batch_run(pw_batch* b) {
   if (!b) return fail(PW_EINVAL, "null batch");
   cudaError_t e;
   if (b->ndirect) {
-    smu_tables_kernel<<<b->ndirect, 256, 0, b->stream>>>(b->dev_smu_t);
+    if ((e = pwi::launch_smu_list_tables(b->dev_smu_t, b->ndirect, b->stream)) != cudaSuccess)
+      return cuda_fail(e, "batch S/mu tables launch");
     for (const auto& r : b->rounds)
       for (int N : r.Ns)
-        if ((e = pwi::launch_smu(N, b->dev_smu, pw::smu::Inst{}, b->ndirect, r.chunk, r.mu, b->stream)) != cudaSuccess)
+        if ((e = pwi::launch_smu_list(N, b->dev_smu, b->ndirect, r.chunk, r.mu, b->stream)) != cudaSuccess)
           return cuda_fail(e, "batch S/mu launch");
     if (b->ndirect == b->n) return PW_OK;
   }

@@ -170,11 +170,31 @@ __global__ void __launch_bounds__(256) write_kernel(WriteArgs p) {
 // Parameter gradients of the amplitude-masked GSM source W0 = A a(x1) a(x2) G(x1, x2) from the adjoint array
 // R = kappa conj e(k1) e(k2) [D + Hermitian cross], which is never stored: with
 //   t(x1, x2) = Re R(x1, x2) G(x1, x2) a(x1),
-// a block takes one column x2 after another and adds, over x1,
+// a block takes NC neighbouring columns x2 = (c, d .. d + NC - 1) after one another and adds, over x1,
 //   sum t (r^2(x1) + r^2(x2)), sum t |x1 - x2|^2, sum t   (r^2 and |x1 - x2|^2 in pixels^2),
 // the last one also as the mask gradient of x2.  Re R = kappa [Re(conj e1 (e2 D)) + Re(al1 be2 + al2 be1) / 2].
-// A thread owns one b and walks over a; N^4 terms of about 25 instructions, 85 million at N = 96.  FP32 terms
-// and per-thread sums (N^2 / threads terms each), FP64 over threads and columns, in a fixed order.
+// A thread owns one b and walks over a; what depends on x1 alone is loaded once for the NC columns (one
+// column at a time took 254 us at N = 96, six loads a term).  N^4 terms of about 20 instructions, 85
+// million at N = 96.  FP32 terms and per-thread sums (N^2 / threads terms each), pairs of floats over threads
+// and columns (FP64 additions there were 40 % of the kernel), FP64 over blocks, in a fixed order.
+struct Pair {  // an unevaluated sum h + l, about 48 bits
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float s = h + x, z = s - h;
+    l += (h - (s - z)) + (x - z);
+    h = s;
+  }
+  __device__ __forceinline__ void add(Pair o) {
+    add(o.h);
+    l += o.l;
+  }
+  __device__ __forceinline__ Pair from(int lanes) const {  // the pair of the lane `lanes` further down
+    Pair o;
+    o.h = __shfl_down_sync(0xffffffffu, h, lanes);
+    o.l = __shfl_down_sync(0xffffffffu, l, lanes);
+    return o;
+  }
+};
 struct GradArgs {
   int N;
   const float2* Eout;
@@ -189,9 +209,10 @@ struct GradArgs {
   float gscale;           // 4 c A
 };
 
-template <bool CROSS>
+template <bool CROSS, int NC>
 __global__ void __launch_bounds__(256) grad_kernel(GradArgs p) {
-  __shared__ double red[4][8];
+  __shared__ double red[3][8];
+  __shared__ float col[NC][256];
   extern __shared__ float2 ea[];  // N: e of one axis
   const int N = p.N, M = N / 2, rows = blockDim.x / N;
   const int b = threadIdx.x % N, a0 = threadIdx.x / N;
@@ -199,63 +220,84 @@ __global__ void __launch_bounds__(256) grad_kernel(GradArgs p) {
   for (int i = threadIdx.x; i < N; i += blockDim.x) ea[i] = axis_e(p.Eout, p.q, i);
   __syncthreads();
   const float2 eb = ea[b];
-  double tS = 0.0, tM = 0.0, tA = 0.0;
+  const float rb = (float)((b - M) * (b - M));
+  Pair tot[3];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k2 = blockIdx.x; k2 < N * N; k2 += gridDim.x) {
-    const int c = k2 / N, d = k2 - c * N;
-    float sS = 0.f, sM = 0.f, sA = 0.f;
+  for (int k2 = NC * blockIdx.x; k2 < N * N; k2 += NC * gridDim.x) {
+    const int c = k2 / N, d = k2 - c * N;  // NC divides N: one row c
+    float sS[NC], sM[NC], sA[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) sS[j] = sM[j] = sA[j] = 0.f;
     if (on) {
-      const float2 e2 = cscale(cmul(ea[c], ea[d]), p.kappa);
-      float2 al2 = make_float2(0.f, 0.f), be2 = al2;
-      if (CROSS) {
-        al2 = cscale(__ldg(p.al + k2), 0.5f * p.kappa);
-        be2 = cscale(__ldg(p.be + k2), 0.5f * p.kappa);
+      float2 f2[NC], al2[CROSS ? NC : 1], be2[CROSS ? NC : 1];
+      float gb[NC], fb[NC];
+      int v[NC];
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        f2[j] = cmul(cconj(eb), cscale(cmul(ea[c], ea[d + j]), p.kappa));  // conj e(b) kappa e(c) e(d)
+        if (CROSS) {
+          al2[j] = cscale(__ldg(p.al + k2 + j), 0.5f * p.kappa);
+          be2[j] = cscale(__ldg(p.be + k2 + j), 0.5f * p.kappa);
+        }
+        gb[j] = __ldg(p.gtab + b * N + d + j);
+        v[j] = b - d - j;
+        fb[j] = (float)(v[j] * v[j]);
+        v[j] += v[j] < 0 ? N : 0;
       }
-      int v = b - d;
-      const float fb = (float)(v * v), rb = (float)((b - M) * (b - M)), gb = __ldg(p.gtab + b * N + d);
-      v += v < 0 ? N : 0;
-      const float2 f2 = cmul(cconj(eb), e2);  // conj e(b) kappa e(c) e(d)
-#pragma unroll 4
+#pragma unroll 2
       for (int a = a0; a < N; a += rows) {
         int u = a - c;
-        const float fa = (float)(u * u), ra = (float)((a - M) * (a - M));
+        const float fa = (float)(u * u), r1 = (float)((a - M) * (a - M)) + rb;
         u += u < 0 ? N : 0;
-        const float2 z = cmul(f2, __ldg(p.D + u * N + v)), e1 = ea[a];
-        float R = fmaf(e1.x, z.x, e1.y * z.y);
-        if (CROSS) {
-          const float2 al1 = __ldg(p.al + a * N + b), be1 = __ldg(p.be + a * N + b);
-          R += fmaf(al1.x, be2.x, fmaf(-al1.y, be2.y, fmaf(al2.x, be1.x, -al2.y * be1.y)));
-        }
-        float m = gb * __ldg(p.gtab + a * N + c);
+        const float2 e1 = ea[a];
+        const float2* Du = p.D + u * N;
+        float m = __ldg(p.gtab + a * N + c);
         if (p.amask) m *= __ldg(p.amask + a * N + b);
-        const float tt = R * m;
-        sS = fmaf(tt, ra + rb, sS);
-        sM = fmaf(tt, fa + fb, sM);
-        sA += tt;
+        float2 al1 = make_float2(0.f, 0.f), be1 = al1;
+        if (CROSS) {
+          al1 = __ldg(p.al + a * N + b);
+          be1 = __ldg(p.be + a * N + b);
+        }
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const float2 z = cmul(f2[j], __ldg(Du + v[j]));
+          float R = fmaf(e1.x, z.x, e1.y * z.y);
+          if (CROSS) {
+            R = fmaf(al1.x, be2[j].x, R);
+            R = fmaf(-al1.y, be2[j].y, R);
+            R = fmaf(al2[j].x, be1.x, R);
+            R = fmaf(-al2[j].y, be1.y, R);
+          }
+          const float tt = R * (m * gb[j]);
+          sS[j] = fmaf(tt, r1, sS[j]);
+          sM[j] = fmaf(tt, fa + fb[j], sM[j]);
+          sA[j] += tt;
+        }
       }
-      const float rc = (float)((c - M) * (c - M) + (d - M) * (d - M));
-      sS = fmaf(rc, sA, sS);
     }
-    const float a2 = p.amask ? __ldg(p.amask + k2) : 1.f;
-    tS += (double)sS * a2 * p.d2;
-    tM += (double)sM * a2 * p.d2;
-    tA += (double)sA * a2;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+      const float rc = (float)((c - M) * (c - M) + (d + j - M) * (d + j - M));
+      const float a2 = p.amask ? __ldg(p.amask + k2 + j) : 1.f;
+      tot[0].add(fmaf(rc, sA[j], sS[j]) * a2);
+      tot[1].add(sM[j] * a2);
+      tot[2].add(sA[j] * a2);
+    }
     if (p.gmask) {
-      double x = (double)sA;
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      __syncthreads();  // red[3] of the previous column is read
-      if (lane == 0) red[3][warp] = x;
+      __syncthreads();  // col of the previous columns is read
+#pragma unroll
+      for (int j = 0; j < NC; ++j) col[j][threadIdx.x] = sA[j];
       __syncthreads();
-      if (threadIdx.x == 0) {
-        double y = 0.0;
-        for (int w = 0; w < nw; ++w) y += red[3][w];
-        p.gmask[k2] = (float)(p.gscale * y);
+      for (int j = warp; j < NC; j += nw) {
+        Pair x;
+        for (int i = lane; i < (int)blockDim.x; i += 32) x.add(col[j][i]);
+        for (int o = 16; o > 0; o >>= 1) x.add(x.from(o));
+        if (lane == 0) p.gmask[k2 + j] = (float)(p.gscale * ((double)x.h + (double)x.l));
       }
     }
   }
-  double v[3] = {tS, tM, tA};
   for (int k = 0; k < 3; ++k) {
-    double x = v[k];
+    double x = (double)tot[k].h + (double)tot[k].l;
     for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
     if (lane == 0) red[k][warp] = x;
   }
@@ -263,7 +305,7 @@ __global__ void __launch_bounds__(256) grad_kernel(GradArgs p) {
   if (threadIdx.x < 3) {
     double x = 0.0;
     for (int w = 0; w < nw; ++w) x += red[threadIdx.x][w];
-    p.part[(size_t)blockIdx.x * 3 + threadIdx.x] = x;
+    p.part[(size_t)blockIdx.x * 3 + threadIdx.x] = threadIdx.x < 2 ? x * p.d2 : x;
   }
 }
 

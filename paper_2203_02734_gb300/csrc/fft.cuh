@@ -13,45 +13,54 @@
 
 namespace pw {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+// Complex values are float2, or double2 where a small transform is wanted to more digits (smu.cuh).
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float2 make_c(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ double2 make_c(double x, double y) { return make_double2(x, y); }
+template <class C> using real_t = decltype(C::x);
+
+template <class C> __device__ __forceinline__ C cadd(C a, C b) { return make_c(a.x + b.x, a.y + b.y); }
+template <class C> __device__ __forceinline__ C csub(C a, C b) { return make_c(a.x - b.x, a.y - b.y); }
+template <class C> __device__ __forceinline__ C cmul(C a, C b) {
+  return make_c(fma_(a.x, b.x, -a.y * b.y), fma_(a.x, b.y, a.y * b.x));
 }
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+template <class C> __device__ __forceinline__ C cconj(C a) { return make_c(a.x, -a.y); }
+template <class C> __device__ __forceinline__ C cscale(C a, real_t<C> s) { return make_c(a.x * s, a.y * s); }
 // a * (S i), S = +-1
-template <int S> __device__ __forceinline__ float2 mul_si(float2 a) {
-  return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+template <int S, class C> __device__ __forceinline__ C mul_si(C a) {
+  return S > 0 ? make_c(-a.y, a.x) : make_c(a.y, -a.x);
 }
 // a * (c + S i s)
-template <int S> __device__ __forceinline__ float2 mul_cs(float2 a, float c, float s) {
-  return S > 0 ? make_float2(fmaf(a.x, c, -a.y * s), fmaf(a.y, c, a.x * s))
-               : make_float2(fmaf(a.x, c, a.y * s), fmaf(a.y, c, -a.x * s));
+template <int S, class C> __device__ __forceinline__ C mul_cs(C a, double cd, double sd) {
+  const real_t<C> c = (real_t<C>)cd, s = (real_t<C>)sd;
+  return S > 0 ? make_c(fma_(a.x, c, -a.y * s), fma_(a.y, c, a.x * s))
+               : make_c(fma_(a.x, c, a.y * s), fma_(a.y, c, -a.x * s));
 }
 
 // cos(pi/4), cos(pi/8), sin(pi/8), sqrt(3)/2
-constexpr float kR2 = 0.70710678118654752440f;
-constexpr float kC8 = 0.92387953251128675613f;
-constexpr float kS8 = 0.38268343236508977173f;
-constexpr float kH3 = 0.86602540378443864676f;
+constexpr double kR2 = 0.70710678118654752440;
+constexpr double kC8 = 0.92387953251128675613;
+constexpr double kS8 = 0.38268343236508977173;
+constexpr double kH3 = 0.86602540378443864676;
 
 // In-place length-R DFT with kernel exp(S 2 pi i n k / R), natural order in and out.
 template <int R, int S> struct Dft;
 
 template <int S> struct Dft<2, S> {
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 t = v[0];
+  template <class C> __device__ __forceinline__ static void run(C* v) {
+    C t = v[0];
     v[0] = cadd(t, v[1]);
     v[1] = csub(t, v[1]);
   }
 };
 
 template <int S> struct Dft<3, S> {
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 t = cadd(v[1], v[2]);
-    float2 u = cscale(mul_si<S>(csub(v[1], v[2])), kH3);
-    float2 m = make_float2(fmaf(-0.5f, t.x, v[0].x), fmaf(-0.5f, t.y, v[0].y));
+  template <class C> __device__ __forceinline__ static void run(C* v) {
+    const real_t<C> half = (real_t<C>)-0.5;
+    C t = cadd(v[1], v[2]);
+    C u = cscale(mul_si<S>(csub(v[1], v[2])), (real_t<C>)kH3);
+    C m = make_c(fma_(half, t.x, v[0].x), fma_(half, t.y, v[0].y));
     v[0] = cadd(v[0], t);
     v[1] = cadd(m, u);
     v[2] = csub(m, u);
@@ -59,9 +68,9 @@ template <int S> struct Dft<3, S> {
 };
 
 template <int S> struct Dft<4, S> {
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-    float2 t2 = cadd(v[1], v[3]), t3 = mul_si<S>(csub(v[1], v[3]));
+  template <class C> __device__ __forceinline__ static void run(C* v) {
+    C t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
+    C t2 = cadd(v[1], v[3]), t3 = mul_si<S>(csub(v[1], v[3]));
     v[0] = cadd(t0, t2);
     v[2] = csub(t0, t2);
     v[1] = cadd(t1, t3);
@@ -70,9 +79,9 @@ template <int S> struct Dft<4, S> {
 };
 
 template <int S> struct Dft<8, S> {
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 e[4] = {v[0], v[2], v[4], v[6]};
-    float2 o[4] = {v[1], v[3], v[5], v[7]};
+  template <class C> __device__ __forceinline__ static void run(C* v) {
+    C e[4] = {v[0], v[2], v[4], v[6]};
+    C o[4] = {v[1], v[3], v[5], v[7]};
     Dft<4, S>::run(e);
     Dft<4, S>::run(o);
     o[1] = mul_cs<S>(o[1], kR2, kR2);
@@ -87,8 +96,8 @@ template <int S> struct Dft<8, S> {
 };
 
 template <int S> struct Dft<16, S> {
-  __device__ __forceinline__ static void run(float2* v) {
-    float2 e[8], o[8];
+  template <class C> __device__ __forceinline__ static void run(C* v) {
+    C e[8], o[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       e[k] = v[2 * k];
@@ -113,14 +122,14 @@ template <int S> struct Dft<16, S> {
 
 // Inter-stage twiddles: input r of butterfly j times w^(r k), k = j mod NS,
 // w = exp(SIGN 2 pi i/(NS R)) = tw[N/(NS R)] (tw[m] = exp(-2 pi i m/N), conjugated for SIGN > 0).
-template <int N, int R, int NS, int SIGN>
-__device__ __forceinline__ void twiddle(float2* v, int j, const float2* tw) {
+template <int N, int R, int NS, int SIGN, class C>
+__device__ __forceinline__ void twiddle(C* v, int j, const C* tw) {
   if constexpr (NS > 1) {
     const int k = j % NS;
     constexpr int STEP = N / (NS * R);
 #pragma unroll
     for (int r = 1; r < R; ++r) {
-      float2 w = tw[r * k * STEP];
+      C w = tw[r * k * STEP];
       if (SIGN > 0) w.y = -w.y;
       v[r] = cmul(v[r], w);
     }
@@ -191,10 +200,10 @@ __device__ __forceinline__ void fft_stage_stream(const float2* tw, Load load, St
 
 // The same stage over LINES independent lines, lanes walking across lines (x[pos * pitch + line] in
 // shared memory is then read and written contiguously by a warp).
-template <int N, int R, int NS, int SIGN, int LINES, int NT, class Load, class Mid, class Store>
-__device__ __forceinline__ void line_stage(const float2* tw, Load load, Mid mid, Store store) {
+template <int N, int R, int NS, int SIGN, int LINES, int NT, class C, class Load, class Mid, class Store>
+__device__ __forceinline__ void line_stage(const C* tw, Load load, Mid mid, Store store) {
   constexpr int NJ = N / R, NB = NJ * LINES, PER = (NB + NT - 1) / NT;
-  float2 v[PER][R];
+  C v[PER][R];
 #pragma unroll
   for (int it = 0; it < PER; ++it) {
     const int u = threadIdx.x + it * NT, line = u % LINES, j = u / LINES;

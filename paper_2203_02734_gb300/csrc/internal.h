@@ -7,7 +7,8 @@
 
 namespace pw {
 namespace smu {
-struct Inst;
+template <class C> struct Inst;
+template <class C> struct TabArgs;
 }
 }  // namespace pw
 
@@ -37,9 +38,10 @@ struct PlaneArgs {
 cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s,
                             cudaEvent_t* ev);
 
-// S and mu without the CSDA (smu.cuh) of the instances of grid size N and launch round `chunk` in
-// list[0 .. n) (device), or of the one instance `one` where list is null (n = 1).
-cudaError_t launch_smu(int N, const pw::smu::Inst* list, const pw::smu::Inst& one, int n, int chunk, bool any_mu,
-                       cudaStream_t s);
+// S and mu without the CSDA (smu.cuh): the tables of n instances, then those of grid size N and launch round
+// `chunk` among them (device lists, FP32); or one instance (FP64).
+cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<float2>* list, int n, cudaStream_t s);
+cudaError_t launch_smu_list(int N, const pw::smu::Inst<float2>* list, int n, int chunk, bool any_mu, cudaStream_t s);
+cudaError_t launch_smu_one(const pw::smu::TabArgs<double2>& t, const pw::smu::Inst<double2>& q, cudaStream_t s);
 
 }  // namespace pwi

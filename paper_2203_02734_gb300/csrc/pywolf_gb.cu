@@ -23,6 +23,7 @@
 #include "delta.cuh"
 #include "grad.cuh"
 #include "plane.cuh"
+#include "smu.cuh"
 #include "r128.cuh"
 #include "r96.cuh"
 
@@ -818,6 +819,14 @@ pw_status propagate_planes(pw_csd* h, double z) {
   return PW_OK;
 }
 
+// Aperture as n_i^2 + n_j^2 <= threshold: the integer floor of the table kernel's FP64 threshold (r^2 is an
+// integer, the same decision), -1 for none.
+int aperture_threshold(const pw_csd* h) {
+  if (!(h->aperture > 0.0)) return -1;
+  const double rp = h->aperture / h->d, thr = rp * rp;
+  return thr >= 2147483647.0 ? 2147483647 : (int)std::floor(thr);
+}
+
 // Tables of a sparse source (delta.cuh) into the work buffer: D, and with a row al and be.
 cudaError_t delta_tables(pw_csd* h, pw::delta::TabArgs& t) {
   const int N = h->N, G = pw::delta::table_groups(N);
@@ -897,16 +906,52 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
   R128Extra x{};
   x.Ein = h->Ein;
   x.mask = reinterpret_cast<const float2*>(h->mask);
-  x.ap_ithr = -1;
+  x.ap_ithr = aperture_threshold(h);
   x.err = h->err;
-  if (h->aperture > 0.0) {
-    const double rp = h->aperture / h->d;
-    const double thr = rp * rp;  // the FP64 threshold of the table kernel; r^2 is an integer
-    x.ap_ithr = thr >= 2147483647.0 ? 2147483647 : (int)std::floor(thr);
-  }
   cudaError_t e = dispatch(h->N, herm, h->vmap, a, b, x, h->stream, next_events(h));
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch");
   to_output_plane(h, lz / (h->N * h->d), herm);
+  return PW_OK;
+}
+
+// S and mu(P1, .) after a propagation of the recorded GSM source, without it (smu.cuh).
+pw_status gsm_s_mu(pw_csd* h, double z, bool farfield, int iP, int jP, float* S, pw_c32* mu) {
+  if (h->kind != SRC_GSM) return fail(PW_ESTATE, "no Gaussian Schell-model source recorded for the current plane");
+  if (h->Nz > 0 || !supported(h->N) || h->N < 4)
+    return fail(PW_EUNSUPPORTED, "S and mu alone need an unpadded grid with an FFT plan, N >= 4");
+  const int N = h->N;
+  const double d = h->d, lam = h->lambda, lz = lam * z, dx = lz / (N * d), base = d * d / (2.0 * lam);
+  const double invf = h->lens_f != 0.0 ? 1.0 / h->lens_f : 0.0;
+  double2* w = reinterpret_cast<double2*>(h->work);  // 6 N^2 values of scratch, then 5.5 N of tables
+  pw::smu::TabArgs<double2> t{};
+  t.N = N;
+  t.Kin = farfield ? -base * invf : base * (1.0 / z - invf);
+  t.Kout = dx * dx / (2.0 * lz);
+  t.gs = d * d / (4.0 * h->sigma_S * h->sigma_S);
+  t.gm = d * d / (2.0 * h->sigma_mu * h->sigma_mu);
+  t.tw = w + (size_t)6 * N * N;
+  t.P1 = t.tw + 2 * N;
+  t.Eout = t.P1 + N;
+  t.k = reinterpret_cast<double*>(t.Eout + N);
+  t.K = t.k + N;
+  pw::smu::Inst<double2> q{};
+  q.N = N;
+  q.iP = iP;
+  q.jP = jP;
+  q.factor = (d * d / lz) * (d * d / lz) * h->A / (4.0 * N * N);
+  q.tw = t.tw;
+  q.P1 = t.P1;
+  q.P1l = t.P1;  // not used in FP64
+  q.Eout = t.Eout;
+  q.k = t.k;
+  q.K = t.K;
+  q.mask = reinterpret_cast<const float2*>(h->mask);
+  q.ap_ithr = aperture_threshold(h);
+  q.scratch = w;
+  q.S = S;
+  q.mu = reinterpret_cast<float2*>(mu);
+  const cudaError_t e = pwi::launch_smu_one(t, q, h->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "S/mu launch (GSM source)");
   return PW_OK;
 }
 
@@ -1465,10 +1510,16 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
     const int rows = std::max(1, 256 / N), nt = (rows * N + 31) / 32 * 32;
     const pw::delta::GradArgs ga{N, h->Eout, t.q, t.D, t.al, t.be, h->gtab, a->dev_amask, (float)s, (float)(d * d),
                                  h->gpart, a->dev_grad_amask, (float)(4.0 * c * a->amplitude)};
-    g.rows = std::min(NN, num_sms() * (2048 / nt));
+    const int nc = N % 4 == 0 ? 4 : 2;  // columns a block takes together
     const size_t sh = N * sizeof(float2);
-    if (has_mu) pw::delta::grad_kernel<true><<<g.rows, nt, sh, st>>>(ga);
-    else pw::delta::grad_kernel<false><<<g.rows, nt, sh, st>>>(ga);
+    auto grad = [&](auto k) -> cudaError_t {  // one wave of resident blocks
+      const cudaError_t r = persistent_grid(k, nt, sh, NN / nc, &g.rows);
+      if (r == cudaSuccess) k<<<g.rows, nt, sh, st>>>(ga);
+      return r;
+    };
+    if (nc == 4) e = has_mu ? grad(pw::delta::grad_kernel<true, 4>) : grad(pw::delta::grad_kernel<false, 4>);
+    else e = has_mu ? grad(pw::delta::grad_kernel<true, 2>) : grad(pw::delta::grad_kernel<false, 2>);
+    if (e != cudaSuccess) return done(cuda_fail(e, "gradient launch"));
     pw::gsm_gradient_reduce<<<1, 256, 0, st>>>(g);
     if ((e = cudaGetLastError()) != cudaSuccess) return done(cuda_fail(e, "gradient launch"));
   }
@@ -1492,6 +1543,17 @@ pw_status pw_propagate_fresnel_adjoint(pw_csd* h, double z_m, const pw_adjoint* 
 pw_status pw_propagate_farfield_adjoint(pw_csd* h, double z_m, const pw_adjoint* a) {
   g_err.clear();
   return adjoint(h, z_m, true, a);
+}
+
+pw_status pw_gsm_s_mu(pw_csd* h, double z_m, int farfield, int iP, int jP, float* dev_S, pw_c32* dev_mu) {
+  g_err.clear();
+  if (!h || !dev_S) return fail(PW_EINVAL, "null argument");
+  if (!finite_pos(z_m)) return fail(PW_EINVAL, "propagation distance must be finite and > 0 (got %g)", z_m);
+  if (!aligned(dev_S, 4)) return fail(PW_EINVAL, "dev_S must be 4-byte aligned");
+  if (dev_mu && !aligned(dev_mu, 8)) return fail(PW_EINVAL, "dev_mu must be 8-byte aligned");
+  if (iP < 0 || jP < 0 || iP >= h->N || jP >= h->N)
+    return fail(PW_EINVAL, "P1 = (%d, %d) outside the %d x %d grid", iP, jP, h->N, h->N);
+  return gsm_s_mu(h, z_m, farfield != 0, iP, jP, dev_S, dev_mu);
 }
 
 pw_status pw_propagate_fresnel(pw_csd* h, double z_m) {

@@ -11,8 +11,10 @@
 // axis): C is the inverse transform of |P^|^2, and R that of
 //   K(m) K(n) conj P^(2 iP - m, 2 jP - n), K = the transform of k,
 // so an instance costs a few FFTs of (2N)^2 points in place of an N^4 array.  (The 4D route took 0.99 ms
-// for one instance at N = 128, 87 ms for a batch of 192.)  Everything but the small tables is FP32, as
-// on the 4D route.
+// for one instance at N = 128, 87 ms for a batch of 192.)  A batch runs in FP32, as the 4D route did.  A few
+// lags carry most of S, so their rounding errors do not average out as the 4D route's did: for the forward
+// pass of an inverse problem, whose loss may be the small difference of two S, the single call runs in
+// FP64 (C = double2; 8 MFLOP at N = 96).
 //   k1: columns b, transform over a              -> X1[m][b]   (L x N)
 //   k2: rows m, transform over b; |P^|^2 back to v, times k(v), to b' -> Z1[m][b'];
 //       the R product back to d                  -> Z2[m][d]   (L x N each)
@@ -29,35 +31,38 @@
 namespace pw {
 namespace smu {
 
+template <class C>
 struct Inst {
+  using R = real_t<C>;
   int N, iP, jP;
   int chunk;            // launch round: instances of one round have scratch of their own
-  float factor;         // s A / L^2
-  const float2* tw;     // L twiddles exp(-2 pi i m / L)
-  const float2* P1;     // N: Ein(i) h(i)
-  const float2* Eout;   // N
-  const float* k;       // N: k(u)
-  const float* K;       // L: transform of k over |u| < N
+  double factor;        // s A / L^2
+  const C* tw;          // L twiddles exp(-2 pi i m / L)
+  const C* P1;          // N: Ein(i) h(i)
+  const C* P1l;         // N: what rounding P1 left out
+  const C* Eout;        // N
+  const R* k;           // N: k(u)
+  const R* K;           // L: transform of k over |u| < N
   const float2* mask;   // N x N or nullptr
   int ap_ithr;          // aperture, as in batch.cuh
-  float2* scratch;      // 3 L N values
+  C* scratch;           // 3 L N values
   float* S;             // N x N
   float2* mu;           // N x N or nullptr
 };
 
 template <int N> __host__ __device__ constexpr int lines() { return N % 16 == 0 ? (N >= 256 ? 8 : 16) : N % 8 == 0 ? 8 : N; }
 template <int N> __host__ __device__ constexpr int threads() { return N >= 64 ? 256 : 128; }
-template <int N> constexpr size_t smem_bytes() {
-  return (size_t)(2 * 2 * N * (lines<N>() + 1) + 3 * N) * sizeof(float2);
+template <int N, class C> constexpr size_t smem_bytes() {
+  return (size_t)(2 * 2 * N * (lines<N>() + 1) + 3 * N) * sizeof(C);
 }
 
 // In-place transform of the block's lines (length LEN, natural order), after a barrier and ending with one.
-template <int LEN, int SIGN, int LINES, int NT, int I = 0>
-__device__ __forceinline__ void fft_lines(float2* x, const float2* tw) {
+template <int LEN, int SIGN, int LINES, int NT, int I = 0, class C>
+__device__ __forceinline__ void fft_lines(C* x, const C* tw) {
   if constexpr (I < Plan<LEN>::stages) {
     constexpr int LP = LINES + 1;
     auto ld = [x](int line, int pos) { return x[pos * LP + line]; };
-    auto st = [x](int line, int pos, float2 v) { x[pos * LP + line] = v; };
+    auto st = [x](int line, int pos, C v) { x[pos * LP + line] = v; };
     line_stage<LEN, StageInfo<LEN, I>::R, StageInfo<LEN, I>::NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
     __syncthreads();
     fft_lines<LEN, SIGN, LINES, NT, I + 1>(x, tw);
@@ -65,52 +70,76 @@ __device__ __forceinline__ void fft_lines(float2* x, const float2* tw) {
 }
 
 // The tables of a block: tw (L) and twN (N = every other entry).
-template <int N>
-__device__ __forceinline__ void load_tw(const Inst& in, float2* tw, float2* twN) {
+template <int N, class C>
+__device__ __forceinline__ void load_tw(const Inst<C>& in, C* tw, C* twN) {
   for (int i = threadIdx.x; i < 2 * N; i += threads<N>()) {
-    const float2 v = in.tw[i];
+    const C v = in.tw[i];
     tw[i] = v;
     if (!(i & 1)) twN[i >> 1] = v;
   }
 }
 
+// (a + al)(b + bl) rounded once: the field's rounding errors reach every output alike, so the product
+// of two rounded factors cost mu a third of its accuracy where S is small.
+__device__ __forceinline__ float2 cmul_exact(float2 a, float2 al, float2 b, float2 bl) {
+  auto dot = [](float x, float xl, float y, float yl, float u, float ul, float v, float vl) {  // x y + u v
+    const float p = x * y, q = u * v, s = p + q, z = s - p;
+    const float es = (p - (s - z)) + (q - z);  // exact error of p + q
+    float e = fmaf(x, y, -p) + fmaf(u, v, -q) + es;
+    e = fmaf(x, yl, fmaf(xl, y, e));
+    e = fmaf(u, vl, fmaf(ul, v, e));
+    return s + e;
+  };
+  return make_float2(dot(a.x, al.x, b.x, bl.x, -a.y, -al.y, b.y, bl.y), dot(a.x, al.x, b.y, bl.y, a.y, al.y, b.x, bl.x));
+}
+
+__device__ __forceinline__ double2 cmul_exact(double2 a, double2, double2 b, double2) { return cmul(a, b); }
+
 // P(a, b): source field at a point.
-template <int N>
-__device__ __forceinline__ float2 field(const Inst& in, int a, int b) {
+template <int N, class C>
+__device__ __forceinline__ C field(const Inst<C>& in, int a, int b) {
+  using R = real_t<C>;
   const int na = a - N / 2, nb = b - N / 2;
-  if (in.ap_ithr >= 0 && na * na + nb * nb > in.ap_ithr) return make_float2(0.f, 0.f);
-  float2 v = cmul(__ldg(in.P1 + a), __ldg(in.P1 + b));
-  if (in.mask) v = cmul(v, __ldg(in.mask + a * N + b));
+  if (in.ap_ithr >= 0 && na * na + nb * nb > in.ap_ithr) return make_c((R)0, (R)0);
+  C v = cmul_exact(__ldg(in.P1 + a), __ldg(in.P1l + a), __ldg(in.P1 + b), __ldg(in.P1l + b));
+  if (in.mask) {
+    const float2 m = __ldg(in.mask + a * N + b);
+    v = cmul(v, make_c((R)m.x, (R)m.y));
+  }
   return v;
 }
 
 // x[v] <- k(v) x[v] + k(N - v) x[v + N] for v < N: the weighted lags v and v - N, folded mod N.
-template <int N, int LINES, int NT>
-__device__ __forceinline__ void fold(float2* x, const float* k) {
+template <int N, int LINES, int NT, class C>
+__device__ __forceinline__ void fold(C* x, const real_t<C>* k) {
   constexpr int LP = LINES + 1;
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int line = e % LINES, v = e / LINES;
-    float2 y = cscale(x[v * LP + line], __ldg(k + v));
+    C y = cscale(x[v * LP + line], __ldg(k + v));
     if (v > 0) y = cadd(y, cscale(x[(v + N) * LP + line], __ldg(k + N - v)));
     x[v * LP + line] = y;
   }
   __syncthreads();
 }
 
-__device__ __forceinline__ Inst pick(const Inst* list, const Inst& one) { return list ? list[blockIdx.y] : one; }
+template <class C>
+__device__ __forceinline__ Inst<C> pick(const Inst<C>* list, const Inst<C>& one) {
+  return list ? list[blockIdx.y] : one;
+}
 
-template <int N>
-__global__ void __launch_bounds__(threads<N>()) k1(const Inst* list, Inst one, int chunk) {
+template <int N, class C>
+__global__ void __launch_bounds__(threads<N>()) k1(const Inst<C>* list, Inst<C> one, int chunk) {
+  using R = real_t<C>;
   constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
-  const Inst in = pick(list, one);
+  const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
-  extern __shared__ __align__(16) float2 smem[];
-  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  extern __shared__ __align__(16) unsigned char smem[];
+  C *x = reinterpret_cast<C*>(smem), *tw = x + 2 * L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int b0 = blockIdx.x * LINES;
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, a = e / LINES;
-    x[a * LP + line] = a < N ? field<N>(in, a, b0 + line) : make_float2(0.f, 0.f);
+    x[a * LP + line] = a < N ? field<N, C>(in, a, b0 + line) : make_c((R)0, (R)0);
   }
   __syncthreads();
   fft_lines<L, -1, LINES, NT>(x, tw);
@@ -120,21 +149,22 @@ __global__ void __launch_bounds__(threads<N>()) k1(const Inst* list, Inst one, i
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(threads<N>()) k2(const Inst* list, Inst one, int chunk) {
+template <int N, class C>
+__global__ void __launch_bounds__(threads<N>()) k2(const Inst<C>* list, Inst<C> one, int chunk) {
+  using R = real_t<C>;
   constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
-  const Inst in = pick(list, one);
+  const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
-  extern __shared__ __align__(16) float2 smem[];
-  float2 *x = smem, *y = x + L * LP, *tw = y + L * LP, *twN = tw + L;
+  extern __shared__ __align__(16) unsigned char smem[];
+  C *x = reinterpret_cast<C*>(smem), *y = x + L * LP, *tw = y + L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int m0 = blockIdx.x * LINES;
-  const float2* X1 = in.scratch;
-  float2* Z1 = in.scratch + (size_t)L * N;
-  float2* Z2 = Z1 + (size_t)L * N;
+  const C* X1 = in.scratch;
+  C* Z1 = in.scratch + (size_t)L * N;
+  C* Z2 = Z1 + (size_t)L * N;
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int b = e % L, line = e / L;
-    x[b * LP + line] = b < N ? X1[(m0 + line) * N + b] : make_float2(0.f, 0.f);
+    x[b * LP + line] = b < N ? X1[(m0 + line) * N + b] : make_c((R)0, (R)0);
   }
   __syncthreads();
   fft_lines<L, -1, LINES, NT>(x, tw);  // P^(m, n)
@@ -150,8 +180,8 @@ __global__ void __launch_bounds__(threads<N>()) k2(const Inst* list, Inst one, i
   }
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, n = e / LINES;
-    const float2 v = x[n * LP + line];
-    x[n * LP + line] = make_float2(fmaf(v.x, v.x, v.y * v.y), 0.f);
+    const C v = x[n * LP + line];
+    x[n * LP + line] = make_c(fma_(v.x, v.x, v.y * v.y), (R)0);
   }
   __syncthreads();
   fft_lines<L, +1, LINES, NT>(x, tw);
@@ -172,18 +202,19 @@ __global__ void __launch_bounds__(threads<N>()) k2(const Inst* list, Inst one, i
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(threads<N>()) k3(const Inst* list, Inst one, int chunk) {
+template <int N, class C>
+__global__ void __launch_bounds__(threads<N>()) k3(const Inst<C>* list, Inst<C> one, int chunk) {
+  using R = real_t<C>;
   constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
-  const Inst in = pick(list, one);
+  const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
-  extern __shared__ __align__(16) float2 smem[];
-  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  extern __shared__ __align__(16) unsigned char smem[];
+  C *x = reinterpret_cast<C*>(smem), *tw = x + 2 * L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int b0 = blockIdx.x * LINES;
-  float2* X3 = in.scratch;
-  const float2* Z1 = in.scratch + (size_t)L * N;
-  const float2* Z2 = Z1 + (size_t)L * N;
+  C* X3 = in.scratch;
+  const C* Z1 = in.scratch + (size_t)L * N;
+  const C* Z2 = Z1 + (size_t)L * N;
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, m = e / LINES;
     x[m * LP + line] = Z1[m * N + b0 + line];
@@ -194,7 +225,7 @@ __global__ void __launch_bounds__(threads<N>()) k3(const Inst* list, Inst one, i
   fft_lines<N, -1, LINES, NT>(x, twN);
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int line = e % LINES, a = e / LINES;
-    in.S[a * N + b0 + line] = x[a * LP + line].x * in.factor;
+    in.S[a * N + b0 + line] = (float)(x[a * LP + line].x * (R)in.factor);
   }
   if (!in.mu) return;
   __syncthreads();
@@ -206,7 +237,7 @@ __global__ void __launch_bounds__(threads<N>()) k3(const Inst* list, Inst one, i
   fft_lines<L, +1, LINES, NT>(x, tw);
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int line = e % LINES, c = e / LINES;
-    x[c * LP + line] = cmul(field<N>(in, c, b0 + line), x[c * LP + line]);
+    x[c * LP + line] = cmul(field<N, C>(in, c, b0 + line), x[c * LP + line]);
   }
   __syncthreads();
   fft_lines<N, -1, LINES, NT>(x, twN);
@@ -216,13 +247,14 @@ __global__ void __launch_bounds__(threads<N>()) k3(const Inst* list, Inst one, i
   }
 }
 
-template <int N>
-__global__ void __launch_bounds__(threads<N>()) k4(const Inst* list, Inst one, int chunk) {
+template <int N, class C>
+__global__ void __launch_bounds__(threads<N>()) k4(const Inst<C>* list, Inst<C> one, int chunk) {
+  using R = real_t<C>;
   constexpr int LINES = lines<N>(), LP = LINES + 1, NT = threads<N>(), L = 2 * N;
-  const Inst in = pick(list, one);
+  const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk || !in.mu) return;
-  extern __shared__ __align__(16) float2 smem[];
-  float2 *x = smem, *tw = x + 2 * L * LP, *twN = tw + L;
+  extern __shared__ __align__(16) unsigned char smem[];
+  C *x = reinterpret_cast<C*>(smem), *tw = x + 2 * L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int c0 = blockIdx.x * LINES;
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
@@ -232,71 +264,89 @@ __global__ void __launch_bounds__(threads<N>()) k4(const Inst* list, Inst one, i
   __syncthreads();
   fft_lines<N, -1, LINES, NT>(x, twN);
   const float sp = in.S[in.iP * N + in.jP];
-  const float2 ep = cscale(cconj(cmul(__ldg(in.Eout + in.iP), __ldg(in.Eout + in.jP))), in.factor);
+  const C ep = cscale(cconj(cmul(__ldg(in.Eout + in.iP), __ldg(in.Eout + in.jP))), (R)in.factor);
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int d = e % N, line = e / N, c = c0 + line;
     const float den = sp * in.S[c * N + d];
-    const float2 row = cmul(cmul(ep, cmul(__ldg(in.Eout + c), __ldg(in.Eout + d))), x[d * LP + line]);
-    in.mu[c * N + d] = den > 0.f ? cscale(row, rsqrtf(den)) : make_float2(0.f, 0.f);
+    const C row = cmul(cmul(ep, cmul(__ldg(in.Eout + c), __ldg(in.Eout + d))), x[d * LP + line]);
+    const float inv = rsqrtf(den);
+    in.mu[c * N + d] = den > 0.f ? make_float2((float)row.x * inv, (float)row.y * inv) : make_float2(0.f, 0.f);
   }
 }
 
 // FP64-derived tables of one instance (one block): twiddles, per-axis factors, coherence and its
 // transform.
+template <class C>
 struct TabArgs {
   int N;
   double Kin, Kout;  // turns per n^2 of the input factor (propagator, lens) and of the output propagator
   double gs, gm;     // d^2/(4 sigma_S^2), d^2/(2 sigma_mu^2)
-  float2 *tw, *P1, *Eout;
-  float *k, *K;
+  C *tw, *P1, *P1l, *Eout;  // P1l: float2 only
+  real_t<C> *k, *K;
 };
 
 // The N = blockDim.x-strided work of each table; a block barrier separates k, tw from K.
-__device__ __forceinline__ void tables(const TabArgs& t) {
+__device__ __forceinline__ void put(float2* h, float2* l, int i, double x, double y) {
+  h[i] = make_float2((float)x, (float)y);
+  if (l) l[i] = make_float2((float)(x - (double)(float)x), (float)(y - (double)(float)y));
+}
+__device__ __forceinline__ void put(double2* h, double2*, int i, double x, double y) { h[i] = make_double2(x, y); }
+
+template <class C>
+__device__ __forceinline__ void tables(const TabArgs<C>& t) {
+  using R = real_t<C>;
   const int N = t.N, L = 2 * N, M = N / 2;
   // one FP64 evaluation per thread and step: tasks 0..L-1 tw, then P1, Eout and k of each index
   for (int q = threadIdx.x; q < L + 3 * N; q += blockDim.x) {
-    if (q < L) {
-      t.tw[q] = cis_turns(-(double)q / (double)L);
+    const int kind = q < L ? -1 : (q - L) / N, i = q < L ? q : (q - L) - kind * N;
+    const double n2 = (double)(i - M) * (double)(i - M);
+    if (kind == 2) {
+      t.k[i] = (R)exp(-(double)i * (double)i * t.gm);
       continue;
     }
-    const int kind = (q - L) / N, i = (q - L) - kind * N;
-    const double n2 = (double)(i - M) * (double)(i - M);
-    if (kind == 0) t.P1[i] = cscale(cis_turns(frac_turns(n2 * t.Kin) + 0.5 * (i & 1)), (float)exp(-n2 * t.gs));
-    else if (kind == 1) t.Eout[i] = cis_turns(frac_turns(n2 * t.Kout) + 0.5 * (i & 1));
-    else t.k[i] = (float)exp(-(double)i * (double)i * t.gm);
+    const double turns = kind < 0 ? -(double)i / (double)L : frac_turns(n2 * (kind == 0 ? t.Kin : t.Kout)) + 0.5 * (i & 1);
+    double sn, cs;
+    sincospi(2.0 * frac_turns(turns), &sn, &cs);
+    if (kind < 0) {
+      put(t.tw, (C*)nullptr, i, cs, sn);
+    } else if (kind == 1) {
+      put(t.Eout, (C*)nullptr, i, cs, sn);
+    } else {
+      const double hh = exp(-n2 * t.gs);
+      put(t.P1, t.P1l, i, cs * hh, sn * hh);
+    }
   }
   __syncthreads();
   for (int m = threadIdx.x; m < L; m += blockDim.x) {
-    float acc = 0.f;
+    R acc = 0;
     int j = 0;  // m u mod L
     for (int u = 1; u < N; ++u) {
       j += m;
       j -= j >= L ? L : 0;
-      acc = fmaf(t.k[u], t.tw[j].x, acc);
+      acc = fma_(t.k[u], t.tw[j].x, acc);
     }
-    t.K[m] = fmaf(2.f, acc, t.k[0]);
+    t.K[m] = fma_((R)2, acc, t.k[0]);
   }
 }
 
-template <int N>
-cudaError_t launch(const Inst* list, const Inst& one, int n, int chunk, bool any_mu, cudaStream_t s) {
+template <int N, class C>
+cudaError_t launch(const Inst<C>* list, const Inst<C>& one, int n, int chunk, bool any_mu, cudaStream_t s) {
   constexpr int LINES = lines<N>(), NT = threads<N>();
-  constexpr size_t sm = smem_bytes<N>();
+  constexpr size_t sm = smem_bytes<N, C>();
   static bool ready = false;
   cudaError_t e = cudaSuccess;
   if (!ready) {
-    if ((e = cudaFuncSetAttribute(k1<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k3<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k4<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k1<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k2<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k3<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(k4<N, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
       return e;
     ready = true;
   }
-  k1<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
-  k2<N><<<dim3(2 * N / LINES, n), NT, sm, s>>>(list, one, chunk);
-  k3<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
-  if (any_mu) k4<N><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k1<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k2<N, C><<<dim3(2 * N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k3<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  if (any_mu) k4<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
   return cudaGetLastError();
 }
 

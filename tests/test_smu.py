@@ -82,3 +82,33 @@ def test_batch_without_w_matches_the_handle(N, n, pool, mask):
         if sp >= 1e-2 * Sh.max():
             ok = Sh >= 1e-2 * Sh.max()
             assert np.abs(mub - muh)[ok].max() < 2e-5
+
+
+# The handle's call against the propagation it stands for, at every grid size with a plan; bounds as above.
+@pytest.mark.gpu
+@pytest.mark.parametrize("N", [4, 6, 8, 12, 24, 48, 96, 128])
+@pytest.mark.parametrize("farfield", [False, True])
+def test_handle_s_mu_matches_the_propagation(N, farfield):
+    import torch
+    import paper_2203_02734_gb300 as pw
+    m = torch.from_numpy(WL.to_c64(WL.phase_screen(N, seed=9))).cuda()
+    P1 = (N // 2 - 1, N // 2)
+    c = pw.CSD(N, D, LAM)
+    c.source_gsm(5 * D, 1.5 * D, 1.3)
+    c.source_mask(m)
+    c.source_aperture(0.45 * N * D)
+    c.source_lens(0.6)
+    S = torch.empty(N, N, device="cuda")
+    mu = torch.empty(N, N, dtype=torch.complex64, device="cuda")
+    pw.pw_gsm_s_mu(c.h, 0.3, farfield, *P1, S.data_ptr(), mu.data_ptr())
+    assert abs(c.sampling() / D - 1) < 1e-12  # the current plane is untouched
+    (c.propagate_farfield if farfield else c.propagate_fresnel)(0.3)
+    Sp, mup = c.spectral_density(), c.degree_of_coherence(*P1)
+    with pytest.raises(pw.PwError, match="PW_ESTATE"):
+        pw.pw_gsm_s_mu(c.h, 0.3, farfield, *P1, S.data_ptr(), mu.data_ptr())
+    c.close()
+    Sp, S = Sp.cpu().numpy().astype(np.float64), S.cpu().numpy().astype(np.float64)
+    assert rel(S, Sp) < 2e-6
+    ok = Sp >= 1e-2 * Sp.max()
+    if ok[P1]:
+        assert np.abs((mu - mup).cpu().numpy()[ok]).max() < 2e-5
