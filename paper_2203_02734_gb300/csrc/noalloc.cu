@@ -110,8 +110,7 @@ pw_status run(const CUtensorMap& vmap, const pw::TableArgs& t, const pw::PassAAr
   int ga = 0, gb = 0;
   pw_status st = pass_grids<N>(&ga, &gb);
   if (st != PW_OK) return st;
-  const int NN = N * N;
-  pw::tables_kernel<<<(NN + 255) / 256, 256, 0, s>>>(t);
+  pw::tables_kernel<<<pw::tables_grid(t), pw::TABLE_NT, 0, s>>>(t);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) {
     pw::pass_a_kernel<N, pw::SRC_GSM><<<ga, pw::Plan<N>::NT, pw::pass_a_smem<N>(), s>>>(vmap, a);

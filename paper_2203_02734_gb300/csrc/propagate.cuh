@@ -59,30 +59,41 @@ struct TableArgs {
   float2* Ein;    // N per-axis input factors (-1)^i exp(2 pi i Kin n_i^2), or nullptr
 };
 
-static __global__ void tables_kernel(TableArgs t) {
-  const int N = t.N, M = N / 2;
-  const int NN = N * N;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < NN; idx += gridDim.x * blockDim.x) {
-    const int i = idx / N, j = idx - i * N;
-    const double ni = (double)(i - M), nj = (double)(j - M);
-    const double n2i = ni * ni, n2j = nj * nj;
-    const bool inside = t.ap_thr < 0.0 || (n2i + n2j) <= t.ap_thr;
-    float2 m = t.mask ? t.mask[idx] : make_float2(1.f, 0.f);
-    if (!inside) m = make_float2(0.f, 0.f);
-    const double turns = frac_turns(n2i * t.Kin) + frac_turns(n2j * t.Kin) + 0.5 * ((i + j) & 1);
-    t.F[idx] = cmul(cis_turns(turns), m);
-    if (t.M0) t.M0[idx] = cmul(cis_turns(frac_turns(n2i * t.K0) + frac_turns(n2j * t.K0)), m);
-    if (t.G) {
-      const double dij = (double)(i - j);
-      t.G[idx] = (float)exp(-(n2i + n2j) * t.gs - dij * dij * t.gm);
+// One FP64 sincospi or exp per thread (blockIdx.y: 0 F, 1 the per-axis tables, 2 G, 3 M0), in small blocks
+// spread over the SMs: an SM issues about two FP64 FMAs a cycle, so a block of 256 threads that evaluated
+// five of them each took 10 to 14 us at any N up to 128.
+constexpr int TABLE_NT = 64;
+inline dim3 tables_grid(const TableArgs& t) {
+  return dim3((t.N * t.N + TABLE_NT - 1) / TABLE_NT, t.M0 ? 4 : t.G ? 3 : 2);
+}
+static __global__ void __launch_bounds__(TABLE_NT) tables_kernel(TableArgs t) {
+  const int N = t.N, M = N / 2, NN = N * N, role = blockIdx.y;
+  const int idx = blockIdx.x * TABLE_NT + threadIdx.x;
+  if (role == 1) {
+    for (int q = idx; q < 3 * N; q += gridDim.x * TABLE_NT) {
+      const int kind = q / N, i = q - kind * N;
+      const double n = (double)(i - M), odd = 0.5 * (i & 1);
+      if (kind == 0) t.tw[i] = cis_turns(-(double)i / (double)N);
+      else if (kind == 1) t.Eout[i] = cis_turns(frac_turns(n * n * t.Kout) + odd);
+      else if (t.Ein) t.Ein[i] = cis_turns(frac_turns(n * n * t.Kin) + odd);
     }
-    if (idx < N) {
-      const double nk = (double)(idx - M);
-      t.tw[idx] = cis_turns(-(double)idx / (double)N);
-      t.Eout[idx] = cis_turns(frac_turns(nk * nk * t.Kout) + 0.5 * (idx & 1));
-      if (t.Ein) t.Ein[idx] = cis_turns(frac_turns(nk * nk * t.Kin) + 0.5 * (idx & 1));
-    }
+    return;
   }
+  if (idx >= NN) return;
+  const int i = idx / N, j = idx - i * N;
+  const double ni = (double)(i - M), nj = (double)(j - M);
+  const double n2i = ni * ni, n2j = nj * nj;
+  if (role == 2) {
+    if (!t.G) return;
+    const double dij = (double)(i - j);
+    t.G[idx] = (float)exp(-(n2i + n2j) * t.gs - dij * dij * t.gm);
+    return;
+  }
+  const bool inside = t.ap_thr < 0.0 || (n2i + n2j) <= t.ap_thr;
+  float2 m = t.mask ? t.mask[idx] : make_float2(1.f, 0.f);
+  if (!inside) m = make_float2(0.f, 0.f);
+  if (role == 0) t.F[idx] = cmul(cis_turns(frac_turns(n2i * t.Kin) + frac_turns(n2j * t.Kin) + 0.5 * ((i + j) & 1)), m);
+  else t.M0[idx] = cmul(cis_turns(frac_turns(n2i * t.K0) + frac_turns(n2j * t.K0)), m);
 }
 
 // Sources: the GSM model, an uploaded CSDA, and (dense path) a diagonal source.

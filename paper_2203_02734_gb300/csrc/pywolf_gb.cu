@@ -507,8 +507,8 @@ pw_status make_vmap(pw_csd* h) {
   return st;
 }
 
-// Fill F, M0, G, tw, Eout for a propagation over z (z <= 0: source-plane view only).
-pw_status build_tables(pw_csd* h, double z, bool farfield) {
+// Fill F, G, tw, Eout for a propagation over z (z <= 0: source-plane view only), and M0 where it is used.
+pw_status build_tables(pw_csd* h, double z, bool farfield, bool want_m0 = false) {
   const int N = h->N;
   const double d = h->d, lam = h->lambda;
   pw::TableArgs t{};
@@ -534,14 +534,11 @@ pw_status build_tables(pw_csd* h, double z, bool farfield) {
   }
   t.mask = reinterpret_cast<const float2*>(h->mask);
   t.F = h->F;
-  t.M0 = h->M0;
+  t.M0 = want_m0 ? h->M0 : nullptr;
   t.tw = h->tw;
   t.Eout = h->Eout;
   t.Ein = h->Ein;
-  const int NN = N * N;
-  const int threads = 256;
-  const int blocks = (NN + threads - 1) / threads;
-  pw::tables_kernel<<<blocks, threads, 0, h->stream>>>(t);
+  pw::tables_kernel<<<pw::tables_grid(t), pw::TABLE_NT, 0, h->stream>>>(t);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "table kernel launch");
   return PW_OK;
@@ -608,7 +605,7 @@ cudaError_t launch_axis_tc(const pw::dense_tc::Args& ax, int mode, const unsigne
 // Events as for the FFT passes: the first half of the contractions counts as the first pass.
 pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
   const int N = h->N, Nz = h->Nz > 0 ? h->Nz : N;
-  pw_status st = build_tables(h, z, farfield);  // G and M0 (the FFT factors are not used here)
+  pw_status st = build_tables(h, z, farfield, true);  // G and M0 (the FFT factors are not used here)
   if (st != PW_OK) return st;
   const double d = h->d, lz = h->lambda * z, dx = lz / (Nz * d);
   cudaStream_t s = h->stream;
@@ -959,7 +956,7 @@ pw_status s_mu(pw_csd* h, int iP, int jP, float* S, pw_c32* mu) {
   if (h->kind == SRC_NONE) return fail(PW_ESTATE, "no source set for the current plane");
   // A propagated plane without masks needs no tables: S comes from the pass-B epilogue.
   if (h->kind != SRC_PROPAGATED || has_masks(h)) {
-    pw_status st = build_tables(h, 0.0, false);
+    pw_status st = build_tables(h, 0.0, false, true);
     if (st != PW_OK) return st;
   }
   pw::SMuArgs a{};
