@@ -456,7 +456,7 @@ pw_status pw_batch_run(pw_batch* b) {
       q.row = d.row;
       q.iP = d.iP;
       q.jP = d.jP;
-      e = pwi::dispatch_planes(d.N, b->wmaps[i], q, nullptr, b->stream, nullptr);
+      e = pwi::dispatch_planes(d.N, b->wmaps[i], q, cnt + 2 * b->n + 1, b->stream, nullptr);
       if (e != cudaSuccess) return cuda_fail(e, "batch instance launch");
     }
     return mu();

@@ -34,7 +34,7 @@ struct PlaneArgs {
   float2* row;  // W(P1, .) or nullptr
   int iP, jP;
 };
-// ev: nullptr or three events around the two passes; err: flag of a bounded wait (N = 256 only).
+// ev: nullptr or three events around the two passes; err: flag of a bounded wait that gave up.
 cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s,
                             cudaEvent_t* ev);
 

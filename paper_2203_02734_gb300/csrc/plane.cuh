@@ -221,69 +221,109 @@ __global__ void __launch_bounds__(r96::NT, 2) plane96_kernel(const __grid_consta
 constexpr size_t plane96_smem() { return (size_t)96 * r96::P * sizeof(float2) + 2 * 96 * sizeof(float2); }
 
 // ---------------------------------------------------------------------------------------------
-// N = 128: the register stages of r128.cuh, one CTA per SM.  Stage 3 takes column pairs (16-byte
-// shared-memory accesses) of the warp's own eight buffer rows; each warp leaves its rows
-// a' = warp + 16 i by one TMA store, which drains while the next plane is built.
-__global__ void __launch_bounds__(r128::NT, 1) plane128_kernel(const __grid_constant__ CUtensorMap wmap, Args p) {
+// N = 128: the register stages of r128.cuh, one CTA per SM, each CTA a contiguous range of planes (c' fastest).
+// Reading both factors when a plane starts brings 256 KB into an SM while nothing computes (4096 cycles
+// of its L2 bandwidth, 0.97 ms in all), so they come ahead of time, each warp's own rows by its own bulk
+// copies on its own mbarrier:
+//   - the 8 rows of T of the next plane land in the warp's eight buffer rows as soon as it has read its
+//     stage-3 inputs from them (the second exchange permutes rows by vrow, so these are its own);
+//   - six of its 8 rows of H stay in shared memory while b' is the same (96 KB; two are read through L2).
+// Stage 1 reads and exchange 1 writes only the warp's own rows, so three block barriers a plane are
+// enough.  Results go straight from registers to W, 16 bytes a lane; S and the P1 row are read back from
+// W by diag_row_kernel (tests for them in the store loop were 5 % of the plane's instructions).
+constexpr int HROWS128 = 6;
+constexpr size_t plane128_smem() {
+  return (size_t)(128 * 128 + 16 * HROWS128 * 128 + 2 * 128) * sizeof(float2) + 16 * sizeof(uint64_t);
+}
+__global__ void __launch_bounds__(r128::NT, 1) plane128_kernel(Args p, int* err) {
   using r128::N;
   using r128::NT;
+  constexpr int HR = HROWS128;
   extern __shared__ __align__(1024) float2 smem[];
   float2* buf = smem;
-  float2* tw = buf + N * N;
+  float2* hs = buf + N * N;  // 16 warps x HR rows of H
+  float2* tw = hs + 16 * HR * N;
   float2* eo = tw + N;
+  uint64_t* mbars = reinterpret_cast<uint64_t*>(eo + N);
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (int i = t; i < N; i += NT) {
     tw[i] = p.tw[i];
     eo[i] = p.Eout[i];
   }
-  __syncthreads();
-  for (int bc = blockIdx.x; bc < N * N; bc += gridDim.x) {
+  float2* rows = buf + 8 * warp * N;   // the warp's buffer rows: T rows a = warp + 16 rp
+  float2* hrows = hs + HR * warp * N;  // H rows a = warp + 16 rp, rp < HR
+  uint64_t* mbar = mbars + warp;
+  const int p0 = (int)((long long)blockIdx.x * N * N / gridDim.x), p1 = (int)((long long)(blockIdx.x + 1) * N * N / gridDim.x);
+  // lane 0: copies for plane bc (with H where b' is new to the warp)
+  auto fetch = [&](int bc, bool with_h) {
+    const int bq = bc / N, cq = bc - bq * N;
+    fence_proxy_async_smem();
+    t256::mbar_expect(mbar, (uint32_t)((8 + (with_h ? HR : 0)) * N * sizeof(float2)));
+    for (int rp = 0; rp < 8; ++rp)
+      bulk_g2s(rows + rp * N, p.T + ((size_t)cq * N + warp + 16 * rp) * N, N * sizeof(float2), mbar);
+    if (with_h)
+      for (int rp = 0; rp < HR; ++rp)
+        bulk_g2s(hrows + rp * N, p.H + ((size_t)bq * N + warp + 16 * rp) * N, N * sizeof(float2), mbar);
+  };
+  if (lane == 0) {
+    tc16::mbar_init(mbar);
+    if (p0 < p1) fetch(p0, true);
+  }
+  __syncthreads();  // tw, eo
+  uint32_t parity = 0;
+  int ok = 1;  // a wait that gave up sets *err; the warp then waits no more and its results are invalid
+  for (int bc = p0; bc < p1; ++bc, parity ^= 1u) {
     const int bq = bc / N, cq = bc - bq * N;
     const float2* __restrict__ H = p.H + (size_t)bq * N * N;
-    const float2* __restrict__ T = p.T + (size_t)cq * N * N;
+    float2 hx[8 - HR][4];
+#pragma unroll
+    for (int rp = HR; rp < 8; ++rp)
+#pragma unroll
+      for (int rq = 0; rq < 4; ++rq) hx[rp - HR][rq] = __ldg(H + (warp + 16 * rp) * N + lane + 32 * rq);
+    if (lane == 0 && ok) {
+      ok = tc16::mbar_wait(mbar, parity) ? 1 : 0;
+      if (!ok) atomicExch(err, 1);
+    }
+    __syncwarp();
     float2 v[8][4];
 #pragma unroll
     for (int rp = 0; rp < 8; ++rp)
 #pragma unroll
-      for (int rq = 0; rq < 4; ++rq) {
-        const int ad = (warp + 16 * rp) * N + lane + 32 * rq;
-        v[rp][rq] = cmul(__ldg(H + ad), __ldg(T + ad));
-      }
+      for (int rq = 0; rq < 4; ++rq)
+        v[rp][rq] = cmul(rp < HR ? hrows[rp * N + lane + 32 * rq] : hx[rp < HR ? 0 : rp - HR][rq], rows[rp * N + lane + 32 * rq]);
     r128::dft2d<8, 4, +1, -1>(v);
-    // exchange 1 writes only the warp's own eight buffer rows, which since the last block barrier
-    // only this warp has touched (stage 3, the write-back and its TMA store)
-    if (lane == 0) bulk_wait_read_all();
-    __syncwarp();
+    __syncwarp();  // the warp has read its rows of T; exchange 1 writes them
     float2 w3[2][4][4];
-    r128::stages_23<+1, true, -1, true>(v, w3, buf, tw);
-    __syncwarp();
+    r128::stages_23<+1, true, -1, true>(v, w3, buf, tw, [&]() {
+      __syncwarp();
+      if (lane == 0 && ok && bc + 1 < p1) fetch(bc + 1, cq == N - 1);
+    });
     const int half = lane >> 4, dq0 = 2 * (lane & 15);
+    float2* Wt = p.W + ((size_t)(warp + 16 * half) * N * N + bc) * N + dq0;
+    float4 ed[4];
+#pragma unroll
+    for (int rq = 0; rq < 4; ++rq) ed[rq] = *reinterpret_cast<const float4*>(eo + dq0 + 32 * rq);
 #pragma unroll
     for (int rp = 0; rp < 4; ++rp) {
-      const int aq = warp + 16 * half + 32 * rp;
-      const float2 ea = cscale(cconj(eo[aq]), p.scale);
+      const float2 ea = cscale(cconj(eo[warp + 16 * half + 32 * rp]), p.scale);
 #pragma unroll
       for (int rq = 0; rq < 4; ++rq) {
-        const int dq = dq0 + 32 * rq;
-        const float4 ed = *reinterpret_cast<const float4*>(eo + dq);
-        const float2 w0 = cmul(cmul(ea, make_float2(ed.x, ed.y)), w3[0][rp][rq]);
-        const float2 w1 = cmul(cmul(ea, make_float2(ed.z, ed.w)), w3[1][rp][rq]);
-        *reinterpret_cast<float4*>(buf + (8 * warp + half + 2 * rp) * N + dq) = make_float4(w0.x, w0.y, w1.x, w1.y);
+        const float2 w0 = cmul(cmul(ea, make_float2(ed[rq].x, ed[rq].y)), w3[0][rp][rq]);
+        const float2 w1 = cmul(cmul(ea, make_float2(ed[rq].z, ed[rq].w)), w3[1][rp][rq]);
+        *reinterpret_cast<float4*>(Wt + (size_t)32 * rp * N * N * N + 32 * rq) = make_float4(w0.x, w0.y, w1.x, w1.y);
       }
     }
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {  // rows a' = warp + 16 i
-      tma_store_5d(&wmap, buf + 8 * warp * N, 0, cq, bq, warp, 0);
-      bulk_commit();
-    }
-    if (warp == (cq & 15) && lane == 0) p.S[cq * N + bq] = buf[vrow<N>(cq) * N + bq].x;
-    if (p.row && bq == p.jP && warp == (p.iP & 15))
-      for (int d = lane; d < N; d += 32) p.row[cq * N + d] = buf[vrow<N>(p.iP) * N + d];
   }
-  if (lane == 0) bulk_wait_all();
+  if (!ok && lane == 0) tc16::mbar_wait(mbar, parity);  // a copy left in flight by a failed wait
+  __syncthreads();
 }
-constexpr size_t plane128_smem() { return (size_t)128 * 128 * sizeof(float2) + 2 * 128 * sizeof(float2); }
+
+__global__ void __launch_bounds__(256) diag_row_kernel(Args p, int N) {
+  const int NN = N * N, x = blockIdx.x * 256 + threadIdx.x;
+  if (x >= NN) return;
+  p.S[x] = p.W[(size_t)x * NN + x].x;
+  if (p.row) p.row[x] = p.W[(size_t)(p.iP * N + p.jP) * NN + x];
+}
 
 // ---------------------------------------------------------------------------------------------
 // N = 256: a plane (512 KB) does not fit an SM, so its rows and its columns are two passes: rows over d

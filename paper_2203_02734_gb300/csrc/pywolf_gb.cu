@@ -25,6 +25,7 @@
 #include "plane.cuh"
 #include "smu.cuh"
 #include "r128.cuh"
+#include "r64.cuh"
 #include "r96.cuh"
 
 namespace {
@@ -238,6 +239,30 @@ cudaError_t launch_b_r96(const pw::PassBArgs& b, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// N = 64: register-resident passes (r64.cuh), three CTAs per SM.
+template <class K>
+cudaError_t grid_r64(K kernel, int* grid) {
+  if (*grid) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw::r64::smem_bytes());
+  return e != cudaSuccess ? e : persistent_grid(kernel, pw::r64::NT, pw::r64::smem_bytes(), 64 * 64, grid);
+}
+
+cudaError_t launch_a_r64(const CUtensorMap& vmap, const pw::PassAArgs& a, cudaStream_t s) {
+  static int grid = 0;
+  const cudaError_t e = grid_r64(pw::r64::pass_a_r64, &grid);
+  if (e != cudaSuccess) return e;
+  pw::r64::pass_a_r64<<<grid, pw::r64::NT, pw::r64::smem_bytes(), s>>>(vmap, a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_b_r64(const pw::PassBArgs& b, cudaStream_t s) {
+  static int grid = 0;
+  const cudaError_t e = grid_r64(pw::r64::pass_b_r64, &grid);
+  if (e != cudaSuccess) return e;
+  pw::r64::pass_b_r64<<<grid, pw::r64::NT, pw::r64::smem_bytes(), s>>>(b);
+  return cudaGetLastError();
+}
+
 // Number of CTAs of the largest grid of `cs`-CTA clusters of `kernel` that can be co-resident.
 template <class K>
 cudaError_t cluster_capacity(K kernel, int cs, int threads, size_t smem, int* grid) {
@@ -339,6 +364,7 @@ cudaError_t launch_passes(bool herm, const CUtensorMap& vmap, const pw::PassAArg
   if constexpr (N == 256) e = x.mask ? launch_a_d256<true>(vmap, a, x, s) : launch_a_d256<false>(vmap, a, x, s);
   else if constexpr (N == 128) e = x.mask ? launch_a_r128<true>(vmap, a, x, s) : launch_a_r128<false>(vmap, a, x, s);
   else if constexpr (N == 96) e = x.mask ? launch_a_r96<true>(vmap, a, x, s) : launch_a_r96<false>(vmap, a, x, s);
+  else if constexpr (N == 64) e = launch_a_r64(vmap, a, s);
   else e = launch_a<N>(vmap, a, s);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
@@ -346,6 +372,7 @@ cudaError_t launch_passes(bool herm, const CUtensorMap& vmap, const pw::PassAArg
   else if (!herm) e = launch_b<N, pw::W_GENERAL>(b, s);
   else if constexpr (N == 128) e = launch_b_r128(b, s);
   else if constexpr (N == 96) e = launch_b_r96(b, s);
+  else if constexpr (N == 64) e = launch_b_r64(b, s);
   else e = launch_b<N, pw::W_HERM>(b, s);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
@@ -369,18 +396,19 @@ cudaError_t dispatch(int N, bool herm, const CUtensorMap& vmap, const pw::PassAA
 using pwi::PlaneArgs;
 
 template <int N>
-cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
+cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s, cudaEvent_t* ev) {
   namespace P = pw::plane;
   constexpr size_t N3 = (size_t)N * N * N;
   static int grid = 0;  // of the plane kernel
   cudaError_t e;
   constexpr auto kernel = [] {
-    if constexpr (N == 96) return P::plane96_kernel;
+    if constexpr (N == 64) return pw::r64::plane64_kernel;
+    else if constexpr (N == 96) return P::plane96_kernel;
     else if constexpr (N == 128) return P::plane128_kernel;
     else return P::plane_kernel<N>;
   }();
-  constexpr int nt = N == 96 ? pw::r96::NT : N == 128 ? pw::r128::NT : pw::Plan<N>::NT;
-  constexpr size_t smem = N == 96 ? P::plane96_smem() : N == 128 ? P::plane128_smem() : P::plane_smem<N>();
+  constexpr int nt = N == 64 ? pw::r64::NT : N == 96 ? pw::r96::NT : N == 128 ? pw::r128::NT : pw::Plan<N>::NT;
+  constexpr size_t smem = N == 64 ? pw::r64::smem_bytes() : N == 96 ? P::plane96_smem() : N == 128 ? P::plane128_smem() : P::plane_smem<N>();
   if (grid == 0) {
     if ((e = cudaFuncSetAttribute(P::table_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)P::tab_smem<N>())) != cudaSuccess ||
@@ -394,7 +422,14 @@ cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, cudaStrea
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
   const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, q.row, q.iP, q.jP};
-  kernel<<<grid, nt, smem, s>>>(wmap, a);
+  if constexpr (N == 128) {
+    kernel<<<grid, nt, smem, s>>>(a, err);
+    P::diag_row_kernel<<<N * N / 256, 256, 0, s>>>(a, N);
+  } else if constexpr (N == 64) {
+    kernel<<<grid, nt, smem, s>>>(a);
+  } else {
+    kernel<<<grid, nt, smem, s>>>(wmap, a);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
   return cudaSuccess;
@@ -438,7 +473,7 @@ cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, 
   switch (N) {
 #define PW_CASE(NN) \
   case NN:          \
-    return launch_planes<NN>(wmap, q, s, ev);
+    return launch_planes<NN>(wmap, q, err, s, ev);
     PW_CASE(2) PW_CASE(4) PW_CASE(6) PW_CASE(8) PW_CASE(12) PW_CASE(16) PW_CASE(24)
     PW_CASE(32) PW_CASE(48) PW_CASE(64) PW_CASE(96) PW_CASE(128)
 #undef PW_CASE
@@ -1005,10 +1040,10 @@ pw_status encode_vmap(CUtensorMap* map, void* work, int N) {
   return PW_OK;
 }
 
-// 5D map of W for the plane kernels: a plane (b', c') is the N rows W(a', b', c', .), left whole (N <= 96), or
-// at N = 128 as the eight rows a' = w + 16 i of one warp; at N = 256 the column pass's tiles, 64 floats
-// of every a.
+// 5D map of W for the plane kernels: a plane (b', c') is the N rows W(a', b', c', .), left whole (N <= 96); at
+// N = 256 the column pass's tiles, 64 floats of every a.  (N = 64 and 128 need none.)
 pw_status encode_wmap(CUtensorMap* map, void* W, int N) {
+  if (N == 64 || N == 128) return PW_OK;
   auto enc = encode_tiled();
   if (!enc) return fail(PW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
@@ -1021,10 +1056,10 @@ pw_status encode_wmap(CUtensorMap* map, void* W, int N) {
     if (r != CUDA_SUCCESS) return fail(PW_ECUDA, "cuTensorMapEncodeTiled (column tiles of W) failed (CUresult %d)", (int)r);
     return PW_OK;
   }
-  const cuuint64_t n = N, row = 2 * n * sizeof(float), lo = N == 128 ? 16 : n;
-  const cuuint64_t dims[5] = {2 * n, n, n, lo, n / lo};
-  const cuuint64_t strides[4] = {row, row * n, row * n * n, row * n * n * lo};
-  const cuuint32_t box[5] = {(cuuint32_t)(2 * N), 1, 1, (cuuint32_t)(N == 128 ? 1 : N), (cuuint32_t)(N == 128 ? 8 : 1)};
+  const cuuint64_t n = N, row = 2 * n * sizeof(float);
+  const cuuint64_t dims[5] = {2 * n, n, n, n, 1};
+  const cuuint64_t strides[4] = {row, row * n, row * n * n, row * n * n * n};
+  const cuuint32_t box[5] = {(cuuint32_t)(2 * N), 1, 1, (cuuint32_t)N, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 5, W, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(PW_ECUDA, "cuTensorMapEncodeTiled (planes of W) failed (CUresult %d)", (int)r);

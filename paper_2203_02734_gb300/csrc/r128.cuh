@@ -70,10 +70,15 @@ __device__ __forceinline__ void twiddle2d(float2 (&v)[RP][RQ], const float2* tw,
 // Contract: buf is free on entry (all threads passed a barrier after its last use).
 // PAIR: the thread's stage-3 butterflies are the column pair 2 (lane mod 16) + i of row
 // jp3 = warp + 16 (lane / 16) instead, read 16 bytes at a time: w3[i][rp][rq] then holds the
-// transform at (jp3 + 32 rp, 2 (lane mod 16) + i + 32 rq).  Signs: SIGN along p, SQ along q.
-template <int SIGN, bool ROWS = false, int SQ = SIGN, bool PAIR = false>
+// transform at (jp3 + 32 rp, 2 (lane mod 16) + i + 32 rq).  Signs: SIGN along p, SQ along q.  after_read()
+// runs once the thread has read its stage-3 inputs (buf may be refilled after a warp or block barrier,
+// as ROWS or not).
+struct NoHook {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <int SIGN, bool ROWS = false, int SQ = SIGN, bool PAIR = false, class Hook = NoHook>
 __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][4], float2* buf,
-                                         const float2* tw) {
+                                         const float2* tw, Hook after_read = Hook{}) {
   auto row = [](int p) { return ROWS ? vrow<N>(p) : p; };
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 #pragma unroll
@@ -106,6 +111,7 @@ __device__ __forceinline__ void stages_23(float2 (&v)[8][4], float2 (&w3)[2][4][
         w3[0][rp][rq] = make_float2(x.x, x.y);
         w3[1][rp][rq] = make_float2(x.z, x.w);
       }
+    after_read();
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       twiddle2d<4, 4, SIGN, SQ>(w3[i], tw, jp3, jq + i);
