@@ -5,9 +5,15 @@
 
 namespace {
 __global__ void __launch_bounds__(256) list_tables_kernel(const pw::smu::TabArgs<float2>* t) {
-  pw::smu::tables(t[blockIdx.x]);
+  const pw::smu::TabArgs<float2> a = t[blockIdx.x];
+  pw::smu::tables(a, threadIdx.x, 256);
+  __syncthreads();
+  pw::smu::table_K(a);
 }
-__global__ void __launch_bounds__(256) one_tables_kernel(pw::smu::TabArgs<double2> t) { pw::smu::tables(t); }
+// One evaluation per thread, in blocks of 64 over the SMs; K is left to k1.
+__global__ void __launch_bounds__(64) one_tables_kernel(pw::smu::TabArgs<double2> t) {
+  pw::smu::tables(t, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
+}
 }  // namespace
 
 namespace pwi {
@@ -30,7 +36,7 @@ cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<float2>* list, int n, 
 }
 
 cudaError_t launch_smu_one(const pw::smu::TabArgs<double2>& t, const pw::smu::Inst<double2>& q, cudaStream_t s) {
-  one_tables_kernel<<<1, 256, 0, s>>>(t);
+  one_tables_kernel<<<(5 * t.N + 63) / 64, 64, 0, s>>>(t);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   switch (q.N) {

@@ -42,7 +42,7 @@ struct Inst {
   const C* P1l;         // N: what rounding P1 left out
   const C* Eout;        // N
   const R* k;           // N: k(u)
-  const R* K;           // L: transform of k over |u| < N
+  R* K;                 // L: transform of k over |u| < N (FP64: written by k1)
   const float2* mask;   // N x N or nullptr
   int ap_ithr;          // aperture, as in batch.cuh
   C* scratch;           // 3 L N values
@@ -50,29 +50,47 @@ struct Inst {
   float2* mu;           // N x N or nullptr
 };
 
-template <int N> __host__ __device__ constexpr int lines() { return N % 16 == 0 ? (N >= 256 ? 8 : 16) : N % 8 == 0 ? 8 : N; }
-template <int N> __host__ __device__ constexpr int threads() { return N >= 64 ? 256 : 128; }
+// Lines per block.  FP32 batches fill the chip with instances, and 16 lines make whole sectors of the column
+// accesses.  FP64 calls are one instance: a line per block puts an SM's FP64 pipe behind each (N = 96: 16
+// lines a block left 6 to 12 blocks, 247 us a call; one line 74 us, with FP64's own radices below 55 us;
+// two lines 58 us).
+template <int N, class C> __host__ __device__ constexpr int lines() {
+  return sizeof(real_t<C>) == 8 ? 1 : N % 16 == 0 ? (N >= 256 ? 8 : 16) : N % 8 == 0 ? 8 : N;
+}
+template <int N, class C> __host__ __device__ constexpr int threads() {
+  return N >= 64 ? 256 : 128;
+}
 template <int N, class C> constexpr size_t smem_bytes() {
-  return (size_t)(2 * 2 * N * (lines<N>() + 1) + 3 * N) * sizeof(C);
+  return (size_t)(2 * 2 * N * (lines<N, C>() + 1) + 3 * N) * sizeof(C);
 }
 
 // In-place transform of the block's lines (length LEN, natural order), after a barrier and ending with one.
-template <int LEN, int SIGN, int LINES, int NT, int I = 0, class C>
+// NS: points already combined (I stages).  FP32 takes the radices of fft.cuh's plans, FP64 fours and then
+// threes and twos: those plans are made for FP32 registers, and at 2 FP64 operations a clock and SM a
+// radix-16 butterfly keeps its warp for 5 us while most warps of the block have none.
+template <int LEN, int SIGN, int LINES, int NT, int NS = 1, int I = 0, class C>
 __device__ __forceinline__ void fft_lines(C* x, const C* tw) {
-  if constexpr (I < Plan<LEN>::stages) {
-    constexpr int LP = LINES + 1;
+  if constexpr (NS < LEN) {
+    constexpr int LP = LINES + 1, REM = LEN / NS;
+    constexpr int RD = REM % 4 == 0 ? 4 : REM % 3 == 0 ? 3 : 2;
     auto ld = [x](int line, int pos) { return x[pos * LP + line]; };
     auto st = [x](int line, int pos, C v) { x[pos * LP + line] = v; };
-    line_stage<LEN, StageInfo<LEN, I>::R, StageInfo<LEN, I>::NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
-    __syncthreads();
-    fft_lines<LEN, SIGN, LINES, NT, I + 1>(x, tw);
+    if constexpr (sizeof(real_t<C>) == 8) {
+      line_stage<LEN, RD, NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
+      __syncthreads();
+      fft_lines<LEN, SIGN, LINES, NT, NS * RD>(x, tw);
+    } else {
+      line_stage<LEN, StageInfo<LEN, I>::R, NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
+      __syncthreads();
+      fft_lines<LEN, SIGN, LINES, NT, NS * StageInfo<LEN, I>::R, I + 1>(x, tw);
+    }
   }
 }
 
 // The tables of a block: tw (L) and twN (N = every other entry).
 template <int N, class C>
 __device__ __forceinline__ void load_tw(const Inst<C>& in, C* tw, C* twN) {
-  for (int i = threadIdx.x; i < 2 * N; i += threads<N>()) {
+  for (int i = threadIdx.x; i < 2 * N; i += threads<N, C>()) {
     const C v = in.tw[i];
     tw[i] = v;
     if (!(i & 1)) twN[i >> 1] = v;
@@ -128,15 +146,27 @@ __device__ __forceinline__ Inst<C> pick(const Inst<C>* list, const Inst<C>& one)
 }
 
 template <int N, class C>
-__global__ void __launch_bounds__(threads<N>()) k1(const Inst<C>* list, Inst<C> one, int chunk) {
+__global__ void __launch_bounds__(threads<N, C>()) k1(const Inst<C>* list, Inst<C> one, int chunk) {
   using R = real_t<C>;
-  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  constexpr int L = 2 * N, LINES = lines<N, C>(), LP = LINES + 1, NT = threads<N, C>();
   const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
   extern __shared__ __align__(16) unsigned char smem[];
   C *x = reinterpret_cast<C*>(smem), *tw = x + 2 * L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int b0 = blockIdx.x * LINES;
+  if constexpr (sizeof(R) == 8) {
+    if (b0 == N) {  // the last block: K
+      for (int e = threadIdx.x; e < L * LINES; e += NT) {
+        const int line = e % LINES, u = e / LINES;
+        x[u * LP + line] = make_c(line || u == N ? (R)0 : __ldg(in.k + (u < N ? u : L - u)), (R)0);
+      }
+      __syncthreads();
+      fft_lines<L, -1, LINES, NT>(x, tw);
+      for (int m = threadIdx.x; m < L; m += NT) in.K[m] = x[m * LP].x;
+      return;
+    }
+  }
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, a = e / LINES;
     x[a * LP + line] = a < N ? field<N, C>(in, a, b0 + line) : make_c((R)0, (R)0);
@@ -150,9 +180,9 @@ __global__ void __launch_bounds__(threads<N>()) k1(const Inst<C>* list, Inst<C> 
 }
 
 template <int N, class C>
-__global__ void __launch_bounds__(threads<N>()) k2(const Inst<C>* list, Inst<C> one, int chunk) {
+__global__ void __launch_bounds__(threads<N, C>()) k2(const Inst<C>* list, Inst<C> one, int chunk) {
   using R = real_t<C>;
-  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  constexpr int L = 2 * N, LINES = lines<N, C>(), LP = LINES + 1, NT = threads<N, C>();
   const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -203,9 +233,9 @@ __global__ void __launch_bounds__(threads<N>()) k2(const Inst<C>* list, Inst<C> 
 }
 
 template <int N, class C>
-__global__ void __launch_bounds__(threads<N>()) k3(const Inst<C>* list, Inst<C> one, int chunk) {
+__global__ void __launch_bounds__(threads<N, C>()) k3(const Inst<C>* list, Inst<C> one, int chunk) {
   using R = real_t<C>;
-  constexpr int L = 2 * N, LINES = lines<N>(), LP = LINES + 1, NT = threads<N>();
+  constexpr int L = 2 * N, LINES = lines<N, C>(), LP = LINES + 1, NT = threads<N, C>();
   const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk) return;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -248,9 +278,9 @@ __global__ void __launch_bounds__(threads<N>()) k3(const Inst<C>* list, Inst<C> 
 }
 
 template <int N, class C>
-__global__ void __launch_bounds__(threads<N>()) k4(const Inst<C>* list, Inst<C> one, int chunk) {
+__global__ void __launch_bounds__(threads<N, C>()) k4(const Inst<C>* list, Inst<C> one, int chunk) {
   using R = real_t<C>;
-  constexpr int LINES = lines<N>(), LP = LINES + 1, NT = threads<N>(), L = 2 * N;
+  constexpr int LINES = lines<N, C>(), LP = LINES + 1, NT = threads<N, C>(), L = 2 * N;
   const Inst<C> in = pick(list, one);
   if (in.N != N || in.chunk != chunk || !in.mu) return;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -285,19 +315,18 @@ struct TabArgs {
   real_t<C> *k, *K;
 };
 
-// The N = blockDim.x-strided work of each table; a block barrier separates k, tw from K.
 __device__ __forceinline__ void put(float2* h, float2* l, int i, double x, double y) {
   h[i] = make_float2((float)x, (float)y);
   if (l) l[i] = make_float2((float)(x - (double)(float)x), (float)(y - (double)(float)y));
 }
 __device__ __forceinline__ void put(double2* h, double2*, int i, double x, double y) { h[i] = make_double2(x, y); }
 
+// All tables but K; one FP64 evaluation per task: tasks 0..L-1 tw, then P1, Eout and k of each index.
 template <class C>
-__device__ __forceinline__ void tables(const TabArgs<C>& t) {
+__device__ __forceinline__ void tables(const TabArgs<C>& t, int q0, int step) {
   using R = real_t<C>;
   const int N = t.N, L = 2 * N, M = N / 2;
-  // one FP64 evaluation per thread and step: tasks 0..L-1 tw, then P1, Eout and k of each index
-  for (int q = threadIdx.x; q < L + 3 * N; q += blockDim.x) {
+  for (int q = q0; q < L + 3 * N; q += step) {
     const int kind = q < L ? -1 : (q - L) / N, i = q < L ? q : (q - L) - kind * N;
     const double n2 = (double)(i - M) * (double)(i - M);
     if (kind == 2) {
@@ -316,7 +345,13 @@ __device__ __forceinline__ void tables(const TabArgs<C>& t) {
       put(t.P1, t.P1l, i, cs * hh, sn * hh);
     }
   }
-  __syncthreads();
+}
+
+// K by one block, from its own k and tw.
+template <class C>
+__device__ __forceinline__ void table_K(const TabArgs<C>& t) {
+  using R = real_t<C>;
+  const int N = t.N, L = 2 * N;
   for (int m = threadIdx.x; m < L; m += blockDim.x) {
     R acc = 0;
     int j = 0;  // m u mod L
@@ -331,7 +366,7 @@ __device__ __forceinline__ void tables(const TabArgs<C>& t) {
 
 template <int N, class C>
 cudaError_t launch(const Inst<C>* list, const Inst<C>& one, int n, int chunk, bool any_mu, cudaStream_t s) {
-  constexpr int LINES = lines<N>(), NT = threads<N>();
+  constexpr int LINES = lines<N, C>(), NT = threads<N, C>();
   constexpr size_t sm = smem_bytes<N, C>();
   static bool ready = false;
   cudaError_t e = cudaSuccess;
@@ -343,7 +378,7 @@ cudaError_t launch(const Inst<C>* list, const Inst<C>& one, int n, int chunk, bo
       return e;
     ready = true;
   }
-  k1<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
+  k1<N, C><<<dim3(N / LINES + (sizeof(real_t<C>) == 8), n), NT, sm, s>>>(list, one, chunk);
   k2<N, C><<<dim3(2 * N / LINES, n), NT, sm, s>>>(list, one, chunk);
   k3<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
   if (any_mu) k4<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
