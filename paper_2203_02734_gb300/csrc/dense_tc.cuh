@@ -19,8 +19,10 @@
 //
 // Up to Np = 128 a CTA computes all 2 Np output reals of its tile; above, two CTAs compute half of them
 // each (both split the same inputs, the second from L2): an accumulator of at most 256 tensor-memory
-// columns and 113 KB of shared memory let two CTAs share an SM, so that one's first loads (4500 cycles
-// at N = 200) and epilogue (9400) overlap the other's MMAs.  K runs in chunks of 16 complex inputs (32 reals,
+// columns and 113 KB of shared memory let two CTAs share an SM, so that one's set-up and first
+// loads (4100 cycles at N = 200) and epilogue (7000 by columns, 11000 by rows) overlap the other's chunks
+// (2050 cycles each, 624 of them MMA).  One CTA of 512 converter threads with all 2 Np outputs splits every
+// input once, but nothing covers its ends: 22.7 ms a propagation at N = 200 against 19.2.  K runs in chunks of 16 complex inputs (32 reals,
 // two MMA K-steps), 6 MMAs (M 128, N = NOUT, K 16) each.  Q is split once per propagation by
 // qsplit_kernel into a global buffer laid out half by half and chunk by chunk in the canonical K-major
 // layout (no swizzle): per chunk, split s and K-step ks, core matrices [kb < 2][row group < NOUT / 8] of 8
@@ -538,7 +540,16 @@ __global__ void __launch_bounds__(NT, 2) axis_tc_kernel(Args p, const unsigned c
           const int k = kp + k0 + lane;
           if (lane < cnt && k < N) {
             const int rows = row0 < ncols ? min(32u, ncols - row0) : 0;
-            for (int r = 0; r < rows; ++r) p.out[(size_t)(row0 + r) * N + k] = turn[r * 33 + lane];
+            float2* o = p.out + (size_t)row0 * N + k;
+            int r = 0;
+            for (; r + 8 <= rows; r += 8, o += 8 * N) {  // eight loads, then eight stores: one by one 14800 cycles a CTA
+              float2 v[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) v[i] = turn[(r + i) * 33 + lane];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) o[i * N] = v[i];
+            }
+            for (; r < rows; ++r, o += N) *o = turn[r * 33 + lane];
           }
           __syncwarp();
         }
