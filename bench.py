@@ -3,8 +3,8 @@
 
 Metric: 4D CSD points propagated per second (N^4 / time of one full propagation step) and the
 HBM-roofline fraction of the dominant kernel.  One step = reset to the source plane, the source
-(GSM x mask), Fresnel propagation (pass A: source build + input propagators + point-2 2D DFT;
-pass B: point-1 2D DFT + output propagators + S), then S and mu(P1, .) of the output plane.
+(GSM x mask), Fresnel propagation (source tables of N^3 values, one 2D DFT per output plane, output
+propagators, S), then S and mu(P1, .) of the output plane.
 
 Default workload (the headline line): N = 256 (4.3 G points, complex64 CSDA of 34 GB), GSM x a
 seeded unit-modulus phase screen (3 px correlation), dxi = 20 um, lambda = 633 nm, sigma_S =
@@ -213,8 +213,8 @@ def run_reference(args):
 # ----------------------------------------------------------------------------- GPU helpers
 # Per grid size: the committed ncu summary of its pass kernels and the device-code headers they
 # are built from (a recorded traffic figure is used only while those headers are unchanged).
-PROFILED = {128: ("pass_kernels_n128.md", ("cluster.cuh", "fft.cuh", "propagate.cuh", "r128.cuh")),
-            256: ("pass_kernels_n256.md", ("fft.cuh", "propagate.cuh", "r128.cuh", "t256.cuh", "tc16.cuh"))}
+PROFILED = {128: ("pass_kernels_n128.md", ("cluster.cuh", "fft.cuh", "plane.cuh", "propagate.cuh", "r128.cuh")),
+            256: ("pass_kernels_n256.md", ("cluster.cuh", "fft.cuh", "plane.cuh", "propagate.cuh"))}
 
 
 def kernel_source_sha(N=128):
@@ -249,32 +249,33 @@ def recorded_traffic(kernel, N):
 
 
 def roofline_dense(N, pts, avg_a, avg_b, clocks, tc):
-    """Padded workloads: four dense axis contractions, N complex multiply-adds (8 flop) per output
-    point each; the second pass's events span two contractions.
-    CUDA cores (tc False): FP32 FMA work against SMs x 128 FP32 lanes x 2 flop x the maximum SM clock.
-    Tensor cores (tc True): the BF16 MMA flops one launch issues, ceil(N^3 / 128) tiles x
-    Np / 16 chunks x 24 MMAs of 2 x 128 x Np x 16 flop (Np = N rounded up to 16; six split products),
-    against the measured BF16 peak."""
+    """Padded workloads: dense axis contractions, N complex multiply-adds (8 flop) per output point each.
+    CUDA cores (tc False): four of them, the second pass's events span two; FP32 FMA work against
+    SMs x 128 FP32 lanes x 2 flop x the maximum SM clock.
+    Tensor cores (tc True): a GSM source takes two N^4 contractions, the second pass's events span the
+    last; the FP16 MMA flops one launch issues, ceil(N^3 / 128) tiles x Np / 16 chunks x 6 x
+    2 x 128 x 2 Np x 16 flop (Np = N rounded up to 16; three split products in two K-steps), against
+    the measured BF16 peak (the FP16 rate is the same)."""
     import torch
-    avg = avg_b / 2
+    avg = avg_b if tc else avg_b / 2
     fp32_flops = 8.0 * N * pts
     if tc:
         Np = (N + 15) // 16 * 16
         tiles = (N ** 3 + 127) // 128
-        flops = tiles * (Np // 16) * 24 * 2.0 * 128 * Np * 16
+        flops = tiles * (Np // 16) * 6 * 2.0 * 128 * 2 * Np * 16
         try:
             peak, src = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["bf16_tflops"]), "measured"
         except Exception:
             peak, src = 1900.0, "fallback"
         achieved = flops / (avg / 1e3) / 1e12
         return {"bound": "tensor", "kernel": "dense_tc::axis_tc_kernel", "achieved": achieved, "peak": peak,
-                "unit": "TFLOP/s", "frac": achieved / peak, "peak_source": src + " (bf16, burst)", "traffic": None,
+                "unit": "TFLOP/s", "frac": achieved / peak, "peak_source": src + " (bf16 GEMM, burst; fp16 runs at the same rate)", "traffic": None,
                 "algorithmic_flops_per_launch": flops,
                 "fp32_equivalent_tflops": fp32_flops / (avg / 1e3) / 1e12,
-                # the method's own work (8 N flop per output point) against the split-BF16x3 ceiling:
-                # each FP32 product costs six BF16 products, so at most peak / 6 of FP32 work
-                "method_work": {"achieved": fp32_flops / (avg / 1e3) / 1e12, "ceiling": peak / 6.0,
-                                "frac": fp32_flops / (avg / 1e3) / 1e12 / (peak / 6.0), "unit": "TFLOP/s"},
+                # the method's own work (8 N flop per output point) against the ceiling of FP16
+                # operands in two parts: each FP32 product costs three, so at most peak / 3 of FP32 work
+                "method_work": {"achieved": fp32_flops / (avg / 1e3) / 1e12, "ceiling": peak / 3.0,
+                                "frac": fp32_flops / (avg / 1e3) / 1e12 / (peak / 3.0), "unit": "TFLOP/s"},
                 "pass_ms": {"pass_a": avg_a, "pass_b": avg_b}}
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     mhz = (clocks or {}).get("sm_max_mhz") or 2070.0
@@ -406,10 +407,13 @@ def measure(cfg, args, rank, world, dist):
         for _ in range(args.steps):
             step()
 
-    # tables, pass A, pass B, S kernel, mu kernel (N = 256: three passes); padded: tables, dense
-    # tables, source, four axis contractions (+ two matrix splits on the tensor cores), S, mu
-    launches_per_step = ((11 if args.dft != "fp32" and N <= 256 else 9) if cfg.get("Nz")
-                         else (6 if N == 256 and args.dft != "tc_bf16x3" else 5))
+    # tables, plane tables, planes, S kernel, mu kernel; N = 128: + diagonal and row; N = 256: rows and
+    # columns in place of planes; cluster engine: tables, pass A, pass B, S, mu.  Padded: FP32 tables,
+    # source, four contractions, S, mu; tensor cores tables, two matrix splits, GSM tables and their
+    # scale, two table and two N^4 contractions, S, mu
+    tc = args.dft != "fp32" and N <= 256
+    launches_per_step = ((12 if tc else 9) if cfg.get("Nz") else
+                         5 if N < 128 or args.dft == "tc_bf16x3" else 6)
     max_blocks = 400
     pw.pw_csd_enable_timing(h, max(args.steps * max_blocks, args.warmup, 1))
     for _ in range(args.warmup):
@@ -425,7 +429,7 @@ def measure(cfg, args, rank, world, dist):
     if dist:
         dist.barrier()
     ms = statistics.median(blocks)
-    ms_a, ms_b, ms_c, nrec = pw.pw_csd_pass_times3(h)
+    ms_a, ms_b, _, nrec = pw.pw_csd_pass_times3(h)
     clocks = clock.stop(t0, t1) if clock else None
     ms = max_over_ranks(ms, dist, "cuda")
 
@@ -477,13 +481,16 @@ def measure(cfg, args, rank, world, dist):
     pts = N ** 4
     value = job_throughput(world, pts, args.steps, ms / 1e3)
     peak, peak_kind = measured_peak_hbm()
-    avg_a, avg_b, avg_c = (x / max(nrec, 1) for x in (ms_a, ms_b, ms_c))
-    if avg_c > 0:  # N = 256: three streaming passes, 8 + 16 + 16 bytes per point
-        passes = {"pass1": (avg_a, 8 * pts), "pass2": (avg_b, 16 * pts), "pass3": (avg_c, 16 * pts)}
-        engine_bytes = 40
-    else:  # two passes, 8 + 16 bytes per point
+    avg_a, avg_b = (x / max(nrec, 1) for x in (ms_a, ms_b))
+    if N == 256 and args.dft == "tc_bf16x3":  # cluster engine: V written, then read and W written
         passes = {"pass_a": (avg_a, 8 * pts), "pass_b": (avg_b, 16 * pts)}
         engine_bytes = 24
+    elif N == 256:  # rows of the planes written into W, columns in place; O(N^3) tables with the rows
+        passes = {"rows256": (avg_a, 8 * pts), "cols256": (avg_b, 16 * pts)}
+        engine_bytes = 24
+    else:  # two tables of N^3 values, then every output plane written once
+        passes = {"plane_tables": (avg_a, 16 * N ** 3), "planes": (avg_b, 8 * pts)}
+        engine_bytes = 8
     kern = max(passes, key=lambda k: passes[k][0])
     avg, bytes_launch = passes[kern]
     achieved = bytes_launch / (avg / 1e3) / 1e9
@@ -505,9 +512,8 @@ def measure(cfg, args, rank, world, dist):
                      "pass_ms": {k: v[0] for k, v in passes.items()},
                      "pass_hbm_frac": {k: v[1] / (v[0] / 1e3) / 1e9 / peak for k, v in passes.items()},
                      "engine_bytes_per_point": engine_bytes,
-                     "step_hbm_frac": (24 * pts / (ms / args.steps / 1e3) / 1e9) / peak,
-                     "step_hbm_frac_note": "24 bytes per point, the two-pass minimum of the method, over "
-                                           "the measured peak"},
+                     "step_hbm_frac": (engine_bytes * pts / (ms / args.steps / 1e3) / 1e9) / peak,
+                     "step_hbm_frac_note": "the engine's bytes per point over the measured peak"},
         "e2e": {"value": job_throughput(world, pts, args.steps, te), "unit": UNIT,
                 "h2d_bytes_per_step": mask_h.numel() * 8, "d2h_bytes_per_step": S_h.numel() * 4 + mu_h.numel() * 8,
                 "result_matches_device_path": same},
@@ -563,8 +569,8 @@ def batch_instances():
 
 
 def run_batch(args):
-    """Batched polychromatic run: all instances in one persistent launch, captured once in a CUDA
-    graph and replayed; S and mu of every instance.  Reported next to the plain path (the
+    """Batched polychromatic run: S and mu of every instance, four kernels per grid size, captured once
+    in a CUDA graph and replayed.  Reported next to the plain path (the
     single-instance calls, one instance after the other) on the same GPU."""
     import torch
     import paper_2203_02734_gb300 as pw
@@ -605,6 +611,9 @@ def run_batch(args):
     pw.pw_batch_check(b)
     ms = e0.elapsed_time(e1) / args.steps
     pts = sum(sp["N"] ** 4 for sp in specs)
+    # 14 N^2 complex values between the four kernels of an instance (mostly in L2), S and mu
+    smu_bytes = sum(128 * sp["N"] ** 2 for sp in specs)
+    launches = 1 + 4 * len(CFG["Ns"])  # tables, then k1-k4 of every grid size (one round of scratch)
     # plain path: the same instances through the single-instance calls, one after the other
     maxN = max(sp["N"] for sp in specs)
     W = torch.empty(maxN ** 4, dtype=torch.complex64, device="cuda")
@@ -646,13 +655,13 @@ def run_batch(args):
                        "Ns": list(CFG["Ns"]), "zs": list(CFG["zs"]), "n_freq": CFG["n_freq"],
                        "outputs": "S and mu per instance", "pool": pool, "chunk": chunk,
                        "launch": "autotuned mode: %s, replayed from a CUDA graph" % mode},
-            "roofline": {"bound": "hbm", "kernel": "whole batch (V written by pass A, read by the S/mu pass)",
-                         "achieved": 16.0 * pts / (ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
-                         "frac": 16.0 * pts / (ms * 1e-3) / 1e9 / peak, "peak_source": peak_src, "traffic": None,
-                         "algorithmic_bytes_per_point": 16},
+            "roofline": {"bound": "latency", "kernel": "smu::k1-k4: S and mu from (2N)^2 transforms, no N^4 array",
+                         "achieved": smu_bytes / (ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
+                         "frac": smu_bytes / (ms * 1e-3) / 1e9 / peak, "peak_source": peak_src, "traffic": None,
+                         "algorithmic_bytes": smu_bytes},
             "plain_path": {"value": pts / (ms_plain / 1e3), "unit": UNIT, "ms_per_step": ms_plain,
                            "what": "the same instances through the single-instance calls, one after another"},
-            "gpu_launches": (4 if mode.startswith("persistent") else 2 + 2 * len(specs)) * args.steps,
+            "gpu_launches": launches * args.steps,
             "clocks": clocks}
     print(json.dumps(line), flush=True)
 

@@ -79,8 +79,9 @@ size_t pw_csda_bytes(int N);
  *   lambda_m  wavelength in metres (finite, > 0); omega = 2 pi c / lambda     (Eq. q_factor)
  *   dev_W     device buffer of >= pw_csda_bytes(N) bytes: holds an uploaded source CSDA
  *             (pw_source_array may point here) and receives every propagated CSDA
- *   dev_work  device buffer of >= pw_csda_bytes(N) bytes, scratch for the half-transformed
- *             CSDA between the two passes; must not overlap dev_W
+ *   dev_work  device buffer of >= pw_csda_bytes(N) bytes, scratch of every call on the handle
+ *             (tables of a GSM source's planes, the half-transformed CSDA of an uploaded array);
+ *             must not overlap dev_W
  *   stream    cudaStream_t to enqueue on (NULL = legacy default stream)
  * Returns PW_EINVAL / PW_ESIZE / PW_EUNSUPPORTED for bad arguments, PW_ECUDA if the small
  * per-handle tables cannot be allocated.  *out is NULL on failure. */
@@ -131,7 +132,7 @@ pw_status pw_source_mask(pw_csd* h, const pw_c32* dev_mask);
  * previous run or built by the user).  dev_W0 (N^4 complex64, device) may be dev_W itself.
  * hermitian != 0 declares W0(xi2, xi1) = conj W0(xi1, xi2) (true of every CSD, Sec. 3.3), which
  * lets the second pass store its output rows contiguously; hermitian == 0 selects the
- * general (strided-store) second pass for N <= 128.  The three-pass engine at N = 256 and the
+ * general (strided-store) second pass for N <= 128.  The three passes at N = 256 and the
  * dense path never use Hermiticity and need no declaration.  Read during the next propagation. */
 pw_status pw_source_array(pw_csd* h, const pw_c32* dev_W0, int hermitian);
 
@@ -164,11 +165,10 @@ pw_status pw_gsm_gradient(pw_csd* h, double sigma_S_m, double sigma_mu_m, double
  * the call builds that source in-kernel, propagates it back (P^H, Fresnel over z from the output
  * sampling dx onto the source grid d = lambda z / (N dx)) and forms the requested gradients:
  *   dev_grad3 / dev_grad_amask: dL/d(sigma_S, sigma_mu, A) and dL/da of the amplitude-masked GSM
- *     source W0 = A a(xi1) a(xi2) G (Sec. 5.4) that the forward propagation started from, reduced
- *     in the epilogue of the adjoint's second pass (W0bar is never stored; at N = 256 it goes
- *     through dev_W and one gradient kernel);
+ *     source W0 = A a(xi1) a(xi2) G (Sec. 5.4) that the forward propagation started from, summed
+ *     from W0bar's closed form (W0bar is never stored);
  *   grad_W0: dL/dRe W0 + i dL/dIm W0 for W0 taken as a general complex N^4 array, written into
- *     dev_W (a second, non-Hermitian adjoint propagation when both kinds are asked with a mu term).
+ *     dev_W.
  * The handle's current sampling must be the forward's output sampling dx (true right after the
  * forward propagation, or after pw_csd_reset(h, dx)); the current plane's contents are not used.
  * dev_work is used as scratch; dev_W is overwritten (the gradient with grad_W0, else unspecified).
@@ -240,9 +240,9 @@ pw_status pw_csd_set_padding(pw_csd* h, int Nz);
 pw_status pw_csd_get_padding(const pw_csd* h, int* Nz);
 
 /* Arithmetic of the DFT work that has a tensor-core form:
- *   - the first radix-16 stage of the first pass at N = 256 (FFT path, GSM sources; all other
- *     stages and FFT grid sizes always run FP32 codelets on the CUDA cores), and
- *   - the four dense axis contractions of the padded / no-FFT-plan path (N <= 256).
+ *   - the first radix-16 stage at N = 256 (FFT path, GSM sources, a two-pass engine of its own; all
+ *     other stages and FFT grid sizes always run FP32 codelets on the CUDA cores), and
+ *   - the dense axis contractions of the padded / no-FFT-plan path (N <= 256).
  *   PW_DFT_AUTO (default): the faster of the two per path, as measured on GB300: FP32 codelets on
  *     the FFT paths, the tensor cores for the dense contractions (N <= 256; FP32 above).
  *   PW_DFT_FP32: FP32 on the CUDA cores everywhere (codelets with FP64-derived twiddles, dense FP32
@@ -272,15 +272,16 @@ pw_status pw_csd_get_dft_mode(const pw_csd* h, int* mode);
 
 /* Per-pass timing (measurement aid, no counterpart in the paper).  pw_csd_enable_timing
  * creates CUDA events for up to max_props propagations (0 disables and frees them); each
- * later propagation records events on the handle's stream around its first pass (source +
- * point-2 DFT) and second pass (point-1 DFT + output chirp + S).  pw_csd_pass_times waits
+ * later propagation records events on the handle's stream around its first pass (an array's
+ * point-2 DFT; a GSM source's tables, at N = 256 with the row pass; half of the dense contractions)
+ * and its second (the rest).  pw_csd_pass_times waits
  * for the recorded events, returns the summed milliseconds of each pass and how many
  * propagations were recorded, and restarts the count.  Propagations beyond max_props are
  * not recorded. */
 pw_status pw_csd_enable_timing(pw_csd* h, int max_props);
 pw_status pw_csd_pass_times(pw_csd* h, double* ms_first, double* ms_second, int* count);
-/* The same with the engine's passes apart: at N = 256 (three streaming passes) ms_first is the
- * first pass, ms_second and ms_third the second and third; elsewhere ms_third is 0. */
+/* The same with the engine's passes apart: for an uploaded array at N = 256 (three streaming passes)
+ * ms_first is the first pass, ms_second and ms_third the second and third; elsewhere ms_third is 0. */
 pw_status pw_csd_pass_times3(pw_csd* h, double* ms_first, double* ms_second, double* ms_third, int* count);
 
 /* ---- Batched runs: many instances in one persistent launch --------------------------------
@@ -319,7 +320,7 @@ typedef struct pw_batch pw_batch; /* opaque */
 enum { PW_BATCH_PERSISTENT = 0, PW_BATCH_SEQUENCED = 1 };
 
 /* Bytes of device workspace pw_batch_create needs for these instances and this pool depth
- * (tables, work list, counters and `pool` half-transformed buffers of the largest N). */
+ * (tables, work list, counters and `pool` scratch buffers of N^4 values of the largest N). */
 size_t pw_batch_workspace_bytes(const pw_instance* inst, int n, int pool);
 
 /* Validate the instances (N in {16, 32, 64, 96, 128}, finite positive lengths, P1 inside the

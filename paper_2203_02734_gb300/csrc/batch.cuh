@@ -13,7 +13,8 @@
 // wait is bounded (about a second of clock64 cycles); when it gives up it sets the error flag,
 // the item is skipped, and the host reads PW_ETIMEOUT.
 //
-// Per instance the passes are those of the single-instance path: pass A builds the GSM x masks x
+// (Instances of GSM sources that keep only S and mu run on smu.cuh instead, unless a stall is injected.)
+// Per instance the passes are those of an uploaded array's path: pass A builds the GSM x masks x
 // input propagators slice, runs the direct 2D DFT and stores it into the instance's V slot in the
 // tiled corner-turn layout; pass B gathers a column, runs the inverse-sign 2D DFT, applies the
 // scale and output propagators and keeps S (diagonal) and the mu numerator W(P1, x) (the element

@@ -16,9 +16,6 @@ __device__ __forceinline__ unsigned cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// The same in two halves: memory written before the arrival is visible after the wait.
-__device__ __forceinline__ void cluster_sync_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Address of `local` (a shared-memory location of this CTA) in the shared memory of CTA `rank`.
 __device__ __forceinline__ unsigned map_rank(const void* local, unsigned rank) {
   unsigned r;

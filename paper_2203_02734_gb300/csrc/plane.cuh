@@ -230,7 +230,8 @@ constexpr size_t plane96_smem() { return (size_t)96 * r96::P * sizeof(float2) + 
 //   - six of its 8 rows of H stay in shared memory while b' is the same (96 KB; two are read through L2).
 // Stage 1 reads and exchange 1 writes only the warp's own rows, so three block barriers a plane are
 // enough.  Results go straight from registers to W, 16 bytes a lane; S and the P1 row are read back from
-// W by diag_row_kernel (tests for them in the store loop were 5 % of the plane's instructions).
+// W by diag_row_kernel (tests for them in the store loop were 5 % of the plane's instructions).  0.844 ms:
+// bound by issue, 62 % active at 77 instructions a point; the write of W alone would take 0.32 ms.
 constexpr int HROWS128 = 6;
 constexpr size_t plane128_smem() {
   return (size_t)(128 * 128 + 16 * HROWS128 * 128 + 2 * 128) * sizeof(float2) + 16 * sizeof(uint64_t);

@@ -1,5 +1,6 @@
 // pywolf_gb.cu -- C ABI of include/pywolf_gb.h: handle state, argument checks, FP64 table
-// set-up and the launch sequence of one propagation (tables -> pass A -> pass B).
+// set-up and the launch sequence of one propagation (by source: planes, passes over an array, closed
+// form, dense contractions).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -86,7 +87,7 @@ struct pw_csd {
   float2* tw;
   float2* Eout;
   float2* Ein;    // per-axis input factors
-  float* S;       // S of the last propagated plane (pass-B epilogue)
+  float* S;       // S of the last propagated plane (the last pass's epilogue)
   int* err;       // device flag: a bounded wait in a kernel gave up
   unsigned* maxes;  // dense path: bits of the largest input component of each contraction (8 slots)
   // adjoint scratch (O(N^2)): the adjoint source (diagonal, P1 row), partial sums, the
@@ -913,8 +914,8 @@ pw_status propagate(pw_csd* h, double z, bool farfield) {
   pw_status st = build_tables(h, z, farfield);
   if (st != PW_OK) return st;
   // GSM sources: plane by plane, one 2D transform over (a, d) per (b', c') from tables of N^3 values
-  // (N = 128: 0.97 against 1.67 ms on the two general passes; N = 256: 16.5 against 31.3 ms; N = 32: 2 us
-  // less).  The exception is the tensor-core comparison mode at N = 256.
+  // (N = 128: 0.87 against 1.67 ms on the two general passes; N = 96: 0.31 against 0.68; N = 256: 16.3
+  // against 31.3 ms; N = 32: 2 us less).  The exception is the tensor-core comparison mode at N = 256.
   const bool tc256 = h->N == 256 && h->dft_mode == PW_DFT_TC_BF16X3;
   if (h->kind == SRC_GSM && !tc256) return propagate_planes(h, z);
   if (h->kind == SRC_DIAGONAL) return propagate_diagonal(h, z);
@@ -989,7 +990,7 @@ pw_status gsm_s_mu(pw_csd* h, double z, bool farfield, int iP, int jP, float* S,
 
 pw_status s_mu(pw_csd* h, int iP, int jP, float* S, pw_c32* mu) {
   if (h->kind == SRC_NONE) return fail(PW_ESTATE, "no source set for the current plane");
-  // A propagated plane without masks needs no tables: S comes from the pass-B epilogue.
+  // A propagated plane without masks needs no tables: S comes from the last pass's epilogue.
   if (h->kind != SRC_PROPAGATED || has_masks(h)) {
     pw_status st = build_tables(h, 0.0, false, true);
     if (st != PW_OK) return st;
