@@ -377,7 +377,7 @@ pw_status pw_batch_destroy(pw_batch* b);
  * latency-critical loops that cannot afford the implicit device synchronisation of
  * cudaMalloc / cudaFree.  It computes what pw_csd_create + pw_source_gsm + pw_source_aperture
  * + pw_source_lens + pw_source_mask + pw_propagate_fresnel + pw_spectral_density compute on a
- * new handle, without a handle: the half-transformed CSDA and the small tables live in one
+ * new handle, without a handle: the scratch (N > 16: the half-transformed CSDA) and the small tables live in one
  * fixed device array inside the library (8 MiB + 12.5 KiB, held by every device that loads the
  * library until the process exits), so N is limited to 2 <= N <= 32 (even, pw_supported_n);
  * larger N returns PW_EINVAL with a message naming the limit.

@@ -17,6 +17,7 @@
 
 #include "../../include/pywolf_gb.h"
 #include "propagate.cuh"
+#include "small.cuh"
 
 namespace pwi {
 void set_last_error(const char* msg);  // pywolf_gb.cu: message returned by pw_last_error()
@@ -127,6 +128,19 @@ pw_status run(const CUtensorMap& vmap, const pw::TableArgs& t, const pw::PassAAr
   return PW_OK;
 }
 
+// N <= 16: the tables, then every output plane from them (15.4 us in three launches at N = 16, 11.5 in two).
+template <int N>
+pw_status run_small(const pw::TableArgs& t, const pw::small::Args& a, cudaStream_t s) {
+  pw::tables_kernel<<<pw::tables_grid(t), pw::TABLE_NT, 0, s>>>(t);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = pw::small::launch<N>(a, s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(PW_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
+  }
+  return PW_OK;
+}
+
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {
@@ -202,6 +216,21 @@ extern "C" pw_status pw_propagate_gsm_fresnel_noalloc(int N, double dxi_m, doubl
   t.tw = tw;
   t.Eout = Eout;
 
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  const double lz = lam * z_m;
+  const float scale = (float)((d * d / lz) * (d * d / lz));
+  const pw::small::Args q{F, G, tw, Eout, reinterpret_cast<float2*>(dev_W_out), dev_S_out, (float)amplitude, scale,
+                          nullptr, 0, 0};
+  switch (N) {
+    case 2: return run_small<2>(t, q, s);
+    case 4: return run_small<4>(t, q, s);
+    case 6: return run_small<6>(t, q, s);
+    case 8: return run_small<8>(t, q, s);
+    case 12: return run_small<12>(t, q, s);
+    case 16: return run_small<16>(t, q, s);
+    default: break;
+  }
+
   // TMA map of V in the tiled layout (host-side descriptor, no allocation).
   auto enc = encode_fn();
   if (!enc) return fail(PW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
@@ -229,17 +258,8 @@ extern "C" pw_status pw_propagate_gsm_fresnel_noalloc(int N, double dxi_m, doubl
   b.Eout = Eout;
   b.W = reinterpret_cast<float2*>(dev_W_out);
   b.S = dev_S_out;
-  const double lz = lam * z_m;
-  b.scale = (float)((d * d / lz) * (d * d / lz));
-
-  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  b.scale = scale;
   switch (N) {
-    case 2: return run<2>(vmap, t, a, b, s);
-    case 4: return run<4>(vmap, t, a, b, s);
-    case 6: return run<6>(vmap, t, a, b, s);
-    case 8: return run<8>(vmap, t, a, b, s);
-    case 12: return run<12>(vmap, t, a, b, s);
-    case 16: return run<16>(vmap, t, a, b, s);
     case 24: return run<24>(vmap, t, a, b, s);
     case 32: return run<32>(vmap, t, a, b, s);
     default: break;

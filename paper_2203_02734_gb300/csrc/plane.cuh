@@ -12,7 +12,8 @@
 // W(a', b', c', .) are final, so the whole propagation writes its 8 bytes a point once and reads the
 // tables from L2.  (The general path moves 24 bytes a point, 40 at N = 256.)
 //   table_kernel: N^2 columns of length N of each table, into the work buffer.
-//   plane kernels (N <= 128): one (b', c') per CTA iteration.
+//   plane kernels (24 <= N <= 128; r64.cuh at N = 64, small.cuh with its own tables up to N = 16): one
+//   (b', c') per CTA iteration.
 //   N = 256: the rows (a, d) and the columns of a plane in two passes, 24 bytes a point.
 #pragma once
 #include <cuda.h>
@@ -118,7 +119,7 @@ __device__ __forceinline__ void plane_s_row(const Args& p, const float2* buf, At
 }
 
 // ---------------------------------------------------------------------------------------------
-// N <= 64: the generic shared-memory 2D transform of propagate.cuh, one plane per block iteration;
+// N <= 48 (from N = 24; small.cuh below): the generic shared-memory 2D transform of propagate.cuh, one plane per block iteration;
 // the natural-order plane leaves by one TMA tensor store (box {2 N floats, 1, 1, N} of W).
 template <int N> constexpr size_t plane_smem() {
   return (size_t)N * pitch<N>() * sizeof(float2) + 2 * N * sizeof(float2);

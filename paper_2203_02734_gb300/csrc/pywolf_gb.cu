@@ -24,6 +24,7 @@
 #include "delta.cuh"
 #include "grad.cuh"
 #include "plane.cuh"
+#include "small.cuh"
 #include "smu.cuh"
 #include "r128.cuh"
 #include "r64.cuh"
@@ -396,6 +397,16 @@ cudaError_t dispatch(int N, bool herm, const CUtensorMap& vmap, const pw::PassAA
 
 using pwi::PlaneArgs;
 
+// N <= 16: tables and planes in one kernel (small.cuh), timed as the planes.
+template <int N>
+cudaError_t launch_small(const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
+  cudaError_t e;
+  if (ev && ((e = cudaEventRecord(ev[0], s)) != cudaSuccess || (e = cudaEventRecord(ev[1], s)) != cudaSuccess)) return e;
+  const pw::small::Args a{q.F, q.G, q.tw, q.Eout, q.W, q.S, q.A, q.scale, q.row, q.iP, q.jP};
+  if ((e = pw::small::launch<N>(a, s)) != cudaSuccess) return e;
+  return ev ? cudaEventRecord(ev[2], s) : cudaSuccess;
+}
+
 template <int N>
 cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, int* err, cudaStream_t s, cudaEvent_t* ev) {
   namespace P = pw::plane;
@@ -475,8 +486,12 @@ cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, 
 #define PW_CASE(NN) \
   case NN:          \
     return launch_planes<NN>(wmap, q, err, s, ev);
-    PW_CASE(2) PW_CASE(4) PW_CASE(6) PW_CASE(8) PW_CASE(12) PW_CASE(16) PW_CASE(24)
-    PW_CASE(32) PW_CASE(48) PW_CASE(64) PW_CASE(96) PW_CASE(128)
+    PW_CASE(24) PW_CASE(32) PW_CASE(48) PW_CASE(64) PW_CASE(96) PW_CASE(128)
+#undef PW_CASE
+#define PW_CASE(NN) \
+  case NN:          \
+    return launch_small<NN>(q, s, ev);
+    PW_CASE(2) PW_CASE(4) PW_CASE(6) PW_CASE(8) PW_CASE(12) PW_CASE(16)
 #undef PW_CASE
     case 256:
       return launch_planes256(wmap, q, err, s, ev);
@@ -1044,7 +1059,7 @@ pw_status encode_vmap(CUtensorMap* map, void* work, int N) {
 // 5D map of W for the plane kernels: a plane (b', c') is the N rows W(a', b', c', .), left whole (N <= 96); at
 // N = 256 the column pass's tiles, 64 floats of every a.  (N = 64 and 128 need none.)
 pw_status encode_wmap(CUtensorMap* map, void* W, int N) {
-  if (N == 64 || N == 128) return PW_OK;
+  if (N <= pw::small::MAX_N || N == 64 || N == 128) return PW_OK;
   auto enc = encode_tiled();
   if (!enc) return fail(PW_ECUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};

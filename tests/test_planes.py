@@ -72,3 +72,30 @@ def test_planes_against_the_general_passes(N, farfield, aperture, lens, mask):
     assert np.array_equal(out[0][1].real, M[d[:, None], d[None, :], d[:, None], d[None, :]].real)
     ok = out[1][1].real >= 1e-2 * out[1][1].real.max()  # mu: 1 / sqrt(S) amplifies W's error tenfold at most
     assert np.abs(out[0][2] - out[1][2])[ok].max() < 2e-5
+
+
+# The allocation-free call shares the kernel of N <= 16 (small.cuh); direct sums of N terms per axis stay
+# within the bound above (2^-24 sqrt(4 N) x 3 <= 1.5e-6 at N = 16 each).
+@pytest.mark.gpu
+@pytest.mark.parametrize("N", [2, 4, 6, 8, 12, 16, 24])
+@pytest.mark.parametrize("aperture,mask", [(False, True), (True, False)])
+def test_noalloc_against_the_general_passes(N, aperture, mask):
+    import torch
+    import paper_2203_02734_gb300 as pw
+    gsm, z = (5 * D, 1.5 * D, 0.8), 0.3
+    m = torch.from_numpy(WL.to_c64(WL.phase_screen(N, seed=4))).cuda() if mask else None
+    ap = 0.4 * N * D if aperture else 0.0
+    W, S = torch.zeros((N,) * 4, dtype=torch.complex64, device="cuda"), torch.zeros((N, N), device="cuda")
+    pw.pw_propagate_gsm_fresnel_noalloc(N, D, LAM, z, *gsm, ap, 0.0, m.data_ptr() if mask else None, W.data_ptr(),
+                                        W.numel() * 8, S.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    c = pw.CSD(N, D, LAM)
+    c.source_array(torch.from_numpy(WL.to_c64(oracle_source(N, D, LAM, gsm=gsm))).cuda())
+    if aperture:
+        c.source_aperture(ap)
+    if mask:
+        c.source_mask(m)
+    c.propagate_fresnel(z)
+    c128 = lambda t: t.cpu().numpy().astype(np.complex128)  # noqa: E731
+    assert rel(c128(W), c128(c.W)) < 3e-6
+    assert rel(c128(S), c128(c.spectral_density())) < 3e-6
+    c.close()
