@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(r128::NT, 1) plane128_kernel(Args p, int* err)
   }
   __syncthreads();  // tw, eo
   uint32_t parity = 0;
-  int ok = 1;  // a wait that gave up sets *err; the warp then waits no more and its results are invalid
-  for (int bc = p0; bc < p1; ++bc, parity ^= 1u) {
+  int ok = 1;  // (lane 0) a wait that gave up sets *err; the warp then waits and copies no more, its results are
+               // invalid, and parity stays that of the phase in flight for the last wait below
+  for (int bc = p0; bc < p1; ++bc, parity ^= (uint32_t)ok) {
     const int bq = bc / N, cq = bc - bq * N;
     const float2* __restrict__ H = p.H + (size_t)bq * N * N;
     float2 hx[8 - HR][4];
