@@ -30,14 +30,16 @@ class _Model:
 
     def outputs(self):
         """New S and mu tensors (they belong to the caller's graph)."""
-        return self.new(torch.float32), self.new(torch.complex64)
+        NN = (self.N, self.N)
+        return self.new((NN, torch.float32), (NN, torch.complex64))
 
-    def new(self, dtype, *shape):
-        """A device tensor that the handle's stream may still be writing when it is freed."""
-        t = torch.empty(shape or (self.N, self.N), dtype=dtype, device=self.dev)
+    def new(self, *specs):
+        """Device tensors (shape, dtype) that the handle's stream may still be writing when they are freed."""
+        out = [torch.empty(shape, dtype=dtype, device=self.dev) for shape, dtype in specs]
         if torch.cuda.current_stream(self.dev) != self.csd.stream:
-            t.record_stream(self.csd.stream)
-        return t
+            for t in out:
+                t.record_stream(self.csd.stream)
+        return out
 
     def propagate_and_read(self):
         h = self.csd.h
@@ -130,7 +132,7 @@ class _GSMFn(torch.autograd.Function):
         if gS is None and gmu is None:
             return None, None, None, None, None
         sS, sM, A = ctx.params
-        g, gmask = m.new(torch.float64, 3), m.new(torch.float32)
+        g, gmask = m.new((3, torch.float64), ((m.N, m.N), torch.float32))
         keep = m.adjoint(gS, gmu, S, mu, sigma_S_m=sS, sigma_mu_m=sM, amplitude=A, dev_amask=am.data_ptr(),
                          dev_grad3=g.data_ptr(), dev_grad_amask=gmask.data_ptr())
         del keep

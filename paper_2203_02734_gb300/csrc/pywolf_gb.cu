@@ -75,6 +75,7 @@ struct pw_csd {
   double sigma_S, sigma_mu, A;
   const pw_c32* W0;
   const float* diag;  // diagonal source values (SRC_DIAGONAL)
+  int grad_rows[2];   // blocks of the adjoint's gradient kernel without and with a mu term (0: not queried yet)
   int hermitian;
   // masks of the current plane
   double aperture;  // <= 0: none
@@ -1528,7 +1529,7 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
   g.gtab = h->gtab;
   g.qtab = h->qtab;
   g.g3 = a->dev_grad3 ? a->dev_grad3 : h->g3tmp;
-  pw::gsm_gradient_tables<<<(NN + 255) / 256, 256, 0, st>>>(g);
+  if (params || farfield) pw::gsm_gradient_tables<<<(NN + 255) / 256, 256, 0, st>>>(g);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return done(cuda_fail(e, "adjoint set-up launch"));
 
@@ -1561,7 +1562,9 @@ pw_status adjoint(pw_csd* h, double z, bool farfield, const pw_adjoint* a) {
     const int nc = N % 4 == 0 ? 4 : 2;  // columns a block takes together
     const size_t sh = N * sizeof(float2);
     auto grad = [&](auto k) -> cudaError_t {  // one wave of resident blocks
-      const cudaError_t r = persistent_grid(k, nt, sh, NN / nc, &g.rows);
+      int& rows_of_k = h->grad_rows[has_mu];
+      const cudaError_t r = rows_of_k ? cudaSuccess : persistent_grid(k, nt, sh, NN / nc, &rows_of_k);
+      g.rows = rows_of_k;
       if (r == cudaSuccess) k<<<g.rows, nt, sh, st>>>(ga);
       return r;
     };
