@@ -298,8 +298,8 @@ pw_status pw_csd_pass_times3(pw_csd* h, double* ms_first, double* ms_second, dou
  *     work (bounded waits, see pw_batch_check);
  *   PW_BATCH_SEQUENCED: one after the other on the single-instance kernels (each fills the GPU).
  * The default is SEQUENCED when every instance has N >= 64, else PERSISTENT.  In both modes the
- * intermediate arrays share a pool of `pool` buffers of the largest N (instance i uses slot
- * i mod pool).  pw_batch_run enqueues only device work (no allocation, no synchronisation), so
+ * intermediate arrays share a pool of `pool` buffers of the largest N (the instances with dev_W use
+ * them in turn).  pw_batch_run enqueues only device work (no allocation, no synchronisation), so
  * the caller may capture it in a CUDA graph and replay it. */
 typedef struct pw_instance {
   int N;                 /* grid size: 16, 32, 64, 96 or 128 */

@@ -25,7 +25,7 @@ def _nvcc():
 
 
 def _deps():
-    return SRCS + glob.glob(os.path.join(HERE, "csrc", "*.cuh")) + [os.path.join(ROOT, "include", "pywolf_gb.h")]
+    return SRCS + glob.glob(os.path.join(HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(HERE, "csrc", "*.h")) + [os.path.join(ROOT, "include", "pywolf_gb.h")]
 
 
 def up_to_date():

@@ -129,31 +129,18 @@ bool direct(const pw_batch* b, int i) {
   return b->inst[i].W == nullptr && !(b->mode == PW_BATCH_PERSISTENT && stalled(b));
 }
 
+// The instances in the launch.
+std::vector<int> members(const pw_batch* b) {
+  std::vector<int> m;
+  for (int i = 0; i < b->n; ++i)
+    if (!direct(b, i)) m.push_back(i);
+  return m;
+}
+
 pw_status build_items(pw_batch* b) {
-  std::vector<pw::batch::Item> items;
-  // One pass = J = ceil(S / chunk) items.  N = 128 (register-resident engine, whose pass B
-  // gathers 8 bytes from every 32-byte run of V): strided items, item j takes slices j, j + J,
-  // j + 2 J, ..., so that neighbouring CTAs gather the columns of one run together.  Other sizes:
-  // contiguous ranges of chunk slices (measured slightly faster there).
-  auto add = [&](int i, int pass) {
-    if (direct(b, i) || (pass == 0 && b->stalled[i])) return;
-    const int S = b->inst[i].slices;
-    const int J = (S + b->chunk - 1) / b->chunk;
-    for (int j = 0; j < J; ++j) {
-      if (b->inst[i].N == 128) items.push_back({i, pass, j, (S - j + J - 1) / J, J});
-      else items.push_back({i, pass, j * b->chunk, j + 1 < J ? b->chunk : S - j * b->chunk, 1});
-    }
-  };
-  // Lookahead of L instances: A(0) .. A(L-1), then B(i), A(i + L) for i = 0, 1, ...  B(i) waits
-  // for A(i), listed L phases earlier; A(i + L) reuses the slot of instance i + L - pool and waits
-  // for its pass B, listed pool - L phases earlier.  L = pool - 2 (at least 1) leaves two phases
-  // between every wait and the items it waits on, and every awaited item precedes its waiter.
-  const int L = b->pool >= 3 ? b->pool - 2 : 1;
-  for (int i = 0; i < L && i < b->n; ++i) add(i, 0);
-  for (int i = 0; i < b->n; ++i) {
-    add(i, 1);
-    if (i + L < b->n) add(i + L, 0);
-  }
+  std::vector<int> Ns;
+  for (const auto& d : b->inst) Ns.push_back(d.N);
+  const std::vector<pw::batch::Item> items = pw::batch::items(members(b), Ns, b->stalled, b->chunk, b->pool);
   if ((int)items.size() > b->L.max_items) return fail(PW_EINVAL, "item list exceeds the workspace");
   b->nitems = (int)items.size();
   cudaError_t e = cudaMemcpyAsync(b->base + b->L.items, items.data(), items.size() * sizeof(pw::batch::Item),
@@ -163,8 +150,8 @@ pw_status build_items(pw_batch* b) {
   return PW_OK;
 }
 
-// Uploads what depends on which instances run on smu.cuh: the FP64 table arguments, the mu outputs of
-// the others, the smu.cuh descriptors, and the item list.  The descriptors sit at the end of the
+// Uploads what depends on which instances run on smu.cuh: the FP64 table arguments, the slots and mu outputs
+// of the others, the smu.cuh descriptors, and the item list.  The descriptors sit at the end of the
 // item area, in the room of the items that these instances do not have (2560 bytes each at least);
 // their scratch is the V pool, in as many rounds as it takes.
 pw_status upload(pw_batch* b) {
@@ -202,8 +189,17 @@ pw_status upload(pw_batch* b) {
   char* tail = b->base + (b->L.items + sizeof(pw::batch::Item) * (size_t)b->L.max_items) / 256 * 256 - lb - tb;
   b->dev_smu = reinterpret_cast<pw::smu::Inst<float2>*>(tail);
   b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs<float2>*>(tail + lb);
-  cudaError_t e = cudaMemcpyAsync(b->base + b->L.targs, targs.data(), sizeof(pw::TableArgs) * n, cudaMemcpyHostToDevice,
+  const std::vector<pw::batch::Place> at = pw::batch::places(members(b), n, b->pool);
+  for (int i = 0; i < n; ++i) {
+    pw::batch::Inst& d = b->inst[i];
+    d.prev = at[i].prev;
+    d.V = reinterpret_cast<float2*>(b->base + b->L.pool + b->L.slot_bytes * at[i].slot);
+    d.vmap = d.N == 128 ? b->base + b->L.tmaps + sizeof(CUtensorMap) * at[i].slot : nullptr;
+  }
+  cudaError_t e = cudaMemcpyAsync(b->base + b->L.inst, b->inst.data(), sizeof(pw::batch::Inst) * n, cudaMemcpyHostToDevice,
                                   b->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(b->base + b->L.targs, targs.data(), sizeof(pw::TableArgs) * n, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->base + b->L.mu, mus.data(), sizeof(float2*) * n, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess && b->ndirect)
@@ -312,8 +308,6 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     d.Eout = Eo;
     d.Ein = Ei;
     d.mask = reinterpret_cast<const float2*>(q.dev_mask);
-    d.V = reinterpret_cast<float2*>(b->base + L.pool + L.slot_bytes * (i % pool));
-    d.vmap = N == 128 ? b->base + L.tmaps + sizeof(CUtensorMap) * (i % pool) : nullptr;
     d.W = reinterpret_cast<float2*>(q.dev_W);
     d.S = q.dev_S;
     mus[i] = reinterpret_cast<float2*>(q.dev_mu);
@@ -384,9 +378,8 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
       }
     }
   }
-  cudaError_t e = cudaMemcpyAsync(b->base + L.inst, b->inst.data(), sizeof(pw::batch::Inst) * n,
-                                  cudaMemcpyHostToDevice, b->stream);
-  if (e == cudaSuccess && any128)
+  cudaError_t e = cudaSuccess;
+  if (any128)
     e = cudaMemcpyAsync(b->base + L.tmaps, maps.data(), sizeof(CUtensorMap) * pool, cudaMemcpyHostToDevice,
                         b->stream);
   if (e == cudaSuccess)  // counters and the error flag start at zero (the workspace may hold old data)
@@ -427,8 +420,7 @@ pw_status pw_batch_run(pw_batch* b) {
   int maxNN = 0;
   for (const auto& d : b->inst) maxNN = d.slices > maxNN ? d.slices : maxNN;
   dim3 tg((maxNN + 255) / 256, b->n);
-  pw::batch::batch_tables_kernel<<<tg, 256, 0, b->stream>>>(reinterpret_cast<const pw::TableArgs*>(b->base + b->L.targs),
-                                                          b->mode == PW_BATCH_PERSISTENT ? cnt + b->n : nullptr);
+  pw::batch::batch_tables_kernel<<<tg, 256, 0, b->stream>>>(reinterpret_cast<const pw::TableArgs*>(b->base + b->L.targs));
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "batch tables launch");
   // mu of the instances that are not on smu.cuh (the others' entries are null)
   auto mu = [&]() -> pw_status {
@@ -465,7 +457,6 @@ pw_status pw_batch_run(pw_batch* b) {
   g.inst = reinterpret_cast<const pw::batch::Inst*>(b->base + b->L.inst);
   g.items = reinterpret_cast<const pw::batch::Item*>(b->base + b->L.items);
   g.nitems = b->nitems;
-  g.pool = b->pool;
   g.next = cnt + 2 * b->n;
   g.doneA = cnt;
   g.doneB = cnt + b->n;

@@ -6,8 +6,8 @@
 // are strided (item j takes slices j, j + J, ...), so the CTAs that claim consecutive items work
 // on neighbouring slices at the same time: in pass B the g columns that share each 32-byte run of
 // V are gathered together, while the run is in L2.  A pass-B item of instance i first waits until
-// all pass-A slices of i are done; a pass-A item of instance i whose half-transformed buffer slot
-// is shared with instance i - P (P = pool depth) first waits until pass B of i - P is done.
+// all pass-A slices of i are done; a pass-A item of instance i first waits until pass B of the instance that
+// used its half-transformed buffer slot before it is done (batch_plan.h).
 // Because items are claimed in list order and every awaited item precedes its waiter in the
 // list, a waiting CTA always waits on items already claimed by running CTAs: no deadlock.  Each
 // wait is bounded (about a second of clock64 cycles); when it gives up it sets the error flag,
@@ -22,6 +22,7 @@
 // asks for it.  N = 128 runs on the register-resident engine (r128.cuh); the other sizes on the
 // generic shared-memory Stockham engine.
 #pragma once
+#include "batch_plan.h"
 #include "propagate.cuh"
 #include "r128.cuh"
 
@@ -34,6 +35,7 @@ struct Inst {
   int N;
   int iP, jP;
   int slices;  // N * N
+  int prev;    // instance of the launch that used this one's slot before it, or -1
   float A;
   float scale;
   const float2* F;  // N x N input factors (propagators, lens, aperture, mask, checkerboard)
@@ -50,17 +52,10 @@ struct Inst {
   int ap_ithr;         // aperture: n_i^2 + n_j^2 <= ap_ithr (integer floor of the FP64 bound), < 0 = none
 };
 
-struct Item {
-  int inst;
-  int pass;  // 0 = A, 1 = B
-  int first, count, stride;
-};
-
 struct Args {
   const Inst* inst;
   const Item* items;
   int nitems;
-  int pool;
   int* next;    // item counter
   int* doneA;   // per instance: pass-A slices done
   int* doneB;   // per instance: pass-B slices done
@@ -379,8 +374,7 @@ __global__ void __launch_bounds__(NT, 1) batch_kernel(Args g) {
     if (threadIdx.x == 0) {
       bool ok = true;
       if (it.pass == 1) ok = wait_ge(g.doneA + it.inst, in.slices, g.wait_cycles);
-      else if (it.inst >= g.pool)
-        ok = wait_ge(g.doneB + it.inst - g.pool, g.inst[it.inst - g.pool].slices, g.wait_cycles);
+      else if (in.prev >= 0) ok = wait_ge(g.doneB + in.prev, g.inst[in.prev].slices, g.wait_cycles);
       if (!ok) atomicOr(g.err, 1);
       s_ok = ok;
     }
@@ -409,14 +403,10 @@ __global__ void __launch_bounds__(NT, 1) batch_kernel(Args g) {
 }
 
 // The FP64 tables of every instance (blockIdx.y = instance), as tables_kernel does for one.
-// An instance with N = 0 is not in the launch (smu.cuh): its passes count as done for the instances
-// that take its slot (doneB: nullptr outside the persistent mode).
-__global__ void batch_tables_kernel(const TableArgs* targs, int* doneB) {
+// An instance with N = 0 is not in the launch (smu.cuh).
+__global__ void batch_tables_kernel(const TableArgs* targs) {
   const TableArgs t = targs[blockIdx.y];
-  if (t.N == 0) {
-    if (doneB && blockIdx.x == 0 && threadIdx.x == 0) doneB[blockIdx.y] = 1 << 30;
-    return;
-  }
+  if (t.N == 0) return;
   const int N = t.N, M = N / 2, NN = N * N;
   for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < NN; idx += gridDim.x * blockDim.x) {
     const int i = idx / N, j = idx - i * N;
