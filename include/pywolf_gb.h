@@ -324,7 +324,7 @@ enum { PW_BATCH_PERSISTENT = 0, PW_BATCH_SEQUENCED = 1 };
 size_t pw_batch_workspace_bytes(const pw_instance* inst, int n, int pool);
 
 /* Validate the instances (N in {16, 32, 64, 96, 128}, finite positive lengths, P1 inside the
- * grid, dev_S given), lay out the caller-owned workspace (>= pw_batch_workspace_bytes) and upload
+ * grid, dev_S given, dev_W and the workspace 16-byte aligned, dev_mu and dev_mask 8, dev_S 4), lay out the caller-owned workspace (>= pw_batch_workspace_bytes) and upload
  * the descriptors and the work list (synchronises `stream`).  The output pointers are kept. */
 pw_status pw_batch_create(pw_batch** out, const pw_instance* inst, int n, int pool, void* dev_workspace,
                           size_t workspace_bytes, void* stream);

@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <cstdint>
 #include <cstdio>
 #include <vector>
 
@@ -36,6 +37,8 @@ pw_status cuda_fail(cudaError_t e, const char* what) {
 bool finite_pos(double v) { return std::isfinite(v) && v > 0.0; }
 
 bool batch_n(int N) { return N == 16 || N == 32 || N == 64 || N == 96 || N == 128; }
+
+bool aligned(const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -235,6 +238,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
   if (!in || n <= 0) return fail(PW_EINVAL, "need at least one instance");
   if (pool <= 0) return fail(PW_EINVAL, "pool depth must be >= 1");
   if (!dev_ws) return fail(PW_EINVAL, "workspace is null");
+  if (!aligned(dev_ws, 16)) return fail(PW_EINVAL, "the workspace must be 16-byte aligned");
   for (int i = 0; i < n; ++i) {
     const pw_instance& q = in[i];
     if (!batch_n(q.N)) return fail(PW_EUNSUPPORTED, "instance %d: N = %d (batched runs take N in {16, 32, 64, 96, 128})", i, q.N);
@@ -245,6 +249,8 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
       return fail(PW_EINVAL, "instance %d: amplitude, aperture and focal length must be finite", i);
     if (q.iP < 0 || q.jP < 0 || q.iP >= q.N || q.jP >= q.N) return fail(PW_EINVAL, "instance %d: P1 outside the grid", i);
     if (!q.dev_S) return fail(PW_EINVAL, "instance %d: dev_S is required", i);
+    if (!aligned(q.dev_W, 16) || !aligned(q.dev_S, 4) || !aligned(q.dev_mu, 8) || !aligned(q.dev_mask, 8))
+      return fail(PW_EINVAL, "instance %d: misaligned device pointer (dev_W 16 bytes, dev_mu and dev_mask 8, dev_S 4)", i);
   }
   const Layout L = layout(in, n, pool);
   if (ws_bytes < L.total) return fail(PW_ESIZE, "workspace needs %zu bytes (got %zu)", L.total, ws_bytes);

@@ -108,3 +108,15 @@ def test_no_device_reports_cuda_error(lib):
     with pytest.raises(lib.PwError, match="PW_ECUDA"):
         lib.pw_csd_create(32, 20e-6, 633e-9, FAKE_W, nb, FAKE_WORK, nb)
     assert "cudaMalloc" in lib.pw_last_error()
+
+
+@pytest.mark.parametrize("N", [16, 32, 64, 96, 128])
+@pytest.mark.parametrize("field,step", [("dev_W", 8), ("dev_S", 2), ("dev_mu", 4), ("dev_mask", 4), ("workspace", 8)])
+def test_batch_rejects_misaligned_pointers(lib, N, field, step):
+    q = lib.pw_instance()
+    q.N, q.dxi_m, q.lambda_m, q.z_m, q.sigma_S_m, q.sigma_mu_m, q.amplitude = N, 20e-6, 633e-9, 0.5, 1e-4, 3e-5, 1.0
+    for k, name in enumerate(("dev_W", "dev_S", "dev_mu", "dev_mask")):
+        setattr(q, name, FAKE_W + (k << 40) + (step if name == field else 0))
+    nb = lib.pw_batch_workspace_bytes([q], 2)
+    with pytest.raises(lib.PwError, match="PW_EINVAL.*aligned"):
+        lib.pw_batch_create([q], 2, FAKE_WORK + (step if field == "workspace" else 0), nb)
