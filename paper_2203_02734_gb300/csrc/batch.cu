@@ -100,8 +100,8 @@ struct pw_batch {
   int mode;  // PW_BATCH_PERSISTENT or PW_BATCH_SEQUENCED
   std::vector<CUtensorMap> wmaps;  // per instance with W: its planes (plane.cuh)
   std::vector<pw::TableArgs> targs;   // FP64 tables, uploaded with N = 0 for the instances on smu.cuh
-  std::vector<pw::smu::Inst<float2>> smu;     // the instances on smu.cuh, by pw_instance index where direct
-  std::vector<pw::smu::TabArgs<float2>> smu_t;
+  std::vector<pw::smu::Inst<pwi::Wide>> smu;     // the instances on smu.cuh, by pw_instance index where direct
+  std::vector<pw::smu::TabArgs<pwi::Wide>> smu_t;
   std::vector<float2*> mus;           // dev_mu of every instance
   struct Round {                      // one launch round of the instances on smu.cuh
     int chunk;
@@ -110,8 +110,8 @@ struct pw_batch {
   };
   std::vector<Round> rounds;
   int ndirect;                        // instances on smu.cuh
-  const pw::smu::Inst<float2>* dev_smu;
-  const pw::smu::TabArgs<float2>* dev_smu_t;
+  const pw::smu::Inst<pwi::Wide>* dev_smu;
+  const pw::smu::TabArgs<pwi::Wide>* dev_smu_t;
   char* base;
   Layout L;
   cudaStream_t stream;
@@ -162,8 +162,8 @@ pw_status upload(pw_batch* b) {
   const size_t pool_bytes = b->L.slot_bytes * b->pool;
   std::vector<pw::TableArgs> targs(b->targs);
   std::vector<float2*> mus(b->mus);
-  std::vector<pw::smu::Inst<float2>> list;
-  std::vector<pw::smu::TabArgs<float2>> tabs;
+  std::vector<pw::smu::Inst<pwi::Wide>> list;
+  std::vector<pw::smu::TabArgs<pwi::Wide>> tabs;
   b->rounds.clear();
   size_t used = 0;
   int chunk = 0;
@@ -171,8 +171,8 @@ pw_status upload(pw_batch* b) {
     if (!direct(b, i)) continue;
     targs[i].N = 0;
     mus[i] = nullptr;
-    pw::smu::Inst<float2> q = b->smu[i];
-    const size_t need = align256((size_t)6 * q.N * q.N * sizeof(float2));
+    pw::smu::Inst<pwi::Wide> q = b->smu[i];
+    const size_t need = align256((size_t)6 * q.N * q.N * sizeof(pwi::Wide));
     if (used + need > pool_bytes) {
       ++chunk;
       used = 0;
@@ -182,16 +182,16 @@ pw_status upload(pw_batch* b) {
     r.mu = r.mu || q.mu;
     if (std::find(r.Ns.begin(), r.Ns.end(), q.N) == r.Ns.end()) r.Ns.push_back(q.N);
     q.chunk = chunk;
-    q.scratch = reinterpret_cast<float2*>(b->base + b->L.pool + used);
+    q.scratch = reinterpret_cast<pwi::Wide*>(b->base + b->L.pool + used);
     used += need;
     list.push_back(q);
     tabs.push_back(b->smu_t[i]);
   }
   b->ndirect = (int)list.size();
-  const size_t lb = align256(list.size() * sizeof(pw::smu::Inst<float2>)), tb = align256(tabs.size() * sizeof(pw::smu::TabArgs<float2>));
+  const size_t lb = align256(list.size() * sizeof(pw::smu::Inst<pwi::Wide>)), tb = align256(tabs.size() * sizeof(pw::smu::TabArgs<pwi::Wide>));
   char* tail = b->base + (b->L.items + sizeof(pw::batch::Item) * (size_t)b->L.max_items) / 256 * 256 - lb - tb;
-  b->dev_smu = reinterpret_cast<pw::smu::Inst<float2>*>(tail);
-  b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs<float2>*>(tail + lb);
+  b->dev_smu = reinterpret_cast<pw::smu::Inst<pwi::Wide>*>(tail);
+  b->dev_smu_t = reinterpret_cast<pw::smu::TabArgs<pwi::Wide>*>(tail + lb);
   const std::vector<pw::batch::Place> at = pw::batch::places(members(b), n, b->pool);
   for (int i = 0; i < n; ++i) {
     pw::batch::Inst& d = b->inst[i];
@@ -206,9 +206,9 @@ pw_status upload(pw_batch* b) {
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->base + b->L.mu, mus.data(), sizeof(float2*) * n, cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess && b->ndirect)
-    e = cudaMemcpyAsync(tail, list.data(), list.size() * sizeof(pw::smu::Inst<float2>), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(tail, list.data(), list.size() * sizeof(pw::smu::Inst<pwi::Wide>), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess && b->ndirect)
-    e = cudaMemcpyAsync(tail + lb, tabs.data(), tabs.size() * sizeof(pw::smu::TabArgs<float2>), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(tail + lb, tabs.data(), tabs.size() * sizeof(pw::smu::TabArgs<pwi::Wide>), cudaMemcpyHostToDevice, b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (e != cudaSuccess) return cuda_fail(e, "uploading the batch descriptors");
   return build_items(b);
@@ -343,30 +343,27 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     t.tw = tw;
     t.Eout = Eo;
     t.Ein = Ei;
-    // smu.cuh: its tables take the place of F (6.5 N of the N^2 values)
-    pw::smu::TabArgs<float2>& ta = b->smu_t[i];
+    // smu.cuh: its tables take the place of F (88 N of the 8 N^2 bytes)
+    pw::smu::TabArgs<pwi::Wide>& ta = b->smu_t[i];
     ta.N = N;
     ta.Kin = t.Kin;
     ta.Kout = t.Kout;
     ta.gs = t.gs;
     ta.gm = t.gm;
-    ta.tw = F;
+    ta.tw = reinterpret_cast<pwi::Wide*>(F);
     ta.P1 = ta.tw + 2 * N;
-    ta.P1l = ta.P1 + N;
-    ta.Eout = ta.P1l + N;
-    ta.k = reinterpret_cast<float*>(ta.Eout + N);
-    ta.K = ta.k + N;
-    pw::smu::Inst<float2>& si = b->smu[i];
+    ta.Eout = ta.P1 + N;
+    ta.k = reinterpret_cast<pw::real_t<pwi::Wide>*>(ta.Eout + N);
+    pw::smu::Inst<pwi::Wide>& si = b->smu[i];
     si.N = N;
     si.iP = q.iP;
     si.jP = q.jP;
-    si.factor = (double)d.scale * q.amplitude / (4.0 * (double)NN);
+    si.factor = (q.dxi_m * q.dxi_m / lz) * (q.dxi_m * q.dxi_m / lz) * q.amplitude / (4.0 * (double)NN);
     si.tw = ta.tw;
     si.P1 = ta.P1;
-    si.P1l = ta.P1l;
     si.Eout = ta.Eout;
     si.k = ta.k;
-    si.K = ta.K;
+    si.K = ta.k + N;
     si.mask = d.mask;
     si.ap_ithr = d.ap_ithr;
     si.S = q.dev_S;

@@ -13,7 +13,8 @@
 
 namespace pw {
 
-// Complex values are float2, or double2 where a small transform is wanted to more digits (smu.cuh).
+// Complex values are float2, or double2 and float pairs (ff.cuh) where a small transform is wanted to more digits
+// (smu.cuh).
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float2 make_c(float x, float y) { return make_float2(x, y); }
@@ -253,9 +254,7 @@ PW_PLAN(48, 192, 16, 3)
 PW_PLAN(64, 256, 8, 8)
 PW_PLAN(96, 384, 8, 4, 3)
 PW_PLAN(128, 512, 16, 8)
-PW_PLAN(192, 256, 8, 8, 3)   // 192, 256, 512: single lines only (plane.cuh, smu.cuh)
-PW_PLAN(256, 256, 16, 16)
-PW_PLAN(512, 256, 8, 8, 8)
+PW_PLAN(256, 256, 16, 16)   // single lines only (plane.cuh)
 #undef PW_PLAN
 
 template <int N, int I> struct StageInfo {

@@ -6,6 +6,7 @@
 #include "../../include/pywolf_gb.h"
 
 namespace pw {
+struct ff2;
 namespace smu {
 template <class C> struct Inst;
 template <class C> struct TabArgs;
@@ -13,6 +14,8 @@ template <class C> struct TabArgs;
 }  // namespace pw
 
 namespace pwi {
+
+using Wide = pw::ff2;  // arithmetic of the batch's S and mu (smu.cuh)
 
 // Sets the thread's message returned by pw_last_error().
 void set_last_error(const char* msg);
@@ -39,9 +42,9 @@ cudaError_t dispatch_planes(int N, const CUtensorMap& wmap, const PlaneArgs& q, 
                             cudaEvent_t* ev);
 
 // S and mu without the CSDA (smu.cuh): the tables of n instances, then those of grid size N and launch round
-// `chunk` among them (device lists, FP32); or one instance (FP64).
-cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<float2>* list, int n, cudaStream_t s);
-cudaError_t launch_smu_list(int N, const pw::smu::Inst<float2>* list, int n, int chunk, bool any_mu, cudaStream_t s);
+// `chunk` among them (device lists, float pairs); or one instance (FP64).
+cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<Wide>* list, int n, cudaStream_t s);
+cudaError_t launch_smu_list(int N, const pw::smu::Inst<Wide>* list, int n, int chunk, bool any_mu, cudaStream_t s);
 cudaError_t launch_smu_one(const pw::smu::TabArgs<double2>& t, const pw::smu::Inst<double2>& q, cudaStream_t s);
 
 }  // namespace pwi

@@ -982,7 +982,6 @@ pw_status gsm_s_mu(pw_csd* h, double z, bool farfield, int iP, int jP, float* S,
   t.P1 = t.tw + 2 * N;
   t.Eout = t.P1 + N;
   t.k = reinterpret_cast<double*>(t.Eout + N);
-  t.K = t.k + N;
   pw::smu::Inst<double2> q{};
   q.N = N;
   q.iP = iP;
@@ -990,10 +989,9 @@ pw_status gsm_s_mu(pw_csd* h, double z, bool farfield, int iP, int jP, float* S,
   q.factor = (d * d / lz) * (d * d / lz) * h->A / (4.0 * N * N);
   q.tw = t.tw;
   q.P1 = t.P1;
-  q.P1l = t.P1;  // not used in FP64
   q.Eout = t.Eout;
   q.k = t.k;
-  q.K = t.K;
+  q.K = t.k + N;
   q.mask = reinterpret_cast<const float2*>(h->mask);
   q.ap_ithr = aperture_threshold(h);
   q.scratch = w;

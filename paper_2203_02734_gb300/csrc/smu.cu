@@ -1,16 +1,14 @@
-// smu.cu -- instantiations of smu.cuh: batches in FP32, single calls in FP64.
+// smu.cu -- instantiations of smu.cuh: batches on float pairs, single calls in FP64.
 #include "smu.cuh"
 
 #include "internal.h"
 
 namespace {
-__global__ void __launch_bounds__(256) list_tables_kernel(const pw::smu::TabArgs<float2>* t) {
-  const pw::smu::TabArgs<float2> a = t[blockIdx.x];
+__global__ void __launch_bounds__(256) list_tables_kernel(const pw::smu::TabArgs<pwi::Wide>* t) {
+  const pw::smu::TabArgs<pwi::Wide> a = t[blockIdx.x];
   pw::smu::tables(a, threadIdx.x, 256);
-  __syncthreads();
-  pw::smu::table_K(a);
 }
-// One evaluation per thread, in blocks of 64 over the SMs; K is left to k1.
+// One evaluation per thread, in blocks of 64 over the SMs.
 __global__ void __launch_bounds__(64) one_tables_kernel(pw::smu::TabArgs<double2> t) {
   pw::smu::tables(t, blockIdx.x * 64 + threadIdx.x, gridDim.x * 64);
 }
@@ -18,11 +16,11 @@ __global__ void __launch_bounds__(64) one_tables_kernel(pw::smu::TabArgs<double2
 
 namespace pwi {
 
-cudaError_t launch_smu_list(int N, const pw::smu::Inst<float2>* list, int n, int chunk, bool any_mu, cudaStream_t s) {
+cudaError_t launch_smu_list(int N, const pw::smu::Inst<Wide>* list, int n, int chunk, bool any_mu, cudaStream_t s) {
   switch (N) {
 #define PW_CASE(NN) \
   case NN:          \
-    return pw::smu::launch<NN, float2>(list, {}, n, chunk, any_mu, s);
+    return pw::smu::launch<NN, Wide>(list, {}, n, chunk, any_mu, s);
     PW_CASE(16) PW_CASE(32) PW_CASE(64) PW_CASE(96) PW_CASE(128)
 #undef PW_CASE
     default:
@@ -30,7 +28,7 @@ cudaError_t launch_smu_list(int N, const pw::smu::Inst<float2>* list, int n, int
   }
 }
 
-cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<float2>* list, int n, cudaStream_t s) {
+cudaError_t launch_smu_list_tables(const pw::smu::TabArgs<Wide>* list, int n, cudaStream_t s) {
   list_tables_kernel<<<n, 256, 0, s>>>(list);
   return cudaGetLastError();
 }

@@ -11,10 +11,12 @@
 // axis): C is the inverse transform of |P^|^2, and R that of
 //   K(m) K(n) conj P^(2 iP - m, 2 jP - n), K = the transform of k,
 // so an instance costs a few FFTs of (2N)^2 points in place of an N^4 array.  (The 4D route took 0.99 ms
-// for one instance at N = 128, 87 ms for a batch of 192.)  A batch runs in FP32, as the 4D route did.  A few
-// lags carry most of S, so their rounding errors do not average out as the 4D route's did: for the forward
-// pass of an inverse problem, whose loss may be the small difference of two S, the single call runs in
-// FP64 (C = double2; 8 MFLOP at N = 96).
+// for one instance at N = 128, 87 ms for a batch of 192.)  A few lags carry most of S, so every output takes the
+// rounding of the largest: in FP32 the relative error of S was 1e-3 where S is 1e-4 of its maximum (the 4D route,
+// whose errors average over N^2 terms, 1e-5), and some dim S came out negative.  So a batch runs on pairs of
+// floats (ff.cuh), which leaves the rounding of the outputs alone: 2.6e-8 of S in L2, 6e-8 at every point,
+// against 1.8e-7 and 6e-6 in FP32 on well-lit outputs.  192 instances of N = 64 to 128 take 0.69 ms; 0.26 ms in
+// FP32, 2.62 ms in FP64.  The single call, for a host loop that waits for it, runs in FP64 (8 MFLOP at N = 96).
 //   k1: columns b, transform over a              -> X1[m][b]   (L x N)
 //   k2: rows m, transform over b; |P^|^2 back to v, times k(v), to b' -> Z1[m][b'];
 //       the R product back to d                  -> Z2[m][d]   (L x N each)
@@ -26,6 +28,9 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
+#include "ff.cuh"
 #include "propagate.cuh"
 
 namespace pw {
@@ -36,13 +41,12 @@ struct Inst {
   using R = real_t<C>;
   int N, iP, jP;
   int chunk;            // launch round: instances of one round have scratch of their own
-  double factor;        // s A / L^2
+  R factor;             // s A / L^2
   const C* tw;          // L twiddles exp(-2 pi i m / L)
   const C* P1;          // N: Ein(i) h(i)
-  const C* P1l;         // N: what rounding P1 left out
   const C* Eout;        // N
   const R* k;           // N: k(u)
-  R* K;                 // L: transform of k over |u| < N (FP64: written by k1)
+  R* K;                 // L: transform of k over |u| < N (written by k1)
   const float2* mask;   // N x N or nullptr
   int ap_ithr;          // aperture, as in batch.cuh
   C* scratch;           // 3 L N values
@@ -50,13 +54,21 @@ struct Inst {
   float2* mu;           // N x N or nullptr
 };
 
-// Lines per block.  FP32 batches fill the chip with instances, and 16 lines make whole sectors of the column
-// accesses.  FP64 calls are one instance: a line per block puts an SM's FP64 pipe behind each (N = 96: 16
-// lines a block left 6 to 12 blocks, 247 us a call; one line 74 us, with FP64's own radices below 55 us;
-// two lines 58 us).
-template <int N, class C> __host__ __device__ constexpr int lines() {
-  return sizeof(real_t<C>) == 8 ? 1 : N % 16 == 0 ? (N >= 256 ? 8 : 16) : N % 8 == 0 ? 8 : N;
+template <class C> __device__ __forceinline__ C ldc(const C* p) { return __ldg(p); }
+__device__ __forceinline__ ff2 ldc(const ff2* p) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
+  return make_c(ff(v.x, v.y), ff(v.z, v.w));
 }
+__device__ __forceinline__ ff ldc(const ff* p) {
+  const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+  return ff(v.x, v.y);
+}
+
+// Lines per block.  Batches (float pairs) fill the chip with instances, and four 16-byte lines fill the
+// 64-byte runs of the column accesses (polychromatic batch of 192: 1216 / 799 / 687 / 736 us with 1 / 2 / 4 / 8 lines).  FP64
+// calls are one instance: a line per block puts an SM's FP64 pipe behind each (N = 96: 16 lines a block left 6
+// to 12 blocks, 247 us a call; one line 74 us, with the radices below 55 us; two lines 58 us).
+template <int N, class C> __host__ __device__ constexpr int lines() { return std::is_same<C, ff2>::value ? 4 : 1; }
 template <int N, class C> __host__ __device__ constexpr int threads() {
   return N >= 64 ? 256 : 128;
 }
@@ -65,25 +77,19 @@ template <int N, class C> constexpr size_t smem_bytes() {
 }
 
 // In-place transform of the block's lines (length LEN, natural order), after a barrier and ending with one.
-// NS: points already combined (I stages).  FP32 takes the radices of fft.cuh's plans, FP64 fours and then
-// threes and twos: those plans are made for FP32 registers, and at 2 FP64 operations a clock and SM a
-// radix-16 butterfly keeps its warp for 5 us while most warps of the block have none.
-template <int LEN, int SIGN, int LINES, int NT, int NS = 1, int I = 0, class C>
+// NS: points already combined.  Radices are fours and then threes and twos: fft.cuh's plans are made for FP32
+// registers, and at 2 FP64 operations a clock and SM a radix-16 butterfly keeps its warp for 5 us while most
+// warps of the block have none.
+template <int LEN, int SIGN, int LINES, int NT, int NS = 1, class C>
 __device__ __forceinline__ void fft_lines(C* x, const C* tw) {
   if constexpr (NS < LEN) {
     constexpr int LP = LINES + 1, REM = LEN / NS;
     constexpr int RD = REM % 4 == 0 ? 4 : REM % 3 == 0 ? 3 : 2;
     auto ld = [x](int line, int pos) { return x[pos * LP + line]; };
     auto st = [x](int line, int pos, C v) { x[pos * LP + line] = v; };
-    if constexpr (sizeof(real_t<C>) == 8) {
-      line_stage<LEN, RD, NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
-      __syncthreads();
-      fft_lines<LEN, SIGN, LINES, NT, NS * RD>(x, tw);
-    } else {
-      line_stage<LEN, StageInfo<LEN, I>::R, NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
-      __syncthreads();
-      fft_lines<LEN, SIGN, LINES, NT, NS * StageInfo<LEN, I>::R, I + 1>(x, tw);
-    }
+    line_stage<LEN, RD, NS, SIGN, LINES, NT>(tw, ld, SyncMid{}, st);
+    __syncthreads();
+    fft_lines<LEN, SIGN, LINES, NT, NS * RD>(x, tw);
   }
 }
 
@@ -97,29 +103,13 @@ __device__ __forceinline__ void load_tw(const Inst<C>& in, C* tw, C* twN) {
   }
 }
 
-// (a + al)(b + bl) rounded once: the field's rounding errors reach every output alike, so the product
-// of two rounded factors cost mu a third of its accuracy where S is small.
-__device__ __forceinline__ float2 cmul_exact(float2 a, float2 al, float2 b, float2 bl) {
-  auto dot = [](float x, float xl, float y, float yl, float u, float ul, float v, float vl) {  // x y + u v
-    const float p = x * y, q = u * v, s = p + q, z = s - p;
-    const float es = (p - (s - z)) + (q - z);  // exact error of p + q
-    float e = fmaf(x, y, -p) + fmaf(u, v, -q) + es;
-    e = fmaf(x, yl, fmaf(xl, y, e));
-    e = fmaf(u, vl, fmaf(ul, v, e));
-    return s + e;
-  };
-  return make_float2(dot(a.x, al.x, b.x, bl.x, -a.y, -al.y, b.y, bl.y), dot(a.x, al.x, b.y, bl.y, a.y, al.y, b.x, bl.x));
-}
-
-__device__ __forceinline__ double2 cmul_exact(double2 a, double2, double2 b, double2) { return cmul(a, b); }
-
 // P(a, b): source field at a point.
 template <int N, class C>
 __device__ __forceinline__ C field(const Inst<C>& in, int a, int b) {
   using R = real_t<C>;
   const int na = a - N / 2, nb = b - N / 2;
-  if (in.ap_ithr >= 0 && na * na + nb * nb > in.ap_ithr) return make_c((R)0, (R)0);
-  C v = cmul_exact(__ldg(in.P1 + a), __ldg(in.P1l + a), __ldg(in.P1 + b), __ldg(in.P1l + b));
+  if (in.ap_ithr >= 0 && na * na + nb * nb > in.ap_ithr) return make_c((R)0.f, (R)0.f);
+  C v = cmul(ldc(in.P1 + a), ldc(in.P1 + b));
   if (in.mask) {
     const float2 m = __ldg(in.mask + a * N + b);
     v = cmul(v, make_c((R)m.x, (R)m.y));
@@ -133,8 +123,8 @@ __device__ __forceinline__ void fold(C* x, const real_t<C>* k) {
   constexpr int LP = LINES + 1;
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int line = e % LINES, v = e / LINES;
-    C y = cscale(x[v * LP + line], __ldg(k + v));
-    if (v > 0) y = cadd(y, cscale(x[(v + N) * LP + line], __ldg(k + N - v)));
+    C y = cscale(x[v * LP + line], ldc(k + v));
+    if (v > 0) y = cadd(y, cscale(x[(v + N) * LP + line], ldc(k + N - v)));
     x[v * LP + line] = y;
   }
   __syncthreads();
@@ -155,21 +145,19 @@ __global__ void __launch_bounds__(threads<N, C>()) k1(const Inst<C>* list, Inst<
   C *x = reinterpret_cast<C*>(smem), *tw = x + 2 * L * LP, *twN = tw + L;
   load_tw<N>(in, tw, twN);
   const int b0 = blockIdx.x * LINES;
-  if constexpr (sizeof(R) == 8) {
-    if (b0 == N) {  // the last block: K
-      for (int e = threadIdx.x; e < L * LINES; e += NT) {
-        const int line = e % LINES, u = e / LINES;
-        x[u * LP + line] = make_c(line || u == N ? (R)0 : __ldg(in.k + (u < N ? u : L - u)), (R)0);
-      }
-      __syncthreads();
-      fft_lines<L, -1, LINES, NT>(x, tw);
-      for (int m = threadIdx.x; m < L; m += NT) in.K[m] = x[m * LP].x;
-      return;
+  if (b0 == N) {  // the last block: K
+    for (int e = threadIdx.x; e < L * LINES; e += NT) {
+      const int line = e % LINES, u = e / LINES;
+      x[u * LP + line] = make_c(line || u == N ? (R)0.f : ldc(in.k + (u < N ? u : L - u)), (R)0.f);
     }
+    __syncthreads();
+    fft_lines<L, -1, LINES, NT>(x, tw);
+    for (int m = threadIdx.x; m < L; m += NT) in.K[m] = x[m * LP].x;
+    return;
   }
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, a = e / LINES;
-    x[a * LP + line] = a < N ? field<N, C>(in, a, b0 + line) : make_c((R)0, (R)0);
+    x[a * LP + line] = a < N ? field<N, C>(in, a, b0 + line) : make_c((R)0.f, (R)0.f);
   }
   __syncthreads();
   fft_lines<L, -1, LINES, NT>(x, tw);
@@ -194,7 +182,7 @@ __global__ void __launch_bounds__(threads<N, C>()) k2(const Inst<C>* list, Inst<
   C* Z2 = Z1 + (size_t)L * N;
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int b = e % L, line = e / L;
-    x[b * LP + line] = b < N ? X1[(m0 + line) * N + b] : make_c((R)0, (R)0);
+    x[b * LP + line] = b < N ? X1[(m0 + line) * N + b] : make_c((R)0.f, (R)0.f);
   }
   __syncthreads();
   fft_lines<L, -1, LINES, NT>(x, tw);  // P^(m, n)
@@ -204,14 +192,14 @@ __global__ void __launch_bounds__(threads<N, C>()) k2(const Inst<C>* list, Inst<
       int mm = 2 * in.iP - (m0 + line), nn = 2 * in.jP - n;
       mm += mm < 0 ? L : 0;
       nn += nn < 0 ? L : 0;
-      y[n * LP + line] = cscale(cconj(x[nn * LP + line]), __ldg(in.K + mm) * __ldg(in.K + n));
+      y[n * LP + line] = cscale(cconj(x[nn * LP + line]), ldc(in.K + mm) * ldc(in.K + n));
     }
     __syncthreads();
   }
   for (int e = threadIdx.x; e < L * LINES; e += NT) {
     const int line = e % LINES, n = e / LINES;
     const C v = x[n * LP + line];
-    x[n * LP + line] = make_c(fma_(v.x, v.x, v.y * v.y), (R)0);
+    x[n * LP + line] = make_c(fma_(v.x, v.x, v.y * v.y), (R)0.f);
   }
   __syncthreads();
   fft_lines<L, +1, LINES, NT>(x, tw);
@@ -255,7 +243,7 @@ __global__ void __launch_bounds__(threads<N, C>()) k3(const Inst<C>* list, Inst<
   fft_lines<N, -1, LINES, NT>(x, twN);
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int line = e % LINES, a = e / LINES;
-    in.S[a * N + b0 + line] = (float)(x[a * LP + line].x * (R)in.factor);
+    in.S[a * N + b0 + line] = (float)(x[a * LP + line].x * in.factor);
   }
   if (!in.mu) return;
   __syncthreads();
@@ -294,34 +282,27 @@ __global__ void __launch_bounds__(threads<N, C>()) k4(const Inst<C>* list, Inst<
   __syncthreads();
   fft_lines<N, -1, LINES, NT>(x, twN);
   const float sp = in.S[in.iP * N + in.jP];
-  const C ep = cscale(cconj(cmul(__ldg(in.Eout + in.iP), __ldg(in.Eout + in.jP))), (R)in.factor);
+  const C ep = cscale(cconj(cmul(ldc(in.Eout + in.iP), ldc(in.Eout + in.jP))), in.factor);
   for (int e = threadIdx.x; e < N * LINES; e += NT) {
     const int d = e % N, line = e / N, c = c0 + line;
     const float den = sp * in.S[c * N + d];
-    const C row = cmul(cmul(ep, cmul(__ldg(in.Eout + c), __ldg(in.Eout + d))), x[d * LP + line]);
+    const C row = cmul(cmul(ep, cmul(ldc(in.Eout + c), ldc(in.Eout + d))), x[d * LP + line]);
     const float inv = rsqrtf(den);
     in.mu[c * N + d] = den > 0.f ? make_float2((float)row.x * inv, (float)row.y * inv) : make_float2(0.f, 0.f);
   }
 }
 
-// FP64-derived tables of one instance (one block): twiddles, per-axis factors, coherence and its
-// transform.
+// FP64-derived tables of one instance: twiddles, per-axis factors, coherence.
 template <class C>
 struct TabArgs {
   int N;
   double Kin, Kout;  // turns per n^2 of the input factor (propagator, lens) and of the output propagator
   double gs, gm;     // d^2/(4 sigma_S^2), d^2/(2 sigma_mu^2)
-  C *tw, *P1, *P1l, *Eout;  // P1l: float2 only
-  real_t<C> *k, *K;
+  C *tw, *P1, *Eout;
+  real_t<C>* k;
 };
 
-__device__ __forceinline__ void put(float2* h, float2* l, int i, double x, double y) {
-  h[i] = make_float2((float)x, (float)y);
-  if (l) l[i] = make_float2((float)(x - (double)(float)x), (float)(y - (double)(float)y));
-}
-__device__ __forceinline__ void put(double2* h, double2*, int i, double x, double y) { h[i] = make_double2(x, y); }
-
-// All tables but K; one FP64 evaluation per task: tasks 0..L-1 tw, then P1, Eout and k of each index.
+// One FP64 evaluation per task: tasks 0..L-1 tw, then P1, Eout and k of each index.
 template <class C>
 __device__ __forceinline__ void tables(const TabArgs<C>& t, int q0, int step) {
   using R = real_t<C>;
@@ -337,30 +318,13 @@ __device__ __forceinline__ void tables(const TabArgs<C>& t, int q0, int step) {
     double sn, cs;
     sincospi(2.0 * frac_turns(turns), &sn, &cs);
     if (kind < 0) {
-      put(t.tw, (C*)nullptr, i, cs, sn);
+      t.tw[i] = make_c((R)cs, (R)sn);
     } else if (kind == 1) {
-      put(t.Eout, (C*)nullptr, i, cs, sn);
+      t.Eout[i] = make_c((R)cs, (R)sn);
     } else {
       const double hh = exp(-n2 * t.gs);
-      put(t.P1, t.P1l, i, cs * hh, sn * hh);
+      t.P1[i] = make_c((R)(cs * hh), (R)(sn * hh));
     }
-  }
-}
-
-// K by one block, from its own k and tw.
-template <class C>
-__device__ __forceinline__ void table_K(const TabArgs<C>& t) {
-  using R = real_t<C>;
-  const int N = t.N, L = 2 * N;
-  for (int m = threadIdx.x; m < L; m += blockDim.x) {
-    R acc = 0;
-    int j = 0;  // m u mod L
-    for (int u = 1; u < N; ++u) {
-      j += m;
-      j -= j >= L ? L : 0;
-      acc = fma_(t.k[u], t.tw[j].x, acc);
-    }
-    t.K[m] = fma_((R)2, acc, t.k[0]);
   }
 }
 
@@ -378,7 +342,7 @@ cudaError_t launch(const Inst<C>* list, const Inst<C>& one, int n, int chunk, bo
       return e;
     ready = true;
   }
-  k1<N, C><<<dim3(N / LINES + (sizeof(real_t<C>) == 8), n), NT, sm, s>>>(list, one, chunk);
+  k1<N, C><<<dim3(N / LINES + 1, n), NT, sm, s>>>(list, one, chunk);
   k2<N, C><<<dim3(2 * N / LINES, n), NT, sm, s>>>(list, one, chunk);
   k3<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
   if (any_mu) k4<N, C><<<dim3(N / LINES, n), NT, sm, s>>>(list, one, chunk);
