@@ -8,11 +8,15 @@
 // Np = N rounded up to 16.  Each operand is x = x1 + x2 with x1 = fp16(x), x2 = fp16(x - x1): 22 to 24
 // bits of x, and D accumulates x1 q1 + x1 q2 + x2 q1 (the dropped x2 q2 is below 2^-23).  FP16 has no
 // exponent to spare, so both operands are scaled by powers of two: Q by 2^10 (|A| = 1), X so that the
-// largest component of the whole input array comes to [2^13, 2^14).  Values down to 2^-29 of the largest
-// keep their two full parts and the absolute floor is 2^-39 of it; an output of a full set of
-// contractions mixes every input with unit-modulus weights, so its FP32 rounding noise (2^-24 of the
-// largest terms) covers that floor.  Every contraction leaves the largest component of its output for the
-// next one (max_out / max_in); the first takes it from the source.
+// largest component of the whole input array comes to [2^13, 2^14).  Values down to 2^-16 of the largest
+// keep their 22 bits, smaller ones an absolute error of 2^-39 of it (a relative 2^-18 at 2^-20).  An output of
+// a full set of contractions mixes every input with unit-modulus weights, so its FP32 rounding noise (2^-24 of
+// the largest terms) covers that floor.  Every contraction leaves the largest component of its output for the
+// next one (max_out / max_in); the first takes it from the source.  The tables of a GSM source are not such a
+// full set: a and d of H(a, b', d) T(a, c', d) only meet the other point's mask in the product, which may
+// leave nothing but lines where both tables are small.  So there every column (a, d) has a scale of its own.
+// (With one scale for a table, an opaque disc of 32 pixels before a beam of sigma_S = 5 pixels, N = 90, cost 5e-3
+// of W; now 1e-7.)
 // Measured against FP64 (relative L2 of W): 1.7e-6 at N = 200 padded to 512, 2.9e-6 at N = 90, where BF16
 // operands in three parts with six products gave 2.1e-6 and 5.4e-6: the error is that of the accumulation,
 // which has half as many steps now.
@@ -138,23 +142,27 @@ struct TableArgs {
   const float2* M0;
   float A;
   float2 *H0, *T0;     // N^3 each: [a][b][d], [a][c][d]
-  unsigned* max;       // [0], [1]: largest components of H0 and T0
+  unsigned* max;       // 2 x N x N: largest component of each column (a, d) of H0, then of T0
 };
-__global__ void __launch_bounds__(256) table_source_kernel(TableArgs p) {
-  const int N = p.N;
-  const size_t N3 = (size_t)N * N * N;
-  float mh = 0.f, mt = 0.f;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N3; idx += (size_t)gridDim.x * blockDim.x) {
-    const int a = (int)(idx / ((size_t)N * N)), bd = (int)(idx - (size_t)a * N * N), b = bd / N;
-    const float2 h = cscale(cconj(__ldg(p.M0 + a * N + b)), p.A * __ldg(p.G + bd));
-    const float2 t = cscale(__ldg(p.M0 + bd), __ldg(p.G + a * N + b));
-    p.H0[idx] = h;
-    p.T0[idx] = t;
-    mh = fmaxf(mh, fmaxf(fabsf(h.x), fabsf(h.y)));
-    mt = fmaxf(mt, fmaxf(fabsf(t.x), fabsf(t.y)));
-  }
-  warp_max(p.max, mh);
-  warp_max(p.max + 1, mt);
+constexpr int TS_D = 32, TS_B = 8;  // a block: 32 columns d of one a, of H0 (blockIdx.z = 0) or T0, in 8 shares of b or c
+__global__ void __launch_bounds__(TS_D * TS_B) table_source_kernel(TableArgs p) {
+  __shared__ float share[TS_B][TS_D];
+  const int N = p.N, tx = threadIdx.x % TS_D, ty = threadIdx.x / TS_D, d = blockIdx.x * TS_D + tx, a = blockIdx.y;
+  const bool h = blockIdx.z == 0;
+  const size_t col = (size_t)a * N * N + d;
+  float m = 0.f;
+  if (d < N)
+    for (int b = ty; b < N; b += TS_B) {
+      const int ab = a * N + b, bd = b * N + d;
+      const float2 v = h ? cscale(cconj(__ldg(p.M0 + ab)), p.A * __ldg(p.G + bd)) : cscale(__ldg(p.M0 + bd), __ldg(p.G + ab));
+      (h ? p.H0 : p.T0)[col + (size_t)b * N] = v;
+      m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
+    }
+  share[ty][tx] = m;
+  __syncthreads();
+  if (ty != 0 || d >= N) return;
+  for (int k = 1; k < TS_B; ++k) m = fmaxf(m, share[k][tx]);
+  p.max[((h ? 0 : N) + a) * N + d] = __float_as_uint(m);
 }
 // Largest |H T| over the N^4 array: for each (a, d) the largest |H| over b' times the largest |T| over c'.
 __global__ void __launch_bounds__(256) table_max_kernel(int N, const float2* __restrict__ H, const float2* __restrict__ T,
@@ -240,6 +248,7 @@ struct Args {
   const float2* M0; // IN_MASK
   const float2 *H, *T;       // IN_PRODUCT (j = (a, b', c'))
   const unsigned* max_in;    // bits of the largest input component
+  const unsigned* max_col;   // IN_COLS: the same of each column j, in place of max_in; or nullptr
   unsigned* max_out;         // the same of the output, or nullptr
   int stall;  // failure-detection test (0 = off): CTA 0 never copies operand chunk `stall` (> 0), or never
               // announces A tile -stall (< 0)
@@ -284,7 +293,7 @@ __global__ void __launch_bounds__(NT, 2) axis_tc_kernel(Args p, const unsigned c
   const long long L = p.L;
   // 32-bit column arithmetic: j < N^3 <= 2^24 and L <= N^3
   const unsigned ncols = (unsigned)p.ncols, Lu = (unsigned)L;
-  const int sexp = scale_exp(*p.max_in);
+  int sexp = 0;  // exponent of the input scale; per column, thread t's being that of its epilogue too
 
   // the converter's inputs: eight values of a chunk, loaded two chunks ahead (three sets in turn).
   // ROWS: n = 16 c + 2 (t mod 8) + {0, 1} of the columns tile * 128 + t / 8 + 32 i, i < 4.
@@ -310,11 +319,13 @@ __global__ void __launch_bounds__(NT, 2) axis_tc_kernel(Args p, const unsigned c
       }
     }
     src = MODE == IN_PRODUCT ? p.T : p.in + (size_t)(tile * 128 + (t >> 3)) * N + 2 * l8;
+    sexp = scale_exp(*p.max_in);
   } else {
     const unsigned j = tile * 128 + m;
     live[0] = t < 256 && j < ncols;
     const unsigned jj = live[0] ? j : 0u;
     src = p.in + (size_t)(jj / Lu) * L * N + jj % Lu;
+    sexp = scale_exp(p.max_col ? p.max_col[jj] : *p.max_in);
   }
   auto load = [&](int c, float2 (&x)[8]) {
     if constexpr (ROWS) {

@@ -706,23 +706,25 @@ pw_status propagate_dense(pw_csd* h, double z, bool farfield, bool herm) {
     h->stall = 0;
     if (sa.mode == pw::SRC_GSM) {
       const size_t N3 = (size_t)N * N * N;
-      T::TableArgs ta{N, h->G, h->M0, (float)h->A, Xf, Xf + N3, mx};
-      T::table_source_kernel<<<num_sms() * 8, 256, 0, s>>>(ta);
+      unsigned* cm = reinterpret_cast<unsigned*>(h->adj_c);  // 2 N^2 column maxima in the adjoint's scratch
+      T::TableArgs ta{N, h->G, h->M0, (float)h->A, Xf, Xf + N3, cm};
+      T::table_source_kernel<<<dim3((N + T::TS_D - 1) / T::TS_D, N, 2), T::TS_D * T::TS_B, 0, s>>>(ta);
       float2 *H = Wf, *Tt = Wf + N3;
       ax.L = N;
       ax.ncols = (long long)NN;
       ax.in = ta.H0;
       ax.out = H;
-      ax.max_in = mx;
+      ax.max_col = cm;
       if ((e = launch_axis_tc(ax, T::IN_COLS, q + qb, h->err, s)) != cudaSuccess) return cuda_fail(e, "table contraction");
       ax.in = ta.T0;
       ax.out = Tt;
-      ax.max_in = mx + 1;
+      ax.max_col = cm + NN;
       if ((e = launch_axis_tc(ax, T::IN_COLS, q, h->err, s)) != cudaSuccess) return cuda_fail(e, "table contraction");
       T::table_max_kernel<<<(NN + 255) / 256, 256, 0, s>>>(N, H, Tt, mx + 2);
       ax.L = 1;
       ax.ncols = (long long)N3;
       ax.in = nullptr;
+      ax.max_col = nullptr;
       ax.H = H;
       ax.T = Tt;
       ax.out = Xf;

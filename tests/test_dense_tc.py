@@ -9,6 +9,7 @@ is 1e-6, so the two stay within 1e-5."""
 import numpy as np
 import pytest
 
+import oracle as O
 import workloads as WL
 
 pytestmark = pytest.mark.gpu
@@ -71,3 +72,28 @@ def test_non_finite_input_stays_in_its_propagation():
     W0[3, 4, 5, 6] = complex(float("inf"), 0.0)
     W, S = _run(N, 0, 2, lambda c, pw, _: c.source_array(W0, False), False)
     assert not bool(torch.isfinite(W).any())  # every output takes every input
+
+
+# Masks that leave only the tail of the source: in the tables a and d meet the other point's mask only in the
+# product (see dense_tc.cuh).  Against FP64 on sampled rows; FP32 accumulation as above, 1e-5.
+@pytest.mark.parametrize("sM", [1.5, 50.0])
+@pytest.mark.parametrize("N,Nz,kind", [(90, 0, "disc"), (90, 0, "opening"), (54, 80, "disc"), (136, 0, "opening")])
+def test_gsm_tail_through_a_mask(N, Nz, kind, sM):
+    import torch
+    import paper_2203_02734_gb300 as pw
+    n, sS = np.arange(N) - N // 2, N / 18
+    r2 = n[:, None] ** 2 + n[None, :] ** 2
+    m = (r2 >= (6.4 * sS) ** 2) if kind == "disc" else ((n[:, None] - int(8 * sS)) ** 2 + n[None, :] ** 2 <= 9)
+    m = WL.to_c64(WL.phase_screen(N, seed=4) * m)
+    z, rows = 0.3, [(N // 2, N // 2), (3, N - 2), (N // 3, N // 2 + 5)]
+    c = pw.CSD(N, D, LAM)
+    pw.pw_csd_set_padding(c.h, Nz)
+    pw.pw_csd_set_dft_mode(c.h, 2)
+    c.source_gsm(sS * D, sM * D, 1.0)
+    c.source_mask(torch.from_numpy(m).cuda())
+    c.propagate_fresnel(z)
+    pw.pw_csd_check(c.h)
+    ref = O.propagate_rows_gsm_padded(m.astype(complex), N, D, LAM, z, sS * D, sM * D, 1.0, rows, Nz or N)
+    out = np.array([c.W[r].cpu().numpy() for r in rows]).astype(complex)
+    assert np.linalg.norm(out - ref) < 1e-5 * np.linalg.norm(ref)
+    c.close()
