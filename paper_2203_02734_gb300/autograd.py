@@ -28,18 +28,26 @@ class _Model:
         self.csd = CSD(N, self.dxi, self.lam, device=device)
         self.dev = self.csd.W.device
 
+    def other_stream(self):
+        """The caller's stream where it is not the handle's, else None."""
+        cur = torch.cuda.current_stream(self.dev)
+        return None if cur == self.csd.stream else cur
+
+    def meet(self, other):
+        """Neither the caller's stream nor the handle's runs on before the other has come to this point (the
+        tensors of a call are the caller's stream's, the handle's stream reads and writes them)."""
+        if other is not None:
+            other.wait_stream(self.csd.stream)
+            self.csd.stream.wait_stream(other)
+
     def outputs(self):
         """New S and mu tensors (they belong to the caller's graph)."""
         NN = (self.N, self.N)
         return self.new((NN, torch.float32), (NN, torch.complex64))
 
     def new(self, *specs):
-        """Device tensors (shape, dtype) that the handle's stream may still be writing when they are freed."""
-        out = [torch.empty(shape, dtype=dtype, device=self.dev) for shape, dtype in specs]
-        if torch.cuda.current_stream(self.dev) != self.csd.stream:
-            for t in out:
-                t.record_stream(self.csd.stream)
-        return out
+        """Device tensors (shape, dtype)."""
+        return [torch.empty(shape, dtype=dtype, device=self.dev) for shape, dtype in specs]
 
     def propagate_and_read(self):
         h = self.csd.h
@@ -66,8 +74,11 @@ class _Model:
         adj.iP, adj.jP = self.P1
         for k, v in kw.items():
             setattr(adj, k, v)
+        other = self.other_stream()
+        self.meet(other)
         abi.pw_csd_reset(h, self.dx)  # the output plane's sampling
         (abi.pw_propagate_farfield_adjoint if self.farfield else abi.pw_propagate_fresnel_adjoint)(h, self.z, adj)
+        self.meet(other)
         return keep
 
     def close(self):
@@ -108,7 +119,10 @@ class _GSMFn(torch.autograd.Function):
         m = model.m
         h = m.csd.h
         am = amask.detach().to(torch.float32).contiguous()
+        other = m.other_stream()
+        m.meet(other)  # the handle's earlier calls have read mask_c
         model.mask_c.real.copy_(am)  # the amplitude mask as a complex mask (argument marshalling)
+        m.meet(other)
         abi.pw_csd_reset(h, m.dxi)
         params = (float(sigma_S), float(sigma_mu), float(A))
         abi.pw_source_gsm(h, *params)
@@ -118,6 +132,7 @@ class _GSMFn(torch.autograd.Function):
             abi.pw_gsm_s_mu(h, m.z, m.farfield, m.P1[0], m.P1[1], S.data_ptr(), mu.data_ptr())
         else:
             S, mu = m.propagate_and_read()
+        m.meet(other)
         ctx.model = model
         ctx.params = params
         ctx.like = [(x.device, x.dtype) if torch.is_tensor(x) else None for x in (sigma_S, sigma_mu, A)]
@@ -166,9 +181,12 @@ class _CSDFn(torch.autograd.Function):
         m = model.m
         h = m.csd.h
         W0c = W0.detach().to(torch.complex64).contiguous()
+        other = m.other_stream()
+        m.meet(other)
         abi.pw_csd_reset(h, m.dxi)
         abi.pw_source_array(h, W0c.data_ptr(), 1 if model.hermitian else 0)
         S, mu = m.propagate_and_read()
+        m.meet(other)
         ctx.model = model
         ctx.save_for_backward(S, mu)
         ctx.set_materialize_grads(False)
