@@ -93,7 +93,7 @@ class GSMPropagation:
     def __init__(self, N, dxi, lam, z, P1=None, farfield=False, device=None):
         self.m = _Model(N, dxi, lam, z, P1, farfield, device)
         self.mask_c = torch.zeros((N, N), dtype=torch.complex64, device=self.m.dev)
-        # S and mu need no CSDA where the library has the direct form (an FFT plan, N >= 4)
+        # S and mu need no CSDA where the library has the direct form (an FFT plan, N >= 4, no zero padding)
         self.direct = N >= 4 and abi.pw_supported_n(N)
 
     def __call__(self, sigma_S, sigma_mu, A, amask):
@@ -127,7 +127,7 @@ class _GSMFn(torch.autograd.Function):
         params = (float(sigma_S), float(sigma_mu), float(A))
         abi.pw_source_gsm(h, *params)
         abi.pw_source_mask(h, model.mask_c.data_ptr())
-        if model.direct:
+        if model.direct and abi.pw_csd_get_padding(h) == m.N:
             S, mu = m.outputs()
             abi.pw_gsm_s_mu(h, m.z, m.farfield, m.P1[0], m.P1[1], S.data_ptr(), mu.data_ptr())
         else:

@@ -307,3 +307,23 @@ def test_tensor_core_wait_timeout_is_reported_and_recovers(stall):
     c.close()
     Wr, _ = O.propagate_padded(O.gsm_source(N, D, SS, SM), D, LAM, z, Nz)
     assert rel(W, Wr) < 1e-5
+
+
+@pytest.mark.parametrize("N,Nz", [(16, 40), (32, 48)])
+def test_autograd_forward_on_a_padded_handle(N, Nz):
+    """A padded handle has no direct S and mu: the model's forward is the padded propagation, as on any handle."""
+    import torch
+    import paper_2203_02734_gb300 as pw
+    from paper_2203_02734_gb300.autograd import GSMPropagation
+    P1, a = (N // 2, N // 2 - 1), 0.5 + 0.5 * torch.rand(N, N, generator=torch.Generator().manual_seed(1)).cuda()
+    model = GSMPropagation(N, D, LAM, 0.4, P1=P1)
+    pw.pw_csd_set_padding(model.m.csd.h, Nz)
+    S, mu = model(5 * D, 1.5 * D, 1.2, a)
+    c = pw.CSD(N, D, LAM)
+    pw.pw_csd_set_padding(c.h, Nz)
+    c.source_gsm(5 * D, 1.5 * D, 1.2)
+    c.source_mask(a.to(torch.complex64))
+    c.propagate_fresnel(0.4)
+    assert torch.equal(S, c.spectral_density()) and torch.equal(torch.view_as_real(mu), torch.view_as_real(c.degree_of_coherence(*P1)))
+    c.close()
+    model.close()
