@@ -117,6 +117,7 @@ struct pw_batch {
   cudaStream_t stream;
   std::vector<pw::batch::Inst> inst;
   std::vector<int> stalled;  // instances whose pass-A items are left out (failure-detection test)
+  std::vector<float> scales;   // scale times amplitude of every instance
   std::vector<double> dx_out;  // output sampling of every instance (lambda z / (N dxi))
   int nitems;
   long long wait_cycles;
@@ -295,7 +296,9 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     d.slices = (int)NN;
     d.A = (float)q.amplitude;
     const double lz = q.lambda_m * q.z_m;
-    d.scale = (float)((q.dxi_m * q.dxi_m / lz) * (q.dxi_m * q.dxi_m / lz));
+    const double s2 = (q.dxi_m * q.dxi_m / lz) * (q.dxi_m * q.dxi_m / lz);
+    d.scale = (float)s2;
+    b->scales.push_back((float)(s2 * q.amplitude));
     float2* F = reinterpret_cast<float2*>(b->base + off);
     off = align256(off + NN * sizeof(float2));
     float* G = reinterpret_cast<float*>(b->base + off);
@@ -358,7 +361,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     si.N = N;
     si.iP = q.iP;
     si.jP = q.jP;
-    si.factor = (q.dxi_m * q.dxi_m / lz) * (q.dxi_m * q.dxi_m / lz) * q.amplitude / (4.0 * (double)NN);
+    si.factor = s2 * q.amplitude / (4.0 * (double)NN);
     si.tw = ta.tw;
     si.P1 = ta.P1;
     si.Eout = ta.Eout;
@@ -448,6 +451,7 @@ pw_status pw_batch_run(pw_batch* b) {
       q.S = d.S;
       q.A = d.A;
       q.scale = d.scale;
+      q.scale_A = b->scales[i];
       q.row = d.row;
       q.iP = d.iP;
       q.jP = d.jP;

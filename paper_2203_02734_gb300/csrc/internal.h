@@ -33,7 +33,7 @@ struct PlaneArgs {
   float2* work;  // 2 N^3 table values
   float2* W;
   float* S;
-  float A, scale;
+  float A, scale, scale_A;  // scale_A = scale A, rounded once
   float2* row;  // W(P1, .) or nullptr
   int iP, jP;
 };

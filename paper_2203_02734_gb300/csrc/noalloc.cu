@@ -218,9 +218,8 @@ extern "C" pw_status pw_propagate_gsm_fresnel_noalloc(int N, double dxi_m, doubl
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const double lz = lam * z_m;
-  const float scale = (float)((d * d / lz) * (d * d / lz));
-  const pw::small::Args q{F, G, tw, Eout, reinterpret_cast<float2*>(dev_W_out), dev_S_out, (float)amplitude, scale,
-                          nullptr, 0, 0};
+  const double s2 = (d * d / lz) * (d * d / lz);
+  const pw::small::Args q{F, G, tw, Eout, reinterpret_cast<float2*>(dev_W_out), dev_S_out, (float)(s2 * amplitude), nullptr, 0, 0};
   switch (N) {
     case 2: return run_small<2>(t, q, s);
     case 4: return run_small<4>(t, q, s);
@@ -258,7 +257,7 @@ extern "C" pw_status pw_propagate_gsm_fresnel_noalloc(int N, double dxi_m, doubl
   b.Eout = Eout;
   b.W = reinterpret_cast<float2*>(dev_W_out);
   b.S = dev_S_out;
-  b.scale = scale;
+  b.scale = (float)s2;
   switch (N) {
     case 24: return run<24>(vmap, t, a, b, s);
     case 32: return run<32>(vmap, t, a, b, s);

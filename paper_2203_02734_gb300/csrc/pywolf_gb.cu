@@ -403,7 +403,7 @@ template <int N>
 cudaError_t launch_small(const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
   cudaError_t e;
   if (ev && ((e = cudaEventRecord(ev[0], s)) != cudaSuccess || (e = cudaEventRecord(ev[1], s)) != cudaSuccess)) return e;
-  const pw::small::Args a{q.F, q.G, q.tw, q.Eout, q.W, q.S, q.A, q.scale, q.row, q.iP, q.jP};
+  const pw::small::Args a{q.F, q.G, q.tw, q.Eout, q.W, q.S, q.scale_A, q.row, q.iP, q.jP};
   if ((e = pw::small::launch<N>(a, s)) != cudaSuccess) return e;
   return ev ? cudaEventRecord(ev[2], s) : cudaSuccess;
 }
@@ -864,6 +864,7 @@ pw_status propagate_planes(pw_csd* h, double z) {
   q.S = h->S;
   q.A = (float)h->A;
   q.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
+  q.scale_A = (float)((h->d * h->d / lz) * (h->d * h->d / lz) * h->A);
   cudaError_t e = pwi::dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch (GSM source)");
   to_output_plane(h, lz / (h->N * h->d), true);
