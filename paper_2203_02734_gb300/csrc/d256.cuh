@@ -126,11 +126,10 @@ __device__ __forceinline__ void p_stages(float2 (&u)[2][16], float2* slab, const
 // kernel needs no more shared memory than the FP32 one: at 6 KB more, the occupancy calculator
 // fits one CTA per SM instead of two (15 clusters of 8 instead of 36, measured).
 // A bounded wait that gives up sets *err and leaves the stage's outputs zero.
-template <int CS, int SRC, bool MASK, bool TC = false>
+template <int CS, bool MASK, bool TC = false>
 __global__ void __launch_bounds__(Geo<CS>::NT, Geo<CS>::MINB)
     pass_a_d256(const __grid_constant__ CUtensorMap vmap, PassAArgs p, const float2* __restrict__ Ein,
                 const float2* __restrict__ mask, int ap_ithr, int* err) {
-  constexpr bool ARRAY = SRC == SRC_ARRAY;
   constexpr int RPC = Geo<CS>::RPC, NT = Geo<CS>::NT, HALF = Geo<CS>::HALF;
   static_assert(!TC || NT == 256, "the tensor-core stage maps thread t to vector t of two 128-row tiles");
   extern __shared__ __align__(1024) float2 smem[];
@@ -166,29 +165,24 @@ __global__ void __launch_bounds__(Geo<CS>::NT, Geo<CS>::MINB)
   constexpr int g = vgroup<N>();
   for (int ab = cluster; ab < N * N; ab += nclusters) {
     const int a = ab / N, b = ab - a * N;
-    if (SRC == SRC_GSM) {
-      for (int i = t; i < N; i += NT) {
-        gA[i] = p.G[a * N + i];
-        gB[i] = p.G[b * N + i];
-      }
+    for (int i = t; i < N; i += NT) {
+      gA[i] = p.G[a * N + i];
+      gB[i] = p.G[b * N + i];
     }
     __syncthreads();
     float2 fab = inside(a, b) ? cmul(ein[a], ein[b]) : make_float2(0.f, 0.f);
     if (MASK) fab = cmul(fab, __ldg(mask + a * N + b));
-    float2 s_ab = cconj(fab);
-    if (SRC == SRC_GSM) s_ab = cscale(s_ab, p.A);
-    const float2* W0 = ARRAY ? p.W0 + (size_t)ab * N * N : nullptr;
+    const float2 s_ab = cscale(cconj(fab), p.A);
     float2 v[2][16];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c = RPC * (int)rank + rg + HALF * h;
-      const float2 sc = SRC == SRC_GSM ? cmul(s_ab, cscale(ein[c], gA[c])) : cmul(s_ab, ein[c]);
+      const float2 sc = cmul(s_ab, cscale(ein[c], gA[c]));
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
         const int d = jq + 16 * r;
-        float2 x = cmul(sc, SRC == SRC_GSM ? cscale(ein[d], gB[d]) : ein[d]);
+        float2 x = cmul(sc, cscale(ein[d], gB[d]));
         if (MASK) x = cmul(x, __ldg(mask + c * N + d));
-        if (ARRAY) x = cmul(x, __ldg(W0 + (size_t)c * N + d));
         bool keep = inside(c, d);
         v[h][r] = keep ? x : make_float2(0.f, 0.f);
       }

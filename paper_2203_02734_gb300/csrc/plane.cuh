@@ -119,8 +119,8 @@ __device__ __forceinline__ void plane_s_row(const Args& p, const float2* buf, At
 }
 
 // ---------------------------------------------------------------------------------------------
-// N <= 48 (from N = 24; small.cuh below): the generic shared-memory 2D transform of propagate.cuh, one plane per block iteration;
-// the natural-order plane leaves by one TMA tensor store (box {2 N floats, 1, 1, N} of W).
+// N = 24 to 48 (small.cuh up to 16): the generic shared-memory 2D transform of propagate.cuh, one plane per
+// block iteration; the natural-order plane leaves by one TMA tensor store (box {2 N floats, 1, 1, N} of W).
 template <int N> constexpr size_t plane_smem() {
   return (size_t)N * pitch<N>() * sizeof(float2) + 2 * N * sizeof(float2);
 }

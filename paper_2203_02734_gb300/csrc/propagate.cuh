@@ -119,7 +119,6 @@ template <int N> __host__ __device__ constexpr int vgroup() { return vgroup_of(N
 // Row of c' along V's c' index.  At N = 128 the eight rows c' = w + 16 i that one pass-A warp
 // finishes are adjacent (8 w + i), so that the warp leaves them by one TMA store; other N keep c'.
 template <int N> __host__ __device__ constexpr int vrow(int c) { return N == 128 ? 8 * (c & 15) + (c >> 4) : c; }
-template <int N> __host__ __device__ constexpr int vrow_inv(int r) { return N == 128 ? 16 * (r & 7) + (r >> 3) : r; }
 // offset of V(a, b, c', d') in the V layout
 template <int N>
 __device__ __forceinline__ size_t v_offset(int ab, int c, int d) {

@@ -323,14 +323,14 @@ cudaError_t launch_a_d256(const CUtensorMap& vmap, const pw::PassAArgs& a, const
     // clusters of 8 instead of 36, measured). This one allocates 128 of an SM's 512 columns and
     // has the registers, threads and shared memory of its FP32 twin, which caps residency at two
     // CTAs per SM, so it takes the twin's grid (two per SM co-resident, measured: 53.8 -> 32.3 ms).
-    cudaError_t e = cudaFuncSetAttribute(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, true>,
+    cudaError_t e = cudaFuncSetAttribute(pw::d256::pass_a_d256<CS, MASK, true>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pw::d256::pass_a_smem<CS>());
     if (e != cudaSuccess) return e;
-    e = cluster_capacity(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, false>, CS, pw::d256::Geo<CS>::NT,
+    e = cluster_capacity(pw::d256::pass_a_d256<CS, MASK, false>, CS, pw::d256::Geo<CS>::NT,
                          pw::d256::pass_a_smem<CS>(), &grid);
     if (e != cudaSuccess) return e;
   }
-  return launch_clusters(pw::d256::pass_a_d256<CS, pw::SRC_GSM, MASK, true>, CS, pw::d256::Geo<CS>::NT,
+  return launch_clusters(pw::d256::pass_a_d256<CS, MASK, true>, CS, pw::d256::Geo<CS>::NT,
                          pw::d256::pass_a_smem<CS>(), &grid, s, vmap, a, x.Ein, x.mask, x.ap_ithr, x.err);
 }
 

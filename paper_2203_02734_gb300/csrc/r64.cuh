@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(NT, CTAS) pass_b_r64(PassBArgs p) {
   }
   auto prefetch = [&](int cd) {
     if (t == 0 && cd < N * N)
-      bulk_prefetch_l2(p.V + ((size_t)(cd / g) * g + cd % g) * N * N, (unsigned)(N * N * sizeof(float2)));
+      bulk_prefetch_l2(p.V + (size_t)cd * N * N, (unsigned)(N * N * sizeof(float2)));
   };
   prefetch(blockIdx.x);
   prefetch(blockIdx.x + gridDim.x);
