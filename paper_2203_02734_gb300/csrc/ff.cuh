@@ -1,9 +1,11 @@
 // ff.cuh -- pairs of floats: an unevaluated sum h + l, about 48 bits, for transforms that need more than FP32 and
 // would wait for the FP64 pipe (2 operations a clock and SM against 128 in FP32).
 //
-// Sums are Knuth's two-sum, products Dekker's with the error term from an FMA; the low parts are added in FP32 and
-// the pair renormalised.  The intrinsics keep the compiler from contracting a product and a sum into one FMA,
-// which would change the error terms.  The range is FP32's: below about 2^-102 the low part fades out.
+// Sums are Knuth's two-sum, products Dekker's with the error term from an FMA; the low parts are added in FP32.  The
+// pair is not renormalised: two-sums hold for any pair, over a transform the low part grows to some units of the
+// high part's last place, and its own rounding stays near 2^-46 of the largest value.  The intrinsics keep the
+// compiler from contracting a product and a sum into one FMA, which would change the error terms.  The range is
+// FP32's: below about 2^-102 the low part fades out.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -22,10 +24,6 @@ struct __align__(16) ff2 {
 };
 
 namespace ffx {
-__device__ __forceinline__ ff fast2(float h, float e) {  // |h| >= |e|
-  const float s = __fadd_rn(h, e);
-  return ff(s, __fsub_rn(e, __fsub_rn(s, h)));
-}
 __device__ __forceinline__ float err_of_sum(float a, float b, float s) {
   const float z = __fsub_rn(s, a);
   return __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
@@ -39,19 +37,19 @@ __device__ __forceinline__ ff dot(ff a, ff b, ff c, ff d) {
   e = __fmaf_rn(a.l, b.h, e);
   e = __fmaf_rn(c.h, d.l, e);
   e = __fmaf_rn(c.l, d.h, e);
-  return fast2(s, e);
+  return ff(s, e);
 }
 }  // namespace ffx
 
 __device__ __forceinline__ ff operator-(ff a) { return ff(-a.h, -a.l); }
 __device__ __forceinline__ ff operator+(ff a, ff b) {
   const float s = __fadd_rn(a.h, b.h);
-  return ffx::fast2(s, __fadd_rn(ffx::err_of_sum(a.h, b.h, s), __fadd_rn(a.l, b.l)));
+  return ff(s, __fadd_rn(ffx::err_of_sum(a.h, b.h, s), __fadd_rn(a.l, b.l)));
 }
 __device__ __forceinline__ ff operator-(ff a, ff b) { return a + (-b); }
 __device__ __forceinline__ ff operator*(ff a, ff b) {
   const float p = __fmul_rn(a.h, b.h);
-  return ffx::fast2(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
+  return ff(p, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.h, b.h, -p))));
 }
 
 // The names that the codelets of fft.cuh use.

@@ -254,7 +254,6 @@ PW_PLAN(48, 192, 16, 3)
 PW_PLAN(64, 256, 8, 8)
 PW_PLAN(96, 384, 8, 4, 3)
 PW_PLAN(128, 512, 16, 8)
-PW_PLAN(256, 256, 16, 16)   // single lines only (plane.cuh)
 #undef PW_PLAN
 
 template <int N, int I> struct StageInfo {

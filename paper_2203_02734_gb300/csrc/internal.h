@@ -34,7 +34,8 @@ struct PlaneArgs {
   float2* W;
   float* S;
   float A, scale, scale_A;  // scale_A = scale A, rounded once
-  float2* row;  // W(P1, .) or nullptr
+  pw::ff2* tw2;  // N = 256: room for N twiddles
+  float2* row;   // W(P1, .) or nullptr
   int iP, jP;
 };
 // ev: nullptr or three events around the two passes; err: flag of a bounded wait that gave up.

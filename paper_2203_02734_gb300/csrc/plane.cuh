@@ -11,7 +11,7 @@
 // and no corner turn: at N <= 128 a plane (a, d) lives in one SM's registers and its result rows
 // W(a', b', c', .) are final, so the whole propagation writes its 8 bytes a point once and reads the
 // tables from L2.  (The general path moves 24 bytes a point, 40 at N = 256.)
-//   table_kernel: N^2 columns of length N of each table, into the work buffer.
+//   table_kernel (table256_kernel): N^2 columns of length N of each table, into the work buffer.
 //   plane kernels (24 <= N <= 128; r64.cuh at N = 64, small.cuh with its own tables up to N = 16): one
 //   (b', c') per CTA iteration.
 //   N = 256: the rows (a, d) and the columns of a plane in two passes, 24 bytes a point.
@@ -19,6 +19,7 @@
 #include <cuda.h>
 #include <cstdint>
 
+#include "ff.cuh"
 #include "propagate.cuh"
 #include "r128.cuh"
 #include "r96.cuh"
@@ -94,6 +95,57 @@ __global__ void __launch_bounds__(tab_nt<N>()) table_kernel(TabArgs p) {
     float2* T = p.T + (size_t)a * N + d0;
     auto out = [=](int line, int c, float2 v) { T[(size_t)c * N * N + line] = cmul(__ldg(E + c), v); };
     table_lines<N, -1>(x, tw, gen, out);
+  }
+}
+
+// N = 256: the same on pairs of floats (ff.cuh), rounded once at the end.  A line of a table goes into 256 planes, and
+// most of a row W(P1, .) lies where the planes cancel: the rounding of the FP32 transforms took mu's error from 2.8e-7
+// (three passes) to 4.1e-7, here 2.6e-7 (S 1.1e-7, 1.3e-7, 0.9e-7).  16.65 ms a propagation against 16.28 ms with
+// FP32 tables, bound by FP32 issue; 4 to 16 columns a block and 128 to 512 threads within 0.07 ms of each other.
+constexpr int TAB_L256 = 16, TAB_NT256 = 256, TAB_P256 = TAB_L256 + 1;
+constexpr size_t table256_smem() { return (size_t)(256 * TAB_P256 + 256) * sizeof(ff2); }
+
+__global__ void __launch_bounds__(256) table256_tw_kernel(ff2* tw) {
+  double sn, cs;
+  sincospi(-2.0 * (double)threadIdx.x / 256.0, &sn, &cs);
+  tw[threadIdx.x] = make_c(ff(cs), ff(sn));
+}
+
+template <int SIGN, int NS = 1>
+__device__ __forceinline__ void table256_stages(ff2* x, const ff2* tw) {
+  if constexpr (NS < 256) {
+    auto ld = [x](int line, int pos) { return x[pos * TAB_P256 + line]; };
+    auto st = [x](int line, int pos, ff2 v) { x[pos * TAB_P256 + line] = v; };
+    line_stage<256, 4, NS, SIGN, TAB_L256, TAB_NT256>(tw, ld, SyncMid{}, st);
+    __syncthreads();
+    table256_stages<SIGN, 4 * NS>(x, tw);
+  }
+}
+
+__global__ void __launch_bounds__(TAB_NT256) table256_kernel(TabArgs p, const ff2* __restrict__ tw2) {
+  constexpr int N = 256;
+  extern __shared__ __align__(1024) float2 smem[];
+  ff2* x = reinterpret_cast<ff2*>(smem);
+  ff2* tw = x + N * TAB_P256;
+  tw[threadIdx.x] = tw2[threadIdx.x];
+  const int a = blockIdx.x / (N / TAB_L256), d0 = (blockIdx.x % (N / TAB_L256)) * TAB_L256;
+  const bool h = blockIdx.y == 0;
+  const ff A = ff(p.A);
+  for (int e = threadIdx.x; e < N * TAB_L256; e += TAB_NT256) {
+    const int line = e % TAB_L256, b = e / TAB_L256;  // b, or c of T
+    const float2 f = __ldg(p.F + (h ? a * N + b : b * N + d0 + line));
+    const ff g = h ? A * ff(__ldg(p.G + b * N + d0 + line)) : ff(__ldg(p.G + a * N + b));
+    x[b * TAB_P256 + line] = make_c(ff(f.x) * g, ff(h ? -f.y : f.y) * g);
+  }
+  __syncthreads();
+  if (h) table256_stages<+1>(x, tw);
+  else table256_stages<-1>(x, tw);
+  float2* out = (h ? p.H : p.T) + (size_t)a * N + d0;
+  for (int e = threadIdx.x; e < N * TAB_L256; e += TAB_NT256) {
+    const int line = e % TAB_L256, k = e / TAB_L256;
+    const float2 E = __ldg(p.Eout + k);
+    const ff2 v = cmul(x[k * TAB_P256 + line], make_c(ff(E.x), ff(h ? -E.y : E.y)));
+    out[(size_t)k * N * N + line] = make_float2((float)v.x, (float)v.y);
   }
 }
 

@@ -455,8 +455,8 @@ cudaError_t launch_planes256(const CUtensorMap& wmap, const PlaneArgs& q, int* e
   static int grid = 0;  // of the column kernel
   cudaError_t e;
   if (grid == 0) {
-    if ((e = cudaFuncSetAttribute(P::table_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)P::tab_smem<N>())) != cudaSuccess ||
+    if ((e = cudaFuncSetAttribute(P::table256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)P::table256_smem())) != cudaSuccess ||
         (e = cudaFuncSetAttribute(P::rows256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)P::rows256_smem())) != cudaSuccess ||
         (e = cudaFuncSetAttribute(P::cols256_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -466,7 +466,8 @@ cudaError_t launch_planes256(const CUtensorMap& wmap, const PlaneArgs& q, int* e
   }
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
   const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, q.A};
-  P::table_kernel<N><<<dim3(N * (N / P::tab_lines<N>()), 2), P::tab_nt<N>(), P::tab_smem<N>(), s>>>(ta);
+  P::table256_tw_kernel<<<1, N, 0, s>>>(q.tw2);
+  P::table256_kernel<<<dim3(N * (N / P::TAB_L256), 2), P::TAB_NT256, P::table256_smem(), s>>>(ta, q.tw2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, nullptr, 0, 0};
   P::rows256_kernel<<<N * (N / 16) * (N / P::ROWS_C), P::NT256, P::rows256_smem(), s>>>(a);
@@ -864,6 +865,7 @@ pw_status propagate_planes(pw_csd* h, double z) {
   q.S = h->S;
   q.A = (float)h->A;
   q.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
+  q.tw2 = reinterpret_cast<pw::ff2*>(h->gpart);  // N = 256: in the adjoint's scratch
   q.scale_A = (float)((h->d * h->d / lz) * (h->d * h->d / lz) * h->A);
   cudaError_t e = pwi::dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch (GSM source)");

@@ -15,7 +15,7 @@
 // rounding of the largest: in FP32 the relative error of S was 1e-3 where S is 1e-4 of its maximum (the 4D route,
 // whose errors average over N^2 terms, 1e-5), and some dim S came out negative.  So a batch runs on pairs of
 // floats (ff.cuh), which leaves the rounding of the outputs alone: 2.6e-8 of S in L2, 6e-8 at every point,
-// against 1.8e-7 and 6e-6 in FP32 on well-lit outputs.  192 instances of N = 64 to 128 take 0.69 ms; 0.26 ms in
+// against 1.8e-7 and 6e-6 in FP32 on well-lit outputs.  192 instances of N = 64 to 128 take 0.62 ms; 0.26 ms in
 // FP32, 2.62 ms in FP64.  The single call, for a host loop that waits for it, runs in FP64 (8 MFLOP at N = 96).
 //   k1: columns b, transform over a              -> X1[m][b]   (L x N)
 //   k2: rows m, transform over b; |P^|^2 back to v, times k(v), to b' -> Z1[m][b'];
@@ -64,10 +64,11 @@ __device__ __forceinline__ ff ldc(const ff* p) {
   return ff(v.x, v.y);
 }
 
-// Lines per block.  Batches (float pairs) fill the chip with instances, and four 16-byte lines fill the
-// 64-byte runs of the column accesses (polychromatic batch of 192: 1216 / 799 / 687 / 736 us with 1 / 2 / 4 / 8 lines).  FP64
-// calls are one instance: a line per block puts an SM's FP64 pipe behind each (N = 96: 16 lines a block left 6
-// to 12 blocks, 247 us a call; one line 74 us, with the radices below 55 us; two lines 58 us).
+// Lines per block.  Batches (float pairs) fill the chip with instances, and four 16-byte lines make 64-byte runs of
+// the column accesses (polychromatic batch of 192, pairs renormalised after every operation: 1216 / 799 / 687 /
+// 736 us with 1 / 2 / 4 / 8 lines; 621 us without that).  FP64 calls are one instance: a line per block puts an SM's
+// FP64 pipe behind each (N = 96: 16 lines a block left 6 to 12 blocks, 247 us a call; one line 74 us, with the
+// radices below 55 us; two lines 58 us).
 template <int N, class C> __host__ __device__ constexpr int lines() { return std::is_same<C, ff2>::value ? 4 : 1; }
 template <int N, class C> __host__ __device__ constexpr int threads() {
   return N >= 64 ? 256 : 128;

@@ -143,3 +143,28 @@ def test_handle_point_by_point(N, far):
         pw.pw_gsm_s_mu(c.h, 0.3, far, *ref[2], S.data_ptr(), mu.data_ptr())
         _check(S, mu, ref)
     c.close()
+
+
+# N = 256: the planes' S and mu after the propagation are as accurate as the three passes that they replaced, whose
+# relative L2 errors over these sources were 1.2e-7 and 1.9e-7 in the mean; 1.3e-7 and 2.2e-7 allow for the library's
+# rounding elsewhere.
+@pytest.mark.gpu
+def test_planes_n256_are_as_accurate_as_the_passes():
+    import torch
+    import paper_2203_02734_gb300 as pw
+    N, P1, eS, emu = 256, (256 // 2 - 256 // 8, 256 // 2 + 1), [], []
+    c = pw.CSD(N, D, LAM)
+    for i, (z, ap, m) in enumerate([(0.5, 0.0, WL.phase_screen(N, seed=1)), (0.3, 0.4 * N * D, None), (1.1, 0.0, WL.amplitude_mask(N, seed=3))]):
+        args = (5 * D, (0.7 + 0.1 * i) * D, 0.6 + 0.3 * i)
+        m = None if m is None else WL.to_c64(m)
+        c.reset(D)
+        c.source_gsm(*args)
+        c.source_aperture(ap)
+        if m is not None:
+            c.source_mask(torch.from_numpy(m).cuda())
+        c.propagate_fresnel(z)
+        S, mu = exact(N, LAM, z, False, *args, ap, 0.0, m, P1)
+        eS.append(rel(c.spectral_density().cpu().numpy().astype(np.float64), S))
+        emu.append(rel(c.degree_of_coherence(*P1).cpu().numpy().astype(complex), mu))
+    c.close()
+    assert np.mean(eS) < 1.3e-7 and np.mean(emu) < 2.2e-7, (eS, emu)
