@@ -117,7 +117,7 @@ struct pw_batch {
   cudaStream_t stream;
   std::vector<pw::batch::Inst> inst;
   std::vector<int> stalled;  // instances whose pass-A items are left out (failure-detection test)
-  std::vector<float> scales;   // scale times amplitude of every instance
+  std::vector<double> A, scale;  // amplitude and scale of every instance
   std::vector<double> dx_out;  // output sampling of every instance (lambda z / (N dxi))
   int nitems;
   long long wait_cycles;
@@ -298,7 +298,8 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     const double lz = q.lambda_m * q.z_m;
     const double s2 = (q.dxi_m * q.dxi_m / lz) * (q.dxi_m * q.dxi_m / lz);
     d.scale = (float)s2;
-    b->scales.push_back((float)(s2 * q.amplitude));
+    b->scale.push_back(s2);
+    b->A.push_back(q.amplitude);
     float2* F = reinterpret_cast<float2*>(b->base + off);
     off = align256(off + NN * sizeof(float2));
     float* G = reinterpret_cast<float*>(b->base + off);
@@ -353,6 +354,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     ta.Kout = t.Kout;
     ta.gs = t.gs;
     ta.gm = t.gm;
+    ta.amp = std::sqrt(std::sqrt(std::fabs(q.amplitude)));
     ta.tw = reinterpret_cast<pwi::Wide*>(F);
     ta.P1 = ta.tw + 2 * N;
     ta.Eout = ta.P1 + N;
@@ -361,7 +363,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     si.N = N;
     si.iP = q.iP;
     si.jP = q.jP;
-    si.factor = s2 * q.amplitude / (4.0 * (double)NN);
+    si.factor = (q.amplitude < 0.0 ? -s2 : s2) / (4.0 * (double)NN);
     si.tw = ta.tw;
     si.P1 = ta.P1;
     si.Eout = ta.Eout;
@@ -449,9 +451,8 @@ pw_status pw_batch_run(pw_batch* b) {
       q.work = d.V;
       q.W = d.W;
       q.S = d.S;
-      q.A = d.A;
-      q.scale = d.scale;
-      q.scale_A = b->scales[i];
+      q.A = b->A[i];
+      q.scale = b->scale[i];
       q.row = d.row;
       q.iP = d.iP;
       q.jP = d.jP;

@@ -33,7 +33,7 @@ struct PlaneArgs {
   float2* work;  // 2 N^3 table values
   float2* W;
   float* S;
-  float A, scale, scale_A;  // scale_A = scale A, rounded once
+  double A, scale;
   pw::ff2* tw2;  // N = 256: room for N twiddles
   float2* row;   // W(P1, .) or nullptr
   int iP, jP;

@@ -219,7 +219,8 @@ extern "C" pw_status pw_propagate_gsm_fresnel_noalloc(int N, double dxi_m, doubl
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const double lz = lam * z_m;
   const double s2 = (d * d / lz) * (d * d / lz);
-  const pw::small::Args q{F, G, tw, Eout, reinterpret_cast<float2*>(dev_W_out), dev_S_out, (float)(s2 * amplitude), nullptr, 0, 0};
+  const pw::small::Scale sA(s2, amplitude);
+  const pw::small::Args q{F, G, tw, Eout, reinterpret_cast<float2*>(dev_W_out), dev_S_out, sA.scale, sA.pow2, nullptr, 0, 0};
   switch (N) {
     case 2: return run_small<2>(t, q, s);
     case 4: return run_small<4>(t, q, s);

@@ -403,7 +403,8 @@ template <int N>
 cudaError_t launch_small(const PlaneArgs& q, cudaStream_t s, cudaEvent_t* ev) {
   cudaError_t e;
   if (ev && ((e = cudaEventRecord(ev[0], s)) != cudaSuccess || (e = cudaEventRecord(ev[1], s)) != cudaSuccess)) return e;
-  const pw::small::Args a{q.F, q.G, q.tw, q.Eout, q.W, q.S, q.scale_A, q.row, q.iP, q.jP};
+  const pw::small::Scale sA(q.scale, q.A);
+  const pw::small::Args a{q.F, q.G, q.tw, q.Eout, q.W, q.S, sA.scale, sA.pow2, q.row, q.iP, q.jP};
   if ((e = pw::small::launch<N>(a, s)) != cudaSuccess) return e;
   return ev ? cudaEventRecord(ev[2], s) : cudaSuccess;
 }
@@ -430,11 +431,11 @@ cudaError_t launch_planes(const CUtensorMap& wmap, const PlaneArgs& q, int* err,
       return e;
   }
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, q.A};
+  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, (float)q.A};
   P::table_kernel<N><<<dim3(N * (N / P::tab_lines<N>()), 2), P::tab_nt<N>(), P::tab_smem<N>(), s>>>(ta);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
-  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, q.row, q.iP, q.jP};
+  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, (float)q.scale, q.row, q.iP, q.jP};
   if constexpr (N == 128) {
     kernel<<<grid, nt, smem, s>>>(a, err);
     P::diag_row_kernel<<<N * N / 256, 256, 0, s>>>(a, N);
@@ -465,11 +466,11 @@ cudaError_t launch_planes256(const CUtensorMap& wmap, const PlaneArgs& q, int* e
       return e;
   }
   if (ev && (e = cudaEventRecord(ev[0], s)) != cudaSuccess) return e;
-  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, q.A};
+  const P::TabArgs ta{q.F, q.G, q.tw, q.Eout, q.work, q.work + N3, (float)q.A};
   P::table256_tw_kernel<<<1, N, 0, s>>>(q.tw2);
   P::table256_kernel<<<dim3(N * (N / P::TAB_L256), 2), P::TAB_NT256, P::table256_smem(), s>>>(ta, q.tw2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, q.scale, nullptr, 0, 0};
+  const P::Args a{ta.H, ta.T, q.tw, q.Eout, q.W, q.S, (float)q.scale, nullptr, 0, 0};
   P::rows256_kernel<<<N * (N / 16) * (N / P::ROWS_C), P::NT256, P::rows256_smem(), s>>>(a);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
@@ -863,10 +864,9 @@ pw_status propagate_planes(pw_csd* h, double z) {
   q.work = reinterpret_cast<float2*>(h->work);
   q.W = reinterpret_cast<float2*>(h->W);
   q.S = h->S;
-  q.A = (float)h->A;
-  q.scale = (float)((h->d * h->d / lz) * (h->d * h->d / lz));
+  q.A = h->A;
+  q.scale = (h->d * h->d / lz) * (h->d * h->d / lz);
   q.tw2 = reinterpret_cast<pw::ff2*>(h->gpart);  // N = 256: in the adjoint's scratch
-  q.scale_A = (float)((h->d * h->d / lz) * (h->d * h->d / lz) * h->A);
   cudaError_t e = pwi::dispatch_planes(h->N, h->wmap, q, h->err, h->stream, ev);
   if (e != cudaSuccess) return cuda_fail(e, "propagation kernel launch (GSM source)");
   to_output_plane(h, lz / (h->N * h->d), true);
@@ -983,6 +983,7 @@ pw_status gsm_s_mu(pw_csd* h, double z, bool farfield, int iP, int jP, float* S,
   t.Kout = dx * dx / (2.0 * lz);
   t.gs = d * d / (4.0 * h->sigma_S * h->sigma_S);
   t.gm = d * d / (2.0 * h->sigma_mu * h->sigma_mu);
+  t.amp = 1.0;
   t.tw = w + (size_t)6 * N * N;
   t.P1 = t.tw + 2 * N;
   t.Eout = t.P1 + N;

@@ -10,6 +10,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "fft.cuh"
 
 namespace pw {
@@ -24,9 +26,20 @@ struct Args {
   const float2* Eout;  // N output factors
   float2* W;
   float* S;
-  float scale;  // s A
+  float scale, pow2;  // s A = scale pow2
   float2* row;  // optional: row[x] = W(P1, x), P1 = (iP, jP)
   int iP, jP;
+};
+
+// The scale s A in two factors: a power of two that goes to the source without rounding, so that a large A meets weak
+// masks there and not after their product, and the rest, rounded once.
+struct Scale {
+  float scale, pow2;
+  Scale(double s, double A) {
+    int k = 0;
+    scale = (float)(s * std::frexp(A, &k));
+    pow2 = std::ldexp(1.0f, k);
+  }
 };
 
 template <int N>
@@ -41,7 +54,7 @@ __global__ void __launch_bounds__(N * N) kernel(Args p) {
   const float2 e = cmul(cconj(p.Eout[bp]), p.Eout[cp]);  // of H T
   const float2 eo = cmul(cconj(p.Eout[i]), p.Eout[j]);   // of (a', d')
   __syncthreads();
-  fb[t] = cmul(cconj(f), cconj(tw[j * bp % N]));  // (a, b) = (i, j)
+  fb[t] = cmul(cscale(cconj(f), p.pow2), cconj(tw[j * bp % N]));  // (a, b) = (i, j)
   fc[t] = cmul(f, tw[i * cp % N]);                // (c, d) = (i, j)
   __syncthreads();
   // Sums in four shares: as one chain each, they took the error of W from 1.55e-7 (general passes) to 1.82e-7 at

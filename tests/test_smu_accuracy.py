@@ -168,3 +168,43 @@ def test_planes_n256_are_as_accurate_as_the_passes():
         emu.append(rel(c.degree_of_coherence(*P1).cpu().numpy().astype(complex), mu))
     c.close()
     assert np.mean(eS) < 1.3e-7 and np.mean(emu) < 2.2e-7, (eS, emu)
+
+
+# A strong source behind weak masks: A |m|^2 = 1 with A = 2^126 and |m| = 2^-63 gives what A = 1 and |m| = 1 give (powers
+# of two round nothing), since products are formed where the range of FP32 holds them.
+@pytest.mark.gpu
+@pytest.mark.parametrize("N", [16, 32, 64, 96, 128])
+@pytest.mark.parametrize("keep", [False, True])
+def test_range_of_amplitude_and_mask(N, keep):
+    import torch
+    import paper_2203_02734_gb300 as pw
+    m = torch.from_numpy(WL.to_c64(WL.phase_screen(N, seed=7))).cuda()
+    P1, out = (N // 2, N // 2 - 1), []
+    for A, w in [(1.0, 1.0), (2.0 ** 126, 2.0 ** -63)]:
+        S = torch.empty(N, N, device="cuda")
+        mu = torch.empty(N, N, dtype=torch.complex64, device="cuda")
+        W = torch.empty((N,) * 4 if keep else (1,), dtype=torch.complex64, device="cuda")
+        mask = m * w
+        q = pw.pw_instance()
+        q.N, q.dxi_m, q.lambda_m, q.z_m, q.sigma_S_m, q.sigma_mu_m, q.amplitude = N, D, LAM, 0.3, 5 * D, 1.5 * D, A
+        (q.iP, q.jP), q.dev_S, q.dev_mu, q.dev_mask = P1, S.data_ptr(), mu.data_ptr(), mask.data_ptr()
+        if keep:
+            q.dev_W = W.data_ptr()
+        nb = pw.pw_batch_workspace_bytes([q], 1)
+        ws = torch.empty(nb, dtype=torch.uint8, device="cuda")
+        b = pw.pw_batch_create([q], 1, ws.data_ptr(), nb, torch.cuda.current_stream().cuda_stream)
+        pw.pw_batch_set_mode(b, pw.PW_BATCH_SEQUENCED)
+        pw.pw_batch_run(b)
+        pw.pw_batch_check(b)
+        pw.pw_batch_destroy(b)
+        c = pw.CSD(N, D, LAM)
+        c.source_gsm(5 * D, 1.5 * D, A)
+        c.source_mask(mask)
+        Sh, muh = torch.empty_like(S), torch.empty_like(mu)
+        pw.pw_gsm_s_mu(c.h, 0.3, False, *P1, Sh.data_ptr(), muh.data_ptr())
+        c.propagate_fresnel(0.3)
+        out.append((S, mu, W, Sh, muh, c.W, c.spectral_density()))
+        c.close()
+    for x, y in zip(*out):
+        if x.numel() > 1:
+            assert float(torch.linalg.vector_norm(x - y)) <= 3e-7 * float(torch.linalg.vector_norm(x))
