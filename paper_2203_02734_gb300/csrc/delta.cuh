@@ -74,7 +74,8 @@ __global__ void tables_kernel(TabArgs p, int G) {
       w.y = -w.y;
       float dv = __ldg(p.d + a * N + b);
       if (a * N + b == xp) dv -= fix;
-      s = cadd(s, cscale(w, p.A * dv * (f.x * f.x + f.y * f.y)));
+      const float ad = p.A * dv;  // |F|^2 alone would underflow behind weak masks
+      s = cadd(s, cscale(w, fmaf(ad * f.x, f.x, ad * f.y * f.y)));
     } else {
       s = cadd(s, cmul(w, cmul(f, __ldg(p.cross + a * N + b))));
     }

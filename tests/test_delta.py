@@ -51,3 +51,23 @@ def test_diagonal_against_the_general_passes(N, farfield, masked):
         c.close()
     assert rel(out[0][0], out[1][0]) < 2e-6
     assert rel(out[0][1], out[1][1]) < 2e-6
+
+
+# A strong source behind weak masks: 2^120 behind 2^-70 is 2^-20 behind 1 (powers of two round nothing).
+@pytest.mark.gpu
+@pytest.mark.parametrize("N", [16, 96])
+def test_range_of_weight_and_mask(N):
+    import torch
+    import paper_2203_02734_gb300 as pw
+    d = torch.rand(N, N, device="cuda", generator=torch.Generator(device="cuda").manual_seed(N))
+    m = torch.from_numpy(WL.to_c64(WL.amplitude_mask(N, seed=2))).cuda()
+    out = []
+    for A, w in [(2.0 ** -20, 1.0), (2.0 ** 120, 2.0 ** -70)]:
+        c = pw.CSD(N, D, LAM)
+        pw.pw_source_diagonal(c.h, d.data_ptr(), A)
+        c.source_mask(m * w)
+        c.propagate_fresnel(0.3)
+        out.append((c.W, c.spectral_density()))
+        c.close()
+    for x, y in zip(*out):
+        assert float(torch.linalg.vector_norm(x - y)) <= 3e-7 * float(torch.linalg.vector_norm(x))
