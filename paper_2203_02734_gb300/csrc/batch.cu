@@ -354,7 +354,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     ta.Kout = t.Kout;
     ta.gs = t.gs;
     ta.gm = t.gm;
-    ta.amp = std::sqrt(std::sqrt(std::fabs(q.amplitude)));
+    ta.amp = std::sqrt(std::sqrt(s2 * std::fabs(q.amplitude) / (4.0 * (double)NN)));
     ta.tw = reinterpret_cast<pwi::Wide*>(F);
     ta.P1 = ta.tw + 2 * N;
     ta.Eout = ta.P1 + N;
@@ -363,7 +363,7 @@ pw_status pw_batch_create(pw_batch** out, const pw_instance* in, int n, int pool
     si.N = N;
     si.iP = q.iP;
     si.jP = q.jP;
-    si.factor = (q.amplitude < 0.0 ? -s2 : s2) / (4.0 * (double)NN);
+    si.factor = q.amplitude < 0.0 ? -1.0 : 1.0;
     si.tw = ta.tw;
     si.P1 = ta.P1;
     si.Eout = ta.Eout;

@@ -37,8 +37,9 @@ struct Scale {
   float scale, pow2;
   Scale(double s, double A) {
     int k = 0;
-    scale = (float)(s * std::frexp(A, &k));
-    pow2 = std::ldexp(1.0f, k);
+    const double m = std::frexp(A, &k);  // A = 2 m 2^(k - 1): the power of any finite float is one
+    scale = (float)(s * 2.0 * m);
+    pow2 = std::ldexp(1.0f, k - 1);
   }
 };
 

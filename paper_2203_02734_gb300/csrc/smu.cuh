@@ -41,7 +41,7 @@ struct Inst {
   using R = real_t<C>;
   int N, iP, jP;
   int chunk;            // launch round: instances of one round have scratch of their own
-  R factor;             // s A / L^2, without the power of A that P1 carries
+  R factor;             // s A / L^2 (float pairs: its sign, the rest is in P1)
   const C* tw;          // L twiddles exp(-2 pi i m / L)
   const C* P1;          // N: Ein(i) h(i)
   const C* Eout;        // N
@@ -299,8 +299,8 @@ struct TabArgs {
   int N;
   double Kin, Kout;  // turns per n^2 of the input factor (propagator, lens) and of the output propagator
   double gs, gm;     // d^2/(4 sigma_S^2), d^2/(2 sigma_mu^2)
-  double amp;        // factor of P1: |A|^(1/4) puts |A| into |P^|^2 and P R, so that FP32's range has to hold no more
-                     // than the product of the source and its masks
+  double amp;        // factor of P1: with (s |A| / L^2)^(1/4) the sums between are of the size of S, whatever A and
+                     // the masks are by themselves (float pairs have FP32's range; FP64: 1)
   C *tw, *P1, *Eout;
   real_t<C>* k;
 };
