@@ -36,9 +36,9 @@ class _Model:
     def meet(self, other):
         """Neither the caller's stream nor the handle's runs on before the other has come to this point (the
         tensors of a call are the caller's stream's, the handle's stream reads and writes them)."""
-        if other is not None:
-            other.wait_stream(self.csd.stream)
+        if other is not None:  # in this order also under capture of the caller's stream
             self.csd.stream.wait_stream(other)
+            other.wait_stream(self.csd.stream)
 
     def outputs(self):
         """New S and mu tensors (they belong to the caller's graph)."""

@@ -62,3 +62,26 @@ def test_other_stream_gives_the_same(kind, direct):
         for r, o in zip(ref, out):
             assert torch.equal(torch.view_as_real(r) if r.is_complex() else r, torch.view_as_real(o) if o.is_complex() else o)
     model.close()
+
+
+def test_capture_on_another_stream():
+    import torch
+    from paper_2203_02734_gb300.autograd import GSMPropagation
+    N, a = 32, torch.cuda.Stream()
+    x = _inputs("gsm", N, torch)
+    with torch.cuda.stream(a):
+        model = GSMPropagation(N, D, LAM, 0.5)
+    torch.cuda.synchronize()
+    with torch.no_grad():
+        ref = [t.clone() for t in model(5 * D, 1.5 * D, 1.2, x)]
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            out = model(5 * D, 1.5 * D, 1.2, x)
+    for t in out:
+        t.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for r, o in zip(ref, out):
+        assert torch.equal(torch.view_as_real(r) if r.is_complex() else r, torch.view_as_real(o) if o.is_complex() else o)
+    model.close()
