@@ -408,12 +408,12 @@ def measure(cfg, args, rank, world, dist):
             step()
 
     # tables, plane tables, planes, S kernel, mu kernel; N = 128: + diagonal and row; N = 256: rows and
-    # columns in place of planes; cluster engine: tables, pass A, pass B, S, mu.  Padded: FP32 tables,
+    # columns in place of planes, + the plane tables' twiddles; cluster engine: tables, pass A, pass B, S, mu.  Padded: FP32 tables,
     # source, four contractions, S, mu; tensor cores tables, two matrix splits, GSM tables and their
     # scale, two table and two N^4 contractions, S, mu
     tc = args.dft != "fp32" and N <= 256
     launches_per_step = ((12 if tc else 9) if cfg.get("Nz") else
-                         5 if N < 128 or args.dft == "tc_bf16x3" else 6)
+                         5 if N < 128 or args.dft == "tc_bf16x3" else 7 if N == 256 else 6)
     max_blocks = 400
     pw.pw_csd_enable_timing(h, max(args.steps * max_blocks, args.warmup, 1))
     for _ in range(args.warmup):
@@ -611,8 +611,8 @@ def run_batch(args):
     pw.pw_batch_check(b)
     ms = e0.elapsed_time(e1) / args.steps
     pts = sum(sp["N"] ** 4 for sp in specs)
-    # 14 N^2 complex values between the four kernels of an instance (mostly in L2), S and mu
-    smu_bytes = sum(128 * sp["N"] ** 2 for sp in specs)
+    # 14 N^2 complex values of 16 bytes between the four kernels of an instance (mostly in L2), S and mu
+    smu_bytes = sum(240 * sp["N"] ** 2 for sp in specs)
     launches = 1 + 4 * len(CFG["Ns"])  # tables, then k1-k4 of every grid size (one round of scratch)
     # plain path: the same instances through the single-instance calls, one after the other
     maxN = max(sp["N"] for sp in specs)
@@ -655,7 +655,7 @@ def run_batch(args):
                        "Ns": list(CFG["Ns"]), "zs": list(CFG["zs"]), "n_freq": CFG["n_freq"],
                        "outputs": "S and mu per instance", "pool": pool, "chunk": chunk,
                        "launch": "autotuned mode: %s, replayed from a CUDA graph" % mode},
-            "roofline": {"bound": "latency", "kernel": "smu::k1-k4: S and mu from (2N)^2 transforms, no N^4 array",
+            "roofline": {"bound": "issue", "kernel": "smu::k1-k4: S and mu from (2N)^2 transforms on float pairs, no N^4 array",
                          "achieved": smu_bytes / (ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                          "frac": smu_bytes / (ms * 1e-3) / 1e9 / peak, "peak_source": peak_src, "traffic": None,
                          "algorithmic_bytes": smu_bytes},

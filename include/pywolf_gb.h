@@ -291,7 +291,8 @@ pw_status pw_csd_pass_times3(pw_csd* h, double* ms_first, double* ms_second, dou
  * it yields S (Eq. defS) and mu(P1, .) (Eq. defMu) of its output plane, and the whole propagated
  * CSDA when dev_W is given.  Instances without dev_W need no CSDA at all: S is the transform of the
  * correlation of the source field times its coherence and mu's row two convolutions, O(N^2 log N)
- * work each, all of them together in a few launches in either mode.  For the instances with dev_W
+ * work each, on pairs of floats (the error of S is the rounding of its FP32 values and at most 1e-12 of its
+ * maximum), all of them together in a few launches in either mode.  For the instances with dev_W
  * there are two execution modes (pw_batch_set_mode, chosen by pw_batch_autotune):
  *   PW_BATCH_PERSISTENT: all of them in one persistent launch that walks a work list of
  *     (instance, pass, slice chunk) items; pass-B work of an instance starts after its pass-A
@@ -329,9 +330,10 @@ size_t pw_batch_workspace_bytes(const pw_instance* inst, int n, int pool);
 pw_status pw_batch_create(pw_batch** out, const pw_instance* inst, int n, int pool, void* dev_workspace,
                           size_t workspace_bytes, void* stream);
 
-/* Enqueue one batched run on the batch's stream: FP64 tables of every instance, then (persistent
- * mode) counter reset + the persistent launch or (sequenced mode) two pass launches per
- * instance, then mu.  Asynchronous; no allocation; capturable in a CUDA graph. */
+/* Enqueue one batched run on the batch's stream.  Instances without dev_W: their FP64 tables, then four
+ * launches per grid size that leave S and mu.  Instances with dev_W: their FP64 tables, then (persistent
+ * mode) counter reset + the persistent launch or (sequenced mode) the launches of one propagation after the
+ * other, then mu.  Asynchronous; no allocation; capturable in a CUDA graph. */
 pw_status pw_batch_run(pw_batch* b);
 
 /* Synchronise and report PW_ETIMEOUT if a bounded dependency wait of a run gave up since the

@@ -2,7 +2,7 @@
 // callers that cannot allocate device memory: applications whose framework reserves all
 // device memory in its own pool and forbids libraries to call the CUDA allocator, and
 // latency-critical loops that cannot afford the implicit device synchronisation of
-// cudaMalloc / cudaFree.  The half-transformed CSDA and the small tables live in one
+// cudaMalloc / cudaFree.  The small tables (and above N = 16 the half-transformed CSDA) live in one
 // file-scope device array of fixed size instead of handle memory and a work buffer.
 #include <cuda.h>
 #include <cuda_runtime.h>
