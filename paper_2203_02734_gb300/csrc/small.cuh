@@ -54,12 +54,12 @@ __global__ void __launch_bounds__(N * N) kernel(Args p) {
   const float2 f = p.F[t];
   const float2 e = cmul(cconj(p.Eout[bp]), p.Eout[cp]);  // of H T
   const float2 eo = cmul(cconj(p.Eout[i]), p.Eout[j]);   // of (a', d')
-  __syncthreads();
-  fb[t] = cmul(cscale(cconj(f), p.pow2), cconj(tw[j * bp % N]));  // (a, b) = (i, j)
-  fc[t] = cmul(f, tw[i * cp % N]);                // (c, d) = (i, j)
+  fb[t] = cmul(cscale(cconj(f), p.pow2), cconj(p.tw[j * bp % N]));  // (a, b) = (i, j)
+  fc[t] = cmul(f, p.tw[i * cp % N]);                                // (c, d) = (i, j)
   __syncthreads();
   // Sums in four shares: as one chain each, they took the error of W from 1.55e-7 (general passes) to 1.82e-7 at
-  // N = 16; in shares, and with A in the scale, 1.53e-7 in the same time.
+  // N = 16; in shares, and with A in the scale, 1.53e-7.  (Their time is made up for by a barrier less, with the first
+  // twiddles from memory, and by indices i a mod N in place of running ones: two launches 7.05 -> 6.96 us in a graph.)
   auto total = [](const float2 (&v)[4]) { return cadd(cadd(v[0], v[1]), cadd(v[2], v[3])); };
   auto add = [](float2& s, float2 v, float2 w) {  // s += v w
     s = make_float2(fmaf(v.x, w.x, fmaf(-v.y, w.y, s.x)), fmaf(v.x, w.y, fmaf(v.y, w.x, s.y)));
@@ -77,23 +77,13 @@ __global__ void __launch_bounds__(N * N) kernel(Args p) {
   x[t] = cmul(cmul(total(h), total(u)), e);
   __syncthreads();
   float2 r[4] = {};
-  int m = 0;  // d d' mod N
 #pragma unroll
-  for (int d = 0; d < N; ++d) {
-    add(r[d & 3], x[i * N + d], tw[m]);
-    m += j;
-    m -= m >= N ? N : 0;
-  }
+  for (int d = 0; d < N; ++d) add(r[d & 3], x[i * N + d], tw[j * d % N]);
   y[t] = total(r);  // (a, d')
   __syncthreads();
   float2 q[4] = {};
-  m = 0;  // a a' mod N
 #pragma unroll
-  for (int a = 0; a < N; ++a) {
-    add(q[a & 3], y[a * N + j], cconj(tw[m]));
-    m += i;
-    m -= m >= N ? N : 0;
-  }
+  for (int a = 0; a < N; ++a) add(q[a & 3], y[a * N + j], cconj(tw[i * a % N]));
   const float2 s = total(q);
   const float2 w = cscale(cmul(s, eo), p.scale);  // W(a' = i, b', c', d' = j)
   p.W[(size_t)((i * N + bp) * N + cp) * N + j] = w;
